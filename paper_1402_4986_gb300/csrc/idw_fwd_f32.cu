@@ -2,8 +2,10 @@
 // for one problem or a batch of independent problems in one launch.
 //
 // Pipeline (one call): coordinate range scan -> staging -> persistent
-// all-pairs sweep -> combine (FP64 division) with the FP64 slow path of
-// flagged queries.
+// all-pairs sweep -> combine (FP64 division) -> for problems of more than
+// 2048 points, the search for the exact hits among the flagged queries and
+// the results of those queries (smaller problems' flagged queries are
+// finished by the combine).
 //
 // The sweep is the paper's tiled kernel (Sec. 4.2: the data are read once
 // per block of prediction points, tile by tile) rebuilt for sm_103a:
@@ -397,18 +399,43 @@ __global__ void __launch_bounds__(Var<V>::NT, 512 / Var<V>::NT)
 // every warp's loads are coalesced across its 32 queries, and the 8 partial
 // sums are added in a fixed order, so the result is deterministic.  The
 // CTA's flagged queries are then redone one after another by all 256
-// threads (a query's slow path reads all n points).  Block 0 finally clears
+// threads when their problem is small; a query's slow path reads all n
+// points, so those of a larger problem are listed for the two kernels after
+// this one, which spread each search over the GPU.  Block 0 finally clears
 // the per-problem range words the range scan and staging of this call used,
 // so the next call (or graph replay) starts from zero without a memset.
 constexpr int kCombineQueries = 32;
 constexpr int kCombineLanes = 8;
 static_assert(kCombineQueries * kCombineLanes == kSlowThreads, "the combine CTA runs the slow path");
 
+// Flagged queries of problems up to this many points stay with their CTA:
+// one FP64 recomputation of 2048 points keeps one SM's FP64 pipe busy for
+// about 14 us (100,003 points: 690 us), and the two kernels that share larger
+// ones out cost about 3 us a call.
+constexpr int kSlowInlinePoints = 2048;
+
+// A listed query: problem, query, the lowest coincident data index found so
+// far (INT_MAX: none), and how many slices of its FP64 sums are done.
+struct SlowItem {
+  int32_t problem, query, hit;
+  unsigned done;
+};
+static_assert(sizeof(SlowItem) == 16, "slow list record");
+
+// The list, then the slices' FP64 sums, in the staged tiles' memory, which
+// nothing reads after the sweep.  A list of c queries is summed in at most
+// max(c, grid) slices, so `cap` queries fit; further ones stay with their CTA.
+struct SlowList {
+  SlowItem* item;
+  SlowSums* part;
+  unsigned cap;
+};
+
 template <int CAP, int QT>
 __global__ void __launch_bounds__(kCombineQueries * kCombineLanes)
     combine_kernel(const __grid_constant__ Table<CAP> t, const float4* __restrict__ partial,
                    int64_t total_slots, int64_t units, int grid, const float* __restrict__ scales,
-                   double p, Control* __restrict__ ctrl) {
+                   double p, Control* __restrict__ ctrl, const SlowList slow) {
   __shared__ float4 red[kCombineLanes][kCombineQueries];
   __shared__ int2 flagged[kCombineQueries];
   __shared__ int nflagged;
@@ -456,7 +483,11 @@ __global__ void __launch_bounds__(kCombineQueries * kCombineLanes)
     const double s0 = double(h0) + double(l0), s1 = double(h1) + double(l1);
     if (!(s0 > kTinySumPerPoint * double(I.n)) || !isfinite(s0) || !isfinite(s1) ||
         (p >= 2.0 && s0 > kHugeSumPow2Up)) {
-      flagged[atomicAdd(&nflagged, 1)] = make_int2(k, static_cast<int>(j));
+      const unsigned slot = I.n > kSlowInlinePoints ? atomicAdd(&ctrl->flagged, 1u) : slow.cap;
+      if (slot < slow.cap)
+        slow.item[slot] = SlowItem{k, static_cast<int32_t>(j), INT_MAX, 0u};
+      else
+        flagged[atomicAdd(&nflagged, 1)] = make_int2(k, static_cast<int>(j));
     } else {
       I.out[j] = static_cast<float>(s1 / s0);
       // Weights were computed on coordinates scaled by s: w = s^-p w_true.
@@ -476,6 +507,144 @@ __global__ void __launch_bounds__(kCombineQueries * kCombineLanes)
   }
   if (blockIdx.x == 0)
     for (int c = threadIdx.x; c < t.count; c += blockDim.x) ctrl->maxbits[c] = 0u;
+}
+
+// Exact hits of the listed queries.  A work item is a group of up to 32
+// listed queries and one of S equal slices of their problem's points, S
+// chosen so that the items fill the grid: every point is read once per group
+// and compared with the group's queries from shared memory, and the lowest
+// coincident index is kept with an atomic minimum.
+constexpr int kSlowGroup = 32;
+
+template <int CAP>
+__global__ void __launch_bounds__(kSlowThreads)
+    slow_search_kernel(const __grid_constant__ Table<CAP> t, const Control* __restrict__ ctrl,
+                       const SlowList slow) {
+  __shared__ float2 q[kSlowGroup];
+  __shared__ int prob[kSlowGroup];
+  pdl_trigger();
+  pdl_wait();
+  const int64_t count = min(ctrl->flagged, slow.cap);
+  const int64_t groups = (count + kSlowGroup - 1) / kSlowGroup;
+  if (groups == 0) return;
+  const int64_t slices = max(int64_t(1), gridDim.x / groups);
+  for (int64_t w = blockIdx.x; w < groups * slices; w += gridDim.x) {
+    const int64_t e0 = w / slices * kSlowGroup, sl = w % slices;
+    const int ne = static_cast<int>(min(int64_t(kSlowGroup), count - e0));
+    __syncthreads();  // the previous item's group is no longer read
+    if (threadIdx.x < ne) {
+      const SlowItem it = slow.item[e0 + threadIdx.x];
+      const float* p = t.inst[it.problem].queries + 2 * int64_t(it.query);
+      q[threadIdx.x] = make_float2(p[0], p[1]);
+      prob[threadIdx.x] = it.problem;
+    }
+    __syncthreads();
+    for (int a = 0; a < ne;) {  // runs of the same problem (uniform across the CTA)
+      int b = a + 1;
+      while (b < ne && prob[b] == prob[a]) ++b;
+      const Instance& I = t.inst[prob[a]];
+      slow_scan(I.data, sl * I.n / slices, (sl + 1) * I.n / slices,
+                [&](int64_t i, float x, float y) {
+                  for (int e = a; e < b; ++e)
+                    if (q[e].x == x && q[e].y == y)
+                      atomicMin(&slow.item[e0 + e].hit, static_cast<int32_t>(i));
+                  return false;
+                });
+      a = b;
+    }
+  }
+}
+
+// Results of the listed queries: a hit's z, or Eq. 1 in FP64.  A query
+// without a hit is one whose FP32 sums left FP32's range; among them are the
+// queries that shared a reciprocal with a hit (their weight there is NaN).
+// Its points are cut into S slices, S chosen so that all such queries'
+// slices fill the grid (counted when the list is short; a list of more than
+// kSlowThreads queries fills it by itself); each slice's sums are scaled by
+// its own d2_min, and a warp of the CTA that finishes a query's last slice
+// rescales and adds them in a fixed order.  A 100,003-point, 65,537-query call with 16
+// hits spent 860 us on them in the combine, one CTA a query: the FP64 pipe
+// of one SM bounds a query; spread over the GPU they take under 30 us.
+template <int CAP>
+__global__ void __launch_bounds__(kSlowThreads)
+    slow_finish_kernel(const __grid_constant__ Table<CAP> t, const Control* __restrict__ ctrl,
+                       const SlowList slow, double p) {
+  __shared__ int work[kSlowThreads];
+  __shared__ int warp_count[kSlowThreads / 32];
+  __shared__ bool last;
+  pdl_trigger();
+  pdl_wait();
+  const int count = static_cast<int>(min(ctrl->flagged, slow.cap));
+  if (count == 0) return;
+  const int tid = threadIdx.x;
+  // Hits: one thread each.
+  for (int f = blockIdx.x * kSlowThreads + tid; f < count; f += gridDim.x * kSlowThreads) {
+    const SlowItem it = slow.item[f];
+    if (it.hit == INT_MAX) continue;
+    const Instance& I = t.inst[it.problem];
+    const int64_t j = it.query;
+    slow_write_hit<float, float>(I.data, it.hit, &I.out[j], I.s0_out ? &I.s0_out[j] : nullptr,
+                                 I.hit_out ? &I.hit_out[j] : nullptr);
+  }
+  const bool short_list = count <= kSlowThreads;
+  int sums = count;
+  if (short_list) {  // the queries without a hit, in list order
+    const bool mine = tid < count && slow.item[tid].hit == INT_MAX;
+    const unsigned vote = __ballot_sync(0xffffffffu, mine);
+    if ((tid & 31) == 0) warp_count[tid >> 5] = __popc(vote);
+    __syncthreads();
+    int before = 0;
+    sums = 0;
+    for (int w = 0; w < kSlowThreads / 32; ++w) {
+      if (w < (tid >> 5)) before += warp_count[w];
+      sums += warp_count[w];
+    }
+    if (mine) work[before + __popc(vote & ((1u << (tid & 31)) - 1))] = tid;
+    __syncthreads();
+    if (sums == 0) return;
+  }
+  const int slices = max(1, int(gridDim.x) / sums);
+  for (int64_t w = blockIdx.x; w < int64_t(sums) * slices; w += gridDim.x) {
+    const int e = static_cast<int>(w / slices), sl = static_cast<int>(w % slices);
+    const int f = short_list ? work[e] : e;
+    const SlowItem it = slow.item[f];
+    if (it.hit != INT_MAX) continue;  // uniform across the CTA
+    const Instance& I = t.inst[it.problem];
+    const int64_t j = it.query;
+    const SlowSums s = slow_sums<float>(I.data, int64_t(sl) * I.n / slices,
+                                        int64_t(sl + 1) * I.n / slices, I.queries[2 * j],
+                                        I.queries[2 * j + 1], p);
+    if (tid == 0) {
+      slow.part[w] = s;
+      __threadfence();
+      last = atomicAdd(&slow.item[f].done, 1u) + 1u == unsigned(slices);
+    }
+    __syncthreads();
+    if (last && tid < 32) {  // one warp, lanes over the slices, a fixed shuffle tree
+      __threadfence();
+      const double* P = reinterpret_cast<const double*>(slow.part + (w - sl));
+      double dmin = INFINITY;
+      for (int k = tid; k < slices; k += 32) dmin = fmin(dmin, __ldcg(P + 3 * k));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xffffffffu, dmin, o));
+      SlowSums sum{dmin, 0.0, 0.0};
+      for (int k = tid; k < slices; k += 32) {
+        // A slice at infinity (d2_min = +inf) holds zeros, or NaN to keep.
+        const double dk = __ldcg(P + 3 * k);
+        const double c = dk == dmin || dk == INFINITY ? 1.0
+                         : p == 2.0                   ? dmin / dk
+                                                      : pow(dmin / dk, 0.5 * p);
+        sum.s0 += __ldcg(P + 3 * k + 1) * c;
+        sum.s1 += __ldcg(P + 3 * k + 2) * c;
+      }
+      sum.s0 = warp_sum(sum.s0);
+      sum.s1 = warp_sum(sum.s1);
+      if (tid == 0)
+        slow_write_sums<float>(sum, p, &I.out[j], I.s0_out ? &I.s0_out[j] : nullptr,
+                               I.hit_out ? &I.hit_out[j] : nullptr);
+    }
+    __syncthreads();  // `last` is rewritten by the next item
+  }
 }
 
 // One thread waits, with the sweep kernels' bounded wait, on a barrier whose
@@ -560,7 +729,7 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
 
   const unsigned gx = static_cast<unsigned>(std::min<int64_t>(1024, (longest + 255) / 256));
   if ((e = launch_pdl(range_kernel<CAP>, dim3(gx, plan.count), dim3(256), 0, stream, t,
-                      maxbits)) != cudaSuccess)
+                      maxbits, &ctrl->flagged)) != cudaSuccess)
     return e;
   const int64_t records = plan.total_stage_tiles * TB;
   const unsigned sgrid = static_cast<unsigned>((records + 255) / 256);
@@ -592,11 +761,32 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
   if (ev && (e = cudaEventRecord(ev->stop, stream)) != cudaSuccess) return e;
 
   const int64_t slots = plan.total_query_tiles * QT;
-  return launch_pdl(combine_kernel<CAP, QT>,
-                    dim3(static_cast<unsigned>((slots + kCombineQueries - 1) / kCombineQueries)),
-                    dim3(kCombineQueries * kCombineLanes), 0, stream, t,
-                    static_cast<const float4*>(partial), slots, plan.units, plan.grid,
-                    static_cast<const float*>(scales), p, ctrl);
+  // Each listed query takes an item and a slice record; the grid's worth of
+  // records more covers short lists cut into more slices.
+  const int slow_grid = 2 * sm_count;
+  SlowList slow;
+  const size_t spare = size_t(slow_grid) * sizeof(SlowSums);
+  slow.cap = static_cast<unsigned>(std::min<size_t>(
+      plan.staged_bytes > spare
+          ? (plan.staged_bytes - spare) / (sizeof(SlowItem) + sizeof(SlowSums))
+          : 0,
+      size_t(INT_MAX)));
+  slow.item = reinterpret_cast<SlowItem*>(ws);
+  slow.part = reinterpret_cast<SlowSums*>(ws + size_t(slow.cap) * sizeof(SlowItem));
+  if ((e = launch_pdl(combine_kernel<CAP, QT>,
+                      dim3(static_cast<unsigned>((slots + kCombineQueries - 1) / kCombineQueries)),
+                      dim3(kCombineQueries * kCombineLanes), 0, stream, t,
+                      static_cast<const float4*>(partial), slots, plan.units, plan.grid,
+                      static_cast<const float*>(scales), p, ctrl, slow)) != cudaSuccess)
+    return e;
+  int64_t most_points = 0;
+  for (int k = 0; k < plan.count; ++k) most_points = std::max(most_points, probs[k].n);
+  if (most_points <= kSlowInlinePoints || slow.cap == 0) return cudaSuccess;  // nothing is listed
+  if ((e = launch_pdl(slow_search_kernel<CAP>, dim3(slow_grid), dim3(kSlowThreads), 0, stream, t,
+                      static_cast<const Control*>(ctrl), slow)) != cudaSuccess)
+    return e;
+  return launch_pdl(slow_finish_kernel<CAP>, dim3(slow_grid), dim3(kSlowThreads), 0, stream, t,
+                    static_cast<const Control*>(ctrl), slow, p);
 }
 
 }  // namespace
