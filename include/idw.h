@@ -283,8 +283,10 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *   IDW_OPT_KNN_SEARCH          0 (default) or 1.  The k-NN search of
  *                               idw_interpolate_knn and idw_knn_backward: 0
  *                               one thread per query, each growing its own
- *                               square of cells at its own pace; 1 the same
- *                               per-query search with the 32 lanes of a warp
+ *                               square of cells at its own pace, or a warp per
+ *                               query where there are few queries or the
+ *                               points around one are far or dense; 1 the
+ *                               per-thread search with the 32 lanes of a warp
  *                               kept in step (the same step and row order,
  *                               each lane's row runs walked as one stream,
  *                               heap inserts merged by the warp together).
@@ -554,9 +556,12 @@ idw_status idw_interpolate_modified(idw_handle_t handle, const float *data_xyz, 
  * keys in shared memory.  Band sizes come from a summed-area table of the
  * cells; once k keys are held, cells whose points provably lie beyond the
  * k-th key are skipped; the search stops once the k-th key is below a
- * conservative FP32 lower bound on the key of any point not yet seen.
- * Workspace as idw_interpolate_local.  Errors as in idw_interpolate, plus
- * IDW_ERR_INVALID_ARG for k outside [1, 64].
+ * conservative FP32 lower bound on the key of any point not yet seen.  For
+ * few queries, and for those whose surroundings are empty or dense, a warp
+ * takes the query instead: it walks the cells of a disc that the table shows
+ * to hold k points.
+ * Workspace as idw_interpolate_local and 4 bytes per query.  Errors as in
+ * idw_interpolate, plus IDW_ERR_INVALID_ARG for k outside [1, 64].
  */
 idw_status idw_interpolate_knn(idw_handle_t handle, const float *data_xyz, int64_t n,
                                const float *queries_xy, int64_t m, double p, int32_t k,
@@ -657,7 +662,7 @@ idw_status idw_knn_backward(idw_handle_t handle, const float *data_xyz, int64_t 
  * index, for any 1 <= k <= 64.  Outputs, NaN and hit rules are those of
  * the one-shot calls.  Both run on `stream` without host synchronisation
  * (graph-capturable once the handle's workspace has grown) and take the
- * handle's workspace: 16 bytes per query and 8 per cell.  The handle must be
+ * handle's workspace: 20 bytes per query and 8 per cell.  The handle must be
  * on the index's device; calling the wrong form's query on an index, a
  * radius above the build radius or k outside [1, 64] gives
  * IDW_ERR_INVALID_ARG.  Several handles (one per stream) may query one

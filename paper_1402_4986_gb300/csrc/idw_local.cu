@@ -97,6 +97,7 @@ struct GridDev {
   float hx0, hy0, inv2;  // cell position u(v) = fl(fl(fl(v/2) - h0) * inv2)
   float rho;             // reach of R in cells, with margin (< 2)
   int gx, gy, cells;
+  unsigned hard;         // k-NN queries the single-thread search left to warps
 };
 
 // Order-preserving unsigned key of a float (for atomic min).
@@ -181,6 +182,7 @@ __device__ void plan_grid(GridDev* grid, double radius, double inv_max_cells, in
   grid->gx = gx;
   grid->gy = gy;
   grid->cells = gx * gy;
+  grid->hard = 0u;
 }
 
 // Bounding box of the finite data points; the last block to finish plans
@@ -1192,9 +1194,35 @@ __device__ __forceinline__ void knn_write_result(KnnHeap& hp, int best_hit, floa
   }
 }
 
+// Whether one thread should search for a query in cell (cx, cy).  With ca
+// cells per point, the square of radius re = ceil((sqrt(2 k ca) - 1) / 2)
+// holds 2k points at the mean density.  Where the square one cell wider holds
+// fewer than k, the search has empty space to cross; where the square holds
+// over 8k + 64, it has a dense cluster to sift; a thread takes ten to a
+// hundred times as long over such a query as over one at the mean density,
+// and its warp waits.  (n = 2^20 points in 64 blobs, 100,000 uniform queries,
+// k = 8: 1.09 ms when every query was one thread's.)
+__device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* __restrict__ sat,
+                                         float cells_per_point, int cx, int cy, int k) {
+  const int re = int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
+  const int W = g.gx + 1;
+  int c[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int rr = re + i;
+    const int ya = max(0, cy - rr), yb = min(g.gy - 1, cy + rr);
+    const int xa = max(0, cx - rr), xb = min(g.gx - 1, cx + rr);
+    if (!dcheck(ya >= 0 && xa >= 0 && yb < g.gy && xb < g.gx, kSiteTable)) return true;
+    c[i] = sat[(yb + 1) * W + xb + 1] - sat[ya * W + xb + 1] - sat[(yb + 1) * W + xa] +
+           sat[ya * W + xa];
+  }
+  return c[1] >= k && c[0] <= 8 * k + 64;
+}
+
 // At most 64 registers (32 one-warp blocks per SM); left to itself the
-// compiler settles on fewer and spills.
-template <int MODE>
+// compiler settles on fewer and spills.  With LIST, queries that are not
+// knn_easy are listed in `hard` for knn_warp_kernel.
+template <int MODE, bool LIST>
 __global__ void __maxnreg__(64)
     knn_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
                      const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
@@ -1203,7 +1231,8 @@ __global__ void __maxnreg__(64)
                      int64_t m,
                      double p, int k, float* __restrict__ out, int32_t* __restrict__ nbr_out,
                      float* __restrict__ kd2_out, int32_t* __restrict__ hit_out,
-                     bool sort_rows) {
+                     bool sort_rows, unsigned* __restrict__ hard_count,
+                     int32_t* __restrict__ hard) {
   extern __shared__ __align__(16) unsigned char knn_smem[];
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= m) return;  // no block-wide barrier in this kernel
@@ -1248,6 +1277,15 @@ __global__ void __maxnreg__(64)
   if (finite2(qx, qy)) {
     const float u = cell_pos(qx, g.hx0, g.inv2), v = cell_pos(qy, g.hy0, g.inv2);
     const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
+    if (LIST && !knn_easy(g, sat, float(g.cells) * rcp_approx(float(n)), cx, cy, k)) {
+      const unsigned lanes = __activemask();  // one atomic for those that are here together
+      const int lane = threadIdx.x & 31, lead = __ffs(lanes) - 1;
+      unsigned at = 0;
+      if (lane == lead) at = atomicAdd(hard_count, unsigned(__popc(lanes)));
+      at = __shfl_sync(lanes, at, lead) + __popc(lanes & ((1u << lane) - 1));
+      if (dcheck(at < m, kSiteScatter)) hard[at] = static_cast<int32_t>(t);
+      return;
+    }
     const float mg = __fmaf_ru(fabsf(u) + fabsf(v), 0x1p-22f, 0x1p-9f);
     const float ax = fmaxf(0.f, fmaxf(u - float(g.gx), -u) - mg);
     const float ay = fmaxf(0.f, fmaxf(v - float(g.gy), -v) - mg);
@@ -1389,6 +1427,380 @@ __global__ void __maxnreg__(64)
   }
   knn_write_result<MODE>(hp, best_hit, qx, qy, j, data, n, p, k, out, nbr_out, kd2_out, hit_out,
                          sort_rows);
+}
+
+// ------------------------------------------------- k-NN, a warp per query
+//
+// The search for calls with few queries, and for the queries of larger calls
+// that one thread would take long over (see knn_easy):
+// 1. a disc around the query that holds at least k points, its radius found
+//    from the summed-area table with 32 radii per probe: the cells inside
+//    three rectangles inscribed in the disc are counted, so the k-th key is
+//    at most the disc's radius squared;
+// 2. every cell the disc reaches is walked (the rows' runs laid end to end,
+//    32 candidates at a time, one coalesced load each); keys up to the bound
+//    are appended to a buffer in shared memory, and whenever it is nearly
+//    full its k smallest keys are kept and the bound drops to the k-th key;
+// 3. the k smallest of the buffer are the selection (keys are distinct, so
+//    the order of candidates does not matter), and the lanes share the sums.
+// Bound by instruction issue (66% of issue slots, 30 of 32 lanes active,
+// about 1250 instructions a query at k = 8); a query costs about as many
+// whether its points lie near or far, which is what the hard queries need.
+constexpr unsigned kWarp = 0xffffffffu;
+
+// kRegs keys per lane: the buffer of 32 kRegs keys is cut back to k when
+// fewer than 32 slots are free, so k <= 32 (kRegs - 1).
+template <int kRegs>
+struct KnnBuffer {
+  static constexpr int kCap = 32 * kRegs;
+  int lane;
+  u64* buf;
+
+  // Keeps the k smallest of the buffer's `cnt` keys (all of them if there are
+  // no more than k) and returns the largest kept; `cnt` becomes their number.
+  // The k-th smallest d^2 is bracketed between lo (fewer than k keys at or
+  // below) and hi (at least k) in the order of the float's bits; the probe
+  // between them assumes keys spread evenly in d^2, as points of even density
+  // are, and every third probe halves the bracket instead, which ends the
+  // search whatever the keys.
+  __device__ u64 prune(int& cnt, int k) {
+    __syncwarp();
+    if (cnt <= 32) return prune_regs<1>(cnt, k);
+    if (cnt <= 64) return prune_regs<2>(cnt, k);
+    return prune_regs<kRegs>(cnt, k);
+  }
+
+  // As prune, for at most 32 R keys.
+  template <int R>
+  __device__ __forceinline__ u64 prune_regs(int& cnt, int k) {
+    int d[R], id[R];  // d^2 bits (not negative) and index; INT_MAX: no key
+    int dmin = INT_MAX, dmax = -1;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int s = lane + i * 32;
+      const u64 key = s < cnt ? buf[s] : u64(0);
+      d[i] = s < cnt ? int(unsigned(key >> 32)) : INT_MAX;
+      id[i] = key_index(key);
+      dmin = min(dmin, d[i]);
+      if (s < cnt) dmax = max(dmax, d[i]);
+    }
+    int hi = __reduce_max_sync(kWarp, dmax), chi = cnt;
+    if (chi > k) {
+      int lo = __reduce_min_sync(kWarp, dmin) - 1, clo = 0;
+      for (int it = 0; hi - lo > 1 && chi != k; ++it) {
+        const float fl = __int_as_float(max(lo, 0)), fh = __int_as_float(hi);
+        const float f = (float(k - clo) - 0.5f) * rcp_approx(float(chi - clo));
+        int mid = it % 3 == 2 || !(fh <= FLT_MAX) ? lo + ((hi - lo) >> 1)
+                                                  : __float_as_int(fmaf(fh - fl, f, fl));
+        mid = max(lo + 1, min(hi - 1, mid));
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < R; ++i) c += d[i] <= mid;
+        c = __reduce_add_sync(kWarp, c);
+        if (c >= k) {
+          hi = mid;
+          chi = c;
+        } else {
+          lo = mid;
+          clo = c;
+        }
+      }
+      int tie = INT_MAX;  // of keys with d^2 == hi, indices up to this one
+      if (chi != k) {     // more than k: the lowest k - clo indices among the ties
+        tie = -1;
+        for (int t = clo; t < k; ++t) {
+          int m = INT_MAX;
+#pragma unroll
+          for (int i = 0; i < R; ++i)
+            if (d[i] == hi && id[i] > tie) m = min(m, id[i]);
+          tie = __reduce_min_sync(kWarp, m);
+        }
+      }
+      int base = 0;
+      dmax = -1;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {  // every lane holds its keys in registers by now
+        const bool keep = d[i] < hi || (d[i] == hi && id[i] <= tie);
+        const unsigned b = __ballot_sync(kWarp, keep);
+        if (keep) {
+          const int at = base + __popc(b & ((1u << lane) - 1));
+          if (dcheck(at < kCap, kSiteHeap)) buf[at] = knn_key(__int_as_float(d[i]), id[i]);
+          dmax = max(dmax, d[i]);
+        } else {
+          d[i] = -1;
+        }
+        base += __popc(b);
+      }
+      cnt = base;
+      hi = __reduce_max_sync(kWarp, dmax);
+      __syncwarp();
+    }
+    int im = -1;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+      if (d[i] == hi) im = max(im, id[i]);
+    return knn_key(__int_as_float(hi), __reduce_max_sync(kWarp, im));
+  }
+};
+
+constexpr int kKnnWarpThreads = 128;
+
+// One query, by a whole warp.
+template <int MODE, int kRegs>
+__device__ __forceinline__ void knn_warp_query(
+    const GridDev& g, u64* keys, float qx, float qy, int j, const float4* __restrict__ sorted,
+    const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
+    const int32_t* __restrict__ sat, const float* __restrict__ data, int64_t n, double p, int k,
+    float* __restrict__ out, int32_t* __restrict__ nbr_out, float* __restrict__ kd2_out,
+    int32_t* __restrict__ hit_out, bool sort_rows) {
+  using Buffer = KnnBuffer<kRegs>;
+  Buffer kb;
+  kb.lane = threadIdx.x % 32;
+  kb.buf = keys;
+  const int lane = kb.lane;
+  int best_hit = INT_MAX;  // this lane's
+  int cnt = 0;             // keys in the buffer (the same in every lane)
+  u64 worst = ~u64(0);     // no key above this one is in the selection
+
+  if (finite2(qx, qy)) {
+    const float u = cell_pos(qx, g.hx0, g.inv2), v = cell_pos(qy, g.hy0, g.inv2);
+    const float mg = __fmaf_ru(fabsf(u) + fabsf(v), 0x1p-22f, 0x1p-9f);
+    const float hh = g.inv2 > 0.f ? 2.f / g.inv2 : 0.f;
+    const float h2 = __fmul_rd(hh, hh) * (1.f - 0x1p-18f);
+    const float ih2 = __frcp_ru(h2);  // +inf for the one-cell grid: nothing is clipped
+    if (g.inv2 > 0.f && fabsf(u) < 0x1p20f && fabsf(v) < 0x1p20f) {
+      // Points in cells xa..xb, ya..yb, clamped into the grid; an empty
+      // rectangle's four entries cancel.  Straight-line code: every lane of
+      // the warp reaches the votes below together.
+      const int W = g.gx + 1;
+      auto rect = [&](int xa, int xb, int ya, int yb) {
+        const int x0 = min(max(xa, 0), g.gx), x1 = min(max(xb + 1, x0), g.gx);
+        const int y0 = min(max(ya, 0), g.gy), y1 = min(max(yb + 1, y0), g.gy);
+        return sat[y1 * W + x1] - sat[y0 * W + x1] - sat[y1 * W + x0] + sat[y0 * W + x0];
+      };
+      // Points in cells that lie inside the disc of radius rho cells: the
+      // union of three inscribed rectangles (corners at 22.5, 45 and 67.5
+      // degrees), each shrunk by mg for the cell-position errors.
+      auto disc_count = [&](float rho) {
+        const float e1 = 0.9238795f * rho - mg, e2 = 0.7071067f * rho - mg,
+                    e3 = 0.3826834f * rho - mg;
+        const int xa1 = int(ceilf(u - e1)), xb1 = int(floorf(u + e1)) - 1;
+        const int xa2 = int(ceilf(u - e2)), xb2 = int(floorf(u + e2)) - 1;
+        const int xa3 = int(ceilf(u - e3)), xb3 = int(floorf(u + e3)) - 1;
+        const int ya1 = int(ceilf(v - e3)), yb1 = int(floorf(v + e3)) - 1;
+        const int ya2 = int(ceilf(v - e2)), yb2 = int(floorf(v + e2)) - 1;
+        const int ya3 = int(ceilf(v - e1)), yb3 = int(floorf(v + e1)) - 1;
+        int c = rect(xa1, xb1, ya1, yb1);
+        c += rect(xa2, xb2, ya2, yb2) - rect(xa2, xb2, ya1, yb1);
+        c += rect(xa3, xb3, ya3, yb3) - rect(xa3, xb3, ya2, yb2);
+        return c;
+      };
+      // Bracket: squares of half-width 5/8 (5/4)^lane cells (the last one, 631,
+      // doubled until it holds k points or cannot: then no bound).  The disc
+      // around the first that holds k does too; the discs that fit into the
+      // square before it do not.
+      auto square = [&](float e) {
+        return rect(int(ceilf(u - e + mg)), int(floorf(u + e - mg)) - 1, int(ceilf(v - e + mg)),
+                    int(floorf(v + e - mg)) - 1);
+      };
+      const float side = 0.625f * ex2_approx(0.32192809f * float(lane));
+      int inside = square(side);
+      unsigned b = __ballot_sync(kWarp, inside >= k);
+      float far = 1.f;
+      while (b == 0 && far < 4096.f) {
+        far *= 2.f;
+        inside = square(side * far);
+        b = __ballot_sync(kWarp, inside >= k) & 0x80000000u;
+      }
+      if (b) {
+        const int f = __ffs(b) - 1;
+        const float s1 = far * __shfl_sync(kWarp, side, f);
+        const float before = __shfl_sync(kWarp, side, max(f - 1, 0));
+        float lo = far > 1.f ? 0.5f * s1 : f > 0 ? before : 0.f;
+        float hi = 1.4142137f * (s1 + mg), step;
+        // 32 radii in between, again while they are over a cell apart.
+        do {
+          step = (hi - lo) * 0x1p-5f;
+          const float probe = lane == 31 ? hi : fmaf(step, float(lane + 1), lo);
+          inside = disc_count(probe);
+          const unsigned in = __ballot_sync(kWarp, inside >= k) | 0x80000000u;  // hi does
+          hi = __shfl_sync(kWarp, probe, __ffs(in) - 1);
+          lo = hi - step;
+        } while (step > 1.f);
+        // An upper bound of the FP32 d^2 of any point in the disc.
+        const float bound = __fadd_ru(
+            __fmul_ru(__fmul_ru(__fmul_ru(hi, hi), __fmul_ru(hh, hh)), 1.f + 0x1p-17f), 0x1p-126f);
+        if (bound <= FLT_MAX) worst = knn_key(bound, -1);
+      }
+    }
+    // Rows whose gap from v, and columns whose gap from u, can hold a key up
+    // to `worst`, rounded outwards (a NaN or infinite bound clips nothing).
+    auto reach2 = [&]() { return __fmul_ru(__fadd_ru(key_d2(worst), 0x1p-126f), ih2); };
+    auto clip = [&](float c, float e, int& first, int& last) {
+      const float fa = ceilf(__fsub_rd(__fsub_rd(__fsub_rd(c, mg), e), 1.f));
+      const float fb = floorf(__fadd_ru(__fadd_ru(c, mg), e));
+      const int nf = int(fminf(fmaxf(float(first), fa), float(last) + 1.f));
+      const int nl = int(fmaxf(fminf(float(last), fb), float(first) - 1.f));
+      first = nf;
+      last = nl;
+    };
+    int row0 = 0, row1 = g.gy - 1;
+    clip(v, __fsqrt_ru(reach2()), row0, row1);
+    for (int y0 = row0; y0 <= row1; y0 += 32) {
+      // This lane's row: its run [a, a + len) of the sorted points.
+      const int yy = y0 + lane;
+      int a = 0, len = 0;
+      if (yy <= row1) {
+        const float gap = fmaxf(0.f, fmaxf(float(yy) - v, v - float(yy + 1)) - mg);
+        const float w2 = reach2(), g2 = __fmul_rd(gap, gap);
+        int ra = 0, rb = g.gx - 1;
+        if (!(g2 > w2)) {
+          clip(u, __fsqrt_ru(__fsub_ru(w2, g2)), ra, rb);
+          if (ra <= rb) {
+            a = cell_start(starts, base, yy * g.gx + ra, g.cells);
+            len = cell_start(starts, base, yy * g.gx + rb + 1, g.cells) - a;
+          }
+        }
+      }
+      // The rows' runs end to end: candidate s belongs to the run whose end
+      // is the first above s.
+      int end = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kWarp, end, o);
+        if (lane >= o) end += x;
+      }
+      const int total = __shfl_sync(kWarp, end, 31);
+      const int shift = a - (end - len);  // candidate s of this run is sorted[s + shift]
+      for (int s0 = 0; s0 < total; s0 += 32) {
+        const int s = s0 + lane;
+        int r = 0;  // the number of runs that end at or before s
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(kWarp, end, r + o - 1) <= s) r += o;
+        const int at = s + __shfl_sync(kWarp, shift, r);
+        u64 key = ~u64(0);
+        bool take = false;
+        if (s < total && dcheck(at >= 0 && at < n, kSiteGather)) {
+          const float4 c = sorted[at];
+          const float d2 = fp32_d2(qx, qy, c.x, c.y);
+          const int idx = __float_as_int(c.w);
+          if (d2 == 0.f && c.x == qx && c.y == qy) best_hit = min(best_hit, idx);
+          key = knn_key(d2, idx);
+          take = key <= worst;
+        }
+        const unsigned b = __ballot_sync(kWarp, take);
+        const int slot = cnt + __popc(b & ((1u << lane) - 1));
+        if (take && dcheck(slot < Buffer::kCap, kSiteHeap)) kb.buf[slot] = key;
+        cnt += __popc(b);
+        if (cnt > Buffer::kCap - 32) worst = kb.prune(cnt, k);
+      }
+    }
+    if (cnt > 0) worst = kb.prune(cnt, k);  // the largest key of the selection
+    best_hit = __reduce_min_sync(kWarp, best_hit);
+  }
+  __syncwarp();
+
+  if (lane == 0) {
+    if (kd2_out) kd2_out[j] = cnt > 0 ? key_d2(worst) : __int_as_float(0x7fc00000);
+    if (hit_out) hit_out[j] = best_hit != INT_MAX ? best_hit : -1;
+  }
+  if (nbr_out) {
+    int32_t* row = nbr_out + int64_t(j) * k;
+    for (int s = lane; s < k; s += 32) {
+      int at = s;
+      if (s < cnt && sort_rows) {  // the key's rank
+        const u64 key = kb.buf[s];
+        at = 0;
+        for (int o = 0; o < cnt; ++o) at += kb.buf[o] < key;
+      }
+      row[at] = s < cnt ? key_index(kb.buf[s]) : -1;
+    }
+  }
+  if (best_hit != INT_MAX || cnt == 0) {
+    if (lane == 0)
+      out[j] = cnt == 0 ? __int_as_float(0x7fc00000)
+               : dcheck(best_hit >= 0 && best_hit < n, kSiteData) ? data[3 * int64_t(best_hit) + 2]
+                                                                  : 0.f;
+    return;
+  }
+  // Eq. 1 over the selection: compensated FP32 sums per lane, joined by a
+  // fixed tree of error-free additions.
+  const float hpw = static_cast<float>(0.5 * p), nhp = -hpw;
+  u64 hi = 0, lo = 0;
+  for (int s = lane; s < cnt; s += 32) {
+    const u64 key = kb.buf[s];
+    const float w = local_weight<MODE>(key_d2(key), hpw, nhp);
+    if (!dcheck(key_index(key) >= 0 && key_index(key) < n, kSiteData)) continue;
+    two_sum_acc(hi, lo, pk(w, __fmul_rn(w, data[3 * int64_t(key_index(key)) + 2])));
+  }
+  // Lanes from min(cnt, 32) on hold zeros; lane 0 gets the total.
+  for (int o = cnt > 16 ? 16 : cnt > 8 ? 8 : cnt > 4 ? 4 : 2; o > 0; o >>= 1) {
+    const u64 oh = __shfl_xor_sync(kWarp, hi, o), ol = __shfl_xor_sync(kWarp, lo, o);
+    two_sum_acc(hi, lo, oh);
+    lo = add2(lo, ol);
+  }
+  hi = __shfl_sync(kWarp, hi, 0);  // every lane takes the same branch below
+  lo = __shfl_sync(kWarp, lo, 0);
+  float h0, h1, l0, l1;
+  upk(hi, h0, h1);
+  upk(lo, l0, l1);
+  float zv;
+  if (h0 >= kTinyPerMember * float(cnt) && h0 <= FLT_MAX && fabsf(h1) <= FLT_MAX &&
+      fabsf(l1) <= FLT_MAX) {
+    const float z0 = __fdiv_rn(h1, h0);
+    const float res = __fadd_rn(__fmaf_rn(-z0, h0, h1), __fmaf_rn(-z0, l0, l1));
+    zv = __fmaf_rn(res, rcp_approx(h0), z0);
+  } else {
+    // Outside FP32's range (the same in every lane): FP64 over the selected
+    // points, scaled by d2_min^(p/2).
+    double dmin = INFINITY;
+    for (int s = 0; s < cnt; ++s) {
+      const float* x = data + 3 * int64_t(key_index(kb.buf[s]));
+      const double ex = double(qx) - x[0], ey = double(qy) - x[1];
+      dmin = fmin(dmin, ex * ex + ey * ey);
+    }
+    double s0 = 0.0, s1 = 0.0;
+    for (int s = lane; s < cnt; s += 32) {
+      const float* x = data + 3 * int64_t(key_index(kb.buf[s]));
+      const double ex = double(qx) - x[0], ey = double(qy) - x[1];
+      const double w = pow(dmin / (ex * ex + ey * ey), 0.5 * p);
+      s0 += w;
+      s1 += w * double(x[2]);
+    }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+    zv = static_cast<float>(s1 / s0);
+  }
+  if (lane == 0) out[j] = zv;
+}
+
+// The queries of `hard` (null: all m), a warp each.
+template <int MODE, int kRegs>
+__global__ void __launch_bounds__(kKnnWarpThreads)
+    knn_warp_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
+                    const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
+                    const int32_t* __restrict__ sat, const float4* __restrict__ qrec,
+                    const float* __restrict__ data, int64_t n, int64_t m, double p, int k,
+                    float* __restrict__ out, int32_t* __restrict__ nbr_out,
+                    float* __restrict__ kd2_out, int32_t* __restrict__ hit_out, bool sort_rows,
+                    const unsigned* __restrict__ hard_count, const int32_t* __restrict__ hard) {
+  using Buffer = KnnBuffer<kRegs>;
+  __shared__ u64 keys[kKnnWarpThreads / 32][Buffer::kCap];
+  const int64_t count = hard ? int64_t(*hard_count) : m;
+  const int64_t warps = int64_t(gridDim.x) * (kKnnWarpThreads / 32);
+  const GridDev g = *grid;
+  for (int64_t w = (int64_t(blockIdx.x) * kKnnWarpThreads + threadIdx.x) / 32; w < count;
+       w += warps) {  // whole warps: no block-wide barrier in this kernel
+    const int64_t t = hard ? int64_t(hard[w]) : w;
+    if (!dcheck(t >= 0 && t < m && count <= m, kSiteScatter)) continue;
+    const float4 rq = qrec[t];
+    const int j = __float_as_int(rq.z);
+    if (!dcheck(j >= 0 && j < m, kSiteOutput)) continue;
+    knn_warp_query<MODE, kRegs>(g, keys[threadIdx.x / 32], rq.x, rq.y, j, sorted, starts, base, sat,
+                                data, n, p, k, out, nbr_out, kd2_out, hit_out, sort_rows);
+    __syncwarp();  // the buffer is the next query's
+  }
 }
 
 // ------------------------------------------- k-NN, warp-synchronous
@@ -2054,6 +2466,7 @@ LocalLayout local_layout(int64_t n, int64_t m, int64_t max_cells) {
   L.off_sums = off;       off += round_up(size_t(2 * scan_tiles_of(max_cells)) * 4, 256);
   L.off_sorted = off;     off += round_up(size_t(n) * 16, 256);
   L.off_qrec = off;       off += round_up(size_t(m) * 16, 256);
+  L.off_hard = off;       off += round_up(size_t(m) * 4, 256);
   L.off_bpre = off;
   off += round_up(size_t(kMaxBlocksPerAxis) * (kMaxBlocksPerAxis + 1) * 4, 256);
   // (gx + 1)(gy + 1) = cells + gx + gy + 1 entries, cells <= max_cells.
@@ -2324,27 +2737,86 @@ cudaError_t debug_check_failures(unsigned* sites, bool* enabled) {
 #endif
 }
 
+namespace {
+
 size_t knn_smem_bytes(int k) { return size_t(k) * kKnnThreads * sizeof(u64); }
 
+// Up to this many queries, a warp searches for each: a thread per query
+// leaves the GPU idle there.  Measured on a GB300 against n = 2^20 uniform
+// points, whole query call on a prepared index, thread / warp per query:
+// m = 10,007 61 / 43 us at k = 8, 107 / 46 us at k = 32; m = 100,000
+// 69 / 143 us at k = 8, 141 / 168 us at k = 32.
+int64_t knn_warp_queries(int k) { return 8192 + 1024 * int64_t(k); }
+
+// Up to this many queries, those that are not knn_easy go to warps.  Beyond
+// it every warp of the single-thread search has hard queries to overlap with
+// and the GPU is full either way (64 blobs, n = 2^20, k = 8, threads alone /
+// with warps: m = 10,007 1010 / 74 us, 100,000 1090 / 263 us, 2^20
+// 1440 / 1770 us).
+constexpr int64_t kKnnHardQueries = int64_t(1) << 19;
+
+// The search over sorted queries, by warps for few of them, else by threads
+// with warps for the hard ones; the launch arguments both share.
+struct KnnArgs {
+  GridDev* grid;
+  const float4* sorted;
+  const int32_t *starts, *base, *bpre, *sat;
+  const float4* qrec;
+  const float* data;
+  int64_t n, m;
+  double p;
+  int k;
+  float* out;
+  int32_t* nbr_out;
+  float* kd2_out;
+  int32_t* hit_out;
+  bool sort_rows;
+  int32_t* hard;
+};
+
+cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
+  // Rows in search order (the gradients' plain FP32 sums follow it) keep the
+  // single-thread search's order.
+  const bool warps = !a.nbr_out || a.sort_rows;
+  const bool all_warps = warps && a.m <= knn_warp_queries(a.k);
+  int32_t* list = warps && !all_warps && a.m <= kKnnHardQueries ? a.hard : nullptr;
+  unsigned* hard_count = &a.grid->hard;
+  if (!all_warps) {
+    const size_t smem = knn_smem_bytes(a.k);  // below the default limit (k <= 64: 16 KB)
+    auto kernel = list ? (a.p == 2.0 ? knn_query_kernel<kPow2, true> : knn_query_kernel<kPowGeneral, true>)
+                       : (a.p == 2.0 ? knn_query_kernel<kPow2, false>
+                                     : knn_query_kernel<kPowGeneral, false>);
+    kernel<<<static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads), kKnnThreads, smem, s>>>(
+        a.grid, a.sorted, a.starts, a.base, a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out,
+        a.nbr_out, a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
+    if (!list) return cudaGetLastError();
+  }
+  constexpr int per_block = kKnnWarpThreads / 32;
+  // The hard list's length is known on the device only: enough blocks to
+  // fill the GPU stride over it.
+  const int64_t blocks = all_warps ? (a.m + per_block - 1) / per_block : int64_t(sm_count) * 8;
+  auto kernel = a.k <= 32 ? (a.p == 2.0 ? knn_warp_kernel<kPow2, 3> : knn_warp_kernel<kPowGeneral, 3>)
+                          : (a.p == 2.0 ? knn_warp_kernel<kPow2, 4> : knn_warp_kernel<kPowGeneral, 4>);
+  kernel<<<static_cast<unsigned>(blocks), kKnnWarpThreads, 0, s>>>(
+      a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
+      a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
+  return cudaGetLastError();
+}
+
+}  // namespace
 
 cudaError_t launch_knn(const float* data, int64_t n, const float* queries, int64_t m, double p,
                        int k, float* out, int32_t* nbr_out, float* kd2_out, void* workspace,
                        const LocalLayout& L, int sm_count, cudaStream_t s, int32_t* hit_out,
                        bool sort_queries, bool sort_rows, bool warp_search) {
-  const size_t smem = warp_search ? knn_sync_smem_bytes(k) : knn_smem_bytes(k);
   cudaError_t e = cudaSuccess;
+  const size_t sync_smem = knn_sync_smem_bytes(k);
   if (warp_search) {
     e = cudaFuncSetAttribute(knn_sync_kernel<kPow2>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(sync_smem));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(knn_sync_kernel<kPowGeneral>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  } else {
-    e = cudaFuncSetAttribute(knn_query_kernel<kPow2>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(knn_query_kernel<kPowGeneral>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(sync_smem));
   }
   if (e != cudaSuccess) return e;
   e = launch_grid_sort(data, n, queries, m, 0.0, k, workspace, L, sm_count, s, sort_queries);
@@ -2360,11 +2832,16 @@ cudaError_t launch_knn(const float* data, int64_t n, const float* queries, int64
   block_prefix_kernel<<<kMaxBlocksPerAxis, kMaxBlocksPerAxis, 0, s>>>(grid, starts_d, sums, bpre);
   sat_kernel<<<(kMaxCellsPerAxis + 1 + kSatCols - 1) / kSatCols, kSatCols * kSatWarps, 0, s>>>(
       grid, starts_d, sums, sat);
+  if (!warp_search)
+    return launch_knn_search(
+        KnnArgs{reinterpret_cast<GridDev*>(ws + L.off_grid), sorted, starts_d, sums, bpre, sat, qrec,
+                data, n, m, p, k, out, nbr_out, kd2_out, hit_out, sort_rows,
+                reinterpret_cast<int32_t*>(ws + L.off_hard)},
+        sm_count, s);
   const unsigned qgrid = static_cast<unsigned>((m + kKnnThreads - 1) / kKnnThreads);
-  auto kernel = warp_search ? (p == 2.0 ? knn_sync_kernel<kPow2> : knn_sync_kernel<kPowGeneral>)
-                            : (p == 2.0 ? knn_query_kernel<kPow2> : knn_query_kernel<kPowGeneral>);
-  kernel<<<qgrid, kKnnThreads, smem, s>>>(grid, sorted, starts_d, sums, bpre, sat, qrec, data, n,
-                                          m, p, k, out, nbr_out, kd2_out, hit_out, sort_rows);
+  auto kernel = p == 2.0 ? knn_sync_kernel<kPow2> : knn_sync_kernel<kPowGeneral>;
+  kernel<<<qgrid, kKnnThreads, sync_smem, s>>>(grid, sorted, starts_d, sums, bpre, sat, qrec, data, n,
+                                               m, p, k, out, nbr_out, kd2_out, hit_out, sort_rows);
   return cudaGetLastError();
 }
 
@@ -2379,6 +2856,7 @@ __global__ void index_prep_kernel(const GridDev* __restrict__ src, GridDev* __re
   GridDev g = *src;
   g.box_ticket = 0xffffffffu;
   g.scan_ticket = 0xffffffffu;
+  g.hard = 0u;
   if (radius > 0.0 && g.inv2 > 0.f)
     g.rho = __fmaf_ru(__fmul_ru(__double2float_ru(radius), g.inv2), 0.5f + 0x1p-9f, 0x1p-8f);
   *dst = g;
@@ -2445,6 +2923,7 @@ QueryLayout query_layout(int64_t m, int64_t max_cells) {
   Q.off_starts = off;  off += round_up(len, 256);
   Q.off_sums = off;    off += round_up(size_t(2 * scan_tiles_of(max_cells)) * 4, 256);
   Q.off_qrec = off;    off += round_up(size_t(m) * 16, 256);
+  Q.off_hard = off;    off += round_up(size_t(m) * 4, 256);
   Q.bytes = off;
   return Q;
 }
@@ -2524,20 +3003,12 @@ cudaError_t launch_index_knn(const void* index_mem, const IndexLayout& X, const 
                              int64_t m, double p, int k, float* out, int32_t* nbr_out,
                              float* kd2_out, void* workspace, const QueryLayout& Q, int sm_count,
                              cudaStream_t s, bool sort_queries) {
-  const size_t smem = knn_smem_bytes(k);
-  cudaError_t e = cudaFuncSetAttribute(knn_query_kernel<kPow2>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(knn_query_kernel<kPowGeneral>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-  if (e != cudaSuccess) return e;
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
-  e = launch_query_sort(xgrid, queries, m, 0.0, X.max_cells, workspace, Q, sm_count, s,
-                        sort_queries);
+  cudaError_t e = launch_query_sort(xgrid, queries, m, 0.0, X.max_cells, workspace, Q, sm_count, s,
+                                    sort_queries);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  const GridDev* grid = reinterpret_cast<const GridDev*>(ws + Q.off_grid);
   const float4* qrec = reinterpret_cast<const float4*>(ws + Q.off_qrec);
   const int32_t* starts = reinterpret_cast<const int32_t*>(mem + X.off_starts);
   const int32_t* sums = reinterpret_cast<const int32_t*>(mem + X.off_sums);
@@ -2545,16 +3016,11 @@ cudaError_t launch_index_knn(const void* index_mem, const IndexLayout& X, const 
   const float* data = reinterpret_cast<const float*>(mem + X.off_data);
   const int32_t* bpre = reinterpret_cast<const int32_t*>(mem + X.off_bpre);
   const int32_t* sat = reinterpret_cast<const int32_t*>(mem + X.off_sat);
-  const unsigned qgrid = static_cast<unsigned>((m + kKnnThreads - 1) / kKnnThreads);
-  if (p == 2.0)
-    knn_query_kernel<kPow2><<<qgrid, kKnnThreads, smem, s>>>(
-        grid, sorted, starts, sums, bpre, sat, qrec, data, X.n, m, p, k, out, nbr_out, kd2_out,
-        nullptr, true);
-  else
-    knn_query_kernel<kPowGeneral><<<qgrid, kKnnThreads, smem, s>>>(
-        grid, sorted, starts, sums, bpre, sat, qrec, data, X.n, m, p, k, out, nbr_out, kd2_out,
-        nullptr, true);
-  return cudaGetLastError();
+  return launch_knn_search(
+      KnnArgs{reinterpret_cast<GridDev*>(ws + Q.off_grid), sorted, starts, sums, bpre, sat, qrec, data,
+              X.n, m, p, k, out, nbr_out, kd2_out, nullptr, true,
+              reinterpret_cast<int32_t*>(ws + Q.off_hard)},
+      sm_count, s);
 }
 
 }  // namespace idw

@@ -14,7 +14,7 @@ namespace idw {
 struct LocalLayout {
   int64_t max_cells = 0;
   size_t off_grid = 0, off_counts_d = 0, off_counts_q = 0, off_starts_d = 0, off_starts_q = 0;
-  size_t off_sums = 0, off_sorted = 0, off_qrec = 0, off_bpre = 0, off_sat = 0;
+  size_t off_sums = 0, off_sorted = 0, off_qrec = 0, off_hard = 0, off_bpre = 0, off_sat = 0;
   size_t bytes = 0;
 };
 
@@ -89,7 +89,7 @@ IndexLayout index_layout(int64_t n, bool knn);
 
 // Scratch of one query call on a prepared index (in the handle's workspace).
 struct QueryLayout {
-  size_t off_grid = 0, off_counts = 0, off_starts = 0, off_sums = 0, off_qrec = 0;
+  size_t off_grid = 0, off_counts = 0, off_starts = 0, off_sums = 0, off_qrec = 0, off_hard = 0;
   size_t bytes = 0;
 };
 QueryLayout query_layout(int64_t m, int64_t max_cells);

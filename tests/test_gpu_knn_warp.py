@@ -1,0 +1,67 @@
+"""The k-NN search by warps (few queries, or queries whose surroundings are
+empty or dense) against the FP64 oracle: neighbour lists equal, k-th key and
+hits equal, values within the FP32 bar.  Sizes sit at its edges: one and a
+few points, fewer points than k, buffers of 32, 64 and more keys, ties, the
+call sizes where the search changes, and queries outside the data's box."""
+import numpy as np
+import pytest
+
+import oracle
+import synthetic
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(data, queries, k, p=2.0, index=False):
+    import torch
+    import paper_1402_4986_gb300 as idw
+    d, q = torch.from_numpy(data).cuda(), torch.from_numpy(queries).cuda()
+    if index:
+        Z, nbr, kd2 = idw.LocalIndex(d, k=8).knn(q, p, k, neighbours=True, kth_d2=True)
+    else:
+        Z, nbr, kd2 = idw.interpolate_knn(d, q, p, k, neighbours=True, kth_d2=True)
+    idw.sync_status()
+    want = oracle.idw_knn(data, queries, p, k)
+    assert np.array_equal(nbr.cpu().numpy(), want["nbr"])
+    assert np.array_equal(kd2.cpu().numpy(), want["kd2"].astype(np.float32))
+    err = np.abs(Z.cpu().numpy() - want["Z"])
+    assert np.max(err) <= 2e-6 * np.max(np.abs(data[:, 2]))
+
+
+@pytest.mark.parametrize("k", [1, 2, 8, 31, 32, 33, 63, 64])
+@pytest.mark.parametrize("n", [1, 5, 64, 3001])
+def test_few_queries(n, k):
+    prob = synthetic.uniform_problem(n, 203, seed=n + k, exact_hits=min(n, 5))
+    _check(prob["data"], prob["queries"], k, index=n > 64)
+
+
+@pytest.mark.parametrize("k", [1, 8, 40])
+def test_clustered(k):
+    prob = synthetic.config_local(n=20000, m=2000, clustered=True)
+    q = prob["queries"] * 3.0 - 1.0  # a third of the box inside the data's
+    _check(prob["data"], np.ascontiguousarray(q), k, p=3.5)
+
+
+def test_hard_queries_of_a_larger_call():
+    """10,000 queries at k = 1 (above the all-warps size of 9216): the queries
+    far from the blobs go to warps, those inside to threads."""
+    prob = synthetic.config_local(n=30000, m=10000, clustered=True)
+    _check(prob["data"], prob["queries"], 1)
+
+
+def test_ties_and_duplicates():
+    """A lattice (equal distances throughout) with every point doubled, and
+    queries on its points and cell centres: ties go to the lower index."""
+    xy = synthetic.grid_xy(24)
+    xy = np.concatenate([xy, xy])
+    data = synthetic.pack_xyz(xy, np.arange(len(xy), dtype=np.float32) / len(xy))
+    queries = np.concatenate([xy[:100], synthetic.grid_xy(12)]).astype(np.float32)
+    for k in (3, 32, 50):
+        _check(data, np.ascontiguousarray(queries), k)
+
+
+def test_far_queries():
+    """Queries from 10 to 1e9 box widths away."""
+    prob = synthetic.uniform_problem(4000, 12, seed=9)
+    q = (prob["queries"] + np.float32(10.0) ** np.arange(1, 13)[:, None] % np.float32(1e9))
+    _check(prob["data"], np.ascontiguousarray(q.astype(np.float32)), 8)
