@@ -45,6 +45,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 
 #include "idw.h"
 #include "idw_device.cuh"
@@ -97,7 +98,7 @@ struct GridDev {
   float hx0, hy0, inv2;  // cell position u(v) = fl(fl(fl(v/2) - h0) * inv2)
   float rho;             // reach of R in cells, with margin (< 2)
   int gx, gy, cells;
-  unsigned hard;         // k-NN queries the single-thread search left to warps
+  unsigned hard;         // queries the per-thread kernels left to warps
 };
 
 // Order-preserving unsigned key of a float (for atomic min).
@@ -513,6 +514,12 @@ __device__ __forceinline__ float fp32_d2(float qx, float qy, float x, float y) {
 struct Runs {
   int a[5], b[5];
 
+  __device__ __forceinline__ int candidates() const {
+    int c = 0;
+#pragma unroll
+    for (int r = 0; r < 5; ++r) c += b[r] - a[r];
+    return c;
+  }
   __device__ __forceinline__ Runs(const GridDev& g, float qx, float qy,
                                   const int32_t* __restrict__ starts,
                                   const int32_t* __restrict__ base) {
@@ -540,6 +547,67 @@ struct Runs {
   }
 };
 
+// A query's runs laid end to end: candidate s of `total` sits at at(s), so
+// that one lane, or the 32 lanes of a warp side by side, can walk them.
+struct FlatRuns {
+  int end[5], shift[5];  // candidates s < end[r] (and >= end[r - 1]) sit at s + shift[r]
+
+  __device__ __forceinline__ explicit FlatRuns(const Runs& runs) {
+    int e = 0;
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+      shift[r] = runs.a[r] - e;
+      e += runs.b[r] - runs.a[r];
+      end[r] = e;
+    }
+  }
+  __device__ __forceinline__ int total() const { return end[4]; }
+  __device__ __forceinline__ int at(int s) const {
+    int d = shift[0];
+#pragma unroll
+    for (int r = 1; r < 5; ++r) d = s >= end[r - 1] ? shift[r] : d;
+    return s + d;
+  }
+};
+
+// Heavy queries: those with more candidates than `heavy_candidates`.  A
+// thread walks its candidates one load after another while the other lanes
+// wait, so heavy queries are listed and each is given a whole warp by a
+// kernel of their own.  At the mean density a query has about 21 cells of
+// candidates.  Calls that do not fill the GPU (few = true) list queries a
+// little above that; others, whose warps hide each other's loads, only those
+// several times above it.  200,003 points in 64 blobs, 150,001 uniform
+// queries, R for 16 members at the mean density (up to 1400 candidates a
+// query, modified Shepard): values 178 -> 18 us for the heavy queries and
+// 60 us for the rest, query gradients 680 -> 47 and 150 us.
+__device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, bool few) {
+  const float per_cell = float(n) * rcp_approx(float(g.cells));
+  return int(few ? fminf(fmaf(24.f, per_cell, 32.f), 1e9f) : fminf(fmaf(64.f, per_cell, 256.f), 1e9f));
+}
+// Lists query t (any subset of a warp's lanes may call it together).
+__device__ __forceinline__ void list_heavy(int64_t t, int64_t m, unsigned* __restrict__ count,
+                                           int32_t* __restrict__ list) {
+  const unsigned lanes = __activemask();  // one atomic for those that are here together
+  const int lane = threadIdx.x & 31, lead = __ffs(lanes) - 1;
+  unsigned at = 0;
+  if (lane == lead) at = atomicAdd(count, unsigned(__popc(lanes)));
+  at = __shfl_sync(lanes, at, lead) + __popc(lanes & ((1u << lane) - 1));
+  if (dcheck(at < m, kSiteScatter)) list[at] = static_cast<int32_t>(t);
+}
+
+// Error-free sum of the lanes' compensated pairs (both packed lanes), by a
+// fixed tree; lane 0's total is returned to every lane.
+__device__ __forceinline__ void warp_sum_pairs(u64& hi, u64& lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const u64 oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+    two_sum_acc(hi, lo, oh);
+    lo = add2(lo, ol);
+  }
+  hi = __shfl_sync(0xffffffffu, hi, 0);
+  lo = __shfl_sync(0xffffffffu, lo, 0);
+}
+
 // One thread per query, in cell order.  The fast loop takes every candidate
 // with d^2 < r2t, r2t = fl32(R^2) (or the least subnormal when that is 0,
 // so that only d^2 == 0 passes), and sums its FP32 weight.  A coincident
@@ -565,62 +633,53 @@ __device__ __forceinline__ float modified_weight(float d2, float inv_r, float pw
   return ex2_approx(pw * lg2_approx(t));
 }
 
-template <int MODE, int WMODE = kWeightShepard>
-__global__ void __launch_bounds__(kLocalThreads)
-    local_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                       int64_t n, const int32_t* __restrict__ starts,
-                       const int32_t* __restrict__ base, const float4* __restrict__ qrec,
-                       int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
-                       int32_t* __restrict__ count_out, double radius = 0.0) {
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= m) return;
-  const float4 r = qrec[t];
-  const float qx = r.x, qy = r.y;
-  const int j = __float_as_int(r.z);
-  if (!dcheck(j >= 0 && j < m, kSiteOutput)) return;
-  const Runs runs(*grid, qx, qy, starts, base);
-  const float hp = static_cast<float>(0.5 * p), nhp = -hp;
-  const float pw = static_cast<float>(p);
-  const float inv_r = WMODE == kWeightModified ? static_cast<float>(1.0 / radius) : 0.f;
-
-  // (sum w, sum w z) and their TwoSum errors.  The products w z are rounded
-  // once (2^-24), below the error of the MUFU weights themselves (2^-23).
+// One candidate: adds a member's (w, w z) to the compensated pair.  The
+// products w z are rounded once (2^-24), below the error of the MUFU weights
+// themselves (2^-23).
+template <int MODE, int WMODE>
+struct ValueSums {
   u64 hi = 0, lo = 0;
   int cnt = 0;
-#pragma unroll
-  for (int r = 0; r < 5; ++r) {
-#pragma unroll 2
-    for (int k = runs.a[r]; k < runs.b[r]; ++k) {
-      if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
-      const float4 v = sorted[k];
-      const float d2 = fp32_d2(qx, qy, v.x, v.y);
-      if (d2 < r2t) {
-        const float w = WMODE == kWeightModified ? modified_weight<MODE>(d2, inv_r, pw)
-                                                 : local_weight<MODE>(d2, hp, nhp);
-        two_sum_acc(hi, lo, pk(w, __fmul_rn(w, v.z)));
-        ++cnt;
-      }
+  __device__ __forceinline__ void consider(const float4 v, float qx, float qy, float r2t,
+                                           float inv_r, float hp, float pw) {
+    const float d2 = fp32_d2(qx, qy, v.x, v.y);
+    if (d2 < r2t) {
+      const float w = WMODE == kWeightModified ? modified_weight<MODE>(d2, inv_r, pw)
+                                               : local_weight<MODE>(d2, hp, -hp);
+      two_sum_acc(hi, lo, pk(w, __fmul_rn(w, v.z)));
+      ++cnt;
     }
   }
-  if (cnt == 0) {  // no member and no coincident point
-    out[j] = __int_as_float(0x7fc00000);
-    if (count_out) count_out[j] = 0;
-    return;
-  }
-  float h0, h1, l0, l1;
-  upk(hi, h0, h1);
-  upk(lo, l0, l1);
-  if (h0 >= kTinyPerMember * float(cnt) && h0 <= FLT_MAX && fabsf(h1) <= FLT_MAX &&
-      fabsf(l1) <= FLT_MAX) {
+  // Z, if the sums stayed in FP32's range.
+  __device__ __forceinline__ bool value(float& z) const {
+    float h0, h1, l0, l1;
+    upk(hi, h0, h1);
+    upk(lo, l0, l1);
+    if (!(h0 >= kTinyPerMember * float(cnt) && h0 <= FLT_MAX && fabsf(h1) <= FLT_MAX &&
+          fabsf(l1) <= FLT_MAX))
+      return false;
     // Z = (h1 + l1) / (h0 + l0): quotient, then one residual correction.
     const float z0 = __fdiv_rn(h1, h0);
     const float res = __fadd_rn(__fmaf_rn(-z0, h0, h1), __fmaf_rn(-z0, l0, l1));
-    out[j] = __fmaf_rn(res, rcp_approx(h0), z0);
-    if (count_out) count_out[j] = cnt;
-    return;
+    z = __fmaf_rn(res, rcp_approx(h0), z0);
+    return true;
   }
-  // FP64 pass: exact hits first, then the members' d2_min (or, for the
-  // modified weights, their largest base (R - d)/(R d), clamped at 0).
+};
+
+// The FP64 pass of one query, by one lane (WARP false) or a whole warp: exact
+// hits first, then the members' d2_min (or, for the modified weights, their
+// largest base (R - d)/(R d), clamped at 0) and the sums scaled by it.
+struct ValueF64 {
+  float z;
+  int count;
+};
+template <int WMODE, bool WARP>
+__device__ __forceinline__ ValueF64 local_value_f64(const FlatRuns& fr,
+                                                    const float4* __restrict__ sorted, float qx,
+                                                    float qy, double p, float r2f, double radius) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int step = WARP ? 32 : 1;
+  const int first = WARP ? int(threadIdx.x & 31) : 0;
   int best = INT_MAX, members = 0;
   float bestz = 0.f;
   double dmin = INFINITY, tmax = 0.0;
@@ -629,43 +688,145 @@ __global__ void __launch_bounds__(kLocalThreads)
     const double t = isinf(radius) ? 1.0 / d : (radius - d) / (radius * d);
     return t > 0.0 ? t : 0.0;
   };
-#pragma unroll
-  for (int r = 0; r < 5; ++r)
-    for (int k = runs.a[r]; k < runs.b[r]; ++k) {
-      const float4 v = sorted[k];
-      if (v.x == qx && v.y == qy) {
-        const int idx = __float_as_int(v.w);
-        if (idx < best) {
-          best = idx;
-          bestz = v.z;
-        }
-      } else if (fp32_d2(qx, qy, v.x, v.y) < r2f) {
-        const double ex = double(qx) - v.x, ey = double(qy) - v.y;
-        dmin = fmin(dmin, ex * ex + ey * ey);
-        if (WMODE == kWeightModified) tmax = fmax(tmax, base64(ex * ex + ey * ey));
-        ++members;
+  for (int i = first; i < fr.total(); i += step) {
+    const float4 v = sorted[fr.at(i)];
+    if (v.x == qx && v.y == qy) {
+      const int idx = __float_as_int(v.w);
+      if (idx < best) {
+        best = idx;
+        bestz = v.z;
       }
+    } else if (fp32_d2(qx, qy, v.x, v.y) < r2f) {
+      const double ex = double(qx) - v.x, ey = double(qy) - v.y;
+      dmin = fmin(dmin, ex * ex + ey * ey);
+      if (WMODE == kWeightModified) tmax = fmax(tmax, base64(ex * ex + ey * ey));
+      ++members;
     }
-  if (best != INT_MAX || members == 0 || (WMODE == kWeightModified && !(tmax > 0.0))) {
-    out[j] = best != INT_MAX ? bestz : __int_as_float(0x7fc00000);
-    if (count_out) count_out[j] = best != INT_MAX ? -1 : members;
+  }
+  if (WARP) {
+    const int lowest = __reduce_min_sync(kAll, best);
+    const unsigned who = __ballot_sync(kAll, best == lowest);
+    bestz = __shfl_sync(kAll, bestz, __ffs(who) - 1);
+    best = lowest;
+    members = __reduce_add_sync(kAll, members);
+    for (int o = 16; o > 0; o >>= 1) {
+      dmin = fmin(dmin, __shfl_xor_sync(kAll, dmin, o));
+      tmax = fmax(tmax, __shfl_xor_sync(kAll, tmax, o));
+    }
+  }
+  if (best != INT_MAX) return ValueF64{bestz, -1};
+  if (members == 0 || (WMODE == kWeightModified && !(tmax > 0.0)))
+    return ValueF64{__int_as_float(0x7fc00000), members};
+  double s0 = 0.0, s1 = 0.0;
+  for (int i = first; i < fr.total(); i += step) {
+    const float4 v = sorted[fr.at(i)];
+    if (fp32_d2(qx, qy, v.x, v.y) < r2f) {
+      const double ex = double(qx) - v.x, ey = double(qy) - v.y;
+      const double w = WMODE == kWeightModified ? pow(base64(ex * ex + ey * ey) / tmax, p)
+                                                : pow(dmin / (ex * ex + ey * ey), 0.5 * p);
+      s0 += w;
+      s1 += w * double(v.z);
+    }
+  }
+  if (WARP) {
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
+  }
+  return ValueF64{static_cast<float>(s1 / s0), members};
+}
+
+template <int MODE, int WMODE = kWeightShepard>
+__global__ void __launch_bounds__(kLocalThreads)
+    local_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
+                       int64_t n, const int32_t* __restrict__ starts,
+                       const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+                       int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
+                       int32_t* __restrict__ count_out, double radius, bool few,
+                       unsigned* __restrict__ heavy_count, int32_t* __restrict__ heavy) {
+  pdl_trigger();
+  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= m) return;
+  const float4 r = qrec[t];
+  const float qx = r.x, qy = r.y;
+  const int j = __float_as_int(r.z);
+  if (!dcheck(j >= 0 && j < m, kSiteOutput)) return;
+  const Runs runs(*grid, qx, qy, starts, base);
+  if (runs.candidates() > heavy_candidates(*grid, n, few)) {
+    list_heavy(t, m, heavy_count, heavy);
     return;
   }
-  double s0 = 0.0, s1 = 0.0;
+  const float hp = static_cast<float>(0.5 * p);
+  const float pw = static_cast<float>(p);
+  const float inv_r = WMODE == kWeightModified ? static_cast<float>(1.0 / radius) : 0.f;
+  ValueSums<MODE, WMODE> sums;
+  // Four loads in flight: a candidate's FP32 work is short next to its load.
 #pragma unroll
-  for (int r = 0; r < 5; ++r)
+  for (int r = 0; r < 5; ++r) {
+#pragma unroll 4
     for (int k = runs.a[r]; k < runs.b[r]; ++k) {
-      const float4 v = sorted[k];
-      if (fp32_d2(qx, qy, v.x, v.y) < r2f) {
-        const double ex = double(qx) - v.x, ey = double(qy) - v.y;
-        const double w = WMODE == kWeightModified ? pow(base64(ex * ex + ey * ey) / tmax, p)
-                                                  : pow(dmin / (ex * ex + ey * ey), 0.5 * p);
-        s0 += w;
-        s1 += w * double(v.z);
-      }
+      if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
+      sums.consider(sorted[k], qx, qy, r2t, inv_r, hp, pw);
     }
-  out[j] = static_cast<float>(s1 / s0);
-  if (count_out) count_out[j] = members;
+  }
+  float z = __int_as_float(0x7fc00000);  // no member and no coincident point
+  int cnt = sums.cnt;
+  if (cnt > 0 && !sums.value(z)) {
+    const ValueF64 v = local_value_f64<WMODE, false>(FlatRuns(runs), sorted, qx, qy, p, r2f, radius);
+    z = v.z;
+    cnt = v.count;
+  }
+  out[j] = z;
+  if (count_out) count_out[j] = cnt;
+}
+
+// The heavy queries, a warp each: 32 candidates side by side, the lanes'
+// sums joined by a fixed tree of error-free additions.
+constexpr int kHeavyThreads = 128;
+template <int MODE, int WMODE = kWeightShepard>
+__global__ void __launch_bounds__(kHeavyThreads)
+    local_heavy_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
+                       int64_t n, const int32_t* __restrict__ starts,
+                       const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+                       int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
+                       int32_t* __restrict__ count_out, double radius,
+                       const unsigned* __restrict__ heavy_count,
+                       const int32_t* __restrict__ heavy) {
+  pdl_wait();
+  const int64_t count = *heavy_count;
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = int64_t(gridDim.x) * (kHeavyThreads / 32);
+  const float hp = static_cast<float>(0.5 * p), pw = static_cast<float>(p);
+  const float inv_r = WMODE == kWeightModified ? static_cast<float>(1.0 / radius) : 0.f;
+  for (int64_t w = (int64_t(blockIdx.x) * kHeavyThreads + threadIdx.x) / 32; w < count;
+       w += warps) {
+    const int64_t t = heavy[w];
+    if (!dcheck(t >= 0 && t < m, kSiteScatter)) continue;
+    const float4 r = qrec[t];
+    const float qx = r.x, qy = r.y;
+    const int j = __float_as_int(r.z);
+    if (!dcheck(j >= 0 && j < m, kSiteOutput)) continue;
+    const FlatRuns fr(Runs(*grid, qx, qy, starts, base));
+    ValueSums<MODE, WMODE> sums;
+#pragma unroll 2
+    for (int i = lane; i < fr.total(); i += 32) {
+      const int k = fr.at(i);
+      if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
+      sums.consider(sorted[k], qx, qy, r2t, inv_r, hp, pw);
+    }
+    warp_sum_pairs(sums.hi, sums.lo);
+    sums.cnt = __reduce_add_sync(0xffffffffu, sums.cnt);
+    float z = __int_as_float(0x7fc00000);
+    int cnt = sums.cnt;
+    if (cnt > 0 && !sums.value(z)) {  // the same in every lane
+      const ValueF64 v = local_value_f64<WMODE, true>(fr, sorted, qx, qy, p, r2f, radius);
+      z = v.z;
+      cnt = v.count;
+    }
+    if (lane == 0) {
+      out[j] = z;
+      if (count_out) count_out[j] = cnt;
+    }
+  }
 }
 
 // ------------------------------------------------- local-form gradients
@@ -799,6 +960,169 @@ __device__ __forceinline__ float modified_ratio(float a, float b, float lb, floa
   return ex2_approx(pf * (lg2_approx(a) - lb));
 }
 
+// First pass of one query: hit, members, and the sums with weights scaled by
+// the heaviest member so far (the smallest d^2, or for the modified weights
+// the largest base 1/d - 1/R), rescaled as in an online softmax when a
+// heavier one appears, so every scaled weight stays <= 1.  (sum w, sum w z)
+// is a compensated pair, as in the forward pass: Z and g / S0 then stay
+// accurate however many members a query has.
+template <int MODE, int WMODE>
+struct GradSums {
+  static constexpr bool kMod = WMODE == kWeightModified;
+  int best = INT_MAX, members = 0;
+  float d2min = INFINITY, scale = kMod ? 0.f : INFINITY, lsc = 0.f;
+  u64 hi = 0, lo = 0;
+
+  __device__ __forceinline__ static float log_of(float s) {
+    return MODE == kPow2 ? 0.f : lg2_approx(s);
+  }
+  __device__ __forceinline__ void consider(const float4 v, float qx, float qy, float r2f,
+                                           float r2t, float inv_r, float hp, float pf) {
+    const float d2 = fp32_d2(qx, qy, v.x, v.y);
+    if (!(d2 < r2t)) return;
+    if (v.x == qx && v.y == qy) {
+      best = min(best, __float_as_int(v.w));
+      return;
+    }
+    if (!(d2 < r2f)) return;
+    ++members;
+    d2min = fminf(d2min, d2);
+    const float s = kMod ? fmaxf(rsqrt_approx(d2) - inv_r, 0.f) : d2;
+    if (kMod && !(s > 0.f)) return;  // zero weight
+    if (kMod ? s > scale : s < scale) {
+      const float l = log_of(s);
+      if (kMod ? scale > 0.f : members > 1) {
+        // (t_old / t)^p, or (d2 / d2_old)^(p/2): the old sums shrink.
+        const float f = kMod ? modified_ratio<MODE>(scale, s, l, pf)
+                             : grad_weight<MODE>(scale, s, l, hp);
+        hi = mul2(hi, pk(f, f));
+        lo = mul2(lo, pk(f, f));
+      }
+      scale = s;
+      lsc = l;
+    }
+    const float w = kMod ? modified_ratio<MODE>(s, scale, lsc, pf)
+                         : grad_weight<MODE>(s, scale, lsc, hp);
+    two_sum_acc(hi, lo, pk(w, __fmul_rn(w, v.z)));
+  }
+  // The lanes' sums over their shares of one query, joined: each lane's are
+  // rescaled to the heaviest member of all, then added.
+  __device__ __forceinline__ void join(float hp, float pf) {
+    best = __reduce_min_sync(0xffffffffu, best);
+    members = __reduce_add_sync(0xffffffffu, members);
+    float top = scale;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      d2min = fminf(d2min, __shfl_xor_sync(0xffffffffu, d2min, o));
+      const float other = __shfl_xor_sync(0xffffffffu, top, o);
+      top = kMod ? fmaxf(top, other) : fminf(top, other);
+    }
+    const float l = log_of(top);
+    if (kMod ? scale > 0.f && scale < top : scale < INFINITY && scale > top) {
+      const float f = kMod ? modified_ratio<MODE>(scale, top, l, pf)
+                           : grad_weight<MODE>(scale, top, l, hp);
+      hi = mul2(hi, pk(f, f));
+      lo = mul2(lo, pk(f, f));
+    }
+    scale = top;
+    lsc = l;
+    warp_sum_pairs(hi, lo);
+  }
+  __device__ __forceinline__ bool has_weight() const {
+    return members > 0 && (!kMod || scale > 0.f);
+  }
+  // Z = (h1 + l1) / (h0 + l0): quotient, then one residual correction.
+  __device__ __forceinline__ float value(float& s0) const {
+    float h0, h1, l0, l1;
+    upk(hi, h0, h1);
+    upk(lo, l0, l1);
+    s0 = h0 + l0;
+    const float z0 = __fdiv_rn(h1, h0);
+    return __fmaf_rn(__fadd_rn(__fmaf_rn(-z0, h0, h1), __fmaf_rn(-z0, l0, l1)), rcp_approx(h0), z0);
+  }
+};
+
+// Second pass: the sums of dL/dq (x and y) and of the dL/dp share.
+template <int MODE, int WMODE>
+struct GradTerms {
+  float ax = 0.f, ay = 0.f, al = 0.f;
+  __device__ __forceinline__ void consider(const float4 v, float qx, float qy, float r2f,
+                                           float inv_r, float hp, float pf, float Z, float scale,
+                                           float lsc, float lsc2) {
+    constexpr bool kMod = WMODE == kWeightModified;
+    const float dx = __fsub_rn(qx, v.x), dy = __fsub_rn(qy, v.y);
+    const float d2 = __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
+    if (!(d2 < r2f)) return;
+    float w, ar, lt;
+    if (kMod) {
+      const float id = rsqrt_approx(d2);
+      const float tb = fmaxf(id - inv_r, 0.f);
+      if (!(tb > 0.f)) return;
+      w = modified_ratio<MODE>(tb, scale, lsc, pf);
+      ar = (v.z - Z) * w * (id * id) * (id * rcp_approx(tb));  // / (t d^3)
+      lt = lg2_approx(tb) - lsc2;
+    } else {
+      w = grad_weight<MODE>(d2, scale, lsc, hp);
+      ar = (v.z - Z) * w * rcp_approx(d2);  // / d^2
+      lt = lg2_approx(d2) - lsc2;
+    }
+    ax = fmaf(ar, dx, ax);
+    ay = fmaf(ar, dy, ay);
+    al = fmaf((v.z - Z) * w, lt, al);
+  }
+};
+
+// One query's result from its two passes (one lane): its record for the
+// data-side kernel, dL/dq, and its share of dL/dp (returned).
+template <int MODE, int WMODE>
+__device__ __forceinline__ double grad_finish(const GradSums<MODE, WMODE>& sums,
+                                              const GradTerms<MODE, WMODE>& terms, bool second,
+                                              float Z, float s0, float gj, int j, int64_t t,
+                                              const Runs& runs, const float4* __restrict__ sorted,
+                                              float qx, float qy, float r2f, double p,
+                                              double radius, float* __restrict__ grad_q,
+                                              LocalGradRec* __restrict__ rec,
+                                              LocalGradRec64* __restrict__ rec64) {
+  constexpr bool kMod = WMODE == kWeightModified;
+  LocalGradRec out{0.f, 0.f, 0.f, kGradHitNone};
+  float gqx = 0.f, gqy = 0.f;
+  double gp = 0.0;
+  if (sums.best != INT_MAX) {
+    out.code = sums.best;
+    out.c = gj;
+  } else if (sums.has_weight()) {
+    bool f32 = second;
+    if (second) {
+      const float pf = static_cast<float>(p), c = gj / s0, k1 = c * pf;
+      gqx = -k1 * terms.ax;
+      gqy = -k1 * terms.ay;
+      // dL/dp share in FP32 (no FP64 divide): -ln2/2 c al for d^-p,
+      // +ln2 c al for the modified weights (dw/dp = w ln t).
+      const float gpf = (kMod ? 0.6931471805599453f : -0.5f * 0.6931471805599453f) * c * terms.al;
+      gp = gpf;
+      out.code = kGradF32;
+      out.c = c;
+      out.z = Z;
+      out.d2min = sums.scale;
+      f32 = isfinite(Z) && isfinite(gqx) && isfinite(gqy) && isfinite(gpf) && isfinite(c);
+    }
+    if (!f32) {  // FP64: weights scaled by the exact scale
+      const GradF64 r64 = grad_query_f64(runs, sorted, qx, qy, r2f, p, gj, kMod, radius);
+      gqx = r64.gqx;
+      gqy = r64.gqy;
+      gp = r64.gp;
+      out.code = r64.rec.c == 0.0 && r64.rec.d2min == 0.0 ? kGradHitNone : kGradF64;
+      rec64[t] = r64.rec;
+    }
+  }
+  rec[t] = out;
+  if (grad_q) {
+    grad_q[2 * int64_t(j)] = gqx;
+    grad_q[2 * int64_t(j) + 1] = gqy;
+  }
+  return gp;
+}
+
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kLocalThreads)
     local_grad_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
@@ -807,8 +1131,9 @@ __global__ void __launch_bounds__(kLocalThreads)
                             int64_t m, double p, float r2f, float r2t,
                             const float* __restrict__ grad_out, float* __restrict__ grad_q,
                             double* __restrict__ grad_p, LocalGradRec* __restrict__ rec,
-                            LocalGradRec64* __restrict__ rec64, double radius) {
-  constexpr bool kMod = WMODE == kWeightModified;
+                            LocalGradRec64* __restrict__ rec64, double radius, bool few,
+                            unsigned* __restrict__ heavy_count, int32_t* __restrict__ heavy) {
+  pdl_trigger();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   double gp = 0.0;  // this query's share of dL/dp (every lane joins the warp sum)
   if (t < m) {
@@ -816,131 +1141,37 @@ __global__ void __launch_bounds__(kLocalThreads)
     const float qx = r.x, qy = r.y;
     const int j = __float_as_int(r.z);
     if (dcheck(j >= 0 && j < m, kSiteOutput)) {
-      const float gj = grad_out[j];
       const Runs runs(*grid, qx, qy, starts, base);
-      // One pass: hit, members, and the sums with weights scaled by the
-      // heaviest member so far (the smallest d^2, or for the modified
-      // weights the largest base 1/d - 1/R), rescaled as in an online softmax
-      // when a heavier one appears, so every scaled weight stays <= 1.
-      const float hp = static_cast<float>(0.5 * p), pf = static_cast<float>(p);
-      const float inv_r = kMod ? static_cast<float>(1.0 / radius) : 0.f;
-      int best = INT_MAX, members = 0;
-      float d2min = INFINITY, scale = kMod ? 0.f : INFINITY, lsc = 0.f;
-      // (sum w, sum w z) as a compensated pair, as in the forward pass: Z
-      // and g / S0 then stay accurate however many members a query has.
-      u64 hi = 0, lo = 0;
+      if (runs.candidates() > heavy_candidates(*grid, n, few)) {
+        list_heavy(t, m, heavy_count, heavy);
+      } else {
+        const float gj = grad_out[j];
+        const float hp = static_cast<float>(0.5 * p), pf = static_cast<float>(p);
+        const float inv_r = WMODE == kWeightModified ? static_cast<float>(1.0 / radius) : 0.f;
+        GradSums<MODE, WMODE> sums;
 #pragma unroll
-      for (int rr = 0; rr < 5; ++rr)
-        for (int k = runs.a[rr]; k < runs.b[rr]; ++k) {
-          if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
-          const float4 v = sorted[k];
-          const float d2 = fp32_d2(qx, qy, v.x, v.y);
-          if (!(d2 < r2t)) continue;
-          if (v.x == qx && v.y == qy) {
-            best = min(best, __float_as_int(v.w));
-            continue;
+        for (int rr = 0; rr < 5; ++rr)
+#pragma unroll 4
+          for (int k = runs.a[rr]; k < runs.b[rr]; ++k) {
+            if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
+            sums.consider(sorted[k], qx, qy, r2f, r2t, inv_r, hp, pf);
           }
-          if (!(d2 < r2f)) continue;
-          ++members;
-          d2min = fminf(d2min, d2);
-          float w;
-          if (kMod) {
-            const float tb = fmaxf(rsqrt_approx(d2) - inv_r, 0.f);
-            if (!(tb > 0.f)) continue;  // zero weight
-            if (tb > scale) {
-              const float l = MODE == kPow2 ? 0.f : lg2_approx(tb);
-              if (scale > 0.f) {
-                const float f = modified_ratio<MODE>(scale, tb, l, pf);  // (t_old / t)^p
-                hi = mul2(hi, pk(f, f));
-                lo = mul2(lo, pk(f, f));
-              }
-              scale = tb;
-              lsc = l;
-            }
-            w = modified_ratio<MODE>(tb, scale, lsc, pf);
-          } else {
-            if (d2 < scale) {
-              const float l = MODE == kPow2 ? 0.f : lg2_approx(d2);
-              if (members > 1) {
-                const float f = grad_weight<MODE>(scale, d2, l, hp);  // (d2 / d2min_old)^(p/2)
-                hi = mul2(hi, pk(f, f));
-                lo = mul2(lo, pk(f, f));
-              }
-              scale = d2;
-              lsc = l;
-            }
-            w = grad_weight<MODE>(d2, scale, lsc, hp);
-          }
-          two_sum_acc(hi, lo, pk(w, __fmul_rn(w, v.z)));
-        }
-      float h0, h1, l0, l1;
-      upk(hi, h0, h1);
-      upk(lo, l0, l1);
-      const float s0 = h0 + l0;
-      LocalGradRec out{0.f, 0.f, 0.f, kGradHitNone};
-      float gqx = 0.f, gqy = 0.f;
-      if (best != INT_MAX) {
-        out.code = best;
-        out.c = gj;
-      } else if (members > 0 && (!kMod || scale > 0.f)) {
-        bool f32 = d2min >= 0x1p-100f;
-        if (f32) {
-          // Z = (h1 + l1) / (h0 + l0): quotient, then one residual correction.
-          const float z0 = __fdiv_rn(h1, h0);
-          const float Z = __fmaf_rn(__fadd_rn(__fmaf_rn(-z0, h0, h1), __fmaf_rn(-z0, l0, l1)),
-                                    rcp_approx(h0), z0);
-          const float lsc2 = lg2_approx(scale);
-          float ax = 0.f, ay = 0.f, al = 0.f;
+        // A query with members and no hit, in FP32's range, takes the second pass.
+        const bool second =
+            sums.best == INT_MAX && sums.has_weight() && sums.d2min >= 0x1p-100f;
+        float s0 = 1.f, Z = 0.f;
+        GradTerms<MODE, WMODE> terms;
+        if (second) {
+          Z = sums.value(s0);
+          const float lsc2 = lg2_approx(sums.scale);
 #pragma unroll
           for (int rr = 0; rr < 5; ++rr)
-            for (int k = runs.a[rr]; k < runs.b[rr]; ++k) {
-              const float4 v = sorted[k];
-              const float dx = __fsub_rn(qx, v.x), dy = __fsub_rn(qy, v.y);
-              const float d2 = __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
-              if (!(d2 < r2f)) continue;
-              float w, ar, lt;
-              if (kMod) {
-                const float id = rsqrt_approx(d2);
-                const float tb = fmaxf(id - inv_r, 0.f);
-                if (!(tb > 0.f)) continue;
-                w = modified_ratio<MODE>(tb, scale, lsc, pf);
-                ar = (v.z - Z) * w * (id * id) * (id * rcp_approx(tb));  // / (t d^3)
-                lt = lg2_approx(tb) - lsc2;
-              } else {
-                w = grad_weight<MODE>(d2, scale, lsc, hp);
-                ar = (v.z - Z) * w * rcp_approx(d2);  // / d^2
-                lt = lg2_approx(d2) - lsc2;
-              }
-              ax = fmaf(ar, dx, ax);
-              ay = fmaf(ar, dy, ay);
-              al = fmaf((v.z - Z) * w, lt, al);
-            }
-          const float c = gj / s0, k1 = c * pf;
-          gqx = -k1 * ax;
-          gqy = -k1 * ay;
-          // dL/dp share in FP32 (no FP64 divide): -ln2/2 c al for d^-p,
-          // +ln2 c al for the modified weights (dw/dp = w ln t).
-          const float gpf = (kMod ? 0.6931471805599453f : -0.5f * 0.6931471805599453f) * c * al;
-          gp = gpf;
-          out.code = kGradF32;
-          out.c = c;
-          out.z = Z;
-          out.d2min = scale;
-          f32 = isfinite(Z) && isfinite(gqx) && isfinite(gqy) && isfinite(gpf) && isfinite(c);
+#pragma unroll 4
+            for (int k = runs.a[rr]; k < runs.b[rr]; ++k)
+              terms.consider(sorted[k], qx, qy, r2f, inv_r, hp, pf, Z, sums.scale, sums.lsc, lsc2);
         }
-        if (!f32) {  // FP64: weights scaled by the exact scale
-          const GradF64 r64 = grad_query_f64(runs, sorted, qx, qy, r2f, p, gj, kMod, radius);
-          gqx = r64.gqx;
-          gqy = r64.gqy;
-          gp = r64.gp;
-          out.code = r64.rec.c == 0.0 && r64.rec.d2min == 0.0 ? kGradHitNone : kGradF64;
-          rec64[t] = r64.rec;
-        }
-      }
-      rec[t] = out;
-      if (grad_q) {
-        grad_q[2 * int64_t(j)] = gqx;
-        grad_q[2 * int64_t(j) + 1] = gqy;
+        gp = grad_finish<MODE, WMODE>(sums, terms, second, Z, s0, gj, j, t, runs, sorted, qx, qy,
+                                      r2f, p, radius, grad_q, rec, rec64);
       }
     }
   }
@@ -948,6 +1179,63 @@ __global__ void __launch_bounds__(kLocalThreads)
     gp = warp_sum(gp);
     if ((threadIdx.x & 31) == 0 && gp != 0.0) atomicAdd(grad_p, gp);
   }
+}
+
+// The heavy queries' gradients, a warp each.
+template <int MODE, int WMODE = kWeightShepard>
+__global__ void __launch_bounds__(kHeavyThreads)
+    local_grad_heavy_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
+                            int64_t n, const int32_t* __restrict__ starts,
+                            const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+                            int64_t m, double p, float r2f, float r2t,
+                            const float* __restrict__ grad_out, float* __restrict__ grad_q,
+                            double* __restrict__ grad_p, LocalGradRec* __restrict__ rec,
+                            LocalGradRec64* __restrict__ rec64, double radius,
+                            const unsigned* __restrict__ heavy_count,
+                            const int32_t* __restrict__ heavy) {
+  pdl_wait();
+  const int64_t count = *heavy_count;
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = int64_t(gridDim.x) * (kHeavyThreads / 32);
+  const float hp = static_cast<float>(0.5 * p), pf = static_cast<float>(p);
+  const float inv_r = WMODE == kWeightModified ? static_cast<float>(1.0 / radius) : 0.f;
+  double gp = 0.0;  // lane 0: this warp's queries' shares of dL/dp
+  for (int64_t w = (int64_t(blockIdx.x) * kHeavyThreads + threadIdx.x) / 32; w < count;
+       w += warps) {
+    const int64_t t = heavy[w];
+    if (!dcheck(t >= 0 && t < m, kSiteScatter)) continue;
+    const float4 r = qrec[t];
+    const float qx = r.x, qy = r.y;
+    const int j = __float_as_int(r.z);
+    if (!dcheck(j >= 0 && j < m, kSiteOutput)) continue;
+    const Runs runs(*grid, qx, qy, starts, base);
+    const FlatRuns fr(runs);
+    GradSums<MODE, WMODE> sums;
+#pragma unroll 2
+    for (int i = lane; i < fr.total(); i += 32) {
+      const int k = fr.at(i);
+      if (!dcheck(k >= 0 && k < n, kSiteGather)) break;
+      sums.consider(sorted[k], qx, qy, r2f, r2t, inv_r, hp, pf);
+    }
+    sums.join(hp, pf);
+    const bool second = sums.best == INT_MAX && sums.has_weight() && sums.d2min >= 0x1p-100f;
+    float s0 = 1.f, Z = 0.f;
+    GradTerms<MODE, WMODE> terms;
+    if (second) {  // the same in every lane
+      Z = sums.value(s0);
+      const float lsc2 = lg2_approx(sums.scale);
+#pragma unroll 2
+      for (int i = lane; i < fr.total(); i += 32)
+        terms.consider(sorted[fr.at(i)], qx, qy, r2f, inv_r, hp, pf, Z, sums.scale, sums.lsc, lsc2);
+      terms.ax = warp_sum(terms.ax);
+      terms.ay = warp_sum(terms.ay);
+      terms.al = warp_sum(terms.al);
+    }
+    if (lane == 0)
+      gp += grad_finish<MODE, WMODE>(sums, terms, second, Z, s0, grad_out[j], j, t, runs, sorted, qx,
+                                     qy, r2f, p, radius, grad_q, rec, rec64);
+  }
+  if (grad_p && lane == 0 && gp != 0.0) atomicAdd(grad_p, gp);
 }
 
 // The FP64 path's share of one (point, query) pair: (dL/dz, dL/dx, dL/dy).
@@ -996,7 +1284,7 @@ __global__ void __launch_bounds__(kLocalThreads)
   float gz = 0.f, gx = 0.f, gy = 0.f;
 #pragma unroll
   for (int rr = 0; rr < 5; ++rr)
-#pragma unroll 2
+#pragma unroll 4
     for (int t = runs.a[rr]; t < runs.b[rr]; ++t) {
       if (!dcheck(t >= 0 && t < m, kSiteGather)) break;
       const LocalGradRec R = rec[t];  // both loads issue before any branch
@@ -1278,12 +1566,7 @@ __global__ void __maxnreg__(64)
     const float u = cell_pos(qx, g.hx0, g.inv2), v = cell_pos(qy, g.hy0, g.inv2);
     const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
     if (LIST && !knn_easy(g, sat, float(g.cells) * rcp_approx(float(n)), cx, cy, k)) {
-      const unsigned lanes = __activemask();  // one atomic for those that are here together
-      const int lane = threadIdx.x & 31, lead = __ffs(lanes) - 1;
-      unsigned at = 0;
-      if (lane == lead) at = atomicAdd(hard_count, unsigned(__popc(lanes)));
-      at = __shfl_sync(lanes, at, lead) + __popc(lanes & ((1u << lane) - 1));
-      if (dcheck(at < m, kSiteScatter)) hard[at] = static_cast<int32_t>(t);
+      list_heavy(t, m, hard_count, hard);
       return;
     }
     const float mg = __fmaf_ru(fabsf(u) + fabsf(v), 0x1p-22f, 0x1p-9f);
@@ -2440,6 +2723,27 @@ __global__ void __launch_bounds__(256)
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Launches `kernel` allowed to start before the kernel ahead of it in the
+// stream completes (programmatic dependent launch); the kernel itself waits
+// in pdl_wait() before touching memory, so only launch latency overlaps.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t stream,
+                       Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// Calls whose queries, a thread each, leave most of the GPU's warps empty.
+bool few_queries(int64_t m, int sm_count) { return m <= int64_t(sm_count) * 1024; }
+
 int scan_tiles_of(int64_t max_cells) {
   return static_cast<int>((max_cells + 1 + kScanTile - 1) / kScanTile);
 }
@@ -2518,6 +2822,34 @@ cudaError_t launch_grid_sort(const float* data, int64_t n, const float* queries,
 
 }  // namespace
 
+namespace {
+// The values of sorted queries: one thread each, then a warp for each heavy one.
+cudaError_t launch_radius_queries(const GridDev* grid, const float4* sorted, int64_t n,
+                                  const int32_t* starts, const int32_t* base, const float4* qrec,
+                                  int64_t m, double p, float r2f, float r2t, float* out,
+                                  int32_t* count_out, double radius, bool modified, int32_t* heavy,
+                                  unsigned qgrid, int sm_count, cudaStream_t s) {
+  unsigned* heavy_count = &const_cast<GridDev*>(grid)->hard;
+  auto run = [&](auto mode, auto wmode) {
+    constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
+    local_query_kernel<M, W><<<qgrid, kLocalThreads, 0, s>>>(
+        grid, sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
+        few_queries(m, sm_count), heavy_count, heavy);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_pdl(local_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, s, grid,
+                      sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
+                      static_cast<const unsigned*>(heavy_count), static_cast<const int32_t*>(heavy));
+  };
+  using P2 = std::integral_constant<int, kPow2>;
+  using PG = std::integral_constant<int, kPowGeneral>;
+  using WS = std::integral_constant<int, kWeightShepard>;
+  using WM = std::integral_constant<int, kWeightModified>;
+  if (modified) return p == 2.0 ? run(P2{}, WM{}) : run(PG{}, WM{});
+  return p == 2.0 ? run(P2{}, WS{}) : run(PG{}, WS{});
+}
+}  // namespace
+
 cudaError_t launch_local(const float* data, int64_t n, const float* queries, int64_t m, double p,
                          double radius, float* out, int32_t* count_out, void* workspace,
                          const LocalLayout& L, int sm_count, cudaStream_t s, bool sort_queries,
@@ -2534,21 +2866,9 @@ cudaError_t launch_local(const float* data, int64_t n, const float* queries, int
   const float r2f = static_cast<float>(radius * radius);
   const float r2t = r2f > 0.f ? r2f : 0x1p-149f;
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
-  if (modified) {
-    if (p == 2.0)
-      local_query_kernel<kPow2, kWeightModified><<<qgrid, kLocalThreads, 0, s>>>(
-          grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out, radius);
-    else
-      local_query_kernel<kPowGeneral, kWeightModified><<<qgrid, kLocalThreads, 0, s>>>(
-          grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out, radius);
-  } else if (p == 2.0) {
-    local_query_kernel<kPow2><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out);
-  } else {
-    local_query_kernel<kPowGeneral><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out);
-  }
-  return cudaGetLastError();
+  return launch_radius_queries(grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out,
+                               radius, modified, reinterpret_cast<int32_t*>(ws + L.off_hard), qgrid,
+                               sm_count, s);
 }
 
 size_t local_grad_record_bytes(int64_t m) {
@@ -2582,11 +2902,18 @@ cudaError_t launch_local_backward(const float* data, int64_t n, const float* que
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
   const unsigned dgrid = static_cast<unsigned>((n + kLocalThreads - 1) / kLocalThreads);
   const bool data_side = grad_z || grad_xy;
+  unsigned* heavy_count = &reinterpret_cast<GridDev*>(ws + L.off_grid)->hard;
+  int32_t* heavy = reinterpret_cast<int32_t*>(ws + L.off_hard);
   auto run = [&](auto mode, auto wmode) {
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
     local_grad_query_kernel<M, W><<<qgrid, kLocalThreads, 0, s>>>(
         grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec,
-        rec64, radius);
+        rec64, radius, few_queries(m, sm_count), heavy_count, heavy);
+    if ((e = cudaGetLastError()) == cudaSuccess)
+      e = launch_pdl(local_grad_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, s, grid,
+                     sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec,
+                     rec64, radius, static_cast<const unsigned*>(heavy_count),
+                     static_cast<const int32_t*>(heavy));
     if (data_side)
       local_grad_data_kernel<M, W><<<dgrid, kLocalThreads, 0, s>>>(
           grid, sorted, n, starts_d, sums, starts_q, sums_q, qrec, m, rec, rec64, p, r2f, grad_z,
@@ -2601,7 +2928,7 @@ cudaError_t launch_local_backward(const float* data, int64_t n, const float* que
   } else {
     if (p == 2.0) run(P2{}, WS{}); else run(PG{}, WS{});
   }
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 size_t knn_grad_scratch_bytes(int64_t n, int64_t m, int k, bool deterministic) {
@@ -2982,21 +3309,9 @@ cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, cons
   const float r2f = static_cast<float>(radius * radius);
   const float r2t = r2f > 0.f ? r2f : 0x1p-149f;
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
-  if (modified) {
-    if (p == 2.0)
-      local_query_kernel<kPow2, kWeightModified><<<qgrid, kLocalThreads, 0, s>>>(
-          grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out, radius);
-    else
-      local_query_kernel<kPowGeneral, kWeightModified><<<qgrid, kLocalThreads, 0, s>>>(
-          grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out, radius);
-  } else if (p == 2.0) {
-    local_query_kernel<kPow2><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out);
-  } else {
-    local_query_kernel<kPowGeneral><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out);
-  }
-  return cudaGetLastError();
+  return launch_radius_queries(grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out,
+                               radius, modified, reinterpret_cast<int32_t*>(ws + Q.off_hard), qgrid,
+                               sm_count, s);
 }
 
 cudaError_t launch_index_knn(const void* index_mem, const IndexLayout& X, const float* queries,
