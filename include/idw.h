@@ -221,8 +221,8 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *       The persistent grid always fills the GPU, so the number of pieces
  *       each query tile is split into (the split-N factor) follows from the
  *       query-tile size and the problem sizes.
- *   IDW_OPT_FORCE_GENERAL_POWER 0/1: evaluate p = 2 through the log2/exp2
- *       form used for other p (for comparing the two forms).
+ *   IDW_OPT_FORCE_GENERAL_POWER 0/1: evaluate p = 1, 2, 3 and 4 through the
+ *       log2/exp2 form used for other p (for comparing the forms).
  *   IDW_OPT_STAGING_LAYOUT      layout of the staged data tiles: -1 (default)
  *       picks per weight form, 1 at p = 2 and 0 otherwise (the faster of
  *       each on GB300); 0 duplicated pair records (x,x,y,y)+(z,z),

@@ -26,10 +26,16 @@ __host__ __device__ constexpr uint32_t tile_bytes_of() {
 static_assert(tile_bytes_of<0>() == kTileBytes32, "default layout");
 static_assert(tile_bytes_of<1>() % 16 == 0 && tile_bytes_of<2>() % 16 == 0, "bulk copy sizes");
 
-// Padding records of the p = 2 form sit at (2^63, 2^63): for any query with
+// Forms whose query pairs may share a reciprocal, 1/(da db): their padding
+// records sit at a finite place (a product with +inf would give NaN).
+__host__ __device__ constexpr bool shares_reciprocals(int mode) {
+  return mode == kPow2 || mode == kPow4;
+}
+
+// Padding records of those forms sit at (2^63, 2^63): for any query with
 // |coordinate| <= 2^10, d^2 = 2^127, whose reciprocal is subnormal and
 // flushes to 0, and the shared product overflows to +inf, whose reciprocal
-// is 0.  The general form pads at +inf (its log2 is clamped).
+// is 0.  The other forms pad at +inf (log2 is clamped, rsqrt gives 0).
 constexpr float kPadPow2 = 9.223372036854775808e18f;  // 2^63
 
 struct Instance {
@@ -149,7 +155,7 @@ __global__ void __launch_bounds__(256)
   const int64_t lr = r - I.record_base;
   const float s = scale_from_max(maxbits[k]);
   if (lr == 0) scales[k] = s;
-  const float pad = MODE == kPow2 ? kPadPow2 : INFINITY;
+  const float pad = shares_reciprocals(MODE) ? kPadPow2 : INFINITY;
   float x = pad, y = pad, z = 0.f;
   if (lr < I.n) {
     x = I.data[3 * lr] * s;

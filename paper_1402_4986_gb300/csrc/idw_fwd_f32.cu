@@ -21,7 +21,9 @@
 //     except that for one of the query pairs the two pairs share one
 //     reciprocal, 1/(da db), and recover 1/da = db/(da db) with two FMULs;
 //     this moves work from the MUFU pipe (the binding one) to the FMA pipe.
-//     General p: 2^(-(p/2) log2 d^2) with the product's rounding error
+//     p = 1, 3, 4: powers of one MUFU reciprocal square root (1, 3) or
+//     reciprocal (4, shared as at p = 2).
+//     Other p: 2^(-(p/2) log2 d^2) with the product's rounding error
 //     recovered by an FMA and applied to first order;
 //   * sums run in chunks of 64 (p = 2) or 32 points: S0 as a balanced
 //     binary tree, S1 as FMA chains of products joined by a tree; each chunk
@@ -134,12 +136,18 @@ __device__ __forceinline__ u64 weight_pair(u64 d2, bool shared_rcp, u64 half_p2,
                                            u64 neg_half_p2, bool fma_log2 = false) {
   float a, b;
   upk(d2, a, b);
-  if (MODE == kPow2) {
+  if (MODE == kPow2 || MODE == kPow4) {
+    u64 w;
     if (shared_rcp) {
       const float r = rcp_approx(mul_ftz(a, b));  // 1 / (da db)
-      return pk(mul_ftz(b, r), mul_ftz(a, r));
+      w = pk(mul_ftz(b, r), mul_ftz(a, r));
+    } else {
+      w = pk(rcp_approx(a), rcp_approx(b));
     }
-    return pk(rcp_approx(a), rcp_approx(b));
+    return MODE == kPow4 ? mul2f(w, w) : w;
+  } else if (MODE == kPow1 || MODE == kPow3) {
+    const u64 r = pk(rsqrt_approx(a), rsqrt_approx(b));
+    return MODE == kPow3 ? mul2f(mul2f(r, r), r) : r;
   } else {
     // L = log2 d^2, clamped so that +inf (padding) stays finite below; on
     // the MUFU pipe, or for a fixed fraction of the pairs on the FMA pipe.
@@ -326,7 +334,7 @@ __global__ void __launch_bounds__(Var<V>::NT, 512 / Var<V>::NT)
               const u64 dx = sub2(QX[k], xx);
               const u64 dy = sub2(QY[k], yy);
               const u64 d2 = fma2(dy, dy, mul2(dx, dx));
-              const bool shared = k < KSHARED || (k == KALT && (r & 1));
+              const bool shared = shares_reciprocals(MODE) && (k < KSHARED || (k == KALT && (r & 1)));
               const bool fma_log2 = FMA_LOG2 && k == 0 && r % kLog2FmaPeriod == 0;
               const u64 w = weight_pair<MODE>(d2, shared, hp2, nhp2, fma_log2);
               tree_push<SH.tree_levels>(P0[k], w, r, C0[k]);
@@ -882,6 +890,26 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   const int layout = plan.layout >= 0 ? plan.layout : (pow2 ? 1 : 0);
   if (one && plan.variant == 4 && !pow2 && plan.fma_log2)
     return launch_impl<1, 4, kPowGeneral, 0, true>(probs, plan, p, ws, ctrl, sm_count, ev, stream);
+  // p = 1, 3, 4 as powers of one reciprocal (square root): 1 MUFU at 16 per SM
+  // and clock against lg2 at 16 and ex2 at 32.  n = m = 51,200, p = 1 / 3 / 4:
+  // 641 / 700 / 651 us, against 1007 us through log2 and exp2, with errors
+  // against 64 bits at or below that form's (it keeps that form's 32-point
+  // chunks: the 64-point ones of p = 2 were 3% faster and 5% less exact).
+  // Aligned records beat duplicated pairs by 1-2% here as at p = 2.  Forced
+  // variants and layouts, made to study the general form, keep it.
+  if (!plan.force_general && plan.layout < 0 && !plan.fma_log2 &&
+      (plan.variant == 0 || plan.variant == 4)) {
+#define IDW_LAUNCH_POWER(M)                                                                     \
+  if (plan.variant == 0)                                                                        \
+    return one ? launch_impl<1, 0, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)        \
+               : launch_impl<kBatchCap, 0, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream); \
+  return one ? launch_impl<1, 4, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)          \
+             : launch_impl<kBatchCap, 4, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)
+    if (p == 1.0) { IDW_LAUNCH_POWER(kPow1); }
+    if (p == 3.0) { IDW_LAUNCH_POWER(kPow3); }
+    if (p == 4.0) { IDW_LAUNCH_POWER(kPow4); }
+#undef IDW_LAUNCH_POWER
+  }
   if (one && plan.variant == 0) {
     if (pow2 && layout == 0) return launch_impl<1, 0, kPow2, 0>(probs, plan, p, ws, ctrl, sm_count, ev, stream);
     if (pow2 && layout == 2) return launch_impl<1, 0, kPow2, 2>(probs, plan, p, ws, ctrl, sm_count, ev, stream);

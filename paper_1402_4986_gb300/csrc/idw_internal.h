@@ -66,7 +66,9 @@ struct Control {
   unsigned maxbits[kBatchCap];
 };
 
-enum WeightMode : int { kPow2 = 0, kPowGeneral = 1 };
+// Forms of w = (d^2)^(-p/2): p = 2 (a reciprocal), any p (log2 and exp2), and
+// p = 1, 3, 4 (powers of a reciprocal or reciprocal square root).
+enum WeightMode : int { kPow2 = 0, kPowGeneral = 1, kPow1 = 2, kPow3 = 3, kPow4 = 4 };
 
 // Optional events recorded around the all-pairs sweep kernel.
 struct SweepEvents {

@@ -621,11 +621,6 @@ __device__ __forceinline__ void warp_sum_pairs(u64& hi, u64& lo) {
 // square root (relative error ~2^-22) and is clamped at 0 for members that
 // rounding puts at the boundary; a coincident point gives an infinite base.
 constexpr int kWeightShepard = 0, kWeightModified = 1;
-__device__ __forceinline__ float rsqrt_approx(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 template <int MODE>
 __device__ __forceinline__ float modified_weight(float d2, float inv_r, float pw) {
   const float t = fmaxf(rsqrt_approx(d2) - inv_r, 0.f);
