@@ -209,7 +209,9 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *   IDW_OPT_SWEEP_VARIANT       -1 (default: autotuned if enabled; else, at
  *       p = 2, variant 5 for problems with fewer than 4 work units of 256
  *       points x 2048 queries per resident CTA; else 4 when its 4096-query
- *       tiles pad the queries within 1% of variant 0's; else 0) or:
+ *       tiles pad the queries within 1% of variant 0's; else 0; or, where
+ *       smaller tiles are predicted to be faster, 6 or 7: 512 queries per CTA
+ *       with work units of 64 or 256 data points, which cannot be set) or:
  *       0: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal;
  *       1: 2048 queries per CTA, no shared reciprocal;
  *       2: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal

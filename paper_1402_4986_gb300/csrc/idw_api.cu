@@ -33,7 +33,7 @@ struct idw_handle_s {
   idw::Control* ctrl = nullptr;  // device control words
   int occ_f64 = 0, occ_bwd = 0;
   int occ_f64_layout[3] = {};  // plain FP64 form per staging layout
-  int occ_f32[2][idw::kNumSweepVariants] = {};  // [general p][variant]
+  int occ_f32[2][idw::kNumAllVariants] = {};  // [general p][variant]
   // Options (idw_set_option).
   int opt_autotune = 0, opt_variant = -1, opt_force_general = 0, opt_layout = -1;
   int opt_validate = 0;         // scan inputs for NaN / inf before computing

@@ -82,8 +82,10 @@ template <> struct Var<2> { static constexpr int NT = 256, KP = 4, KSH = 1, KALT
 template <> struct Var<3> { static constexpr int NT = 128, KP = 4, KSH = 1, KALT = -1, TBV = 256; };
 template <> struct Var<4> { static constexpr int NT = 512, KP = 4, KSH = 1, KALT = 1, TBV = 256; };
 template <> struct Var<5> { static constexpr int NT = 256, KP = 4, KSH = 1, KALT = -1, TBV = 64; };
+template <> struct Var<6> { static constexpr int NT = 64, KP = 4, KSH = 1, KALT = -1, TBV = 64; };
+template <> struct Var<7> { static constexpr int NT = 64, KP = 4, KSH = 1, KALT = -1, TBV = 256; };
 template <int V> __host__ __device__ constexpr int qt_of() { return Var<V>::NT * 2 * Var<V>::KP; }
-static_assert(kNumSweepVariants == 6, "variant table");
+static_assert(kNumAllVariants == 8, "variant table");
 static_assert(qt_of<0>() == kQueriesPerCtaF32, "default variant is the documented tiling");
 
 struct SweepArgs {
@@ -806,6 +808,8 @@ int sweep_variant_queries_per_cta(int variant) {
     case 3: return qt_of<3>();
     case 4: return qt_of<4>();
     case 5: return qt_of<5>();
+    case 6: return qt_of<6>();
+    case 7: return qt_of<7>();
     default: return qt_of<0>();
   }
 }
@@ -813,10 +817,39 @@ int sweep_variant_queries_per_cta(int variant) {
 int sweep_variant_points_per_unit(int variant) {
   switch (variant) {
     case 5: return Var<5>::TBV;
+    case 6: return Var<6>::TBV;
     default: return TB;
   }
 }
 
+// Predicted clocks of a sweep's longest CTA: its units times a unit's share
+// of an SM.  An SM with w of its 16 warps sweeps 1 - (1 - w/16)^2 of its full
+// rate, `rate` pairs a clock.
+namespace {
+double sweep_clocks(const F32Problem* probs, int count, int variant, int threads, double rate,
+                    int sm_count) {
+  const int64_t qt = sweep_variant_queries_per_cta(variant);
+  const int64_t tb = sweep_variant_points_per_unit(variant);
+  int64_t units = 0;
+  for (int k = 0; k < count; ++k)
+    units += (probs[k].m + qt - 1) / qt * ((probs[k].n + tb - 1) / tb);
+  const int64_t per_sm = 512 / threads, resident = per_sm * sm_count;
+  const int64_t grid = std::min(units, resident);
+  const int64_t longest = (units + grid - 1) / grid;
+  const double ctas = double((grid + sm_count - 1) / sm_count);
+  const double idle = 1.0 - ctas / double(per_sm);
+  return double(longest) * double(qt * tb) * ctas / (rate * (1.0 - idle * idle));
+}
+}  // namespace
+
+// The fixed rule of thumb (large tiles, or 64-point units for small p = 2
+// problems) unless one of the 512-query variants is predicted to be 10%
+// faster: those pad small or uneven query sets less and fill the GPU with
+// smaller pieces, at 80% (64-point units) to 93% of the large tiles' rate.
+// Measured, rule of thumb / 512-query tiles, whole call: p = 2: n = 20,000,
+// m = 1000 35.4 / 30.7 us; n = 70,000, m = 3000 88.7 / 78.6; n = m = 20,000
+// 113.5 / 126.4 (not taken).  p = 3.5: n = m = 4000 70.7 / 38.0; 64 problems of
+// 256 to 8192 points 320 / 275; n = m = 40,000 648 / 687 (not taken).
 int default_sweep_variant(const F32Problem* probs, int count, bool general_form, int sm_count) {
   const int64_t q4 = qt_of<4>(), q0 = qt_of<0>();
   double pad4 = 0, pad0 = 0, units0 = 0;
@@ -825,12 +858,26 @@ int default_sweep_variant(const F32Problem* probs, int count, bool general_form,
     pad0 += double((probs[k].m + q0 - 1) / q0 * q0);
     units0 += double((probs[k].m + q0 - 1) / q0) * double((probs[k].n + TB - 1) / TB);
   }
-  if (!general_form && units0 < 4.0 * sm_count * 2) return 5;
-  return pad4 <= 1.01 * pad0 ? 4 : 0;
+  const int large = !general_form && units0 < 4.0 * sm_count * 2 ? 5 : pad4 <= 1.01 * pad0 ? 4 : 0;
+  // Pairs per SM and clock of a full GPU.
+  const double rate[kNumAllVariants] = {general_form ? 8.5 : 15.1, 0, 0, 0,
+                                        general_form ? 8.65 : 15.35, 14.8, 12.2,
+                                        general_form ? 7.6 : 14.2};
+  int best = large;
+  double t = 0.9 * sweep_clocks(probs, count, large, large == 4 ? 512 : 256, rate[large], sm_count);
+  for (int v : {kSmallTileFine, kSmallTile}) {
+    if (general_form && v == kSmallTileFine) continue;
+    const double tv = sweep_clocks(probs, count, v, 64, rate[v], sm_count);
+    if (tv < t) {
+      best = v;
+      t = tv;
+    }
+  }
+  return best;
 }
 
 int resolve_sweep_variant(int variant, bool general_form) {
-  if (variant < 0 || variant >= kNumSweepVariants) return 0;
+  if (variant < 0 || variant >= kNumAllVariants) return 0;
   // Sub-tile work units need the aligned-AoS staging of the p = 2 form.
   if (general_form && sweep_variant_points_per_unit(variant) != TB) return 0;
   return variant;
@@ -898,11 +945,14 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   // Aligned records beat duplicated pairs by 1-2% here as at p = 2.  Forced
   // variants and layouts, made to study the general form, keep it.
   if (!plan.force_general && plan.layout < 0 && !plan.fma_log2 &&
-      (plan.variant == 0 || plan.variant == 4)) {
+      (plan.variant == 0 || plan.variant == 4 || plan.variant == 7)) {
 #define IDW_LAUNCH_POWER(M)                                                                     \
   if (plan.variant == 0)                                                                        \
     return one ? launch_impl<1, 0, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)        \
                : launch_impl<kBatchCap, 0, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream); \
+  if (plan.variant == 7)                                                                        \
+    return one ? launch_impl<1, 7, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)        \
+               : launch_impl<kBatchCap, 7, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream); \
   return one ? launch_impl<1, 4, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)          \
              : launch_impl<kBatchCap, 4, M, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)
     if (p == 1.0) { IDW_LAUNCH_POWER(kPow1); }
@@ -935,6 +985,13 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
                    : launch_impl<kBatchCap, 5, kPow2, 1>(probs, plan, p, ws, ctrl, sm_count, ev,
                                                          stream);
       return cudaErrorInvalidValue;  // resolve_sweep_variant maps it away for general p
+    case 6:
+      if (pow2)
+        return one ? launch_impl<1, 6, kPow2, 1>(probs, plan, p, ws, ctrl, sm_count, ev, stream)
+                   : launch_impl<kBatchCap, 6, kPow2, 1>(probs, plan, p, ws, ctrl, sm_count, ev,
+                                                         stream);
+      return cudaErrorInvalidValue;
+    case 7: IDW_LAUNCH(7);
     default: IDW_LAUNCH(0);
   }
 #undef IDW_LAUNCH
@@ -968,6 +1025,8 @@ int occupancy_forward_f32(bool general_p, int variant) {
     case 3: return occupancy_variant<3>(general_p);
     case 4: return occupancy_variant<4>(general_p);
     case 5: return general_p ? occupancy_variant<0>(true) : occupancy_variant<5>(false);
+    case 6: return general_p ? occupancy_variant<0>(true) : occupancy_variant<6>(false);
+    case 7: return occupancy_variant<7>(general_p);
     default: return occupancy_variant<0>(general_p);
   }
 }

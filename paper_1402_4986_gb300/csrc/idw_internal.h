@@ -40,6 +40,10 @@ constexpr int kBatchCap = 256;
 // Compiled variants of the FP32 sweep (query-tile size, shared reciprocals);
 // variant 0 is the default tiling above.
 constexpr int kNumSweepVariants = 6;
+// Two more that only the default rule picks, for small problems: 512 queries
+// per CTA (64 threads), work units of 64 (6; p = 2 and p = 1, 3, 4 only) or
+// 256 points (7).
+constexpr int kSmallTileFine = 6, kSmallTile = 7, kNumAllVariants = 8;
 
 // Plain FP64 forward: kQueriesF64 queries per thread; tiles of (x,y) + z.
 constexpr int kThreadsF64 = 128;
@@ -115,7 +119,8 @@ int resolve_sweep_variant(int variant, bool general_form);
 // 256-point work units per resident CTA) use the fine-grained variant 5, so
 // the grid stays full and balanced; otherwise one 512-thread CTA per SM
 // (variant 4) keeps all 16 warps of an SM in step, when its 4096-query
-// tiles pad the queries no more than variant 0's 2048-query tiles (+1%).
+// tiles pad the queries no more than variant 0's 2048-query tiles (+1%).  The
+// 512-query variants 6 and 7 take over where they are predicted to be faster.
 int default_sweep_variant(const F32Problem* probs, int count, bool general_form, int sm_count);
 
 // Enqueues range scan, staging, sweep, combine and slow path for the batch.

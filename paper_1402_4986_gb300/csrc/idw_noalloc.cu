@@ -33,7 +33,7 @@ struct DeviceSetup {
   bool ready = false;
   unsigned char* scratch = nullptr;  // device address of g_noalloc_scratch
   int sm_count = 0;
-  int occ[2][kNumSweepVariants] = {};  // resident CTAs per SM: [general p][variant]
+  int occ[2][kNumAllVariants] = {};  // resident CTAs per SM: [general p][variant]
 };
 
 std::mutex g_setup_mutex;
@@ -66,7 +66,7 @@ idw_status setup_current_device(DeviceSetup* out) {
     s.scratch = static_cast<unsigned char*>(ptr);
     s.sm_count = sms;
     for (int g = 0; g < 2; ++g)
-      for (int v = 0; v < kNumSweepVariants; ++v)
+      for (int v = 0; v < kNumAllVariants; ++v)
         if (resolve_sweep_variant(v, g != 0) == v) s.occ[g][v] = occupancy_forward_f32(g != 0, v);
     s.ready = true;
   }
