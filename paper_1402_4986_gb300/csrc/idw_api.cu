@@ -652,7 +652,8 @@ idw_status idw_backward(idw_handle_t h, const float* data, int64_t n, const floa
   if (st != IDW_OK) return st;
   if (!h->occ_bwd) h->occ_bwd = idw::occupancy_backward_f32();
   idw::BwdPlan bp;
-  idw::plan_backward_f32(n, m, h->sm_count, h->occ_bwd, &bp);
+  const bool both = (grad_query_xy || grad_p) && (grad_z || grad_data_xy);
+  idw::plan_backward_f32(n, m, p, both, h->sm_count, h->occ_bwd, &bp);
   st = ensure_buffer(h, &h->ws, &h->ws_bytes, bp.workspace_bytes);
   if (st != IDW_OK) return st;
   idw::BwdProblem pb{static_cast<const float*>(data), n, static_cast<const float*>(queries), m, p,

@@ -34,6 +34,11 @@ __device__ __forceinline__ u64 sub2f(u64 a, u64 b) {
   asm("sub.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ u64 add2f(u64 a, u64 b) {
+  u64 r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ u64 mul2f(u64 a, u64 b) {
   u64 r;
   asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));

@@ -153,11 +153,17 @@ struct BwdPlan {
   int64_t data_tiles = 0, query_records_tiles = 0, query_reg_tiles = 0, data_reg_tiles = 0;
   int64_t units_q = 0, units_d = 0;
   int grid_q = 0, grid_d = 0;
+  // One sweep for both sides: 0, or the threads per CTA of the variant used.
+  int fused = 0, grid_f = 0;
+  int64_t fused_tiles = 0, fused_data_tiles = 0, panel_tiles = 0;
+  size_t dpart_bytes = 0, dacc_bytes = 0;
   size_t staged_bytes = 0, qtiles_bytes = 0, partial_bytes = 0, gp_bytes = 0, list_bytes = 0,
          dlist_bytes = 0, scale_bytes = 0, workspace_bytes = 0;
 };
 
-void plan_backward_f32(int64_t n, int64_t m, int sm_count, int ctas_per_sm, BwdPlan* plan);
+// both: gradients of both sides (queries or p, and data) are wanted.
+void plan_backward_f32(int64_t n, int64_t m, double p, bool both, int sm_count, int ctas_per_sm,
+                       BwdPlan* plan);
 cudaError_t launch_backward_f32(const BwdProblem& pb, const BwdPlan& plan, void* workspace,
                                 Control* ctrl, int sm_count, cudaStream_t stream);
 int occupancy_backward_f32();
