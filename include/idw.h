@@ -252,12 +252,13 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *                               and k-NN, one-shot and prepared index, and
  *                               idw_knn_backward) sort the queries into the
  *                               grid's cells so that neighbouring threads
- *                               read the same data.  1 keeps the caller's
- *                               order instead, which saves that sort when
- *                               the queries already come in spatial order
- *                               (a raster of prediction points) and costs
- *                               locality when they do not.  Results are the
- *                               same either way.  idw_local_backward always
+ *                               read the same data (a prepared index leaves
+ *                               up to 2^17 radius or 2^15 k-NN queries as they
+ *                               come).  1 keeps the caller's order instead,
+ *                               which saves that sort when the queries already
+ *                               come in spatial order (a raster of prediction
+ *                               points) and costs locality when they do not.
+ *                               Results are the same either way.  idw_local_backward always
  *                               sorts (its data-side pass finds queries by
  *                               cell).
  *   IDW_OPT_DETERMINISTIC       0 (default) or 1.  idw_knn_backward adds the

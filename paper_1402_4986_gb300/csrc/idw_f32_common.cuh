@@ -110,8 +110,8 @@ __device__ __forceinline__ float mul_ftz(float a, float b) {
 // `flagged`, the call's count of queries listed for the slow path (nullable).
 template <int CAP>
 __global__ void __launch_bounds__(256) range_kernel(const __grid_constant__ Table<CAP> t,
-                                                    unsigned* __restrict__ maxbits,
-                                                    unsigned* __restrict__ flagged) {
+                                                    unsigned* maxbits,
+                                                    unsigned* flagged) {
   __shared__ float red[8];
   pdl_trigger();
   pdl_wait();
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) range_kernel(const __grid_constant__ Tabl
 template <int CAP, int MODE, int LAYOUT = 0>
 __global__ void __launch_bounds__(256)
     stage_kernel(const __grid_constant__ Table<CAP> t, int64_t total_records,
-                 const unsigned* __restrict__ maxbits, float* __restrict__ scales) {
+                 const unsigned* maxbits, float* scales) {
   pdl_trigger();
   pdl_wait();
   const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;

@@ -443,9 +443,9 @@ struct SlowList {
 
 template <int CAP, int QT>
 __global__ void __launch_bounds__(kCombineQueries * kCombineLanes)
-    combine_kernel(const __grid_constant__ Table<CAP> t, const float4* __restrict__ partial,
-                   int64_t total_slots, int64_t units, int grid, const float* __restrict__ scales,
-                   double p, Control* __restrict__ ctrl, const SlowList slow) {
+    combine_kernel(const __grid_constant__ Table<CAP> t, const float4* partial,
+                   int64_t total_slots, int64_t units, int grid, const float* scales,
+                   double p, Control* ctrl, const SlowList slow) {
   __shared__ float4 red[kCombineLanes][kCombineQueries];
   __shared__ int2 flagged[kCombineQueries];
   __shared__ int nflagged;
@@ -528,7 +528,7 @@ constexpr int kSlowGroup = 32;
 
 template <int CAP>
 __global__ void __launch_bounds__(kSlowThreads)
-    slow_search_kernel(const __grid_constant__ Table<CAP> t, const Control* __restrict__ ctrl,
+    slow_search_kernel(const __grid_constant__ Table<CAP> t, const Control* ctrl,
                        const SlowList slow) {
   __shared__ float2 q[kSlowGroup];
   __shared__ int prob[kSlowGroup];
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(kSlowThreads)
 // of one SM bounds a query; spread over the GPU they take under 30 us.
 template <int CAP>
 __global__ void __launch_bounds__(kSlowThreads)
-    slow_finish_kernel(const __grid_constant__ Table<CAP> t, const Control* __restrict__ ctrl,
+    slow_finish_kernel(const __grid_constant__ Table<CAP> t, const Control* ctrl,
                        const SlowList slow, double p) {
   __shared__ int work[kSlowThreads];
   __shared__ int warp_count[kSlowThreads / 32];
@@ -669,26 +669,6 @@ __global__ void bounded_wait_selftest_kernel(unsigned* err) {
 }
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// Launches `kernel` allowed to start before the kernel ahead of it in the
-// stream completes (programmatic dependent launch); the kernel itself waits
-// in pdl_wait() before touching memory, so results are as with a plain
-// launch and only launch latency overlaps.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t stream, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
 
 // Raises a kernel's dynamic shared memory limit to `bytes` (needed above
 // 48 KB), once per kernel and device (one flag word per instantiation).

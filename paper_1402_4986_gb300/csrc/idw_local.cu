@@ -66,6 +66,12 @@ constexpr int kMaxBlocksPerAxis = kMaxCellsPerAxis >> kBlockShift;
 // (FTZ) weights: such queries are redone in FP64.
 constexpr float kTinyPerMember = 0x1p-100f;
 
+// Kernels here are launched with programmatic dependent launch: each waits in
+// pdl_wait() for the kernel ahead of it.  Inputs, which that kernel may be
+// writing, are passed without __restrict__: the compiler may move loads
+// through a restricted pointer, which it takes to be untouched by anything
+// else, above that wait, and reads them through the non-coherent path.
+
 // Index checks of a debug build (-DIDW_DEBUG_CHECKS): a failed check sets
 // its site's bit in a device word and the access it guards is skipped; no
 // trap.  Release builds compile every check to `true`.
@@ -186,11 +192,27 @@ __device__ void plan_grid(GridDev* grid, double radius, double inv_max_cells, in
   grid->hard = 0u;
 }
 
+// Zeroes a histogram over `len4` int4s (grid-stride; the scan reads int4s).
+__device__ __forceinline__ void zero_counts(int32_t* counts, int len4) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len4; i += gridDim.x * blockDim.x)
+    reinterpret_cast<int4*>(counts)[i] = make_int4(0, 0, 0, 0);
+}
+// int4s that hold cells + 1 entries.
+__host__ __device__ __forceinline__ int count_int4s(int64_t cells) {
+  return static_cast<int>((cells + 1 + 3) / 4);
+}
+
 // Bounding box of the finite data points; the last block to finish plans
-// the grid.
+// the grid.  Also clears the histograms (over the most cells the plan may
+// have; counts_q may be null).
 __global__ void __launch_bounds__(256)
-    box_plan_kernel(const float* __restrict__ data, int64_t n, GridDev* __restrict__ grid,
-                    double radius, double inv_max_cells, int knn_k) {
+    box_plan_kernel(const float* data, int64_t n, GridDev* grid,
+                    double radius, double inv_max_cells, int knn_k, int64_t max_cells,
+                    int32_t* counts_d, int32_t* counts_q) {
+  pdl_trigger();
+  pdl_wait();
+  zero_counts(counts_d, count_int4s(max_cells));
+  if (counts_q) zero_counts(counts_q, count_int4s(max_cells));
   __shared__ unsigned part[4][8];
   __shared__ bool last;
   unsigned k0 = 0xffffffffu, k1 = 0xffffffffu, k2 = 0xffffffffu, k3 = 0xffffffffu;
@@ -236,18 +258,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Zeroes both histograms over cells + 1 entries rounded up to a multiple of
-// four (the scan reads them as int4).
-__global__ void __launch_bounds__(256)
-    zero_counts_kernel(const GridDev* __restrict__ grid, int32_t* __restrict__ counts_d,
-                       int32_t* __restrict__ counts_q) {
-  const int len = (grid->cells + 1 + 3) & ~3;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x) {
-    counts_d[i] = 0;
-    counts_q[i] = 0;
-  }
-}
-
 // Cell of a data point (-1: a non-finite point, in no cell) and sorting
 // bucket of a query (its cell clamped into the grid).
 __device__ __forceinline__ int data_cell(const GridDev& g, float x, float y) {
@@ -265,9 +275,11 @@ __device__ __forceinline__ int query_bucket(const GridDev& g, float x, float y) 
 
 // Threads [0, n) count data points, [n, n + m) count queries.
 __global__ void __launch_bounds__(256)
-    count_kernel(const GridDev* __restrict__ grid, const float* __restrict__ data, int64_t n,
-                 const float* __restrict__ queries, int64_t m, int32_t* __restrict__ counts_d,
-                 int32_t* __restrict__ counts_q) {
+    count_kernel(const GridDev* grid, const float* data, int64_t n,
+                 const float* queries, int64_t m, int32_t* counts_d,
+                 int32_t* counts_q) {
+  pdl_trigger();
+  pdl_wait();
   const GridDev g = *grid;
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -315,10 +327,12 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t* warp
 // scan in place), so that a cell starts at starts[i] + base[i / kScanTile].
 // The histogram arrays hold a multiple of four entries, 16-byte aligned.
 __global__ void __launch_bounds__(kScanBlock)
-    scan_kernel(GridDev* __restrict__ grid, int32_t* __restrict__ counts_d,
-                int32_t* __restrict__ counts_q, int32_t* __restrict__ starts_d,
-                int32_t* __restrict__ starts_q, int32_t* __restrict__ sums, int max_tiles,
+    scan_kernel(GridDev* grid, int32_t* counts_d,
+                int32_t* counts_q, int32_t* starts_d,
+                int32_t* starts_q, int32_t* sums, int max_tiles,
                 int first) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int32_t warp_tot[kScanBlock / 32];
   __shared__ bool last;
   const int len = grid->cells + 1;
@@ -360,8 +374,8 @@ __global__ void __launch_bounds__(kScanBlock)
   }
 }
 
-__device__ __forceinline__ int cell_start(const int32_t* __restrict__ starts,
-                                          const int32_t* __restrict__ base, int i, int cells) {
+__device__ __forceinline__ int cell_start(const int32_t* starts,
+                                          const int32_t* base, int i, int cells) {
   if (!dcheck(i >= 0 && i <= cells, kSiteCell)) return 0;
   return starts[i] + base[i / kScanTile];
 }
@@ -371,8 +385,10 @@ __device__ __forceinline__ int cell_start(const int32_t* __restrict__ starts,
 // blocks 0 .. bx - 1 of that row.  One CTA per block row, one thread per
 // block; runs after the scan (cell starts are final).
 __global__ void __launch_bounds__(kMaxBlocksPerAxis)
-    block_prefix_kernel(const GridDev* __restrict__ grid, const int32_t* __restrict__ starts,
-                        const int32_t* __restrict__ base, int32_t* __restrict__ bpre) {
+    block_prefix_kernel(const GridDev* grid, const int32_t* starts,
+                        const int32_t* base, int32_t* bpre) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int32_t warp_tot[kMaxBlocksPerAxis / 32];
   const GridDev g = *grid;
   const int bgx = (g.gx + 7) >> kBlockShift, bgy = (g.gy + 7) >> kBlockShift;
@@ -414,8 +430,10 @@ __global__ void __launch_bounds__(kMaxBlocksPerAxis)
 // device).
 constexpr int kSatCols = 32, kSatWarps = 32;
 __global__ void __launch_bounds__(kSatCols * kSatWarps)
-    sat_kernel(const GridDev* __restrict__ grid, const int32_t* __restrict__ starts,
-               const int32_t* __restrict__ base, int32_t* __restrict__ sat) {
+    sat_kernel(const GridDev* grid, const int32_t* starts,
+               const int32_t* base, int32_t* sat) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int32_t part[kSatWarps][kSatCols];
   const GridDev g = *grid;
   if (int(blockIdx.x) * kSatCols > g.gx) return;  // the whole CTA: no barrier is reached
@@ -447,8 +465,10 @@ __global__ void __launch_bounds__(kSatCols * kSatWarps)
 // Query records in the caller's order, (x, y, index, 0): used in place of
 // the query sort when the caller's order is kept.
 __global__ void __launch_bounds__(256)
-    query_identity_kernel(const float* __restrict__ queries, int64_t m,
-                          float4* __restrict__ qrec) {
+    query_identity_kernel(const float* queries, int64_t m,
+                          float4* qrec) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= m) return;
   qrec[j] = make_float4(queries[2 * j], queries[2 * j + 1], __int_as_float(static_cast<int>(j)),
@@ -458,12 +478,14 @@ __global__ void __launch_bounds__(256)
 // Threads [0, n) place data points as (x, y, z, index), [n, n + m) place
 // queries as (x, y, index, 0).
 __global__ void __launch_bounds__(256)
-    scatter_kernel(const GridDev* __restrict__ grid, const float* __restrict__ data, int64_t n,
-                   const float* __restrict__ queries, int64_t m,
-                   const int32_t* __restrict__ starts_d, const int32_t* __restrict__ starts_q,
-                   const int32_t* __restrict__ sums, int max_tiles,
-                   int32_t* __restrict__ cursor_d, int32_t* __restrict__ cursor_q,
-                   float4* __restrict__ sorted, float4* __restrict__ qrec) {
+    scatter_kernel(const GridDev* grid, const float* data, int64_t n,
+                   const float* queries, int64_t m,
+                   const int32_t* starts_d, const int32_t* starts_q,
+                   const int32_t* sums, int max_tiles,
+                   int32_t* cursor_d, int32_t* cursor_q,
+                   float4* sorted, float4* qrec) {
+  pdl_trigger();
+  pdl_wait();
   const GridDev g = *grid;
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -521,8 +543,8 @@ struct Runs {
     return c;
   }
   __device__ __forceinline__ Runs(const GridDev& g, float qx, float qy,
-                                  const int32_t* __restrict__ starts,
-                                  const int32_t* __restrict__ base) {
+                                  const int32_t* starts,
+                                  const int32_t* base) {
     int y0 = 0, y1 = -1;
     float u = 0.f, v = 0.f;
     if (finite2(qx, qy)) {
@@ -585,8 +607,8 @@ __device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, boo
   return int(few ? fminf(fmaf(24.f, per_cell, 32.f), 1e9f) : fminf(fmaf(64.f, per_cell, 256.f), 1e9f));
 }
 // Lists query t (any subset of a warp's lanes may call it together).
-__device__ __forceinline__ void list_heavy(int64_t t, int64_t m, unsigned* __restrict__ count,
-                                           int32_t* __restrict__ list) {
+__device__ __forceinline__ void list_heavy(int64_t t, int64_t m, unsigned* count,
+                                           int32_t* list) {
   const unsigned lanes = __activemask();  // one atomic for those that are here together
   const int lane = threadIdx.x & 31, lead = __ffs(lanes) - 1;
   unsigned at = 0;
@@ -670,7 +692,7 @@ struct ValueF64 {
 };
 template <int WMODE, bool WARP>
 __device__ __forceinline__ ValueF64 local_value_f64(const FlatRuns& fr,
-                                                    const float4* __restrict__ sorted, float qx,
+                                                    const float4* sorted, float qx,
                                                     float qy, double p, float r2f, double radius) {
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int step = WARP ? 32 : 1;
@@ -732,13 +754,14 @@ __device__ __forceinline__ ValueF64 local_value_f64(const FlatRuns& fr,
 
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kLocalThreads)
-    local_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                       int64_t n, const int32_t* __restrict__ starts,
-                       const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+    local_query_kernel(const GridDev* grid, const float4* sorted,
+                       int64_t n, const int32_t* starts,
+                       const int32_t* base, const float4* qrec,
                        int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
-                       int32_t* __restrict__ count_out, double radius, bool few,
-                       unsigned* __restrict__ heavy_count, int32_t* __restrict__ heavy) {
+                       int32_t* count_out, double radius, bool few,
+                       unsigned* heavy_count, int32_t* heavy) {
   pdl_trigger();
+  pdl_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= m) return;
   const float4 r = qrec[t];
@@ -779,13 +802,14 @@ __global__ void __launch_bounds__(kLocalThreads)
 constexpr int kHeavyThreads = 128;
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kHeavyThreads)
-    local_heavy_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                       int64_t n, const int32_t* __restrict__ starts,
-                       const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+    local_heavy_kernel(const GridDev* grid, const float4* sorted,
+                       int64_t n, const int32_t* starts,
+                       const int32_t* base, const float4* qrec,
                        int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
-                       int32_t* __restrict__ count_out, double radius,
-                       const unsigned* __restrict__ heavy_count,
-                       const int32_t* __restrict__ heavy) {
+                       int32_t* count_out, double radius,
+                       const unsigned* heavy_count,
+                       const int32_t* heavy) {
+  pdl_trigger();
   pdl_wait();
   const int64_t count = *heavy_count;
   const int lane = threadIdx.x & 31;
@@ -897,7 +921,7 @@ __device__ __forceinline__ GradTerms64 grad_terms64(double e2, double scale, dou
   return GradTerms64{w, w / (t * e2 * d), log(t / scale)};
 }
 
-__device__ __noinline__ GradF64 grad_query_f64(const Runs runs, const float4* __restrict__ sorted,
+__device__ __noinline__ GradF64 grad_query_f64(const Runs runs, const float4* sorted,
                                                float qx, float qy, float r2f, double p,
                                                float gj, bool modified, double radius) {
   double scale = modified ? 0.0 : INFINITY;  // d2_min, or the largest base t
@@ -1073,11 +1097,11 @@ template <int MODE, int WMODE>
 __device__ __forceinline__ double grad_finish(const GradSums<MODE, WMODE>& sums,
                                               const GradTerms<MODE, WMODE>& terms, bool second,
                                               float Z, float s0, float gj, int j, int64_t t,
-                                              const Runs& runs, const float4* __restrict__ sorted,
+                                              const Runs& runs, const float4* sorted,
                                               float qx, float qy, float r2f, double p,
                                               double radius, float* __restrict__ grad_q,
-                                              LocalGradRec* __restrict__ rec,
-                                              LocalGradRec64* __restrict__ rec64) {
+                                              LocalGradRec* rec,
+                                              LocalGradRec64* rec64) {
   constexpr bool kMod = WMODE == kWeightModified;
   LocalGradRec out{0.f, 0.f, 0.f, kGradHitNone};
   float gqx = 0.f, gqy = 0.f;
@@ -1120,15 +1144,17 @@ __device__ __forceinline__ double grad_finish(const GradSums<MODE, WMODE>& sums,
 
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kLocalThreads)
-    local_grad_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                            int64_t n, const int32_t* __restrict__ starts,
-                            const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+    local_grad_query_kernel(const GridDev* grid, const float4* sorted,
+                            int64_t n, const int32_t* starts,
+                            const int32_t* base, const float4* qrec,
                             int64_t m, double p, float r2f, float r2t,
-                            const float* __restrict__ grad_out, float* __restrict__ grad_q,
-                            double* __restrict__ grad_p, LocalGradRec* __restrict__ rec,
-                            LocalGradRec64* __restrict__ rec64, double radius, bool few,
-                            unsigned* __restrict__ heavy_count, int32_t* __restrict__ heavy) {
+                            const float* grad_out, float* __restrict__ grad_q,
+                            double* __restrict__ grad_p, LocalGradRec* rec,
+                            LocalGradRec64* rec64, double radius, bool few,
+                            unsigned* heavy_count, int32_t* heavy) {
   pdl_trigger();
+  pdl_wait();
+  pdl_wait();
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   double gp = 0.0;  // this query's share of dL/dp (every lane joins the warp sum)
   if (t < m) {
@@ -1179,15 +1205,16 @@ __global__ void __launch_bounds__(kLocalThreads)
 // The heavy queries' gradients, a warp each.
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kHeavyThreads)
-    local_grad_heavy_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                            int64_t n, const int32_t* __restrict__ starts,
-                            const int32_t* __restrict__ base, const float4* __restrict__ qrec,
+    local_grad_heavy_kernel(const GridDev* grid, const float4* sorted,
+                            int64_t n, const int32_t* starts,
+                            const int32_t* base, const float4* qrec,
                             int64_t m, double p, float r2f, float r2t,
-                            const float* __restrict__ grad_out, float* __restrict__ grad_q,
-                            double* __restrict__ grad_p, LocalGradRec* __restrict__ rec,
-                            LocalGradRec64* __restrict__ rec64, double radius,
-                            const unsigned* __restrict__ heavy_count,
-                            const int32_t* __restrict__ heavy) {
+                            const float* grad_out, float* __restrict__ grad_q,
+                            double* __restrict__ grad_p, LocalGradRec* rec,
+                            LocalGradRec64* rec64, double radius,
+                            const unsigned* heavy_count,
+                            const int32_t* heavy) {
+  pdl_trigger();
   pdl_wait();
   const int64_t count = *heavy_count;
   const int lane = threadIdx.x & 31;
@@ -1256,15 +1283,17 @@ __device__ __noinline__ float3 grad_pair_f64_modified(LocalGradRec64 D, float qx
 
 template <int MODE, int WMODE = kWeightShepard>
 __global__ void __launch_bounds__(kLocalThreads)
-    local_grad_data_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                           int64_t n, const int32_t* __restrict__ starts_d,
-                           const int32_t* __restrict__ base_d,
-                           const int32_t* __restrict__ starts_q,
-                           const int32_t* __restrict__ base_q, const float4* __restrict__ qrec,
-                           int64_t m, const LocalGradRec* __restrict__ rec,
-                           const LocalGradRec64* __restrict__ rec64, double p, float r2f,
+    local_grad_data_kernel(const GridDev* grid, const float4* sorted,
+                           int64_t n, const int32_t* starts_d,
+                           const int32_t* base_d,
+                           const int32_t* starts_q,
+                           const int32_t* base_q, const float4* qrec,
+                           int64_t m, const LocalGradRec* rec,
+                           const LocalGradRec64* rec64, double p, float r2f,
                            float* __restrict__ grad_z, float* __restrict__ grad_xy,
                            double radius) {
+  pdl_trigger();
+  pdl_wait();
   constexpr bool kMod = WMODE == kWeightModified;
   const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const GridDev g = *grid;
@@ -1411,12 +1440,12 @@ struct KnnHeap {
 // sort_rows, else heap order).  Shared by both search kernels.
 template <int MODE>
 __device__ __forceinline__ void knn_write_result(KnnHeap& hp, int best_hit, float qx, float qy,
-                                                 int j, const float* __restrict__ data,
+                                                 int j, const float* data,
                                                  int64_t n, double p, int k,
                                                  float* __restrict__ out,
-                                                 int32_t* __restrict__ nbr_out,
+                                                 int32_t* nbr_out,
                                                  float* __restrict__ kd2_out,
-                                                 int32_t* __restrict__ hit_out, bool sort_rows) {
+                                                 int32_t* hit_out, bool sort_rows) {
   const int size = hp.size;
   if (kd2_out) kd2_out[j] = size > 0 ? key_d2(hp.top()) : __int_as_float(0x7fc00000);
   float zv = __int_as_float(0x7fc00000);  // NaN: nothing selected
@@ -1485,7 +1514,7 @@ __device__ __forceinline__ void knn_write_result(KnnHeap& hp, int best_hit, floa
 // hundred times as long over such a query as over one at the mean density,
 // and its warp waits.  (n = 2^20 points in 64 blobs, 100,000 uniform queries,
 // k = 8: 1.09 ms when every query was one thread's.)
-__device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* __restrict__ sat,
+__device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* sat,
                                          float cells_per_point, int cx, int cy, int k) {
   const int re = int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
   const int W = g.gx + 1;
@@ -1507,15 +1536,17 @@ __device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* __rest
 // knn_easy are listed in `hard` for knn_warp_kernel.
 template <int MODE, bool LIST>
 __global__ void __maxnreg__(64)
-    knn_query_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                     const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
-                     const int32_t* __restrict__ bpre, const int32_t* __restrict__ sat,
-                     const float4* __restrict__ qrec, const float* __restrict__ data, int64_t n,
+    knn_query_kernel(const GridDev* grid, const float4* sorted,
+                     const int32_t* starts, const int32_t* base,
+                     const int32_t* bpre, const int32_t* sat,
+                     const float4* qrec, const float* data, int64_t n,
                      int64_t m,
-                     double p, int k, float* __restrict__ out, int32_t* __restrict__ nbr_out,
-                     float* __restrict__ kd2_out, int32_t* __restrict__ hit_out,
-                     bool sort_rows, unsigned* __restrict__ hard_count,
-                     int32_t* __restrict__ hard) {
+                     double p, int k, float* __restrict__ out, int32_t* nbr_out,
+                     float* __restrict__ kd2_out, int32_t* hit_out,
+                     bool sort_rows, unsigned* hard_count,
+                     int32_t* hard) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char knn_smem[];
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (t >= m) return;  // no block-wide barrier in this kernel
@@ -1826,11 +1857,11 @@ constexpr int kKnnWarpThreads = 128;
 // One query, by a whole warp.
 template <int MODE, int kRegs>
 __device__ __forceinline__ void knn_warp_query(
-    const GridDev& g, u64* keys, float qx, float qy, int j, const float4* __restrict__ sorted,
-    const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
-    const int32_t* __restrict__ sat, const float* __restrict__ data, int64_t n, double p, int k,
-    float* __restrict__ out, int32_t* __restrict__ nbr_out, float* __restrict__ kd2_out,
-    int32_t* __restrict__ hit_out, bool sort_rows) {
+    const GridDev& g, u64* keys, float qx, float qy, int j, const float4* sorted,
+    const int32_t* starts, const int32_t* base,
+    const int32_t* sat, const float* data, int64_t n, double p, int k,
+    float* __restrict__ out, int32_t* nbr_out, float* __restrict__ kd2_out,
+    int32_t* hit_out, bool sort_rows) {
   using Buffer = KnnBuffer<kRegs>;
   Buffer kb;
   kb.lane = threadIdx.x % 32;
@@ -2056,13 +2087,15 @@ __device__ __forceinline__ void knn_warp_query(
 // The queries of `hard` (null: all m), a warp each.
 template <int MODE, int kRegs>
 __global__ void __launch_bounds__(kKnnWarpThreads)
-    knn_warp_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                    const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
-                    const int32_t* __restrict__ sat, const float4* __restrict__ qrec,
-                    const float* __restrict__ data, int64_t n, int64_t m, double p, int k,
-                    float* __restrict__ out, int32_t* __restrict__ nbr_out,
-                    float* __restrict__ kd2_out, int32_t* __restrict__ hit_out, bool sort_rows,
-                    const unsigned* __restrict__ hard_count, const int32_t* __restrict__ hard) {
+    knn_warp_kernel(const GridDev* grid, const float4* sorted,
+                    const int32_t* starts, const int32_t* base,
+                    const int32_t* sat, const float4* qrec,
+                    const float* data, int64_t n, int64_t m, double p, int k,
+                    float* __restrict__ out, int32_t* nbr_out,
+                    float* __restrict__ kd2_out, int32_t* hit_out, bool sort_rows,
+                    const unsigned* hard_count, const int32_t* hard) {
+  pdl_trigger();
+  pdl_wait();
   using Buffer = KnnBuffer<kRegs>;
   __shared__ u64 keys[kKnnWarpThreads / 32][Buffer::kCap];
   const int64_t count = hard ? int64_t(*hard_count) : m;
@@ -2120,13 +2153,15 @@ size_t knn_sync_smem_bytes(int k) {
 
 template <int MODE>
 __global__ void __launch_bounds__(kKnnThreads)
-    knn_sync_kernel(const GridDev* __restrict__ grid, const float4* __restrict__ sorted,
-                    const int32_t* __restrict__ starts, const int32_t* __restrict__ base,
-                    const int32_t* __restrict__ bpre, const int32_t* __restrict__ sat,
-                    const float4* __restrict__ qrec, const float* __restrict__ data, int64_t n,
+    knn_sync_kernel(const GridDev* grid, const float4* sorted,
+                    const int32_t* starts, const int32_t* base,
+                    const int32_t* bpre, const int32_t* sat,
+                    const float4* qrec, const float* data, int64_t n,
                     int64_t m, double p, int k, float* __restrict__ out,
-                    int32_t* __restrict__ nbr_out, float* __restrict__ kd2_out,
-                    int32_t* __restrict__ hit_out, bool sort_rows) {
+                    int32_t* nbr_out, float* __restrict__ kd2_out,
+                    int32_t* hit_out, bool sort_rows) {
+  pdl_trigger();
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char knn_smem[];
   constexpr unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x;
@@ -2378,10 +2413,10 @@ struct KnnGradF64 {
   double gp;
   double Z, c, dmin;  // what the pair terms are computed from
 };
-__device__ __noinline__ KnnGradF64 knn_grad_query_f64(const int32_t* __restrict__ row, int cnt,
-                                                      const float* __restrict__ data, float qx,
+__device__ __noinline__ KnnGradF64 knn_grad_query_f64(const int32_t* row, int cnt,
+                                                      const float* data, float qx,
                                                       float qy, double p, float gj,
-                                                      float4* __restrict__ acc) {
+                                                      float4* acc) {
   double dmin = INFINITY;
   for (int s = 0; s < cnt; ++s) {
     const float* x = data + 3 * int64_t(row[s]);
@@ -2433,12 +2468,14 @@ static_assert(sizeof(KnnQState) == 32, "query state layout");
 
 template <int MODE>
 __global__ void __launch_bounds__(kLocalThreads)
-    knn_grad_kernel(const float4* __restrict__ qrec, int64_t m, const float* __restrict__ data,
-                    int64_t n, const int32_t* __restrict__ nbr, const int32_t* __restrict__ hit,
-                    int k, double p, const float* __restrict__ grad_out,
-                    float4* __restrict__ acc, float* __restrict__ grad_q,
+    knn_grad_kernel(const float4* qrec, int64_t m, const float* data,
+                    int64_t n, const int32_t* nbr, const int32_t* hit,
+                    int k, double p, const float* grad_out,
+                    float4* acc, float* __restrict__ grad_q,
                     double* __restrict__ grad_p, KnnQState* __restrict__ qstate,
                     double* __restrict__ gp_query) {
+  pdl_trigger();
+  pdl_wait();
   // qstate (deterministic mode): each query's state is recorded for the
   // point-major pass, acc is null, and dL/dp goes per query to gp_query.
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -2707,8 +2744,10 @@ __global__ void __launch_bounds__(256)
 
 // Copies the per-point accumulators out to the caller's gradient arrays.
 __global__ void __launch_bounds__(256)
-    knn_grad_copy_kernel(const float4* __restrict__ acc, int64_t n, float* __restrict__ grad_z,
+    knn_grad_copy_kernel(const float4* acc, int64_t n, float* __restrict__ grad_z,
                          float* __restrict__ grad_xy) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float4 v = acc[i];
@@ -2717,24 +2756,6 @@ __global__ void __launch_bounds__(256)
 }
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
-
-// Launches `kernel` allowed to start before the kernel ahead of it in the
-// stream completes (programmatic dependent launch); the kernel itself waits
-// in pdl_wait() before touching memory, so only launch latency overlaps.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t stream,
-                       Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
 
 // Calls whose queries, a thread each, leave most of the GPU's warps empty.
 bool few_queries(int64_t m, int sm_count) { return m <= int64_t(sm_count) * 1024; }
@@ -2797,27 +2818,40 @@ cudaError_t launch_grid_sort(const float* data, int64_t n, const float* queries,
   if (e != cudaSuccess) return e;
   const unsigned bgrid = static_cast<unsigned>(
       std::max<int64_t>(1, std::min<int64_t>(int64_t(sm_count) * 4, (n + 255) / 256)));
-  box_plan_kernel<<<bgrid, 256, 0, s>>>(data, n, grid, radius, 1.0 / double(L.max_cells), knn_k);
-  const unsigned zgrid = static_cast<unsigned>(
-      std::min<int64_t>(int64_t(sm_count) * 8, (L.max_cells + 4 + 255) / 256));
-  zero_counts_kernel<<<zgrid, 256, 0, s>>>(grid, counts_d, counts_q);
+  e = launch_pdl(box_plan_kernel, bgrid, 256, 0, s, data, n, grid, radius,
+                 1.0 / double(L.max_cells), knn_k, L.max_cells, counts_d, counts_q);
+  if (e != cudaSuccess) return e;
   // Without the query sort, the queries join none of the three passes and
   // their records are written in the caller's order.
   const int64_t mq = sort_queries ? m : 0;
   const unsigned pgrid = static_cast<unsigned>((n + mq + 255) / 256);
-  count_kernel<<<pgrid, 256, 0, s>>>(grid, data, n, queries, mq, counts_d, counts_q);
-  scan_kernel<<<dim3(max_tiles, sort_queries ? 2 : 1), kScanBlock, 0, s>>>(
-      grid, counts_d, counts_q, starts_d, starts_q, sums, max_tiles, 0);
-  scatter_kernel<<<pgrid, 256, 0, s>>>(grid, data, n, queries, mq, starts_d, starts_q, sums,
-                                       max_tiles, counts_d, counts_q, sorted, qrec);
-  if (!sort_queries && m > 0)
-    query_identity_kernel<<<static_cast<unsigned>((m + 255) / 256), 256, 0, s>>>(queries, m, qrec);
-  return cudaGetLastError();
+  e = launch_pdl(count_kernel, pgrid, 256, 0, s, grid, data, n, queries, mq, counts_d, counts_q);
+  if (e == cudaSuccess)
+    e = launch_pdl(scan_kernel, dim3(max_tiles, sort_queries ? 2 : 1), kScanBlock, 0, s, grid,
+                   counts_d, counts_q, starts_d, starts_q, sums, max_tiles, 0);
+  if (e == cudaSuccess)
+    e = launch_pdl(scatter_kernel, pgrid, 256, 0, s, grid, data, n, queries, mq, starts_d, starts_q,
+                   sums, max_tiles, counts_d, counts_q, sorted, qrec);
+  if (e == cudaSuccess && !sort_queries && m > 0)
+    e = launch_pdl(query_identity_kernel, static_cast<unsigned>((m + 255) / 256), 256, 0, s, queries,
+                   m, qrec);
+  return e;
 }
 
 }  // namespace
 
 namespace {
+// The k-NN search's count tables of the data cells.
+cudaError_t launch_count_tables(const GridDev* grid, const int32_t* starts, const int32_t* base,
+                                int32_t* bpre, int32_t* sat, cudaStream_t s) {
+  cudaError_t e = launch_pdl(block_prefix_kernel, kMaxBlocksPerAxis, kMaxBlocksPerAxis, 0, s, grid,
+                             starts, base, bpre);
+  if (e == cudaSuccess)
+    e = launch_pdl(sat_kernel, (kMaxCellsPerAxis + 1 + kSatCols - 1) / kSatCols,
+                   kSatCols * kSatWarps, 0, s, grid, starts, base, sat);
+  return e;
+}
+
 // The values of sorted queries: one thread each, then a warp for each heavy one.
 cudaError_t launch_radius_queries(const GridDev* grid, const float4* sorted, int64_t n,
                                   const int32_t* starts, const int32_t* base, const float4* qrec,
@@ -2827,14 +2861,13 @@ cudaError_t launch_radius_queries(const GridDev* grid, const float4* sorted, int
   unsigned* heavy_count = &const_cast<GridDev*>(grid)->hard;
   auto run = [&](auto mode, auto wmode) {
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
-    local_query_kernel<M, W><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
-        few_queries(m, sm_count), heavy_count, heavy);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(
+        local_query_kernel<M, W>, qgrid, kLocalThreads, 0, s, grid, sorted, n, starts, base, qrec, m,
+        p, r2f, r2t, out, count_out, radius, few_queries(m, sm_count), heavy_count, heavy);
     if (e != cudaSuccess) return e;
-    return launch_pdl(local_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, s, grid,
+    return launch_pdl(local_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, 0, s, grid,
                       sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
-                      static_cast<const unsigned*>(heavy_count), static_cast<const int32_t*>(heavy));
+                      heavy_count, heavy);
   };
   using P2 = std::integral_constant<int, kPow2>;
   using PG = std::integral_constant<int, kPowGeneral>;
@@ -2876,11 +2909,14 @@ cudaError_t launch_local_backward(const float* data, int64_t n, const float* que
                                   float* grad_xy, float* grad_q, double* grad_p, void* workspace,
                                   const LocalLayout& L, int sm_count, cudaStream_t s,
                                   bool modified) {
-  cudaError_t e = launch_grid_sort(data, n, queries, m, radius, 0, workspace, L, sm_count, s);
-  if (e != cudaSuccess) return e;
+  // Cleared first, so that the kernels after the grid's memset overlap their
+  // launches.
+  cudaError_t e = cudaSuccess;
   if (grad_z && (e = cudaMemsetAsync(grad_z, 0, size_t(n) * 4, s)) != cudaSuccess) return e;
   if (grad_xy && (e = cudaMemsetAsync(grad_xy, 0, size_t(n) * 8, s)) != cudaSuccess) return e;
   if (grad_p && (e = cudaMemsetAsync(grad_p, 0, sizeof(double), s)) != cudaSuccess) return e;
+  e = launch_grid_sort(data, n, queries, m, radius, 0, workspace, L, sm_count, s);
+  if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const GridDev* grid = reinterpret_cast<const GridDev*>(ws + L.off_grid);
   const int32_t* starts_d = reinterpret_cast<const int32_t*>(ws + L.off_starts_d);
@@ -2901,18 +2937,17 @@ cudaError_t launch_local_backward(const float* data, int64_t n, const float* que
   int32_t* heavy = reinterpret_cast<int32_t*>(ws + L.off_hard);
   auto run = [&](auto mode, auto wmode) {
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
-    local_grad_query_kernel<M, W><<<qgrid, kLocalThreads, 0, s>>>(
-        grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec,
-        rec64, radius, few_queries(m, sm_count), heavy_count, heavy);
-    if ((e = cudaGetLastError()) == cudaSuccess)
-      e = launch_pdl(local_grad_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, s, grid,
-                     sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec,
-                     rec64, radius, static_cast<const unsigned*>(heavy_count),
-                     static_cast<const int32_t*>(heavy));
-    if (data_side)
-      local_grad_data_kernel<M, W><<<dgrid, kLocalThreads, 0, s>>>(
-          grid, sorted, n, starts_d, sums, starts_q, sums_q, qrec, m, rec, rec64, p, r2f, grad_z,
-          grad_xy, radius);
+    e = launch_pdl(local_grad_query_kernel<M, W>, qgrid, kLocalThreads, 0, s, grid, sorted, n,
+                   starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec, rec64, radius,
+                   few_queries(m, sm_count), heavy_count, heavy);
+    if (e == cudaSuccess)
+      e = launch_pdl(local_grad_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, 0, s,
+                     grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p,
+                     rec, rec64, radius, heavy_count, heavy);
+    if (e == cudaSuccess && data_side)
+      e = launch_pdl(local_grad_data_kernel<M, W>, dgrid, kLocalThreads, 0, s, grid, sorted, n,
+                     starts_d, sums, starts_q, sums_q, qrec, m, rec, rec64, p, r2f, grad_z, grad_xy,
+                     radius);
   };
   using P2 = std::integral_constant<int, kPow2>;
   using PG = std::integral_constant<int, kPowGeneral>;
@@ -3015,34 +3050,34 @@ cudaError_t launch_knn_backward(const float* data, int64_t n, const float* queri
   float* zbuf = reinterpret_cast<float*>(ws + L.bytes);
   int32_t* hit = reinterpret_cast<int32_t*>(ws + L.bytes + round_up(size_t(m) * 4, 256));
   int32_t* nbr = reinterpret_cast<int32_t*>(ws + L.bytes + 2 * round_up(size_t(m) * 4, 256));
+  const bool data_side = grad_z || grad_xy;
+  float4* acc = data_side && !deterministic
+                    ? reinterpret_cast<float4*>(ws + L.bytes + 2 * round_up(size_t(m) * 4, 256) +
+                                                round_up(size_t(m) * size_t(k) * 4, 256))
+                    : nullptr;
+  // Cleared first, so that the kernels after the grid's memset overlap their
+  // launches.
+  cudaError_t e = cudaSuccess;
+  if (acc && (e = cudaMemsetAsync(acc, 0, size_t(n) * 16, s)) != cudaSuccess) return e;
+  if (grad_p && !deterministic && (e = cudaMemsetAsync(grad_p, 0, sizeof(double), s)) != cudaSuccess)
+    return e;
   // Deterministic mode: rows in key order, so each query's own sums run in
   // one fixed order too.
-  cudaError_t e = launch_knn(data, n, queries, m, p, k, zbuf, nbr, nullptr, workspace, L, sm_count,
-                             s, hit, sort_queries, deterministic, warp_search);
+  e = launch_knn(data, n, queries, m, p, k, zbuf, nbr, nullptr, workspace, L, sm_count, s, hit,
+                 sort_queries, deterministic, warp_search);
   if (e != cudaSuccess) return e;
   if (deterministic)
     return launch_knn_backward_fixed_order(data, n, queries, m, p, k, grad_out, grad_z, grad_xy,
                                            grad_q, grad_p, ws, L, hit, nbr, s);
-  const bool data_side = grad_z || grad_xy;
-  float4* acc = data_side ? reinterpret_cast<float4*>(ws + L.bytes + 2 * round_up(size_t(m) * 4, 256) +
-                                                      round_up(size_t(m) * size_t(k) * 4, 256))
-                          : nullptr;
-  if (acc && (e = cudaMemsetAsync(acc, 0, size_t(n) * 16, s)) != cudaSuccess) return e;
-  if (grad_p && (e = cudaMemsetAsync(grad_p, 0, sizeof(double), s)) != cudaSuccess) return e;
   const float4* qrec = reinterpret_cast<const float4*>(ws + L.off_qrec);
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
-  if (p == 2.0)
-    knn_grad_kernel<kPow2><<<qgrid, kLocalThreads, 0, s>>>(qrec, m, data, n, nbr, hit, k, p,
-                                                           grad_out, acc, grad_q, grad_p,
-                                                           nullptr, nullptr);
-  else
-    knn_grad_kernel<kPowGeneral><<<qgrid, kLocalThreads, 0, s>>>(qrec, m, data, n, nbr, hit, k,
-                                                                 p, grad_out, acc, grad_q, grad_p,
-                                                                 nullptr, nullptr);
-  if (acc)
-    knn_grad_copy_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(acc, n, grad_z,
-                                                                               grad_xy);
-  return cudaGetLastError();
+  e = launch_pdl(p == 2.0 ? knn_grad_kernel<kPow2> : knn_grad_kernel<kPowGeneral>, qgrid,
+                 kLocalThreads, 0, s, qrec, m, data, n, nbr, hit, k, p, grad_out, acc, grad_q, grad_p,
+                 nullptr, nullptr);
+  if (e == cudaSuccess && acc)
+    e = launch_pdl(knn_grad_copy_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, s, acc, n,
+                   grad_z, grad_xy);
+  return e;
 }
 
 cudaError_t debug_check_failures(unsigned* sites, bool* enabled) {
@@ -3108,10 +3143,11 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
     auto kernel = list ? (a.p == 2.0 ? knn_query_kernel<kPow2, true> : knn_query_kernel<kPowGeneral, true>)
                        : (a.p == 2.0 ? knn_query_kernel<kPow2, false>
                                      : knn_query_kernel<kPowGeneral, false>);
-    kernel<<<static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads), kKnnThreads, smem, s>>>(
+    const cudaError_t e = launch_pdl(
+        kernel, static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads), kKnnThreads, smem, s,
         a.grid, a.sorted, a.starts, a.base, a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out,
         a.nbr_out, a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
-    if (!list) return cudaGetLastError();
+    if (e != cudaSuccess || !list) return e;
   }
   constexpr int per_block = kKnnWarpThreads / 32;
   // The hard list's length is known on the device only: enough blocks to
@@ -3119,10 +3155,9 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
   const int64_t blocks = all_warps ? (a.m + per_block - 1) / per_block : int64_t(sm_count) * 8;
   auto kernel = a.k <= 32 ? (a.p == 2.0 ? knn_warp_kernel<kPow2, 3> : knn_warp_kernel<kPowGeneral, 3>)
                           : (a.p == 2.0 ? knn_warp_kernel<kPow2, 4> : knn_warp_kernel<kPowGeneral, 4>);
-  kernel<<<static_cast<unsigned>(blocks), kKnnWarpThreads, 0, s>>>(
-      a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-      a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
-  return cudaGetLastError();
+  return launch_pdl(kernel, static_cast<unsigned>(blocks), kKnnWarpThreads, 0, s, a.grid, a.sorted,
+                    a.starts, a.base, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
+                    a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
 }
 
 }  // namespace
@@ -3151,9 +3186,8 @@ cudaError_t launch_knn(const float* data, int64_t n, const float* queries, int64
   const float4* qrec = reinterpret_cast<const float4*>(ws + L.off_qrec);
   int32_t* bpre = reinterpret_cast<int32_t*>(ws + L.off_bpre);
   int32_t* sat = reinterpret_cast<int32_t*>(ws + L.off_sat);
-  block_prefix_kernel<<<kMaxBlocksPerAxis, kMaxBlocksPerAxis, 0, s>>>(grid, starts_d, sums, bpre);
-  sat_kernel<<<(kMaxCellsPerAxis + 1 + kSatCols - 1) / kSatCols, kSatCols * kSatWarps, 0, s>>>(
-      grid, starts_d, sums, sat);
+  e = launch_count_tables(grid, starts_d, sums, bpre, sat, s);
+  if (e != cudaSuccess) return e;
   if (!warp_search)
     return launch_knn_search(
         KnnArgs{reinterpret_cast<GridDev*>(ws + L.off_grid), sorted, starts_d, sums, bpre, sat, qrec,
@@ -3162,9 +3196,8 @@ cudaError_t launch_knn(const float* data, int64_t n, const float* queries, int64
         sm_count, s);
   const unsigned qgrid = static_cast<unsigned>((m + kKnnThreads - 1) / kKnnThreads);
   auto kernel = p == 2.0 ? knn_sync_kernel<kPow2> : knn_sync_kernel<kPowGeneral>;
-  kernel<<<qgrid, kKnnThreads, sync_smem, s>>>(grid, sorted, starts_d, sums, bpre, sat, qrec, data, n,
-                                               m, p, k, out, nbr_out, kd2_out, hit_out, sort_rows);
-  return cudaGetLastError();
+  return launch_pdl(kernel, qgrid, kKnnThreads, sync_smem, s, grid, sorted, starts_d, sums, bpre, sat,
+                    qrec, data, n, m, p, k, out, nbr_out, kd2_out, hit_out, sort_rows);
 }
 
 namespace {
@@ -3173,8 +3206,8 @@ namespace {
 // For the radius form (radius > 0) the reach is recomputed for the call's
 // radius, which the host has checked is at most the build radius, so rho
 // stays below 2 and the coverage argument of the plan still holds.
-__global__ void index_prep_kernel(const GridDev* __restrict__ src, GridDev* __restrict__ dst,
-                                  double radius) {
+__device__ __forceinline__ void copy_plan(const GridDev* src,
+                                          GridDev* dst, double radius) {
   GridDev g = *src;
   g.box_ticket = 0xffffffffu;
   g.scan_ticket = 0xffffffffu;
@@ -3184,8 +3217,32 @@ __global__ void index_prep_kernel(const GridDev* __restrict__ src, GridDev* __re
   *dst = g;
 }
 
+// First kernel of a query call on an index: the plan copy and, for the query
+// sort, the histogram's clearing, or else the records in the caller's order.
+__global__ void __launch_bounds__(256)
+    index_prep_kernel(const GridDev* src, GridDev* dst, double radius,
+                      int32_t* counts) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) copy_plan(src, dst, radius);
+  zero_counts(counts, count_int4s(src->cells));
+}
+__global__ void __launch_bounds__(256)
+    index_identity_kernel(const GridDev* src, GridDev* dst,
+                          double radius, const float* queries, int64_t m,
+                          float4* qrec) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) copy_plan(src, dst, radius);
+  const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j >= m) return;
+  qrec[j] = make_float4(queries[2 * j], queries[2 * j + 1], __int_as_float(static_cast<int>(j)),
+                        0.f);
+}
+
 // Query side of a call on a prepared index: plan copy, then the counting
-// sort of the queries alone (the scan runs its query half only).
+// sort of the queries alone (the scan runs its query half only), or their
+// records as they come.
 cudaError_t launch_query_sort(const GridDev* xgrid, const float* queries, int64_t m, double radius,
                               int64_t max_cells, void* workspace, const QueryLayout& Q,
                               int sm_count, cudaStream_t s, bool sort_queries) {
@@ -3196,22 +3253,30 @@ cudaError_t launch_query_sort(const GridDev* xgrid, const float* queries, int64_
   int32_t* sums = reinterpret_cast<int32_t*>(ws + Q.off_sums);
   float4* qrec = reinterpret_cast<float4*>(ws + Q.off_qrec);
   const int max_tiles = scan_tiles_of(max_cells);
-  index_prep_kernel<<<1, 1, 0, s>>>(xgrid, grid, radius);
-  if (!sort_queries) {
-    query_identity_kernel<<<static_cast<unsigned>((m + 255) / 256), 256, 0, s>>>(queries, m, qrec);
-    return cudaGetLastError();
-  }
-  const unsigned zgrid = static_cast<unsigned>(
-      std::min<int64_t>(int64_t(sm_count) * 8, (max_cells + 4 + 255) / 256));
-  zero_counts_kernel<<<zgrid, 256, 0, s>>>(grid, counts, counts);
   const unsigned qgrid = static_cast<unsigned>((m + 255) / 256);
-  count_kernel<<<qgrid, 256, 0, s>>>(grid, nullptr, 0, queries, m, counts, counts);
-  scan_kernel<<<dim3(max_tiles, 1), kScanBlock, 0, s>>>(grid, counts, counts, starts, starts, sums,
-                                                        max_tiles, 1);
-  scatter_kernel<<<qgrid, 256, 0, s>>>(grid, nullptr, 0, queries, m, starts, starts, sums,
-                                       max_tiles, counts, counts, nullptr, qrec);
-  return cudaGetLastError();
+  if (!sort_queries)
+    return launch_pdl(index_identity_kernel, qgrid, 256, 0, s, xgrid, grid, radius, queries, m, qrec);
+  const unsigned zgrid = static_cast<unsigned>(
+      std::min<int64_t>(int64_t(sm_count) * 4, (count_int4s(max_cells) + 255) / 256));
+  cudaError_t e = launch_pdl(index_prep_kernel, zgrid, 256, 0, s, xgrid, grid, radius, counts);
+  if (e == cudaSuccess)
+    e = launch_pdl(count_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, counts, counts);
+  if (e == cudaSuccess)
+    e = launch_pdl(scan_kernel, dim3(max_tiles, 1), kScanBlock, 0, s, grid, counts, counts, starts,
+                   starts, sums, max_tiles, 1);
+  if (e == cudaSuccess)
+    e = launch_pdl(scatter_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, starts, starts,
+                   sums, max_tiles, counts, counts, nullptr, qrec);
+  return e;
 }
+
+// Up to this many queries an index call leaves them as they come: the sort's
+// launches and passes (about 15 us) cost more than the locality saves.
+// Uniform queries in random order, index of 2^20 uniform points, sorted / as
+// they come: radius K = 32 m = 10,007 43.7 / 26.9 us, 150,001 56.0 / 45.6; k-NN
+// k = 8 m = 30,000 68.4 / 53.9, k = 32 m = 150,001 204.8 / 213.9 (50,000 points:
+// 146 / 216).
+constexpr int64_t kUnsortedRadius = int64_t(1) << 17, kUnsortedKnn = int64_t(1) << 15;
 
 }  // namespace
 
@@ -3264,26 +3329,26 @@ cudaError_t launch_index_build(const float* data, int64_t n, double radius, int 
   if (e != cudaSuccess) return e;
   const unsigned bgrid = static_cast<unsigned>(
       std::max<int64_t>(1, std::min<int64_t>(int64_t(sm_count) * 4, (n + 255) / 256)));
-  box_plan_kernel<<<bgrid, 256, 0, s>>>(data, n, grid, radius, 1.0 / double(X.max_cells), knn_k);
-  const unsigned zgrid = static_cast<unsigned>(
-      std::min<int64_t>(int64_t(sm_count) * 8, (X.max_cells + 4 + 255) / 256));
-  zero_counts_kernel<<<zgrid, 256, 0, s>>>(grid, counts, counts);
+  e = launch_pdl(box_plan_kernel, bgrid, 256, 0, s, data, n, grid, radius,
+                 1.0 / double(X.max_cells), knn_k, X.max_cells, counts, nullptr);
+  if (e != cudaSuccess) return e;
   const unsigned dgrid = static_cast<unsigned>((n + 255) / 256);
-  count_kernel<<<dgrid, 256, 0, s>>>(grid, data, n, nullptr, 0, counts, counts);
-  scan_kernel<<<dim3(max_tiles, 1), kScanBlock, 0, s>>>(grid, counts, counts, starts, starts, sums,
-                                                        max_tiles, 0);
-  scatter_kernel<<<dgrid, 256, 0, s>>>(grid, data, n, nullptr, 0, starts, starts, sums, max_tiles,
-                                       counts, counts, sorted, nullptr);
+  e = launch_pdl(count_kernel, dgrid, 256, 0, s, grid, data, n, nullptr, 0, counts, counts);
+  if (e == cudaSuccess)
+    e = launch_pdl(scan_kernel, dim3(max_tiles, 1), kScanBlock, 0, s, grid, counts, counts, starts,
+                   starts, sums, max_tiles, 0);
+  if (e == cudaSuccess)
+    e = launch_pdl(scatter_kernel, dgrid, 256, 0, s, grid, data, n, nullptr, 0, starts, starts, sums,
+                   max_tiles, counts, counts, sorted, nullptr);
+  if (e != cudaSuccess) return e;
   if (X.knn) {
     e = cudaMemcpyAsync(mem + X.off_data, data, size_t(n) * 12, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
     int32_t* bpre = reinterpret_cast<int32_t*>(mem + X.off_bpre);
     int32_t* sat = reinterpret_cast<int32_t*>(mem + X.off_sat);
-    block_prefix_kernel<<<kMaxBlocksPerAxis, kMaxBlocksPerAxis, 0, s>>>(grid, starts, sums, bpre);
-    sat_kernel<<<(kMaxCellsPerAxis + 1 + kSatCols - 1) / kSatCols, kSatCols * kSatWarps, 0, s>>>(
-        grid, starts, sums, sat);
+    return launch_count_tables(grid, starts, sums, bpre, sat, s);
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, const float* queries,
@@ -3293,7 +3358,7 @@ cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, cons
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
   cudaError_t e = launch_query_sort(xgrid, queries, m, radius, X.max_cells, workspace, Q, sm_count,
-                                    s, sort_queries);
+                                    s, sort_queries && m > kUnsortedRadius);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const GridDev* grid = reinterpret_cast<const GridDev*>(ws + Q.off_grid);
@@ -3316,7 +3381,7 @@ cudaError_t launch_index_knn(const void* index_mem, const IndexLayout& X, const 
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
   cudaError_t e = launch_query_sort(xgrid, queries, m, 0.0, X.max_cells, workspace, Q, sm_count, s,
-                                    sort_queries);
+                                    sort_queries && m > kUnsortedKnn);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const float4* qrec = reinterpret_cast<const float4*>(ws + Q.off_qrec);
