@@ -101,6 +101,7 @@ struct GridDev {
   unsigned keys[4];      // min x, min y, ~max x, ~max y (order-preserving keys)
   unsigned box_ticket;   // blocks of the box kernel done, minus one
   unsigned scan_ticket;  // scan tiles done, minus one
+  unsigned filled;       // data cells that hold a point, minus one
   float hx0, hy0, inv2;  // cell position u(v) = fl(fl(fl(v/2) - h0) * inv2)
   float rho;             // reach of R in cells, with margin (< 2)
   int gx, gy, cells;
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(kScanBlock)
                 int first) {
   pdl_trigger();
   pdl_wait();
-  __shared__ int32_t warp_tot[kScanBlock / 32];
+  __shared__ int32_t warp_tot[kScanBlock / 32], warp_full[kScanBlock / 32];
   __shared__ bool last;
   const int len = grid->cells + 1;
   const int ntiles = (len + kScanTile - 1) / kScanTile;
@@ -348,10 +349,19 @@ __global__ void __launch_bounds__(kScanBlock)
     in[i4] = make_int4(0, 0, 0, 0);
   }
   // Entries past len are zero: the arrays are cleared up to a multiple of 4.
+  if (half == 0) {
+    const int full = (v.x > 0) + (v.y > 0) + (v.z > 0) + (v.w > 0);
+    const int w = __reduce_add_sync(0xffffffffu, full);
+    if ((threadIdx.x & 31) == 0) warp_full[threadIdx.x >> 5] = w;
+  }
   int32_t total;
   const int32_t before = block_exclusive_scan(v.x + v.y + v.z + v.w, warp_tot, total);
   if (4 * i4 < len)
     out[i4] = make_int4(before, before + v.x, before + v.x + v.y, before + v.x + v.y + v.z);
+  if (half == 0 && threadIdx.x < 32) {  // warp_full was written before the scan's barriers
+    const int w = __reduce_add_sync(0xffffffffu, warp_full[threadIdx.x]);
+    if (threadIdx.x == 0 && w > 0) atomicAdd(&grid->filled, unsigned(w));
+  }
   if (threadIdx.x == 0) {
     sums[half * max_tiles + blockIdx.x] = total;  // published by the ticket
     last = ticket_acq_rel(&grid->scan_ticket) + 1u == unsigned(int(gridDim.y) * ntiles - 1);
@@ -1531,6 +1541,17 @@ __device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* sat,
   return c[1] >= k && c[0] <= 8 * k + 64;
 }
 
+// Whether the data fill their box about evenly: their cells hold at least 70%
+// as many points' cells as evenly random points would (uniform data: 100%; 64
+// blobs: about 10%).  Decides, on the device, between the search by counts and
+// the heap search; on clustered data the former lists too many queries (64
+// blobs, n = m = 2^20, k = 32: 3130 us against 2810 by heaps).
+__device__ __forceinline__ bool knn_even(const GridDev& g, int64_t n) {
+  const float cells = float(g.cells);
+  const float expected = cells * (1.f - ex2_approx(-1.44269504f * float(n) * rcp_approx(cells)));
+  return float(g.filled + 1u) >= 0.7f * expected;
+}
+
 // At most 64 registers (32 one-warp blocks per SM); left to itself the
 // compiler settles on fewer and spills.  With LIST, queries that are not
 // knn_easy are listed in `hard` for knn_warp_kernel.
@@ -1544,12 +1565,12 @@ __global__ void __maxnreg__(64)
                      double p, int k, float* __restrict__ out, int32_t* nbr_out,
                      float* __restrict__ kd2_out, int32_t* hit_out,
                      bool sort_rows, unsigned* hard_count,
-                     int32_t* hard) {
+                     int32_t* hard, bool uneven_only) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(16) unsigned char knn_smem[];
   const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= m) return;  // no block-wide barrier in this kernel
+  if (t >= m || (uneven_only && knn_even(*grid, n))) return;  // no block-wide barrier here
   KnnHeap hp;
   hp.h = reinterpret_cast<u64*>(knn_smem) + threadIdx.x;
   const GridDev g = *grid;
@@ -1736,6 +1757,211 @@ __global__ void __maxnreg__(64)
   }
   knn_write_result<MODE>(hp, best_hit, qx, qy, j, data, n, p, k, out, nbr_out, kd2_out, hit_out,
                          sort_rows);
+}
+
+// ------------------------------------------------- k-NN, one thread, by counts
+//
+// The search for calls that want no neighbour lists, on queries whose
+// surroundings are of even density (others are listed for the two searches
+// below):
+// 1. the summed-area table's count over a square of cells gives the local
+//    density, and with it a disc expected to hold the k nearest with a margin
+//    of four standard deviations of their number;
+// 2. the candidates the disc's cells hold are counted by d^2 into kBins equal
+//    bins, which are the lane's own column in shared memory; the bin in which
+//    the count reaches k bounds the k-th key;
+// 3. the cells within that bound are walked again: candidates of lower bins
+//    are summed at once (z is in the record), those of that bin are kept
+//    aside, and the smallest of them complete the k.
+// A disc that turns out to hold fewer than k points is tried again at 2.5
+// times the area, twice; then, or when more than kAside candidates share the
+// bin, the query is listed.  The selection is that of the other searches: the
+// bin is a monotone function of d^2 and ties are settled by (d^2, index).
+//
+// Against the heap search: no heap and no second gather of z, 8300 warp
+// instructions per 32 queries at k = 32 (17,000) with 17 of 32 lanes active
+// (12).  Bound by the latency of the candidate loads (26 warps an SM, which
+// the counters' 7 KB a warp allow).  Uniform n = m = 2^20, k = 32: 693 us by
+// heaps, 450 us.
+constexpr int kBins = 32;
+constexpr int kAside = 8;
+
+template <int MODE>
+__global__ void __launch_bounds__(kKnnThreads)
+    knn_count_kernel(const GridDev* grid, const float4* sorted, const int32_t* starts,
+                     const int32_t* base, const int32_t* sat, const float4* qrec,
+                     const float* data, int64_t n, int64_t m, double p, int k,
+                     float* __restrict__ out, float* __restrict__ kd2_out,
+                     unsigned* hard_count, int32_t* hard) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ int bins[kBins][kKnnThreads];
+  __shared__ u64 aside_key[kAside][kKnnThreads];
+  __shared__ float aside_z[kAside][kKnnThreads];
+  const int lane = threadIdx.x;
+  const int64_t t = int64_t(blockIdx.x) * kKnnThreads + lane;
+  const GridDev g = *grid;
+  // No block-wide barrier in this kernel: a lane reads its own columns.
+  if (t >= m || !knn_even(g, n)) return;
+  const float4 rq = qrec[t];
+  const float qx = rq.x, qy = rq.y;
+  const int j = __float_as_int(rq.z);
+  if (!dcheck(j >= 0 && j < m, kSiteOutput)) return;
+  if (!finite2(qx, qy)) {
+    out[j] = __int_as_float(0x7fc00000);
+    if (kd2_out) kd2_out[j] = __int_as_float(0x7fc00000);
+    return;
+  }
+  const float u = cell_pos(qx, g.hx0, g.inv2), v = cell_pos(qy, g.hy0, g.inv2);
+  const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
+  const float mg = __fmaf_ru(fabsf(u) + fabsf(v), 0x1p-22f, 0x1p-9f);
+  const float hh = g.inv2 > 0.f ? 2.f / g.inv2 : 0.f;
+  const float h2 = __fmul_rd(hh, hh) * (1.f - 0x1p-18f);
+  const float ih2 = __frcp_ru(h2);
+
+  // Points per cell around the query, from the square that holds 2k points
+  // at the mean density.
+  const float ca = float(g.cells) * rcp_approx(float(n));
+  const int re = int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * ca) - 1.f)));
+  const int ya = max(0, cy - re), yb = min(g.gy - 1, cy + re);
+  const int xa = max(0, cx - re), xb = min(g.gx - 1, cx + re);
+  const int W = g.gx + 1;
+  if (!dcheck(ya >= 0 && xa >= 0 && yb < g.gy && xb < g.gx, kSiteTable)) return;
+  const int held = sat[(yb + 1) * W + xb + 1] - sat[ya * W + xb + 1] - sat[(yb + 1) * W + xa] +
+                   sat[ya * W + xa];
+  // d^2 (in cells) of the disc expected to hold k points, and a margin.
+  const float per = float(held) * rcp_approx(float((yb - ya + 1) * (xb - xa + 1)));
+  const float fk = float(k);
+  float reach = fk * rcp_approx(3.14159265f * per) * (1.f + 4.f * rsqrt_approx(fk));
+  bool listed = !(g.inv2 > 0.f) || 4 * held < k || held > 8 * k + 64 || !(h2 >= 0x1p-100f) ||
+                !(h2 <= 0x1p60f);
+
+  // The runs of the cells that can hold a key up to d2 (rows and columns
+  // rounded outwards), row by row.
+  auto walk = [&](float d2, auto&& take) {
+    const float w2 = __fmul_ru(__fadd_ru(d2, 0x1p-126f), ih2);
+    auto clip = [&](float c, float e, int last, int& lo, int& hi) {
+      const float a = ceilf(__fsub_rd(__fsub_rd(__fsub_rd(c, mg), e), 1.f));
+      const float b = floorf(__fadd_ru(__fadd_ru(c, mg), e));
+      lo = int(fminf(fmaxf(0.f, a), float(last) + 1.f));
+      hi = int(fmaxf(fminf(float(last), b), -1.f));
+    };
+    // Row yy's run; empty beyond the disc.
+    auto run = [&](int yy, int& a, int& b) {
+      a = b = 0;
+      const float gap = fmaxf(0.f, fmaxf(float(yy) - v, v - float(yy + 1)) - mg);
+      const float g2 = __fmul_rd(gap, gap);
+      int ra, rb;
+      clip(u, __fsqrt_ru(__fsub_ru(w2, g2)), g.gx - 1, ra, rb);
+      if (g2 <= w2 && ra <= rb) {
+        a = cell_start(starts, base, yy * g.gx + ra, g.cells);
+        b = cell_start(starts, base, yy * g.gx + rb + 1, g.cells);
+      }
+    };
+    int r0, r1, a = 0, b = 0;
+    clip(v, __fsqrt_ru(w2), g.gy - 1, r0, r1);
+    if (r0 <= r1) run(r0, a, b);
+    for (int yy = r0; yy <= r1; ++yy) {
+      int na = 0, nb = 0;  // the next row's, looked up while this one is walked
+      if (yy < r1) run(yy + 1, na, nb);
+#pragma unroll 4
+      for (int q = a; q < b; ++q) {
+        if (!dcheck(q >= 0 && q < n, kSiteGather)) break;
+        take(sorted[q]);
+      }
+      a = na;
+      b = nb;
+    }
+  };
+
+  int below = 0, cut = -1;  // points in bins below `cut`, the bin where the count reaches k
+  float scale = 0.f, edge = 0.f;
+  // Bin of a d^2 below `edge`: 0 .. kBins - 1, monotone in d^2.
+  auto bin_of = [&](float d2) {
+    return min(__float_as_int(__fmaf_rn(d2, scale, 8388608.f)) - 0x4B000000, kBins - 1);
+  };
+  for (int attempt = 0; !listed && attempt < 3; ++attempt, reach *= 2.5f) {
+    edge = reach * hh * hh;
+    scale = float(kBins) * rcp_approx(edge);
+#pragma unroll
+    for (int b = 0; b < kBins; ++b) bins[b][lane] = 0;
+    walk(edge, [&](const float4 c) {
+      const float d2 = fp32_d2(qx, qy, c.x, c.y);
+      if (d2 < edge) ++bins[bin_of(d2)][lane];
+    });
+    int sum = 0;
+    for (int b = 0; b < kBins; ++b) {
+      const int c = bins[b][lane];
+      if (sum + c >= k) {
+        cut = b;
+        below = sum;
+        break;
+      }
+      sum += c;
+    }
+    if (cut >= 0) break;
+  }
+  if (cut < 0) listed = true;
+
+  const float hp = static_cast<float>(0.5 * p);
+  ValueSums<MODE, kWeightShepard> sums;  // of the selection
+  int best = INT_MAX, aside = 0;
+  float bestz = 0.f, kth = 0.f;
+  auto add = [&](float d2, float z) {
+    const float w = local_weight<MODE>(d2, hp, -hp);
+    two_sum_acc(sums.hi, sums.lo, pk(w, __fmul_rn(w, z)));
+  };
+  if (!listed) {
+    // Any d^2 in bins up to `cut` is below this (bins round to nearest, the
+    // last one reaches up to the edge).
+    const float bound = cut == kBins - 1
+                            ? edge
+                            : (float(cut) + 0.5f) * edge * ((1.f / kBins) * (1.f + 0x1p-18f));
+    walk(bound, [&](const float4 c) {
+      const float d2 = fp32_d2(qx, qy, c.x, c.y);
+      if (d2 < edge) {
+        const int b = bin_of(d2);
+        if (b < cut) {
+          add(d2, c.z);
+        } else if (b == cut) {
+          if (aside < kAside) {
+            aside_key[aside][lane] = knn_key(d2, __float_as_int(c.w));
+            aside_z[aside][lane] = c.z;
+          }
+          ++aside;
+        }
+        if (d2 == 0.f && c.x == qx && c.y == qy && __float_as_int(c.w) < best) {
+          best = __float_as_int(c.w);
+          bestz = c.z;
+        }
+      }
+    });
+    listed = aside > kAside;
+  }
+  if (listed) {
+    list_heavy(t, m, hard_count, hard);
+    return;
+  }
+  // The k - below smallest of the candidates set aside.
+  const int need = k - below;
+  for (int i = 0; i < aside; ++i) {
+    const u64 key = aside_key[i][lane];
+    int rank = 0;
+    for (int o = 0; o < aside; ++o) rank += aside_key[o][lane] < key;
+    if (rank < need) add(key_d2(key), aside_z[i][lane]);
+    if (rank == need - 1) kth = key_d2(key);
+  }
+  sums.cnt = k;
+  float z;
+  if (best != INT_MAX) {
+    z = bestz;
+  } else if (!sums.value(z)) {
+    // Sums outside FP32's range: the warp search redoes the query.
+    list_heavy(t, m, hard_count, hard);
+    return;
+  }
+  out[j] = z;
+  if (kd2_out) kd2_out[j] = kth;
 }
 
 // ------------------------------------------------- k-NN, a warp per query
@@ -3133,31 +3359,40 @@ struct KnnArgs {
 
 cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
   // Rows in search order (the gradients' plain FP32 sums follow it) keep the
-  // single-thread search's order.
+  // heap search's order.
   const bool warps = !a.nbr_out || a.sort_rows;
   const bool all_warps = warps && a.m <= knn_warp_queries(a.k);
+  // Without lists and from k = 17 on, evenly spread data are searched by counts
+  // (uniform n = m = 2^20, heaps / counts: k = 16 389 / 383 us, 24 550 / 454,
+  // 32 723 / 515, 64 1552 / 761); the device decides which of the two runs.
+  const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16;
   int32_t* list = warps && !all_warps && a.m <= kKnnHardQueries ? a.hard : nullptr;
   unsigned* hard_count = &a.grid->hard;
-  if (!all_warps) {
+  const unsigned threads_grid = static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads);
+  const bool pow2 = a.p == 2.0;
+  cudaError_t e = cudaSuccess;
+  if (counted)
+    e = launch_pdl(pow2 ? knn_count_kernel<kPow2> : knn_count_kernel<kPowGeneral>, threads_grid,
+                   kKnnThreads, 0, s, a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n,
+                   a.m, a.p, a.k, a.out, a.kd2_out, hard_count, a.hard);
+  if (e == cudaSuccess && !all_warps) {
     const size_t smem = knn_smem_bytes(a.k);  // below the default limit (k <= 64: 16 KB)
-    auto kernel = list ? (a.p == 2.0 ? knn_query_kernel<kPow2, true> : knn_query_kernel<kPowGeneral, true>)
-                       : (a.p == 2.0 ? knn_query_kernel<kPow2, false>
-                                     : knn_query_kernel<kPowGeneral, false>);
-    const cudaError_t e = launch_pdl(
-        kernel, static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads), kKnnThreads, smem, s,
-        a.grid, a.sorted, a.starts, a.base, a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out,
-        a.nbr_out, a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
-    if (e != cudaSuccess || !list) return e;
+    auto kernel = list ? (pow2 ? knn_query_kernel<kPow2, true> : knn_query_kernel<kPowGeneral, true>)
+                       : (pow2 ? knn_query_kernel<kPow2, false> : knn_query_kernel<kPowGeneral, false>);
+    e = launch_pdl(kernel, threads_grid, kKnnThreads, smem, s, a.grid, a.sorted, a.starts, a.base,
+                   a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out, a.kd2_out,
+                   a.hit_out, a.sort_rows, hard_count, a.hard, counted);
   }
+  if (e != cudaSuccess || (!all_warps && !list && !counted)) return e;
   constexpr int per_block = kKnnWarpThreads / 32;
-  // The hard list's length is known on the device only: enough blocks to
-  // fill the GPU stride over it.
+  // The list's length is known on the device only: enough blocks to fill the
+  // GPU stride over it.
   const int64_t blocks = all_warps ? (a.m + per_block - 1) / per_block : int64_t(sm_count) * 8;
-  auto kernel = a.k <= 32 ? (a.p == 2.0 ? knn_warp_kernel<kPow2, 3> : knn_warp_kernel<kPowGeneral, 3>)
-                          : (a.p == 2.0 ? knn_warp_kernel<kPow2, 4> : knn_warp_kernel<kPowGeneral, 4>);
+  auto kernel = a.k <= 32 ? (pow2 ? knn_warp_kernel<kPow2, 3> : knn_warp_kernel<kPowGeneral, 3>)
+                          : (pow2 ? knn_warp_kernel<kPow2, 4> : knn_warp_kernel<kPowGeneral, 4>);
   return launch_pdl(kernel, static_cast<unsigned>(blocks), kKnnWarpThreads, 0, s, a.grid, a.sorted,
                     a.starts, a.base, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                    a.kd2_out, a.hit_out, a.sort_rows, hard_count, list);
+                    a.kd2_out, a.hit_out, a.sort_rows, hard_count, all_warps ? nullptr : a.hard);
 }
 
 }  // namespace
