@@ -106,6 +106,7 @@ struct GridDev {
   float rho;             // reach of R in cells, with margin (< 2)
   int gx, gy, cells;
   unsigned hard;         // queries the per-thread kernels left to warps
+  unsigned next;         // next group of queries of the uneven-data heap search
 };
 
 // Order-preserving unsigned key of a float (for atomic min).
@@ -191,6 +192,7 @@ __device__ void plan_grid(GridDev* grid, double radius, double inv_max_cells, in
   grid->gy = gy;
   grid->cells = gx * gy;
   grid->hard = 0u;
+  grid->next = 0u;
 }
 
 // Zeroes a histogram over `len4` int4s (grid-stride; the scan reads int4s).
@@ -1552,25 +1554,15 @@ __device__ __forceinline__ bool knn_even(const GridDev& g, int64_t n) {
   return float(g.filled + 1u) >= 0.7f * expected;
 }
 
-// At most 64 registers (32 one-warp blocks per SM); left to itself the
-// compiler settles on fewer and spills.  With LIST, queries that are not
-// knn_easy are listed in `hard` for knn_warp_kernel.
+// Query t, by one thread (no block-wide barrier; `return`s are its own).
 template <int MODE, bool LIST>
-__global__ void __maxnreg__(64)
-    knn_query_kernel(const GridDev* grid, const float4* sorted,
-                     const int32_t* starts, const int32_t* base,
-                     const int32_t* bpre, const int32_t* sat,
-                     const float4* qrec, const float* data, int64_t n,
-                     int64_t m,
-                     double p, int k, float* __restrict__ out, int32_t* nbr_out,
-                     float* __restrict__ kd2_out, int32_t* hit_out,
-                     bool sort_rows, unsigned* hard_count,
-                     int32_t* hard, bool uneven_only) {
-  pdl_trigger();
-  pdl_wait();
+__device__ __forceinline__ void knn_thread_query(
+    const GridDev* grid, const float4* sorted, const int32_t* starts, const int32_t* base,
+    const int32_t* bpre, const int32_t* sat, const float4* qrec, const float* data, int64_t n,
+    int64_t m, double p, int k, float* __restrict__ out, int32_t* nbr_out,
+    float* __restrict__ kd2_out, int32_t* hit_out, bool sort_rows, unsigned* hard_count,
+    int32_t* hard, int64_t t) {
   extern __shared__ __align__(16) unsigned char knn_smem[];
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= m || (uneven_only && knn_even(*grid, n))) return;  // no block-wide barrier here
   KnnHeap hp;
   hp.h = reinterpret_cast<u64*>(knn_smem) + threadIdx.x;
   const GridDev g = *grid;
@@ -1759,6 +1751,44 @@ __global__ void __maxnreg__(64)
                          sort_rows);
 }
 
+// At most 64 registers (32 one-warp blocks per SM); left to itself the
+// compiler settles on fewer and spills.  With LIST, queries that are not
+// knn_easy are listed in `hard` for knn_warp_kernel.  With UNEVEN the kernel
+// runs on data that are not knn_even only, and its blocks, as many as fit the
+// GPU, fetch groups of 32 queries from a counter: 32,768 blocks that return
+// at once take 34 us.
+template <int MODE, bool LIST, bool UNEVEN>
+__global__ void __maxnreg__(64)
+    knn_query_kernel(const GridDev* grid, const float4* sorted,
+                     const int32_t* starts, const int32_t* base,
+                     const int32_t* bpre, const int32_t* sat,
+                     const float4* qrec, const float* data, int64_t n,
+                     int64_t m,
+                     double p, int k, float* __restrict__ out, int32_t* nbr_out,
+                     float* __restrict__ kd2_out, int32_t* hit_out,
+                     bool sort_rows, unsigned* hard_count,
+                     int32_t* hard, unsigned* next) {
+  pdl_trigger();
+  pdl_wait();
+  if (UNEVEN && knn_even(*grid, n)) return;
+  const int lane = threadIdx.x;
+  int64_t group = blockIdx.x;
+  for (;;) {
+    if (UNEVEN) {
+      unsigned fetched = 0;
+      if (lane == 0) fetched = atomicAdd(next, 1u);
+      group = __shfl_sync(0xffffffffu, fetched, 0);
+    }
+    const int64_t t = group * kKnnThreads + lane;
+    if (UNEVEN && group * kKnnThreads >= m) break;
+    if (t < m)
+      knn_thread_query<MODE, LIST>(grid, sorted, starts, base, bpre, sat, qrec, data, n, m, p, k, out,
+                                   nbr_out, kd2_out, hit_out, sort_rows, hard_count, hard, t);
+    if (!UNEVEN) break;
+    __syncwarp();
+  }
+}
+
 // ------------------------------------------------- k-NN, one thread, by counts
 //
 // The search for calls that want no neighbour lists, on queries whose
@@ -1785,9 +1815,10 @@ __global__ void __maxnreg__(64)
 // heaps, 450 us.
 constexpr int kBins = 32;
 constexpr int kAside = 8;
+constexpr int kCountThreads = 64;
 
 template <int MODE>
-__global__ void __launch_bounds__(kKnnThreads)
+__global__ void __launch_bounds__(kCountThreads)
     knn_count_kernel(const GridDev* grid, const float4* sorted, const int32_t* starts,
                      const int32_t* base, const int32_t* sat, const float4* qrec,
                      const float* data, int64_t n, int64_t m, double p, int k,
@@ -1795,11 +1826,11 @@ __global__ void __launch_bounds__(kKnnThreads)
                      unsigned* hard_count, int32_t* hard) {
   pdl_trigger();
   pdl_wait();
-  __shared__ int bins[kBins][kKnnThreads];
-  __shared__ u64 aside_key[kAside][kKnnThreads];
-  __shared__ float aside_z[kAside][kKnnThreads];
+  __shared__ int bins[kBins][kCountThreads];
+  __shared__ u64 aside_key[kAside][kCountThreads];
+  __shared__ float aside_z[kAside][kCountThreads];
   const int lane = threadIdx.x;
-  const int64_t t = int64_t(blockIdx.x) * kKnnThreads + lane;
+  const int64_t t = int64_t(blockIdx.x) * kCountThreads + lane;
   const GridDev g = *grid;
   // No block-wide barrier in this kernel: a lane reads its own columns.
   if (t >= m || !knn_even(g, n)) return;
@@ -3364,24 +3395,38 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
   const bool all_warps = warps && a.m <= knn_warp_queries(a.k);
   // Without lists and from k = 17 on, evenly spread data are searched by counts
   // (uniform n = m = 2^20, heaps / counts: k = 16 389 / 383 us, 24 550 / 454,
-  // 32 723 / 515, 64 1552 / 761); the device decides which of the two runs.
+  // 32 723 / 475, 64 1552 / 718); the device decides which of the two runs.
   const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16;
   int32_t* list = warps && !all_warps && a.m <= kKnnHardQueries ? a.hard : nullptr;
   unsigned* hard_count = &a.grid->hard;
-  const unsigned threads_grid = static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads);
   const bool pow2 = a.p == 2.0;
   cudaError_t e = cudaSuccess;
   if (counted)
-    e = launch_pdl(pow2 ? knn_count_kernel<kPow2> : knn_count_kernel<kPowGeneral>, threads_grid,
-                   kKnnThreads, 0, s, a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n,
+    e = launch_pdl(pow2 ? knn_count_kernel<kPow2> : knn_count_kernel<kPowGeneral>,
+                   static_cast<unsigned>((a.m + kCountThreads - 1) / kCountThreads), kCountThreads, 0,
+                   s, a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n,
                    a.m, a.p, a.k, a.out, a.kd2_out, hard_count, a.hard);
   if (e == cudaSuccess && !all_warps) {
     const size_t smem = knn_smem_bytes(a.k);  // below the default limit (k <= 64: 16 KB)
-    auto kernel = list ? (pow2 ? knn_query_kernel<kPow2, true> : knn_query_kernel<kPowGeneral, true>)
-                       : (pow2 ? knn_query_kernel<kPow2, false> : knn_query_kernel<kPowGeneral, false>);
-    e = launch_pdl(kernel, threads_grid, kKnnThreads, smem, s, a.grid, a.sorted, a.starts, a.base,
-                   a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out, a.kd2_out,
-                   a.hit_out, a.sort_rows, hard_count, a.hard, counted);
+    const unsigned groups = static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads);
+    const unsigned resident = std::min(groups, unsigned(sm_count) * 32);
+    auto heap = [&](auto kernel, unsigned blocks) {
+      return launch_pdl(kernel, blocks, kKnnThreads, smem, s, a.grid, a.sorted, a.starts, a.base,
+                        a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
+                        a.kd2_out, a.hit_out, a.sort_rows, hard_count, a.hard, &a.grid->next);
+    };
+    if (counted && list)
+      e = heap(pow2 ? knn_query_kernel<kPow2, true, true> : knn_query_kernel<kPowGeneral, true, true>,
+               resident);
+    else if (counted)
+      e = heap(pow2 ? knn_query_kernel<kPow2, false, true> : knn_query_kernel<kPowGeneral, false, true>,
+               resident);
+    else if (list)
+      e = heap(pow2 ? knn_query_kernel<kPow2, true, false> : knn_query_kernel<kPowGeneral, true, false>,
+               groups);
+    else
+      e = heap(pow2 ? knn_query_kernel<kPow2, false, false>
+                    : knn_query_kernel<kPowGeneral, false, false>, groups);
   }
   if (e != cudaSuccess || (!all_warps && !list && !counted)) return e;
   constexpr int per_block = kKnnWarpThreads / 32;
@@ -3447,6 +3492,7 @@ __device__ __forceinline__ void copy_plan(const GridDev* src,
   g.box_ticket = 0xffffffffu;
   g.scan_ticket = 0xffffffffu;
   g.hard = 0u;
+  g.next = 0u;
   if (radius > 0.0 && g.inv2 > 0.f)
     g.rho = __fmaf_ru(__fmul_ru(__double2float_ru(radius), g.inv2), 0.5f + 0x1p-9f, 0x1p-8f);
   *dst = g;
