@@ -10,6 +10,7 @@ and autograd plumbing.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 import threading
@@ -76,11 +77,17 @@ def get_handle(device=None) -> Handle:
 
 
 def _stream(t: torch.Tensor):
-    return ctypes.c_void_p(torch.cuda.current_stream(t.device).cuda_stream)
+    """The current stream of ``t``'s device, as an address."""
+    return _raw_stream(t.get_device())
+
+
+# A plain integer, without building a torch.cuda.Stream (2.4 us of a 22 us call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _prec(precision):
@@ -223,24 +230,43 @@ def interpolate_batched(datas, queries_list, p: float = 2.0, outs=None,
         raise ValueError("datas and queries_list differ in length")
     if k == 0:
         return []
-    dev = datas[0].device
+    dev, dt = datas[0].device, _DTYPE[prec]
+    index = datas[0].get_device()  # -1 on the host: refused below
+    # One pass with each problem's checks in one expression (64 problems spent
+    # 0.2 ms in separate checks); what fails it is checked again one by one
+    # for the message.
+    dp, nn, qp, mm = [], [], [], []
     for d, q in zip(datas, queries_list):
-        _check_inputs(d, q, prec)
-        if d.device != dev:
+        ds, qs = d.shape, q.shape
+        if (index < 0 or d.get_device() != index or q.get_device() != index or d.dtype != dt
+                or q.dtype != dt or len(ds) != 2 or ds[1] != 3 or len(qs) != 2 or qs[1] != 2
+                or not d.is_contiguous() or not q.is_contiguous()):
+            _check_inputs(d, q, prec)
             raise ValueError(f"every problem must be on {dev}, got {d.device}")
+        dp.append(d.data_ptr())
+        nn.append(ds[0])
+        qp.append(q.data_ptr())
+        mm.append(qs[0])
     if outs is None:
-        outs = [torch.empty(q.shape[0], dtype=_DTYPE[prec], device=dev) for q in queries_list]
+        outs = [torch.empty(m, dtype=dt, device=dev) for m in mm]
     if len(outs) != k:
         raise ValueError(f"outs must hold {k} tensors, got {len(outs)}")
-    for i, (o, q) in enumerate(zip(outs, queries_list)):
-        _check_buf(o, q.shape[0], _DTYPE[prec], dev, f"outs[{i}]")
+    op = []
+    for i, (o, m) in enumerate(zip(outs, mm)):
+        if (not isinstance(o, torch.Tensor) or o.dtype != dt or o.get_device() != index
+                or o.numel() != m or not o.is_contiguous()):
+            _check_buf(o, m, dt, dev, f"outs[{i}]")
+        op.append(o.data_ptr())
     h = _handle_for(handle, dev)
     P = ctypes.c_void_p * k
     I = ctypes.c_int64 * k
+
+    def addresses(v):
+        return P.from_buffer(array.array("Q", v))
+
     st = h.lib.idw_interpolate_batched(
-        h.ptr, k, P(*[d.data_ptr() for d in datas]), I(*[d.shape[0] for d in datas]),
-        P(*[q.data_ptr() for q in queries_list]), I(*[q.shape[0] for q in queries_list]),
-        float(p), prec, P(*[o.data_ptr() for o in outs]), _stream(datas[0]))
+        h.ptr, k, addresses(dp), I.from_buffer(array.array("q", nn)), addresses(qp),
+        I.from_buffer(array.array("q", mm)), float(p), prec, addresses(op), _stream(datas[0]))
     _lib.check(st, "idw_interpolate_batched", h.ptr)
     return outs
 
