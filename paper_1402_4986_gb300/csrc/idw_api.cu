@@ -507,6 +507,7 @@ idw_status idw_interpolate_saved(idw_handle_t h, const void* data, int64_t n, co
     bp.force_general = h->opt_force_general != 0;
     bp.layout = v == 0 ? h->opt_layout : -1;
     bp.fma_log2 = fma_log2;
+    bp.small_ok = h->opt_variant < 0 && !h->opt_autotune && h->opt_layout < 0 && !fma_log2;
     st = ensure_buffer(h, &h->ws, &h->ws_bytes, bp.workspace_bytes);
     if (st != IDW_OK) return st;
     h->last_variant = v;

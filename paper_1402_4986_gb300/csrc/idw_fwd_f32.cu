@@ -670,6 +670,276 @@ __global__ void bounded_wait_selftest_kernel(unsigned* err) {
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// One launch for a small problem: no staging, workspace or partials.  A
+// cluster of 8 CTAs takes 128 queries; each CTA reads an eighth of the points
+// into shared memory, and its 256 threads are 64 query pairs x 4 interleaved
+// quarters of them.  The cluster agrees on the scale (largest |coordinate| of
+// the points and its own queries) and joins its sums through distributed
+// shared memory; CTA r finishes queries 16 r .. 16 r + 15 and answers its hits
+// itself, a warp for two of them.  Sums are chunks of 16 points (S0 a tree, S1
+// chains of 4 joined by a tree) folded by TwoSum, and no reciprocal is shared:
+// errors against 64 bits are 0.5-0.95 of the sweep's, and a hit leaves its
+// neighbour's sums alone.  Such calls are bound by latency: launches, the
+// loads and three cluster barriers.  Against stage, sweep, combine and slow
+// list, us: n = 1000, m = 1021: 5.8, from 13.8 (p = 2), 5.7 from 19.7 (3), 5.9
+// from 28.9 (2.5); 16 x 16: 6.0 from 13.7; 4096 x 4096: 12.5 from 21.3, all of
+// it hits 25.5 from 94.8; 10,000 x 1600: 19.7 from 24.7, hits 35 from 40.
+// The limits: a cluster's CTAs read a whole slice each, so past 12,288 points
+// hits cost more than in the sweep's list (16,384 x 1024: 52 against 44.5);
+// past 2^24 pairs or 16,384 queries the GPU is full and the sweep's larger
+// tiles are as fast (256 x 16,384: 14.0 against 17.7, 1000 x 16,384: 16.3
+// against 18.1).  Above p = 4 sums leave the fast form's range at ordinary
+// distances, and the slow list spreads their FP64 sums better.
+constexpr int kSmallQueries = 128, kSmallCluster = 8, kSmallThreads = 256;
+constexpr int64_t kSmallPoints = 12288, kSmallMax = 1 << 14, kSmallPairs = int64_t(1) << 24;
+constexpr double kSmallPower = 4.0;
+constexpr int kSmallChunk = 16, kSmallSubs = kSmallThreads / (kSmallQueries / 2);
+constexpr int kSmallStep = kSmallSubs * kSmallChunk;  // a CTA's points are padded to these
+static_assert(kSmallThreads == kSlowThreads, "the CTA runs the slow path");
+
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+// The address of CTA `rank`'s copy of this CTA's shared variable.
+__device__ __forceinline__ uint32_t cluster_address(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+  return r;
+}
+
+struct SmallArgs {
+  const float* data;
+  const float* queries;
+  float* out;
+  double* s0_out;
+  int32_t* hit_out;
+  int32_t n, m;
+  float half_p, neg_half_p;
+  double p;
+};
+
+template <int MODE>
+__global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallThreads)
+    small_kernel(const SmallArgs a) {
+  extern __shared__ float4 rec[];  // the CTA's points, padded
+  __shared__ float4 part[kSmallSubs][kSmallQueries];
+  __shared__ float4 mine[kSmallQueries];                 // this CTA's sums, read by the cluster
+  __shared__ float4 piece[kSmallCluster][kSmallQueries / kSmallCluster];
+  __shared__ float maxima[kSmallCluster];                // written by the cluster
+  __shared__ float wmax[kSmallThreads / 32];
+  __shared__ int flagged[kSmallQueries / kSmallCluster], hit[kSmallQueries / kSmallCluster];
+  __shared__ float2 flagged_q[kSmallQueries / kSmallCluster];
+  __shared__ int nflagged;
+  pdl_trigger();
+  cluster_arrive();  // a peer's shared memory may be written once the peer runs
+  pdl_wait();
+  const int tid = threadIdx.x, rank = blockIdx.x % kSmallCluster;
+  const int q0 = blockIdx.x / kSmallCluster * kSmallQueries;
+  const int first = static_cast<int>(int64_t(a.n) * rank / kSmallCluster);
+  const int count = static_cast<int>(int64_t(a.n) * (rank + 1) / kSmallCluster) - first;
+
+  // Points of the slice, queries of the pair, and the largest |coordinate|.
+  float mx = 0.f;
+  auto seen = [&](float v) {
+    if (fabsf(v) <= FLT_MAX) mx = fmaxf(mx, fabsf(v));
+  };
+#pragma unroll 4
+  for (int i = tid; i < count; i += kSmallThreads) {
+    const float* row = a.data + 3 * int64_t(first + i);
+    const float x = row[0], y = row[1];
+    rec[i] = make_float4(x, y, row[2], 0.f);
+    seen(x);
+    seen(y);
+  }
+  const int pair = tid % (kSmallQueries / 2), sub = tid / (kSmallQueries / 2);
+  const int ja = q0 + pair, jb = ja + kSmallQueries / 2;
+  float qxa = 0.f, qya = 0.f, qxb = 0.f, qyb = 0.f;
+  if (ja < a.m) {
+    qxa = a.queries[2 * ja];
+    qya = a.queries[2 * ja + 1];
+    seen(qxa);
+    seen(qya);
+  }
+  if (jb < a.m) {
+    qxb = a.queries[2 * jb];
+    qyb = a.queries[2 * jb + 1];
+    seen(qxb);
+    seen(qyb);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if ((tid & 31) == 0) wmax[tid >> 5] = mx;
+  if (tid == 0) nflagged = 0;
+  __syncthreads();
+  cluster_wait();
+  if (tid < kSmallCluster) {  // thread t tells CTA t
+    mx = wmax[0];
+    for (int w = 1; w < kSmallThreads / 32; ++w) mx = fmaxf(mx, wmax[w]);
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_address(&maxima[rank], tid)),
+                 "f"(mx)
+                 : "memory");
+  }
+  cluster_arrive();
+  cluster_wait();
+  mx = maxima[0];
+#pragma unroll
+  for (int c = 1; c < kSmallCluster; ++c) mx = fmaxf(mx, maxima[c]);
+  const float scale = scale_from_max(__float_as_uint(mx));
+  const int padded = (count + kSmallStep - 1) / kSmallStep * kSmallStep;
+  for (int i = tid; i < padded; i += kSmallThreads) {  // the rows this thread has written
+    const float4 v = i < count ? rec[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    rec[i] = i < count ? make_float4(v.x * scale, v.y * scale, v.z, 0.f)
+                       : make_float4(INFINITY, INFINITY, 0.f, 0.f);  // weight 0
+  }
+  __syncthreads();
+
+  const u64 QX = pk(qxa * scale, qxb * scale), QY = pk(qya * scale, qyb * scale);
+  const u64 hp2 = pk(a.half_p, a.half_p), nhp2 = pk(a.neg_half_p, a.neg_half_p);
+  u64 h0 = 0, l0 = 0, h1 = 0, l1 = 0;
+#pragma unroll 1
+  for (int c = 0; c < padded; c += kSmallStep) {
+    u64 P0[4], P1[2], T1 = 0, C0 = 0, C1 = 0;
+#pragma unroll
+    for (int r = 0; r < kSmallChunk; ++r) {
+      const float4 v = rec[c + r * kSmallSubs + sub];
+      const u64 dx = sub2(QX, pk(v.x, v.x)), dy = sub2(QY, pk(v.y, v.y));
+      const u64 d2 = fma2(dy, dy, mul2(dx, dx));
+      const u64 w = weight_pair<MODE>(d2, false, hp2, nhp2), zz = pk(v.z, v.z);
+      tree_push<4>(P0, w, r, C0);
+      T1 = r % 4 == 0 ? mul2(w, zz) : fma2(w, zz, T1);
+      if (r % 4 == 3) tree_push<2>(P1, T1, r / 4, C1);
+    }
+    two_sum_acc(h0, l0, C0);
+    two_sum_acc(h1, l1, C1);
+  }
+  two_sum_renorm(h0, l0);
+  two_sum_renorm(h1, l1);
+  float ha, hb, la, lb, ga, gb, ka, kb;
+  upk(h0, ha, hb);
+  upk(l0, la, lb);
+  upk(h1, ga, gb);
+  upk(l1, ka, kb);
+  part[sub][pair] = make_float4(ha, la, ga, ka);
+  part[sub][pair + kSmallQueries / 2] = make_float4(hb, lb, gb, kb);
+  __syncthreads();
+  auto fold = [](float4& t, const float4 v) {
+    two_sum_acc_f32(t.x, t.y, v.x);
+    t.y += v.y;
+    two_sum_acc_f32(t.z, t.w, v.z);
+    t.w += v.w;
+  };
+  if (tid < kSmallQueries) {
+    float4 t = part[0][tid];
+#pragma unroll
+    for (int i = 1; i < kSmallSubs; ++i) fold(t, part[i][tid]);
+    mine[tid] = t;
+  }
+  cluster_arrive();
+  cluster_wait();
+  constexpr int kOwn = kSmallQueries / kSmallCluster;  // queries this CTA finishes
+  if (tid < kSmallQueries) {
+    const int from = tid / kOwn, q = tid % kOwn;
+    const uint32_t p = cluster_address(&mine[rank * kOwn + q], from);
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(p)
+                 : "memory");
+    piece[from][q] = v;
+  }
+  cluster_arrive();  // this CTA has read its peers' sums
+  const int j = q0 + rank * kOwn + tid;
+  if (tid < kOwn && j < a.m) {
+    float4 t = piece[0][tid];
+#pragma unroll
+    for (int c = 1; c < kSmallCluster; ++c) fold(t, piece[c][tid]);
+    const double s0 = double(t.x) + double(t.y), s1 = double(t.z) + double(t.w);
+    if (!(s0 > kTinySumPerPoint * double(a.n)) || !isfinite(s0) || !isfinite(s1) ||
+        (a.p >= 2.0 && s0 > kHugeSumPow2Up)) {
+      const int f = atomicAdd(&nflagged, 1);
+      flagged[f] = j;
+      flagged_q[f] = make_float2(a.queries[2 * j], a.queries[2 * j + 1]);
+    } else {
+      a.out[j] = static_cast<float>(s1 / s0);
+      if (a.s0_out) a.s0_out[j] = s0 * pow(double(scale), a.p);
+      if (a.hit_out) a.hit_out[j] = kNoHit;
+    }
+  }
+  cluster_wait();  // and its peers have read its own: it may leave
+  __syncthreads();
+  const int nf = nflagged;
+  if (nf == 0) return;
+  // A warp looks for the points under two of them: they stay in registers.
+  const int f0 = tid >> 5, f1 = f0 + kSmallThreads / 32;
+  static_assert(kOwn == 2 * (kSmallThreads / 32), "two flagged queries per warp");
+  if (f0 < nf) {
+    const float2 qa = flagged_q[f0], qb = f1 < nf ? flagged_q[f1] : make_float2(NAN, NAN);
+    int ia = INT_MAX, ib = INT_MAX;
+    for (int i0 = tid & 31; i0 < a.n; i0 += 32 * kSlowUnroll) {
+      float x[kSlowUnroll], y[kSlowUnroll];
+#pragma unroll
+      for (int u = 0; u < kSlowUnroll; ++u) {
+        const int i = min(i0 + 32 * u, a.n - 1);
+        x[u] = a.data[3 * i];
+        y[u] = a.data[3 * i + 1];
+      }
+#pragma unroll
+      for (int u = 0; u < kSlowUnroll; ++u) {
+        const int i = min(i0 + 32 * u, a.n - 1);
+        if (x[u] == qa.x && y[u] == qa.y) ia = min(ia, i);
+        if (x[u] == qb.x && y[u] == qb.y) ib = min(ib, i);
+      }
+    }
+    ia = __reduce_min_sync(0xffffffffu, ia);
+    ib = __reduce_min_sync(0xffffffffu, ib);
+    if ((tid & 31) == 0) {
+      hit[f0] = ia;
+      if (f1 < nf) hit[f1] = ib;
+    }
+  }
+  __syncthreads();
+  for (int f = 0; f < nf; ++f) {  // uniform across the CTA
+    const int jf = flagged[f];
+    float* out = &a.out[jf];
+    double* s0 = a.s0_out ? &a.s0_out[jf] : nullptr;
+    int32_t* hj = a.hit_out ? &a.hit_out[jf] : nullptr;
+    if (hit[f] != INT_MAX) {
+      if (tid == 0) slow_write_hit(a.data, hit[f], out, s0, hj);
+      continue;
+    }
+    SlowSums sums{INFINITY, 0.0, 0.0};  // of a query at infinity or NaN: a result of NaN
+    if (isfinite(flagged_q[f].x) && isfinite(flagged_q[f].y))
+      sums = slow_sums<float>(a.data, 0, a.n, flagged_q[f].x, flagged_q[f].y, a.p);
+    if (tid == 0) slow_write_sums(sums, a.p, out, s0, hj);
+  }
+}
+
+cudaError_t launch_small(const F32Problem& pb, double p, bool force_general, cudaStream_t stream) {
+  SmallArgs a{pb.data,
+              pb.queries,
+              pb.out,
+              pb.s0_out,
+              pb.hit_out,
+              static_cast<int32_t>(pb.n),
+              static_cast<int32_t>(pb.m),
+              static_cast<float>(0.5 * p),
+              static_cast<float>(-0.5 * p),
+              p};
+  auto kernel = force_general ? small_kernel<kPowGeneral>
+                : p == 2.0    ? small_kernel<kPow2>
+                : p == 1.0    ? small_kernel<kPow1>
+                : p == 3.0    ? small_kernel<kPow3>
+                : p == 4.0    ? small_kernel<kPow4>
+                              : small_kernel<kPowGeneral>;
+  const unsigned clusters = static_cast<unsigned>((pb.m + kSmallQueries - 1) / kSmallQueries);
+  const int64_t slice = (pb.n + kSmallCluster - 1) / kSmallCluster;
+  const size_t smem = size_t((slice + kSmallStep - 1) / kSmallStep * kSmallStep) * sizeof(float4);
+  return launch_pdl(kernel, dim3(clusters * kSmallCluster), dim3(kSmallThreads), smem, stream, a);
+}
+
 // Raises a kernel's dynamic shared memory limit to `bytes` (needed above
 // 48 KB), once per kernel and device (one flag word per instantiation).
 template <auto KERNEL>
@@ -908,6 +1178,9 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   if (plan.count < 1 || plan.count > kBatchCap) return cudaErrorInvalidValue;
   const bool one = plan.count == 1;
+  if (one && plan.small_ok && !ev && p <= kSmallPower && probs[0].n <= kSmallPoints &&
+      probs[0].m <= kSmallMax && probs[0].n * probs[0].m <= kSmallPairs)
+    return launch_small(probs[0], p, plan.force_general, stream);
   const bool pow2 = (p == 2.0) && !plan.force_general;
   // Default staging layout per weight form (measured fastest on GB300): the
   // aligned AoS record at p = 2, whose one shared load per point leaves the

@@ -101,6 +101,7 @@ extern "C" idw_status idw_interpolate_noalloc(const float* data_xyz, int64_t n,
       resolve_sweep_variant(default_sweep_variant(&pb, 1, general, dev.sm_count), general);
   BatchPlan plan;
   plan_batch_f32(&pb, 1, dev.sm_count, dev.occ[general ? 1 : 0][variant], variant, &plan);
+  plan.small_ok = true;
   if (plan.workspace_bytes > kNoAllocScratchBytes - kControlBytes) return IDW_ERR_WORKSPACE;
 
   Control* ctrl = reinterpret_cast<Control*>(dev.scratch);

@@ -1,0 +1,80 @@
+"""Problems that take the one-launch path (n <= 12288, m <= 16384, n m <= 2^24, p <= 4): parity with
+the FP64 oracle at its edges (cluster slices, chunks, query tiles, the largest
+sizes), hits, FP64 recomputations, saved outputs, NaN and infinities, scales,
+and the sizes just outside it."""
+import numpy as np
+import pytest
+
+import oracle
+import synthetic
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-6  # the FP32 form's bar, of the largest |z|
+
+
+def _dev(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("p", [1.0, 2.0, 3.0, 4.0, 2.5])
+@pytest.mark.parametrize("n,m", [(1, 1), (7, 128), (8, 129), (63, 64), (511, 5), (513, 1000),
+                                 (4095, 700), (4096, 4096), (4096, 4097), (12288, 130),
+                                 (12289, 130), (5, 16384), (5, 16385)])
+def test_parity(p, n, m):
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(n, m, seed=n + m, exact_hits=min(n, m, 6))
+    Z, s0, hit = idw.interpolate_saved(_dev(prob["data"]), _dev(prob["queries"]), p)
+    Z64, hit64 = oracle.idw(prob["data"], prob["queries"], p)
+    assert np.max(np.abs(Z.cpu().numpy() - Z64)) <= TOL * np.max(np.abs(prob["data"][:, 2]))
+    hit = hit.cpu().numpy()
+    assert np.array_equal(hit[hit >= 0], hit64[hit64 >= 0])
+    on = hit64 < 0
+    d = prob["queries"][on, None].astype(np.float64) - prob["data"][None, :, :2].astype(np.float64)
+    # S0 carries the weights' relative errors, 2e-6 in all at p = 4.
+    S0 = ((d ** 2).sum(-1) ** (-0.5 * p)).sum(1)
+    assert np.allclose(s0.cpu().numpy()[on], S0, rtol=2e-6, atol=0.0)
+    assert np.isinf(s0.cpu().numpy()[~on]).all()
+
+
+@pytest.mark.parametrize("p,scale", [(2.0, 2.0 ** -60), (2.0, 2.0 ** 60), (64.0, 1.0), (0.1, 1.0)])
+def test_scales_and_recomputed(p, scale):
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(900, 500, seed=3)
+    d, q = prob["data"].copy(), prob["queries"] * np.float32(scale)
+    d[:, :2] *= np.float32(scale)
+    z = idw.interpolate(_dev(d), _dev(q), p).cpu().numpy()
+    Z64, _ = oracle.idw(prob["data"], prob["queries"], p)
+    assert np.max(np.abs(z - Z64)) <= TOL * np.max(np.abs(d[:, 2]))
+
+
+@pytest.mark.parametrize("p", [2.0, 3.0, 2.5])
+def test_nan_and_infinity(p):
+    import torch
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(300, 300, seed=4)
+    data, q = prob["data"].copy(), prob["queries"].copy()
+    data[17, 0] = np.inf  # weight 0
+    q[5, 1] = np.nan
+    q[9, 0] = np.inf
+    z = idw.interpolate(_dev(data), _dev(q), p)
+    Z64, _ = oracle.idw(np.delete(data, 17, 0), prob["queries"], p)
+    assert torch.isnan(z[[5, 9]]).all()
+    z = np.delete(z.cpu().numpy(), [5, 9])
+    assert np.max(np.abs(z - np.delete(Z64, [5, 9]))) <= TOL * np.max(np.abs(data[:, 2]))
+
+
+def test_same_bits_and_capture():
+    import torch
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(1000, 1021, seed=6, exact_hits=3)
+    d, q = _dev(prob["data"]), _dev(prob["queries"])
+    z = idw.interpolate(d, q, 2.0)
+    out = torch.empty_like(z)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        idw.interpolate(d, q, 2.0, out=out)
+    out.zero_()
+    g.replay()
+    assert torch.equal(out, z)
