@@ -211,10 +211,11 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *       points x 2048 queries per resident CTA; else 4 when its 4096-query
  *       tiles pad the queries within 1% of variant 0's; else 0; or, where
  *       smaller tiles are predicted to be faster, 6 or 7: 512 queries per CTA
- *       with work units of 64 or 256 data points, which cannot be set; one
- *       problem of n <= 12,288, m <= 16,384, n m <= 2^24 and p <= 4 takes one
- *       launch without a sweep, unless a variant, a staging layout, the
- *       autotuner or IDW_OPT_FMA_LOG2 is set) or:
+ *       with work units of 64 or 256 data points, which cannot be set; a
+ *       problem or batch of n <= 12,288 each, n m <= 2^24 and 128 tiles of
+ *       128 queries in all, and p <= 4, takes one launch without a sweep,
+ *       unless a variant, a staging layout, the autotuner or IDW_OPT_FMA_LOG2
+ *       is set) or:
  *       0: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal;
  *       1: 2048 queries per CTA, no shared reciprocal;
  *       2: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal

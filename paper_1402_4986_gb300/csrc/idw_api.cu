@@ -611,6 +611,7 @@ idw_status idw_interpolate_batched(idw_handle_t h, int32_t count, const void* co
     plans.emplace_back();
     idw::plan_batch_f32(&probs[b], c, h->sm_count, ctas_per_sm(h, prec, p, v), v, &plans.back());
     plans.back().force_general = h->opt_force_general != 0;
+    plans.back().small_ok = h->opt_variant < 0 && !h->opt_autotune && h->opt_layout < 0;
     need = std::max(need, plans.back().workspace_bytes);
     h->last_variant = v;
   }

@@ -670,7 +670,7 @@ __global__ void bounded_wait_selftest_kernel(unsigned* err) {
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// One launch for a small problem: no staging, workspace or partials.  A
+// One launch for a small problem or batch: no staging, workspace or partials.  A
 // cluster of 8 CTAs takes 128 queries; each CTA reads an eighth of the points
 // into shared memory, and its 256 threads are 64 query pairs x 4 interleaved
 // quarters of them.  The cluster agrees on the scale (largest |coordinate| of
@@ -682,16 +682,18 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // neighbour's sums alone.  Such calls are bound by latency: launches, the
 // loads and three cluster barriers.  Against stage, sweep, combine and slow
 // list, us: n = 1000, m = 1021: 5.8, from 13.8 (p = 2), 5.7 from 19.7 (3), 5.9
-// from 28.9 (2.5); 16 x 16: 6.0 from 13.7; 4096 x 4096: 12.5 from 21.3, all of
+// from 28.9 (2.5); 16 x 16: 6.0 from 13.7; 4096 x 4096: 14 from 20, all of
 // it hits 25.5 from 94.8; 10,000 x 1600: 19.7 from 24.7, hits 35 from 40.
 // The limits: a cluster's CTAs read a whole slice each, so past 12,288 points
 // hits cost more than in the sweep's list (16,384 x 1024: 52 against 44.5);
-// past 2^24 pairs or 16,384 queries the GPU is full and the sweep's larger
-// tiles are as fast (256 x 16,384: 14.0 against 17.7, 1000 x 16,384: 16.3
-// against 18.1).  Above p = 4 sums leave the fast form's range at ordinary
+// past 2^24 pairs or 128 clusters the GPU is full and the sweep's larger
+// tiles are as fast (1000 x 16,000: 14.1 against 18.7; batches of 4e8 pairs and
+// more 5-10% slower).  Batches: 8 problems of 256 to 2048 points and queries
+// 22.3 us, from 34.1 (on the device 12.4 from 22.8), 128 of 16 to 64 on the
+// device 14.3 from 37.  Above p = 4 sums leave the fast form's range at ordinary
 // distances, and the slow list spreads their FP64 sums better.
 constexpr int kSmallQueries = 128, kSmallCluster = 8, kSmallThreads = 256;
-constexpr int64_t kSmallPoints = 12288, kSmallMax = 1 << 14, kSmallPairs = int64_t(1) << 24;
+constexpr int64_t kSmallPoints = 12288, kSmallClusters = 128, kSmallPairs = int64_t(1) << 24;
 constexpr double kSmallPower = 4.0;
 constexpr int kSmallChunk = 16, kSmallSubs = kSmallThreads / (kSmallQueries / 2);
 constexpr int kSmallStep = kSmallSubs * kSmallChunk;  // a CTA's points are padded to these
@@ -710,20 +712,10 @@ __device__ __forceinline__ uint32_t cluster_address(const void* p, int rank) {
   return r;
 }
 
-struct SmallArgs {
-  const float* data;
-  const float* queries;
-  float* out;
-  double* s0_out;
-  int32_t* hit_out;
-  int32_t n, m;
-  float half_p, neg_half_p;
-  double p;
-};
-
-template <int MODE>
+// Instance::qtile_base counts clusters here.
+template <int CAP, int MODE>
 __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallThreads)
-    small_kernel(const SmallArgs a) {
+    small_kernel(const __grid_constant__ Table<CAP> t, float half_p, float neg_half_p, double p) {
   extern __shared__ float4 rec[];  // the CTA's points, padded
   __shared__ float4 part[kSmallSubs][kSmallQueries];
   __shared__ float4 mine[kSmallQueries];                 // this CTA's sums, read by the cluster
@@ -737,7 +729,9 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
   cluster_arrive();  // a peer's shared memory may be written once the peer runs
   pdl_wait();
   const int tid = threadIdx.x, rank = blockIdx.x % kSmallCluster;
-  const int q0 = blockIdx.x / kSmallCluster * kSmallQueries;
+  const int cluster = blockIdx.x / kSmallCluster;
+  const Instance& a = t.inst[CAP == 1 ? 0 : find_qtile(t, cluster)];
+  const int q0 = (cluster - a.qtile_base) * kSmallQueries;
   const int first = static_cast<int>(int64_t(a.n) * rank / kSmallCluster);
   const int count = static_cast<int>(int64_t(a.n) * (rank + 1) / kSmallCluster) - first;
 
@@ -782,6 +776,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
                  "f"(mx)
                  : "memory");
   }
+  __syncwarp();
   cluster_arrive();
   cluster_wait();
   mx = maxima[0];
@@ -797,7 +792,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
   __syncthreads();
 
   const u64 QX = pk(qxa * scale, qxb * scale), QY = pk(qya * scale, qyb * scale);
-  const u64 hp2 = pk(a.half_p, a.half_p), nhp2 = pk(a.neg_half_p, a.neg_half_p);
+  const u64 hp2 = pk(half_p, half_p), nhp2 = pk(neg_half_p, neg_half_p);
   u64 h0 = 0, l0 = 0, h1 = 0, l1 = 0;
 #pragma unroll 1
   for (int c = 0; c < padded; c += kSmallStep) {
@@ -832,10 +827,10 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
     t.w += v.w;
   };
   if (tid < kSmallQueries) {
-    float4 t = part[0][tid];
+    float4 sum = part[0][tid];
 #pragma unroll
-    for (int i = 1; i < kSmallSubs; ++i) fold(t, part[i][tid]);
-    mine[tid] = t;
+    for (int i = 1; i < kSmallSubs; ++i) fold(sum, part[i][tid]);
+    mine[tid] = sum;
   }
   cluster_arrive();
   cluster_wait();
@@ -853,23 +848,23 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
   cluster_arrive();  // this CTA has read its peers' sums
   const int j = q0 + rank * kOwn + tid;
   if (tid < kOwn && j < a.m) {
-    float4 t = piece[0][tid];
+    float4 sum = piece[0][tid];
 #pragma unroll
-    for (int c = 1; c < kSmallCluster; ++c) fold(t, piece[c][tid]);
-    const double s0 = double(t.x) + double(t.y), s1 = double(t.z) + double(t.w);
+    for (int c = 1; c < kSmallCluster; ++c) fold(sum, piece[c][tid]);
+    const double s0 = double(sum.x) + double(sum.y), s1 = double(sum.z) + double(sum.w);
     if (!(s0 > kTinySumPerPoint * double(a.n)) || !isfinite(s0) || !isfinite(s1) ||
-        (a.p >= 2.0 && s0 > kHugeSumPow2Up)) {
+        (p >= 2.0 && s0 > kHugeSumPow2Up)) {
       const int f = atomicAdd(&nflagged, 1);
       flagged[f] = j;
       flagged_q[f] = make_float2(a.queries[2 * j], a.queries[2 * j + 1]);
     } else {
       a.out[j] = static_cast<float>(s1 / s0);
-      if (a.s0_out) a.s0_out[j] = s0 * pow(double(scale), a.p);
+      if (a.s0_out) a.s0_out[j] = s0 * pow(double(scale), p);
       if (a.hit_out) a.hit_out[j] = kNoHit;
     }
   }
-  cluster_wait();  // and its peers have read its own: it may leave
   __syncthreads();
+  cluster_wait();  // and its peers have read its own: it may leave
   const int nf = nflagged;
   if (nf == 0) return;
   // A warp looks for the points under two of them: they stay in registers.
@@ -912,32 +907,55 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
     }
     SlowSums sums{INFINITY, 0.0, 0.0};  // of a query at infinity or NaN: a result of NaN
     if (isfinite(flagged_q[f].x) && isfinite(flagged_q[f].y))
-      sums = slow_sums<float>(a.data, 0, a.n, flagged_q[f].x, flagged_q[f].y, a.p);
-    if (tid == 0) slow_write_sums(sums, a.p, out, s0, hj);
+      sums = slow_sums<float>(a.data, 0, a.n, flagged_q[f].x, flagged_q[f].y, p);
+    if (tid == 0) slow_write_sums(sums, p, out, s0, hj);
   }
 }
 
-cudaError_t launch_small(const F32Problem& pb, double p, bool force_general, cudaStream_t stream) {
-  SmallArgs a{pb.data,
-              pb.queries,
-              pb.out,
-              pb.s0_out,
-              pb.hit_out,
-              static_cast<int32_t>(pb.n),
-              static_cast<int32_t>(pb.m),
-              static_cast<float>(0.5 * p),
-              static_cast<float>(-0.5 * p),
-              p};
-  auto kernel = force_general ? small_kernel<kPowGeneral>
-                : p == 2.0    ? small_kernel<kPow2>
-                : p == 1.0    ? small_kernel<kPow1>
-                : p == 3.0    ? small_kernel<kPow3>
-                : p == 4.0    ? small_kernel<kPow4>
-                              : small_kernel<kPowGeneral>;
-  const unsigned clusters = static_cast<unsigned>((pb.m + kSmallQueries - 1) / kSmallQueries);
-  const int64_t slice = (pb.n + kSmallCluster - 1) / kSmallCluster;
+int64_t small_clusters(int64_t m) { return (m + kSmallQueries - 1) / kSmallQueries; }
+
+bool small_problems(const F32Problem* probs, int count, double p) {
+  int64_t clusters = 0, pairs = 0;
+  for (int k = 0; k < count; ++k) {
+    if (probs[k].n > kSmallPoints || probs[k].m > kSmallPairs) return false;
+    clusters += small_clusters(probs[k].m);
+    pairs += probs[k].n * probs[k].m;
+  }
+  return p <= kSmallPower && clusters <= kSmallClusters && pairs <= kSmallPairs;
+}
+
+template <int CAP>
+cudaError_t launch_small(const F32Problem* probs, int count, double p, bool force_general,
+                         cudaStream_t stream) {
+  Table<CAP> t;
+  t.count = count;
+  t.pad = 0;
+  int64_t clusters = 0, most = 0;
+  for (int k = 0; k < count; ++k) {
+    Instance& I = t.inst[k];
+    I = Instance{};
+    I.data = probs[k].data;
+    I.queries = probs[k].queries;
+    I.out = probs[k].out;
+    I.s0_out = probs[k].s0_out;
+    I.hit_out = probs[k].hit_out;
+    I.n = static_cast<int32_t>(probs[k].n);
+    I.m = static_cast<int32_t>(probs[k].m);
+    I.qtile_base = static_cast<int32_t>(clusters);
+    clusters += small_clusters(probs[k].m);
+    most = std::max(most, probs[k].n);
+  }
+  auto kernel = force_general ? small_kernel<CAP, kPowGeneral>
+                : p == 2.0    ? small_kernel<CAP, kPow2>
+                : p == 1.0    ? small_kernel<CAP, kPow1>
+                : p == 3.0    ? small_kernel<CAP, kPow3>
+                : p == 4.0    ? small_kernel<CAP, kPow4>
+                              : small_kernel<CAP, kPowGeneral>;
+  const int64_t slice = (most + kSmallCluster - 1) / kSmallCluster;
   const size_t smem = size_t((slice + kSmallStep - 1) / kSmallStep * kSmallStep) * sizeof(float4);
-  return launch_pdl(kernel, dim3(clusters * kSmallCluster), dim3(kSmallThreads), smem, stream, a);
+  return launch_pdl(kernel, dim3(static_cast<unsigned>(clusters * kSmallCluster)),
+                    dim3(kSmallThreads), smem, stream, t, static_cast<float>(0.5 * p),
+                    static_cast<float>(-0.5 * p), p);
 }
 
 // Raises a kernel's dynamic shared memory limit to `bytes` (needed above
@@ -1178,9 +1196,9 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   if (plan.count < 1 || plan.count > kBatchCap) return cudaErrorInvalidValue;
   const bool one = plan.count == 1;
-  if (one && plan.small_ok && !ev && p <= kSmallPower && probs[0].n <= kSmallPoints &&
-      probs[0].m <= kSmallMax && probs[0].n * probs[0].m <= kSmallPairs)
-    return launch_small(probs[0], p, plan.force_general, stream);
+  if (plan.small_ok && !ev && small_problems(probs, plan.count, p))
+    return one ? launch_small<1>(probs, 1, p, plan.force_general, stream)
+               : launch_small<kBatchCap>(probs, plan.count, p, plan.force_general, stream);
   const bool pow2 = (p == 2.0) && !plan.force_general;
   // Default staging layout per weight form (measured fastest on GB300): the
   // aligned AoS record at p = 2, whose one shared load per point leaves the

@@ -1,4 +1,5 @@
-"""Problems that take the one-launch path (n <= 12288, m <= 16384, n m <= 2^24, p <= 4): parity with
+"""Problems and batches that take the one-launch path (n <= 12288, at most 128
+tiles of 128 queries, n m <= 2^24, p <= 4): parity with
 the FP64 oracle at its edges (cluster slices, chunks, query tiles, the largest
 sizes), hits, FP64 recomputations, saved outputs, NaN and infinities, scales,
 and the sizes just outside it."""
@@ -78,3 +79,17 @@ def test_same_bits_and_capture():
     out.zero_()
     g.replay()
     assert torch.equal(out, z)
+
+
+@pytest.mark.parametrize("p", [2.0, 3.0, 2.5])
+@pytest.mark.parametrize("sizes", [[(1, 1), (300, 128), (5, 129), (12288, 3), (64, 700)],
+                                   [(40, 20)] * 128, [(40, 20)] * 129])
+def test_batch(p, sizes):
+    import paper_1402_4986_gb300 as idw
+    probs = [synthetic.uniform_problem(n, m, seed=i, exact_hits=min(n, m, 2))
+             for i, (n, m) in enumerate(sizes)]
+    zs = idw.interpolate_batched([_dev(q["data"]) for q in probs],
+                                 [_dev(q["queries"]) for q in probs], p)
+    for z, q in zip(zs, probs):
+        Z64, _ = oracle.idw(q["data"], q["queries"], p)
+        assert np.max(np.abs(z.cpu().numpy() - Z64)) <= TOL * np.max(np.abs(q["data"][:, 2]))
