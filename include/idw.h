@@ -212,7 +212,7 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *       tiles pad the queries within 1% of variant 0's; else 0; or, where
  *       smaller tiles are predicted to be faster, 6 or 7: 512 queries per CTA
  *       with work units of 64 or 256 data points, which cannot be set; a
- *       problem or batch of n <= 12,288 each, n m <= 2^24 and 128 tiles of
+ *       problem or batch of n <= 12,288 each, n m <= 100 2^20 and 256 tiles of
  *       128 queries in all, and p <= 4, takes one launch without a sweep,
  *       unless a variant, a staging layout, the autotuner or IDW_OPT_FMA_LOG2
  *       is set) or:

@@ -414,9 +414,16 @@ __global__ void __launch_bounds__(Var<V>::NT, 512 / Var<V>::NT)
 // this one, which spread each search over the GPU.  Block 0 finally clears
 // the per-problem range words the range scan and staging of this call used,
 // so the next call (or graph replay) starts from zero without a memset.
-constexpr int kCombineQueries = 32;
-constexpr int kCombineLanes = 8;
-static_assert(kCombineQueries * kCombineLanes == kSlowThreads, "the combine CTA runs the slow path");
+//
+// Lanes per query: 8, or 32 where a query has many pieces (few query tiles),
+// whose loads are otherwise a serial chain.  13,000 x 500 (304 pieces): 22.7
+// us by 8 lanes, 19.8 by 32; 100,000 x 2000 74.8 and 69.6; 12,000 x 12,000 (51
+// pieces) 50.9 and 53.7; 20,000 x 20,000 (31) 111.7 and 117.3.  6 CTAs per SM:
+// left alone the slow path's loads take 64 registers and 4 CTAs (2000 x
+// 100,000: 73.3 us, 70.5), and at 8 CTAs it spills (no faster).
+constexpr int kCombineManyPieces = 128;
+constexpr int kCombineThreads = 256;
+static_assert(kCombineThreads == kSlowThreads, "the combine CTA runs the slow path");
 
 // Flagged queries of problems up to this many points stay with their CTA:
 // one FP64 recomputation of 2048 points keeps one SM's FP64 pipe busy for
@@ -441,11 +448,12 @@ struct SlowList {
   unsigned cap;
 };
 
-template <int CAP, int QT>
-__global__ void __launch_bounds__(kCombineQueries * kCombineLanes)
+template <int CAP, int QT, int kCombineLanes>
+__global__ void __launch_bounds__(kCombineThreads, 6)
     combine_kernel(const __grid_constant__ Table<CAP> t, const float4* partial,
                    int64_t total_slots, int64_t units, int grid, const float* scales,
                    double p, Control* ctrl, const SlowList slow) {
+  constexpr int kCombineQueries = kCombineThreads / kCombineLanes;
   __shared__ float4 red[kCombineLanes][kCombineQueries];
   __shared__ int2 flagged[kCombineQueries];
   __shared__ int nflagged;
@@ -684,16 +692,17 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // list, us: n = 1000, m = 1021: 5.8, from 13.8 (p = 2), 5.7 from 19.7 (3), 5.9
 // from 28.9 (2.5); 16 x 16: 6.0 from 13.7; 4096 x 4096: 14 from 20, all of
 // it hits 25.5 from 94.8; 10,000 x 1600: 19.7 from 24.7, hits 35 from 40.
-// The limits: a cluster's CTAs read a whole slice each, so past 12,288 points
-// hits cost more than in the sweep's list (16,384 x 1024: 52 against 44.5);
-// past 2^24 pairs or 128 clusters the GPU is full and the sweep's larger
-// tiles are as fast (1000 x 16,000: 14.1 against 18.7; batches of 4e8 pairs and
-// more 5-10% slower).  Batches: 8 problems of 256 to 2048 points and queries
+// The limits: a flagged query's CTA reads all points, so past 12,288 of them
+// hits cost more than in the sweep's list (16,384 x 1024: 52 against 44.5).
+// Up to 100 M pairs the launch still wins (10,000 x 10,000: 37 against 42, all
+// hits 85 against 279; 3000 x 30,000: 36.5 against 42); beyond, and past 256
+// clusters, the sweep's larger tiles do more per load (12,000 x 12,000: level;
+// 1000 x 60,000: 42 against 33.5; batches of 4e8 pairs and more 5-10% slower).  Batches: 8 problems of 256 to 2048 points and queries
 // 22.3 us, from 34.1 (on the device 12.4 from 22.8), 128 of 16 to 64 on the
 // device 14.3 from 37.  Above p = 4 sums leave the fast form's range at ordinary
 // distances, and the slow list spreads their FP64 sums better.
 constexpr int kSmallQueries = 128, kSmallCluster = 8, kSmallThreads = 256;
-constexpr int64_t kSmallPoints = 12288, kSmallClusters = 128, kSmallPairs = int64_t(1) << 24;
+constexpr int64_t kSmallPoints = 12288, kSmallClusters = 256, kSmallPairs = int64_t(100) << 20;
 constexpr double kSmallPower = 4.0;
 constexpr int kSmallChunk = 16, kSmallSubs = kSmallThreads / (kSmallQueries / 2);
 constexpr int kSmallStep = kSmallSubs * kSmallChunk;  // a CTA's points are padded to these
@@ -846,6 +855,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
     piece[from][q] = v;
   }
   cluster_arrive();  // this CTA has read its peers' sums
+  __syncthreads();   // and its other warps' share of them is in place
   const int j = q0 + rank * kOwn + tid;
   if (tid < kOwn && j < a.m) {
     float4 sum = piece[0][tid];
@@ -1051,11 +1061,14 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
       size_t(INT_MAX)));
   slow.item = reinterpret_cast<SlowItem*>(ws);
   slow.part = reinterpret_cast<SlowSums*>(ws + size_t(slow.cap) * sizeof(SlowItem));
-  if ((e = launch_pdl(combine_kernel<CAP, QT>,
-                      dim3(static_cast<unsigned>((slots + kCombineQueries - 1) / kCombineQueries)),
-                      dim3(kCombineQueries * kCombineLanes), 0, stream, t,
-                      static_cast<const float4*>(partial), slots, plan.units, plan.grid,
-                      static_cast<const float*>(scales), p, ctrl, slow)) != cudaSuccess)
+  const int64_t pieces = plan.partial_slots / plan.total_query_tiles;  // of a query
+  const int lanes = pieces > kCombineManyPieces ? 32 : 8;
+  auto combine = lanes == 32 ? combine_kernel<CAP, QT, 32> : combine_kernel<CAP, QT, 8>;
+  const int per_cta = kCombineThreads / lanes;
+  if ((e = launch_pdl(combine, dim3(static_cast<unsigned>((slots + per_cta - 1) / per_cta)),
+                      dim3(kCombineThreads), 0, stream, t, static_cast<const float4*>(partial),
+                      slots, plan.units, plan.grid, static_cast<const float*>(scales), p, ctrl,
+                      slow)) != cudaSuccess)
     return e;
   int64_t most_points = 0;
   for (int k = 0; k < plan.count; ++k) most_points = std::max(most_points, probs[k].n);

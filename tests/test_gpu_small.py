@@ -1,5 +1,5 @@
-"""Problems and batches that take the one-launch path (n <= 12288, at most 128
-tiles of 128 queries, n m <= 2^24, p <= 4): parity with
+"""Problems and batches that take the one-launch path (n <= 12288, at most 256
+tiles of 128 queries, n m <= 100 2^20, p <= 4): parity with
 the FP64 oracle at its edges (cluster slices, chunks, query tiles, the largest
 sizes), hits, FP64 recomputations, saved outputs, NaN and infinities, scales,
 and the sizes just outside it."""
@@ -22,7 +22,7 @@ def _dev(a):
 @pytest.mark.parametrize("p", [1.0, 2.0, 3.0, 4.0, 2.5])
 @pytest.mark.parametrize("n,m", [(1, 1), (7, 128), (8, 129), (63, 64), (511, 5), (513, 1000),
                                  (4095, 700), (4096, 4096), (4096, 4097), (12288, 130),
-                                 (12289, 130), (5, 16384), (5, 16385)])
+                                 (12289, 130), (5, 32768), (5, 32769), (12288, 1000)])
 def test_parity(p, n, m):
     import paper_1402_4986_gb300 as idw
     prob = synthetic.uniform_problem(n, m, seed=n + m, exact_hits=min(n, m, 6))
@@ -83,7 +83,7 @@ def test_same_bits_and_capture():
 
 @pytest.mark.parametrize("p", [2.0, 3.0, 2.5])
 @pytest.mark.parametrize("sizes", [[(1, 1), (300, 128), (5, 129), (12288, 3), (64, 700)],
-                                   [(40, 20)] * 128, [(40, 20)] * 129])
+                                   [(40, 20)] * 256, [(40, 129)] * 129])
 def test_batch(p, sizes):
     import paper_1402_4986_gb300 as idw
     probs = [synthetic.uniform_problem(n, m, seed=i, exact_hits=min(n, m, 2))
@@ -93,3 +93,30 @@ def test_batch(p, sizes):
     for z, q in zip(zs, probs):
         Z64, _ = oracle.idw(q["data"], q["queries"], p)
         assert np.max(np.abs(z.cpu().numpy() - Z64)) <= TOL * np.max(np.abs(q["data"][:, 2]))
+
+
+@pytest.mark.parametrize("n,m", [(13000, 500), (30000, 2048), (30000, 2049), (30000, 5000)])
+def test_combine_lanes(n, m):
+    """Problems beyond the one-launch path whose queries have many pieces (one
+    or two query tiles) and few."""
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(n, m, seed=m, exact_hits=3)
+    z = idw.interpolate(_dev(prob["data"]), _dev(prob["queries"]), 2.0).cpu().numpy()
+    Z64, _ = oracle.idw(prob["data"], prob["queries"], 2.0)
+    assert np.max(np.abs(z - Z64)) <= TOL * np.max(np.abs(prob["data"][:, 2]))
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 12288])
+@pytest.mark.parametrize("repeat", range(3))
+def test_all_hits_of_a_full_gpu(n, repeat):
+    """Every query a hit, more clusters than the GPU holds at once."""
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(n, 8192, seed=n + repeat)
+    data = prob["data"]
+    rng = np.random.default_rng(repeat)
+    queries = np.ascontiguousarray(data[rng.integers(0, n, 8192), :2])
+    Z, s0, hit = idw.interpolate_saved(_dev(data), _dev(queries), 2.0)
+    Z64, hit64 = oracle.idw(data, queries, 2.0)
+    assert np.array_equal(hit.cpu().numpy(), hit64)
+    assert np.array_equal(Z.cpu().numpy(), Z64.astype(np.float32))
+    assert np.isinf(s0.cpu().numpy()).all()
