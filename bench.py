@@ -79,15 +79,15 @@ TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "sweep_p2_n1048576_dram.md")
 # and loop overhead not credited): FP32 FMA-pipe ops and MUFU ops by kind.
 #   p = 2      d^2 (2 FADD, FMUL, FFMA), S0 FADD, S1 FFMA; rcp
 #   general p  the same plus t = -(p/2) log2 d^2 (FMUL); lg2, ex2
-#   adjoint    one sweep's term (general p): d^2 (4), the two exponents (2
-#              FMUL), z - Z, (z - Z) v, two FFMA for the x / y sums, and for
-#              dL/dp (z - Z) w, log2 d^2 + shift, an FFMA; lg2 and two ex2
-#              (w and v = w / d^2).  The adjoint evaluates each pair twice
-#              (query sweep and data sweep).
+#   adjoint    both sides of a pair (general p): d^2 (4), the two exponents
+#              (2 FMUL), z - Z, the terms of the x / y sums of query and
+#              point, of dL/dz and, for dL/dp, log2 d^2 + shift; lg2 and two
+#              ex2 (w and v = w / d^2).  The fused sweep evaluates each pair
+#              once for both sides.
 SWEEP_COSTS = {
     "pow2": {"fma": 6.0, "mufu": {"mufu_rcp": 1.0}},
     "general": {"fma": 7.0, "mufu": {"mufu_lg2": 1.0, "mufu_ex2": 1.0}},
-    "adjoint_general": {"fma": 13.0, "mufu": {"mufu_lg2": 1.0, "mufu_ex2": 2.0}},
+    "adjoint_general": {"fma": 17.0, "mufu": {"mufu_lg2": 1.0, "mufu_ex2": 2.0}},
 }
 
 
@@ -447,7 +447,9 @@ def run_ours(args, ws, rank, local):
                                "FP32-compensated (FP64 combine)",
                    "n": n, "m": m, "p": 2.0, "parallelism": f"query shards x{ws}, data replicated",
                    "l2": "flushed between steps (256 MiB write; inputs are 36 MiB)"},
-        "e2e": e2e, "gpu_launches": 4 * args.steps,
+        "e2e": e2e,
+        # range, stage, sweep, combine; above 2048 points the slow list's search and finish.
+        "gpu_launches": (6 if n > 2048 else 4) * args.steps,
         "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
         "error_vs_fp64_oracle": err,
         **({"full_check": full} if full else {}),
@@ -547,10 +549,9 @@ def headline_extras(args, idw, h, data, q, data_np, q_np, single_pairs_s, rates,
     apairs = float(ad.shape[0]) * aq.shape[0]
     adj = {"n": ad.shape[0], "m": aq.shape[0], "p": ap["p"], "forward_ms": f_ms,
            "backward_ms": b_ms, "backward_over_forward": b_ms / f_ms,
-           "backward_pair_evaluations_s": 2 * apairs / (b_ms / 1e3),
+           "backward_pair_evaluations_s": apairs / (b_ms / 1e3),
            "roofline": roofline_block("adjoint_general", apairs / (b_ms / 1e3), rates, sms, mhz,
-                                      "query sweep + data sweep (whole backward call)",
-                                      evaluations_per_pair=2.0)}
+                                      "fused_adj_kernel (whole backward call)")}
     if not args.no_cpu_baseline:
         import oracle
         idx = np.sort(np.random.default_rng(12).choice(aq.shape[0], 256, replace=False))
@@ -796,14 +797,13 @@ def run_adjoint(args):
     pairs = float(n) * m
     rates, sms, mhz = _pipe_context()
     _emit("adjoint: N=M=262144 uniform [0,1)^2, wave field, p=2.5, upstream grad N(0,1); "
-          "backward = query sweep + data sweep (2 pair evaluations per pair)",
+          "backward = one fused sweep for both sides (1 pair evaluation per pair)",
           [{"forward_ms": fwd_ms, "forward_pairs_s": pairs / (fwd_ms / 1e3),
             "backward_ms": bwd_ms, "backward_pairs_s": pairs / (bwd_ms / 1e3),
-            "backward_pair_evaluations_s": 2 * pairs / (bwd_ms / 1e3),
+            "backward_pair_evaluations_s": pairs / (bwd_ms / 1e3),
             "backward_over_forward": bwd_ms / fwd_ms,
             "roofline": roofline_block("adjoint_general", pairs / (bwd_ms / 1e3), rates, sms, mhz,
-                                       "query sweep + data sweep (whole backward call)",
-                                       evaluations_per_pair=2.0),
+                                       "fused_adj_kernel (whole backward call)"),
             "forward_roofline": roofline_block("general", pairs / (fwd_ms / 1e3), rates, sms, mhz,
                                                "sweep_kernel<general p> (whole forward call)")}])
 
