@@ -65,3 +65,44 @@ def test_far_queries():
     prob = synthetic.uniform_problem(4000, 12, seed=9)
     q = (prob["queries"] + np.float32(10.0) ** np.arange(1, 13)[:, None] % np.float32(1e9))
     _check(prob["data"], np.ascontiguousarray(q.astype(np.float32)), 8)
+
+
+def _fastest(call, reps=5):
+    """Microseconds of one call among `reps`, the best of five turns."""
+    import torch
+    start, stop = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    best = float("inf")
+    call()
+    for _ in range(5):
+        start.record()
+        for _ in range(reps):
+            call()
+        stop.record()
+        stop.synchronize()
+        best = min(best, start.elapsed_time(stop) / reps * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("distance", [1e-3, 0.05, 0.4, 3.0])
+@pytest.mark.parametrize("k", [1, 8, 40])
+def test_beyond_each_edge_and_corner(distance, k):
+    prob = synthetic.uniform_problem(20000, 0, seed=k)
+    r = np.random.default_rng(k)
+    along = r.random(24, dtype=np.float32)
+    lo, hi = np.full(24, -distance, np.float32), np.full(24, 1 + distance, np.float32)
+    sides = [lo, along, hi]
+    queries = np.concatenate([np.stack([x, y], 1) for x in sides for y in sides])
+    _check(prob["data"], np.ascontiguousarray(queries), k)
+
+
+def test_beyond_the_edge_takes_no_longer():
+    """Queries up to a box width outside walk the part of their disc that
+    reaches the data, about as many points as those inside walk (2 times as
+    long a call; 28 times when the disc's count ignored the edge)."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(1 << 20, 10007, seed=3)
+    index = idw.LocalIndex(torch.from_numpy(prob["data"]).cuda(), k=8)
+    inside = torch.from_numpy(prob["queries"]).cuda()
+    outside = torch.where(inside < 0.5, inside - 1.0, inside + 1.0)
+    assert _fastest(lambda: index.knn(outside)) <= 8 * _fastest(lambda: index.knn(inside))
