@@ -2027,8 +2027,11 @@ struct KnnBuffer {
   // The k-th smallest d^2 is bracketed between lo (fewer than k keys at or
   // below) and hi (at least k) in the order of the float's bits; the probe
   // between them assumes keys spread evenly in d^2, as points of even density
-  // are, and every third probe halves the bracket instead, which ends the
-  // search whatever the keys.
+  // are, and every third probe halves the bracket instead.  No probe separates
+  // keys of equal d^2 (data on a lattice): after kProbes of them the bracket's
+  // ends move to keys, so that it closes on a tie at once, not bit by bit
+  // (lattice of 2^20 points, queries on it, m = 50,000, k = 64: 212 us, 170 so).
+  static constexpr int kProbes = 6;
   __device__ u64 prune(int& cnt, int k) {
     __syncwarp();
     if (cnt <= 32) return prune_regs<1>(cnt, k);
@@ -2053,7 +2056,7 @@ struct KnnBuffer {
     int hi = __reduce_max_sync(kWarp, dmax), chi = cnt;
     if (chi > k) {
       int lo = __reduce_min_sync(kWarp, dmin) - 1, clo = 0;
-      for (int it = 0; hi - lo > 1 && chi != k; ++it) {
+      for (int it = 0; it < kProbes && hi - lo > 1 && chi != k; ++it) {
         const float fl = __int_as_float(max(lo, 0)), fh = __int_as_float(hi);
         const float f = (float(k - clo) - 0.5f) * rcp_approx(float(chi - clo));
         int mid = it % 3 == 2 || !(fh <= FLT_MAX) ? lo + ((hi - lo) >> 1)
@@ -2068,6 +2071,24 @@ struct KnnBuffer {
           chi = c;
         } else {
           lo = mid;
+          clo = c;
+        }
+      }
+      while (hi - lo > 1 && chi != k) {  // ties: the end that moves goes on to a key
+        const int mid = lo + ((hi - lo) >> 1);
+        int c = 0, at = -1, above = INT_MAX;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          c += d[i] <= mid;
+          at = max(at, d[i] <= mid ? d[i] : -1);
+          above = min(above, d[i] > mid ? d[i] : INT_MAX);
+        }
+        c = __reduce_add_sync(kWarp, c);
+        if (c >= k) {
+          hi = __reduce_max_sync(kWarp, at);
+          chi = c;
+        } else {
+          lo = __reduce_min_sync(kWarp, above) - 1;
           clo = c;
         }
       }

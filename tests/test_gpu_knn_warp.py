@@ -106,3 +106,17 @@ def test_beyond_the_edge_takes_no_longer():
     inside = torch.from_numpy(prob["queries"]).cuda()
     outside = torch.where(inside < 0.5, inside - 1.0, inside + 1.0)
     assert _fastest(lambda: index.knn(outside)) <= 8 * _fastest(lambda: index.knn(inside))
+
+
+@pytest.mark.parametrize("k", [5, 32, 33, 64])
+def test_more_ties_than_the_buffer_holds(k):
+    """Eight places at one distance from the query, 60 points on each, and a
+    few nearer: the tie is wider than any buffer of keys."""
+    step = np.float32(0.25)
+    ring = step * np.array([[3, 4], [4, 3], [-3, 4], [-4, 3], [3, -4], [4, -3], [-3, -4], [5, 0]],
+                           np.float32)
+    near = step * np.array([[1, 0], [0, 2], [2, 2]], np.float32)
+    xy = np.concatenate([np.tile(ring, (60, 1)), near])
+    data = synthetic.pack_xyz(xy, np.linspace(-1, 1, len(xy), dtype=np.float32))
+    _check(data, np.zeros((33, 2), np.float32), k)
+    _check(data, np.zeros((33, 2), np.float32), k, p=3.5, index=True)
