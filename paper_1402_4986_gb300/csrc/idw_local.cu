@@ -106,7 +106,11 @@ struct GridDev {
   float rho;             // reach of R in cells, with margin (< 2)
   int gx, gy, cells;
   unsigned hard;         // queries the per-thread kernels left to warps
+  unsigned left;         // queries the search by counts left to warps or threads
   unsigned next;         // next group of queries of the uneven-data heap search
+  unsigned next_left;    // next group of the queries left
+  unsigned beyond;       // of kSampleQueries queries: those beyond the grid's edge,
+  unsigned dense;        // and those in dense surroundings (see knn_sample)
 };
 
 // Order-preserving unsigned key of a float (for atomic min).
@@ -191,8 +195,8 @@ __device__ void plan_grid(GridDev* grid, double radius, double inv_max_cells, in
   grid->gx = gx;
   grid->gy = gy;
   grid->cells = gx * gy;
-  grid->hard = 0u;
-  grid->next = 0u;
+  grid->hard = grid->left = grid->next = grid->next_left = 0u;
+  grid->beyond = grid->dense = 0u;
 }
 
 // Zeroes a histogram over `len4` int4s (grid-stride; the scan reads int4s).
@@ -261,6 +265,14 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// Up to this many queries an index call leaves them as they come: the sort's
+// launches and passes (about 15 us) cost more than the locality saves.
+// Uniform queries in random order, index of 2^20 uniform points, sorted / as
+// they come: radius K = 32 m = 10,007 43.7 / 26.9 us, 150,001 56.0 / 45.6; k-NN
+// k = 8 m = 30,000 68.4 / 53.9, k = 32 m = 150,001 204.8 / 213.9 (50,000 points:
+// 146 / 216).
+constexpr int64_t kUnsortedRadius = int64_t(1) << 17, kUnsortedKnn = int64_t(1) << 15;
+
 // Cell of a data point (-1: a non-finite point, in no cell) and sorting
 // bucket of a query (its cell clamped into the grid).
 __device__ __forceinline__ int data_cell(const GridDev& g, float x, float y) {
@@ -274,6 +286,11 @@ __device__ __forceinline__ int query_bucket(const GridDev& g, float x, float y) 
   const int cx = clamp_floor(cell_pos(x, g.hx0, g.inv2), 0, g.gx - 1);
   const int cy = clamp_floor(cell_pos(y, g.hy0, g.inv2), 0, g.gy - 1);
   return cy * g.gx + cx;
+}
+
+// Whether a position in cells lies beyond the grid's edge.
+__device__ __forceinline__ bool beyond_grid(const GridDev& g, float u, float v) {
+  return fmaxf(fmaxf(-u, u - float(g.gx)), fmaxf(-v, v - float(g.gy))) > 0.f;
 }
 
 // Threads [0, n) count data points, [n, n + m) count queries.
@@ -487,11 +504,56 @@ __global__ void __launch_bounds__(256)
                         0.f);
 }
 
+// MUFU square root (relative error ~2^-22, subnormal input flushed to 0).
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Radius of the square of cells that holds 2k points at the mean density:
+// ceil((sqrt(2 k ca) - 1) / 2) with ca cells per point.
+__device__ __forceinline__ int knn_square(float cells_per_point, int k) {
+  return int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
+}
+// More than this in that square is dense.
+__device__ __forceinline__ int knn_dense(int k) { return 8 * k + 64; }
+
+// What kSampleQueries of the queries, by a block of as many threads, have
+// around them: counts those beyond the grid's edge and those in dense
+// surroundings, from the cells' starts.
+constexpr int kSampleQueries = 256;
+constexpr int kSampleK = 2;  // with one neighbour a thread is through a cluster soon
+__device__ __forceinline__ void knn_sample(GridDev* out, const GridDev& g, const int32_t* starts,
+                                           const int32_t* base, int64_t n, const float* queries,
+                                           int64_t m, int k) {
+  const int64_t j = m * threadIdx.x / kSampleQueries;
+  const float x = queries[2 * j], y = queries[2 * j + 1];
+  bool beyond = false, dense = false;
+  if (finite2(x, y)) {
+    const float u = cell_pos(x, g.hx0, g.inv2), v = cell_pos(y, g.hy0, g.inv2);
+    const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
+    const int re = knn_square(float(g.cells) * rcp_approx(float(n)), k);
+    int held = 0;
+    for (int yy = max(0, cy - re); yy <= min(g.gy - 1, cy + re); ++yy)
+      held += cell_start(starts, base, yy * g.gx + min(g.gx - 1, cx + re) + 1, g.cells) -
+              cell_start(starts, base, yy * g.gx + max(0, cx - re), g.cells);
+    beyond = beyond_grid(g, u, v);
+    dense = held > knn_dense(k);
+  }
+  const int nb = __syncthreads_count(beyond), nd = __syncthreads_count(dense);
+  if (threadIdx.x == 0) {
+    out->beyond = nb;
+    out->dense = nd;
+  }
+}
+
 // Threads [0, n) place data points as (x, y, z, index), [n, n + m) place
-// queries as (x, y, index, 0).
+// queries as (x, y, index, 0).  With sample_k > 0 the last block samples the
+// call's `all` queries instead.
 __global__ void __launch_bounds__(256)
-    scatter_kernel(const GridDev* grid, const float* data, int64_t n,
-                   const float* queries, int64_t m,
+    scatter_kernel(GridDev* grid, const float* data, int64_t n,
+                   const float* queries, int64_t m, int64_t all, int sample_k,
                    const int32_t* starts_d, const int32_t* starts_q,
                    const int32_t* sums, int max_tiles,
                    int32_t* cursor_d, int32_t* cursor_q,
@@ -499,6 +561,10 @@ __global__ void __launch_bounds__(256)
   pdl_trigger();
   pdl_wait();
   const GridDev g = *grid;
+  if (sample_k > 0 && blockIdx.x == gridDim.x - 1) {
+    knn_sample(grid, g, starts_d, sums, n, queries, all, sample_k);
+    return;
+  }
   const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i < n) {
     const float x = data[3 * i], y = data[3 * i + 1];
@@ -525,13 +591,6 @@ __device__ __forceinline__ float local_weight(float d2, float hp, float nhp) {
   const float tl = fmaf(L, nhp, L * hp);  // exact rounding error of th
   const float e = ex2_approx(th);
   return fmaf(e, tl * 0.6931471805599453f, e);
-}
-
-// MUFU square root (relative error ~2^-22, subnormal input flushed to 0).
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
 }
 
 __device__ __forceinline__ float fp32_d2(float qx, float qy, float x, float y) {
@@ -618,7 +677,9 @@ __device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, boo
   const float per_cell = float(n) * rcp_approx(float(g.cells));
   return int(few ? fminf(fmaf(24.f, per_cell, 32.f), 1e9f) : fminf(fmaf(64.f, per_cell, 256.f), 1e9f));
 }
-// Lists query t (any subset of a warp's lanes may call it together).
+// Lists query t (any subset of a warp's lanes may call it together) from
+// `list` on upwards, or downwards (step = -1).
+template <int step = 1>
 __device__ __forceinline__ void list_heavy(int64_t t, int64_t m, unsigned* count,
                                            int32_t* list) {
   const unsigned lanes = __activemask();  // one atomic for those that are here together
@@ -626,7 +687,7 @@ __device__ __forceinline__ void list_heavy(int64_t t, int64_t m, unsigned* count
   unsigned at = 0;
   if (lane == lead) at = atomicAdd(count, unsigned(__popc(lanes)));
   at = __shfl_sync(lanes, at, lead) + __popc(lanes & ((1u << lane) - 1));
-  if (dcheck(at < m, kSiteScatter)) list[at] = static_cast<int32_t>(t);
+  if (dcheck(at < m, kSiteScatter)) list[step * int64_t(at)] = static_cast<int32_t>(t);
 }
 
 // Error-free sum of the lanes' compensated pairs (both packed lanes), by a
@@ -1518,17 +1579,19 @@ __device__ __forceinline__ void knn_write_result(KnnHeap& hp, int best_hit, floa
   }
 }
 
-// Whether one thread should search for a query in cell (cx, cy).  With ca
-// cells per point, the square of radius re = ceil((sqrt(2 k ca) - 1) / 2)
+// Whether one thread should search for a query in cell (cx, cy) (kEasy).  With
+// ca cells per point, the square of radius re = ceil((sqrt(2 k ca) - 1) / 2)
 // holds 2k points at the mean density.  Where the square one cell wider holds
-// fewer than k, the search has empty space to cross; where the square holds
-// over 8k + 64, it has a dense cluster to sift; a thread takes ten to a
-// hundred times as long over such a query as over one at the mean density,
-// and its warp waits.  (n = 2^20 points in 64 blobs, 100,000 uniform queries,
-// k = 8: 1.09 ms when every query was one thread's.)
-__device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* sat,
-                                         float cells_per_point, int cx, int cy, int k) {
-  const int re = int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
+// fewer than k, the search has empty space to cross (kSparse); where the square
+// holds over 8k + 64, it has a dense cluster to sift (kDense); a thread takes
+// ten to a hundred times as long over such a query as over one at the mean
+// density, and its warp waits.  (n = 2^20 points in 64 blobs, 100,000 uniform
+// queries, k = 8: 1.09 ms when every query was one thread's.)
+enum KnnSurroundings : int { kEasy, kSparse, kDense };
+__device__ __forceinline__ KnnSurroundings knn_surroundings(const GridDev& g, const int32_t* sat,
+                                                            float cells_per_point, int cx, int cy,
+                                                            int k) {
+  const int re = knn_square(cells_per_point, k);
   const int W = g.gx + 1;
   int c[2];
 #pragma unroll
@@ -1536,12 +1599,22 @@ __device__ __forceinline__ bool knn_easy(const GridDev& g, const int32_t* sat,
     const int rr = re + i;
     const int ya = max(0, cy - rr), yb = min(g.gy - 1, cy + rr);
     const int xa = max(0, cx - rr), xb = min(g.gx - 1, cx + rr);
-    if (!dcheck(ya >= 0 && xa >= 0 && yb < g.gy && xb < g.gx, kSiteTable)) return true;
+    if (!dcheck(ya >= 0 && xa >= 0 && yb < g.gy && xb < g.gx, kSiteTable)) return kEasy;
     c[i] = sat[(yb + 1) * W + xb + 1] - sat[ya * W + xb + 1] - sat[(yb + 1) * W + xa] +
            sat[ya * W + xa];
   }
-  return c[1] >= k && c[0] <= 8 * k + 64;
+  return c[1] < k ? kSparse : c[0] > knn_dense(k) ? kDense : kEasy;
 }
+
+// Queries set apart from the single-thread search, in one array of m entries.
+// The hard ones (not easy) are listed from the front, for warps.  Those that
+// the search by counts leaves are listed from the back: up to `few` of them go
+// to warps, more to a thread each.
+struct KnnLists {
+  unsigned *hard, *left;  // the lists' lengths
+  int32_t* query;
+  unsigned few;
+};
 
 // Whether the data fill their box about evenly: their cells hold at least 70%
 // as many points' cells as evenly random points would (uniform data: 100%; 64
@@ -1554,14 +1627,27 @@ __device__ __forceinline__ bool knn_even(const GridDev& g, int64_t n) {
   return float(g.filled + 1u) >= 0.7f * expected;
 }
 
+// Whether the search by counts runs: on even data, unless most queries lie
+// beyond the grid's edge, where its discs find nothing (100,000 queries up to a
+// box width outside, k = 32: 432 us a call, 330 by heaps).
+__device__ __forceinline__ bool knn_by_counts(const GridDev& g, int64_t n) {
+  return knn_even(g, n) && 2 * g.beyond <= kSampleQueries;
+}
+
+// The queries that the heap search lists for warps, besides those in sparse
+// surroundings.
+struct KnnListed {
+  bool dense, beyond;  // in dense surroundings; beyond the grid's edge
+};
+
 // Query t, by one thread (no block-wide barrier; `return`s are its own).
 template <int MODE, bool LIST>
 __device__ __forceinline__ void knn_thread_query(
     const GridDev* grid, const float4* sorted, const int32_t* starts, const int32_t* base,
     const int32_t* bpre, const int32_t* sat, const float4* qrec, const float* data, int64_t n,
     int64_t m, double p, int k, float* __restrict__ out, int32_t* nbr_out,
-    float* __restrict__ kd2_out, int32_t* hit_out, bool sort_rows, unsigned* hard_count,
-    int32_t* hard, int64_t t) {
+    float* __restrict__ kd2_out, int32_t* hit_out, bool sort_rows, const KnnLists& lists,
+    KnnListed listed, int64_t t) {
   extern __shared__ __align__(16) unsigned char knn_smem[];
   KnnHeap hp;
   hp.h = reinterpret_cast<u64*>(knn_smem) + threadIdx.x;
@@ -1604,9 +1690,16 @@ __device__ __forceinline__ void knn_thread_query(
   if (finite2(qx, qy)) {
     const float u = cell_pos(qx, g.hx0, g.inv2), v = cell_pos(qy, g.hy0, g.inv2);
     const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
-    if (LIST && !knn_easy(g, sat, float(g.cells) * rcp_approx(float(n)), cx, cy, k)) {
-      list_heavy(t, m, hard_count, hard);
-      return;
+    if (LIST) {
+      const KnnSurroundings at =
+          knn_surroundings(g, sat, float(g.cells) * rcp_approx(float(n)), cx, cy, k);
+      // One branch, so that the warp comes together again behind it.
+      const bool away = (at == kSparse) | (listed.dense & (at == kDense)) |
+                        (listed.beyond & beyond_grid(g, u, v));
+      if (away) {
+        list_heavy(t, m, lists.hard, lists.query);
+        return;
+      }
     }
     const float mg = __fmaf_ru(fabsf(u) + fabsf(v), 0x1p-22f, 0x1p-9f);
     const float ax = fmaxf(0.f, fmaxf(u - float(g.gx), -u) - mg);
@@ -1752,12 +1845,18 @@ __device__ __forceinline__ void knn_thread_query(
 }
 
 // At most 64 registers (32 one-warp blocks per SM); left to itself the
-// compiler settles on fewer and spills.  With LIST, queries that are not
-// knn_easy are listed in `hard` for knn_warp_kernel.  With UNEVEN the kernel
-// runs on data that are not knn_even only, and its blocks, as many as fit the
-// GPU, fetch groups of 32 queries from a counter: 32,768 blocks that return
-// at once take 34 us.
-template <int MODE, bool LIST, bool UNEVEN>
+// compiler settles on fewer and spills.  With LIST, hard queries are listed;
+// but those in dense surroundings only if they are not most of them, or few:
+// neighbouring threads sift a cluster together, which a warp per query does
+// again for each (64 blobs, n = 2^20, queries in the blobs too, threads / warps:
+// m = 500,000 k = 8 520 / 1605 us, k = 32 880 / 1826; m = 100,000 293 / 440 and
+// 391 / 554; m = 30,000 252 / 235 and 393 / 155).  FROM says which queries it
+// takes: all of them, a block's 32 each; all of them unless they are searched
+// by counts; or those that search left, if they are not few.  In the latter two
+// its blocks, as many as fit the GPU, fetch groups of 32 queries from a counter:
+// 32,768 blocks that return at once take 34 us.
+enum KnnFrom : int { kFromAll, kFromUneven, kFromUnevenFetched, kFromLeft };
+template <int MODE, bool LIST, int FROM>
 __global__ void __maxnreg__(64)
     knn_query_kernel(const GridDev* grid, const float4* sorted,
                      const int32_t* starts, const int32_t* base,
@@ -1766,25 +1865,36 @@ __global__ void __maxnreg__(64)
                      int64_t m,
                      double p, int k, float* __restrict__ out, int32_t* nbr_out,
                      float* __restrict__ kd2_out, int32_t* hit_out,
-                     bool sort_rows, unsigned* hard_count,
-                     int32_t* hard, unsigned* next) {
+                     bool sort_rows, const KnnLists lists, unsigned* next) {
   pdl_trigger();
   pdl_wait();
-  if (UNEVEN && knn_even(*grid, n)) return;
+  constexpr bool fetch = FROM >= kFromUnevenFetched;
+  if ((FROM == kFromUneven || FROM == kFromUnevenFetched) && knn_by_counts(*grid, n)) return;
+  const int64_t count = FROM == kFromLeft ? int64_t(*lists.left) : m;
+  if (FROM == kFromLeft && count <= lists.few) return;
+  KnnListed listed{false, false};
+  if (LIST) {
+    listed.beyond = m <= kUnsortedKnn;
+    listed.dense = m <= lists.few ||
+                   (k >= kSampleK && grid->dense * m <= int64_t(kSampleQueries) * lists.few);
+  }
   const int lane = threadIdx.x;
   int64_t group = blockIdx.x;
   for (;;) {
-    if (UNEVEN) {
+    if (fetch) {
       unsigned fetched = 0;
       if (lane == 0) fetched = atomicAdd(next, 1u);
       group = __shfl_sync(0xffffffffu, fetched, 0);
     }
-    const int64_t t = group * kKnnThreads + lane;
-    if (UNEVEN && group * kKnnThreads >= m) break;
-    if (t < m)
-      knn_thread_query<MODE, LIST>(grid, sorted, starts, base, bpre, sat, qrec, data, n, m, p, k, out,
-                                   nbr_out, kd2_out, hit_out, sort_rows, hard_count, hard, t);
-    if (!UNEVEN) break;
+    int64_t t = group * kKnnThreads + lane;
+    if (fetch && group * kKnnThreads >= count) break;
+    if (t < count) {
+      if (FROM == kFromLeft) t = lists.query[m - 1 - t];
+      if (dcheck(t >= 0 && t < m, kSiteScatter))
+        knn_thread_query<MODE, LIST>(grid, sorted, starts, base, bpre, sat, qrec, data, n, m, p, k,
+                                     out, nbr_out, kd2_out, hit_out, sort_rows, lists, listed, t);
+    }
+    if (!fetch) break;
     __syncwarp();
   }
 }
@@ -1792,8 +1902,8 @@ __global__ void __maxnreg__(64)
 // ------------------------------------------------- k-NN, one thread, by counts
 //
 // The search for calls that want no neighbour lists, on queries whose
-// surroundings are of even density (others are listed for the two searches
-// below):
+// surroundings are of even density (others are left to the two searches below
+// and above, see KnnLists):
 // 1. the summed-area table's count over a square of cells gives the local
 //    density, and with it a disc expected to hold the k nearest with a margin
 //    of four standard deviations of their number;
@@ -1823,7 +1933,7 @@ __global__ void __launch_bounds__(kCountThreads)
                      const int32_t* base, const int32_t* sat, const float4* qrec,
                      const float* data, int64_t n, int64_t m, double p, int k,
                      float* __restrict__ out, float* __restrict__ kd2_out,
-                     unsigned* hard_count, int32_t* hard) {
+                     const KnnLists lists) {
   pdl_trigger();
   pdl_wait();
   __shared__ int bins[kBins][kCountThreads];
@@ -1833,7 +1943,7 @@ __global__ void __launch_bounds__(kCountThreads)
   const int64_t t = int64_t(blockIdx.x) * kCountThreads + lane;
   const GridDev g = *grid;
   // No block-wide barrier in this kernel: a lane reads its own columns.
-  if (t >= m || !knn_even(g, n)) return;
+  if (t >= m || !knn_by_counts(g, n)) return;
   const float4 rq = qrec[t];
   const float qx = rq.x, qy = rq.y;
   const int j = __float_as_int(rq.z);
@@ -1853,7 +1963,7 @@ __global__ void __launch_bounds__(kCountThreads)
   // Points per cell around the query, from the square that holds 2k points
   // at the mean density.
   const float ca = float(g.cells) * rcp_approx(float(n));
-  const int re = int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * ca) - 1.f)));
+  const int re = knn_square(ca, k);
   const int ya = max(0, cy - re), yb = min(g.gy - 1, cy + re);
   const int xa = max(0, cx - re), xb = min(g.gx - 1, cx + re);
   const int W = g.gx + 1;
@@ -1864,8 +1974,11 @@ __global__ void __launch_bounds__(kCountThreads)
   const float per = float(held) * rcp_approx(float((yb - ya + 1) * (xb - xa + 1)));
   const float fk = float(k);
   float reach = fk * rcp_approx(3.14159265f * per) * (1.f + 4.f * rsqrt_approx(fk));
-  bool listed = !(g.inv2 > 0.f) || 4 * held < k || held > 8 * k + 64 || !(h2 >= 0x1p-100f) ||
-                !(h2 <= 0x1p60f);
+  // The disc assumes points on all sides: none for a query beyond the grid's
+  // edge (with two retries each and then a warp each, 2^20 queries up to a box
+  // width outside took 28.7 ms, k = 32).
+  bool listed = !(g.inv2 > 0.f) || beyond_grid(g, u, v) || 4 * held < k || held > knn_dense(k) ||
+                !(h2 >= 0x1p-100f) || !(h2 <= 0x1p60f);
 
   // The runs of the cells that can hold a key up to d2 (rows and columns
   // rounded outwards), row by row.
@@ -1970,7 +2083,7 @@ __global__ void __launch_bounds__(kCountThreads)
     listed = aside > kAside;
   }
   if (listed) {
-    list_heavy(t, m, hard_count, hard);
+    list_heavy<-1>(t, m, lists.left, lists.query + (m - 1));
     return;
   }
   // The k - below smallest of the candidates set aside.
@@ -1987,8 +2100,8 @@ __global__ void __launch_bounds__(kCountThreads)
   if (best != INT_MAX) {
     z = bestz;
   } else if (!sums.value(z)) {
-    // Sums outside FP32's range: the warp search redoes the query.
-    list_heavy(t, m, hard_count, hard);
+    // Sums outside FP32's range: the other searches redo the query.
+    list_heavy<-1>(t, m, lists.left, lists.query + (m - 1));
     return;
   }
   out[j] = z;
@@ -1998,7 +2111,7 @@ __global__ void __launch_bounds__(kCountThreads)
 // ------------------------------------------------- k-NN, a warp per query
 //
 // The search for calls with few queries, and for the queries of larger calls
-// that one thread would take long over (see knn_easy):
+// that one thread would take long over (see knn_surroundings, KnnLists):
 // 1. a disc around the query that holds at least k points, its radius found
 //    from the summed-area table with 32 radii per probe: the cells inside
 //    three rectangles inscribed in the disc are counted, so the k-th key is
@@ -2173,7 +2286,7 @@ __device__ __forceinline__ void knn_warp_query(
       // shares of the cap that the edge cuts off the disc (corners at fixed
       // angles reach 0.92 rho, and a query 500 cells away then walked a cap 40
       // cells deep: 10,007 queries up to a box width outside, n = 2^20, k = 8,
-      // 610 us a call, 64 so).
+      // 610 us a call, 84 so).
       const float bx = fmaxf(0.f, fmaxf(-u, u - float(g.gx)));
       const float by = fmaxf(0.f, fmaxf(-v, v - float(g.gy)));
       const bool over = bx + by == 0.f;
@@ -2385,7 +2498,7 @@ __device__ __forceinline__ void knn_warp_query(
   if (lane == 0) out[j] = zv;
 }
 
-// The queries of `hard` (null: all m), a warp each.
+// The listed queries (or, with no list, all m), a warp each.
 template <int MODE, int kRegs>
 __global__ void __launch_bounds__(kKnnWarpThreads)
     knn_warp_kernel(const GridDev* grid, const float4* sorted,
@@ -2394,17 +2507,19 @@ __global__ void __launch_bounds__(kKnnWarpThreads)
                     const float* data, int64_t n, int64_t m, double p, int k,
                     float* __restrict__ out, int32_t* nbr_out,
                     float* __restrict__ kd2_out, int32_t* hit_out, bool sort_rows,
-                    const unsigned* hard_count, const int32_t* hard) {
+                    const KnnLists lists) {
   pdl_trigger();
   pdl_wait();
   using Buffer = KnnBuffer<kRegs>;
   __shared__ u64 keys[kKnnWarpThreads / 32][Buffer::kCap];
-  const int64_t count = hard ? int64_t(*hard_count) : m;
+  const int64_t hard = lists.query ? int64_t(*lists.hard) : m;
+  const unsigned left = lists.query ? *lists.left : 0u;
+  const int64_t count = hard + (left <= lists.few ? int64_t(left) : 0);
   const int64_t warps = int64_t(gridDim.x) * (kKnnWarpThreads / 32);
   const GridDev g = *grid;
   for (int64_t w = (int64_t(blockIdx.x) * kKnnWarpThreads + threadIdx.x) / 32; w < count;
        w += warps) {  // whole warps: no block-wide barrier in this kernel
-    const int64_t t = hard ? int64_t(hard[w]) : w;
+    const int64_t t = !lists.query ? w : lists.query[w < hard ? w : m - 1 - (w - hard)];
     if (!dcheck(t >= 0 && t < m && count <= m, kSiteScatter)) continue;
     const float4 rq = qrec[t];
     const int j = __float_as_int(rq.z);
@@ -3062,6 +3177,19 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Calls whose queries, a thread each, leave most of the GPU's warps empty.
 bool few_queries(int64_t m, int sm_count) { return m <= int64_t(sm_count) * 1024; }
 
+// Up to this many queries that lie in dense surroundings, or that the search by
+// counts left, a warp searches for each (64 blobs, queries in the blobs too,
+// threads / warps: k = 8, 30,000 of them 252 / 235 us, 100,000 293 / 440; k = 64,
+// 30,000 633 / 220, 100,000 847 / 931).
+int64_t knn_few(int k) {
+  return std::min(16384 + 4096 * int64_t(k), 32768 + 512 * int64_t(k));
+}
+
+// Whether a call's queries are sampled: where the result is asked for.
+bool knn_sampled(int k, int64_t m) {
+  return k >= kSampleK && m > knn_few(k);
+}
+
 int scan_tiles_of(int64_t max_cells) {
   return static_cast<int>((max_cells + 1 + kScanTile - 1) / kScanTile);
 }
@@ -3126,14 +3254,16 @@ cudaError_t launch_grid_sort(const float* data, int64_t n, const float* queries,
   // Without the query sort, the queries join none of the three passes and
   // their records are written in the caller's order.
   const int64_t mq = sort_queries ? m : 0;
+  const int sample_k = knn_sampled(knn_k, m) ? knn_k : 0;
   const unsigned pgrid = static_cast<unsigned>((n + mq + 255) / 256);
   e = launch_pdl(count_kernel, pgrid, 256, 0, s, grid, data, n, queries, mq, counts_d, counts_q);
   if (e == cudaSuccess)
     e = launch_pdl(scan_kernel, dim3(max_tiles, sort_queries ? 2 : 1), kScanBlock, 0, s, grid,
                    counts_d, counts_q, starts_d, starts_q, sums, max_tiles, 0);
   if (e == cudaSuccess)
-    e = launch_pdl(scatter_kernel, pgrid, 256, 0, s, grid, data, n, queries, mq, starts_d, starts_q,
-                   sums, max_tiles, counts_d, counts_q, sorted, qrec);
+    e = launch_pdl(scatter_kernel, pgrid + (sample_k > 0 ? 1 : 0), kSampleQueries, 0, s, grid, data,
+                   n, queries, mq, m, sample_k, starts_d, starts_q, sums, max_tiles, counts_d,
+                   counts_q, sorted, qrec);
   if (e == cudaSuccess && !sort_queries && m > 0)
     e = launch_pdl(query_identity_kernel, static_cast<unsigned>((m + 255) / 256), 256, 0, s, queries,
                    m, qrec);
@@ -3406,14 +3536,16 @@ size_t knn_smem_bytes(int k) { return size_t(k) * kKnnThreads * sizeof(u64); }
 // points, whole query call on a prepared index, thread / warp per query:
 // m = 10,007 61 / 43 us at k = 8, 107 / 46 us at k = 32; m = 100,000
 // 69 / 143 us at k = 8, 141 / 168 us at k = 32.
-int64_t knn_warp_queries(int k) { return 8192 + 1024 * int64_t(k); }
+int64_t knn_warp_queries(int k) { return std::min<int64_t>(8192 + 1024 * int64_t(k), 65536); }
 
-// Up to this many queries, those that are not knn_easy go to warps.  Beyond
-// it every warp of the single-thread search has hard queries to overlap with
-// and the GPU is full either way (64 blobs, n = 2^20, k = 8, threads alone /
-// with warps: m = 10,007 1010 / 74 us, 100,000 1090 / 263 us, 2^20
-// 1440 / 1770 us).
+// Up to this many queries, those that are not easy are listed.  Beyond it
+// every warp of the single-thread search has hard queries to overlap with and
+// the GPU is full either way (64 blobs, n = 2^20, k = 8, threads alone / with
+// warps: m = 10,007 1010 / 74 us, 100,000 1090 / 263 us, 2^20 1440 / 1770 us).
 constexpr int64_t kKnnHardQueries = int64_t(1) << 19;
+constexpr int64_t kCountQueries = 7 * (int64_t(1) << 14);
+constexpr int64_t kUnfetchedQueries = int64_t(1) << 18;
+static_assert(kUnfetchedQueries <= kKnnHardQueries, "these list their hard queries");
 
 // The search over sorted queries, by warps for few of them, else by threads
 // with warps for the hard ones; the launch arguments both share.
@@ -3442,60 +3574,64 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
   // Without lists and from k = 17 on, evenly spread data are searched by counts
   // (uniform n = m = 2^20, heaps / counts: k = 16 389 / 383 us, 24 550 / 454,
   // 32 723 / 475, 64 1552 / 718); the device decides which of the two runs.
-  const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16;
-  int32_t* list = warps && !all_warps && a.m <= kKnnHardQueries ? a.hard : nullptr;
-  unsigned* hard_count = &a.grid->hard;
+  const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16 && (a.k > 32 || a.m > kCountQueries);
+  const bool list = warps && !all_warps && a.m <= kKnnHardQueries;
+  const KnnLists lists{&a.grid->hard, &a.grid->left, all_warps ? nullptr : a.hard,
+                       static_cast<unsigned>(knn_few(a.k))};
   const bool pow2 = a.p == 2.0;
   cudaError_t e = cudaSuccess;
   if (counted)
     e = launch_pdl(pow2 ? knn_count_kernel<kPow2> : knn_count_kernel<kPowGeneral>,
                    static_cast<unsigned>((a.m + kCountThreads - 1) / kCountThreads), kCountThreads, 0,
                    s, a.grid, a.sorted, a.starts, a.base, a.sat, a.qrec, a.data, a.n,
-                   a.m, a.p, a.k, a.out, a.kd2_out, hard_count, a.hard);
+                   a.m, a.p, a.k, a.out, a.kd2_out, lists);
   if (e == cudaSuccess && !all_warps) {
     const size_t smem = knn_smem_bytes(a.k);  // below the default limit (k <= 64: 16 KB)
     const unsigned groups = static_cast<unsigned>((a.m + kKnnThreads - 1) / kKnnThreads);
-    const unsigned resident = std::min(groups, unsigned(sm_count) * 32);
-    auto heap = [&](auto kernel, unsigned blocks) {
+    const unsigned resident = unsigned(sm_count) * 32;
+    auto heap = [&](auto list_these, auto from) {
+      constexpr bool L = decltype(list_these)::value;
+      constexpr int F = decltype(from)::value;
+      auto kernel = pow2 ? knn_query_kernel<kPow2, L, F> : knn_query_kernel<kPowGeneral, L, F>;
+      const unsigned blocks = F < kFromUnevenFetched ? groups : std::min(groups, resident);
+      unsigned* next = F == kFromLeft ? &a.grid->next_left : &a.grid->next;
       // A kernel that starts early has its first blocks placed on the SMs that
       // the one before it leaves free; where all blocks fit at once, they stay
       // so (uniform m = 30,000, k = 32, gradient call: 270 us, 204 started
       // plainly; index call of 100,000, k = 16: 99 and 89).  The short searches
       // for a few neighbours gain more from the early start (m = 10,007, k = 1:
       // 18 us, 22 plainly).
-      if (groups >= unsigned(sm_count) * 32 || a.k < 4)
+      if (groups >= resident || F == kFromLeft || a.k < 4)
         return launch_pdl(kernel, blocks, kKnnThreads, smem, s, a.grid, a.sorted, a.starts, a.base,
                           a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                          a.kd2_out, a.hit_out, a.sort_rows, hard_count, a.hard, &a.grid->next);
+                          a.kd2_out, a.hit_out, a.sort_rows, lists, next);
       kernel<<<blocks, kKnnThreads, smem, s>>>(a.grid, a.sorted, a.starts, a.base, a.bpre, a.sat,
                                                a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                                               a.kd2_out, a.hit_out, a.sort_rows, hard_count, a.hard,
-                                               &a.grid->next);
+                                               a.kd2_out, a.hit_out, a.sort_rows, lists, next);
       return cudaGetLastError();
     };
-    if (counted && list)
-      e = heap(pow2 ? knn_query_kernel<kPow2, true, true> : knn_query_kernel<kPowGeneral, true, true>,
-               resident);
+    using All = std::integral_constant<int, kFromAll>;
+    using Uneven = std::integral_constant<int, kFromUneven>;
+    using Fetched = std::integral_constant<int, kFromUnevenFetched>;
+    using Left = std::integral_constant<int, kFromLeft>;
+    if (counted && a.m <= kUnfetchedQueries)
+      e = heap(std::true_type{}, Uneven{});
     else if (counted)
-      e = heap(pow2 ? knn_query_kernel<kPow2, false, true> : knn_query_kernel<kPowGeneral, false, true>,
-               resident);
-    else if (list)
-      e = heap(pow2 ? knn_query_kernel<kPow2, true, false> : knn_query_kernel<kPowGeneral, true, false>,
-               groups);
+      e = list ? heap(std::true_type{}, Fetched{}) : heap(std::false_type{}, Fetched{});
     else
-      e = heap(pow2 ? knn_query_kernel<kPow2, false, false>
-                    : knn_query_kernel<kPowGeneral, false, false>, groups);
+      e = list ? heap(std::true_type{}, All{}) : heap(std::false_type{}, All{});
+    if (e == cudaSuccess && counted && a.m > knn_few(a.k)) e = heap(std::false_type{}, Left{});
   }
   if (e != cudaSuccess || (!all_warps && !list && !counted)) return e;
   constexpr int per_block = kKnnWarpThreads / 32;
-  // The list's length is known on the device only: enough blocks to fill the
-  // GPU stride over it.
+  // The lists' lengths are known on the device only: enough blocks to fill the
+  // GPU stride over them.
   const int64_t blocks = all_warps ? (a.m + per_block - 1) / per_block : int64_t(sm_count) * 8;
   auto kernel = a.k <= 32 ? (pow2 ? knn_warp_kernel<kPow2, 3> : knn_warp_kernel<kPowGeneral, 3>)
                           : (pow2 ? knn_warp_kernel<kPow2, 4> : knn_warp_kernel<kPowGeneral, 4>);
   return launch_pdl(kernel, static_cast<unsigned>(blocks), kKnnWarpThreads, 0, s, a.grid, a.sorted,
                     a.starts, a.base, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                    a.kd2_out, a.hit_out, a.sort_rows, hard_count, all_warps ? nullptr : a.hard);
+                    a.kd2_out, a.hit_out, a.sort_rows, lists);
 }
 
 }  // namespace
@@ -3549,8 +3685,8 @@ __device__ __forceinline__ void copy_plan(const GridDev* src,
   GridDev g = *src;
   g.box_ticket = 0xffffffffu;
   g.scan_ticket = 0xffffffffu;
-  g.hard = 0u;
-  g.next = 0u;
+  g.hard = g.left = g.next = g.next_left = 0u;
+  g.beyond = g.dense = 0u;
   if (radius > 0.0 && g.inv2 > 0.f)
     g.rho = __fmaf_ru(__fmul_ru(__double2float_ru(radius), g.inv2), 0.5f + 0x1p-9f, 0x1p-8f);
   *dst = g;
@@ -3558,21 +3694,35 @@ __device__ __forceinline__ void copy_plan(const GridDev* src,
 
 // First kernel of a query call on an index: the plan copy and, for the query
 // sort, the histogram's clearing, or else the records in the caller's order.
+// In both the first block also samples the queries of a k-NN call (sample_k > 0).
+struct IndexCells {
+  const int32_t *starts, *base;
+  int64_t n;
+};
+__device__ __forceinline__ void index_plan(const GridDev* src, GridDev* dst, double radius,
+                                           const IndexCells& data, const float* queries, int64_t m,
+                                           int sample_k) {
+  if (blockIdx.x != 0) return;
+  if (threadIdx.x == 0) copy_plan(src, dst, radius);
+  if (sample_k > 0) {
+    __syncthreads();
+    knn_sample(dst, *src, data.starts, data.base, data.n, queries, m, sample_k);
+  }
+}
 __global__ void __launch_bounds__(256)
-    index_prep_kernel(const GridDev* src, GridDev* dst, double radius,
-                      int32_t* counts) {
+    index_prep_kernel(const GridDev* src, GridDev* dst, double radius, const IndexCells data,
+                      const float* queries, int64_t m, int sample_k, int32_t* counts) {
   pdl_trigger();
   pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) copy_plan(src, dst, radius);
+  index_plan(src, dst, radius, data, queries, m, sample_k);
   zero_counts(counts, count_int4s(src->cells));
 }
 __global__ void __launch_bounds__(256)
-    index_identity_kernel(const GridDev* src, GridDev* dst,
-                          double radius, const float* queries, int64_t m,
-                          float4* qrec) {
+    index_identity_kernel(const GridDev* src, GridDev* dst, double radius, const IndexCells data,
+                          const float* queries, int64_t m, int sample_k, float4* qrec) {
   pdl_trigger();
   pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) copy_plan(src, dst, radius);
+  index_plan(src, dst, radius, data, queries, m, sample_k);
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= m) return;
   qrec[j] = make_float4(queries[2 * j], queries[2 * j + 1], __int_as_float(static_cast<int>(j)),
@@ -3582,9 +3732,10 @@ __global__ void __launch_bounds__(256)
 // Query side of a call on a prepared index: plan copy, then the counting
 // sort of the queries alone (the scan runs its query half only), or their
 // records as they come.
-cudaError_t launch_query_sort(const GridDev* xgrid, const float* queries, int64_t m, double radius,
-                              int64_t max_cells, void* workspace, const QueryLayout& Q,
-                              int sm_count, cudaStream_t s, bool sort_queries) {
+cudaError_t launch_query_sort(const GridDev* xgrid, const IndexCells& data, const float* queries,
+                              int64_t m, double radius, int sample_k, int64_t max_cells,
+                              void* workspace, const QueryLayout& Q, int sm_count, cudaStream_t s,
+                              bool sort_queries) {
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   GridDev* grid = reinterpret_cast<GridDev*>(ws + Q.off_grid);
   int32_t* counts = reinterpret_cast<int32_t*>(ws + Q.off_counts);
@@ -3594,28 +3745,22 @@ cudaError_t launch_query_sort(const GridDev* xgrid, const float* queries, int64_
   const int max_tiles = scan_tiles_of(max_cells);
   const unsigned qgrid = static_cast<unsigned>((m + 255) / 256);
   if (!sort_queries)
-    return launch_pdl(index_identity_kernel, qgrid, 256, 0, s, xgrid, grid, radius, queries, m, qrec);
+    return launch_pdl(index_identity_kernel, qgrid, kSampleQueries, 0, s, xgrid, grid, radius, data,
+                      queries, m, sample_k, qrec);
   const unsigned zgrid = static_cast<unsigned>(
       std::min<int64_t>(int64_t(sm_count) * 4, (count_int4s(max_cells) + 255) / 256));
-  cudaError_t e = launch_pdl(index_prep_kernel, zgrid, 256, 0, s, xgrid, grid, radius, counts);
+  cudaError_t e = launch_pdl(index_prep_kernel, zgrid, kSampleQueries, 0, s, xgrid, grid, radius,
+                             data, queries, m, sample_k, counts);
   if (e == cudaSuccess)
     e = launch_pdl(count_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, counts, counts);
   if (e == cudaSuccess)
     e = launch_pdl(scan_kernel, dim3(max_tiles, 1), kScanBlock, 0, s, grid, counts, counts, starts,
                    starts, sums, max_tiles, 1);
   if (e == cudaSuccess)
-    e = launch_pdl(scatter_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, starts, starts,
-                   sums, max_tiles, counts, counts, nullptr, qrec);
+    e = launch_pdl(scatter_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, 0, 0, starts,
+                   starts, sums, max_tiles, counts, counts, nullptr, qrec);
   return e;
 }
-
-// Up to this many queries an index call leaves them as they come: the sort's
-// launches and passes (about 15 us) cost more than the locality saves.
-// Uniform queries in random order, index of 2^20 uniform points, sorted / as
-// they come: radius K = 32 m = 10,007 43.7 / 26.9 us, 150,001 56.0 / 45.6; k-NN
-// k = 8 m = 30,000 68.4 / 53.9, k = 32 m = 150,001 204.8 / 213.9 (50,000 points:
-// 146 / 216).
-constexpr int64_t kUnsortedRadius = int64_t(1) << 17, kUnsortedKnn = int64_t(1) << 15;
 
 }  // namespace
 
@@ -3677,8 +3822,8 @@ cudaError_t launch_index_build(const float* data, int64_t n, double radius, int 
     e = launch_pdl(scan_kernel, dim3(max_tiles, 1), kScanBlock, 0, s, grid, counts, counts, starts,
                    starts, sums, max_tiles, 0);
   if (e == cudaSuccess)
-    e = launch_pdl(scatter_kernel, dgrid, 256, 0, s, grid, data, n, nullptr, 0, starts, starts, sums,
-                   max_tiles, counts, counts, sorted, nullptr);
+    e = launch_pdl(scatter_kernel, dgrid, 256, 0, s, grid, data, n, nullptr, 0, 0, 0, starts, starts,
+                   sums, max_tiles, counts, counts, sorted, nullptr);
   if (e != cudaSuccess) return e;
   if (X.knn) {
     e = cudaMemcpyAsync(mem + X.off_data, data, size_t(n) * 12, cudaMemcpyDeviceToDevice, s);
@@ -3696,8 +3841,8 @@ cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, cons
                                cudaStream_t s, bool sort_queries, bool modified) {
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
-  cudaError_t e = launch_query_sort(xgrid, queries, m, radius, X.max_cells, workspace, Q, sm_count,
-                                    s, sort_queries && m > kUnsortedRadius);
+  cudaError_t e = launch_query_sort(xgrid, IndexCells{}, queries, m, radius, 0, X.max_cells, workspace,
+                                    Q, sm_count, s, sort_queries && m > kUnsortedRadius);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const GridDev* grid = reinterpret_cast<const GridDev*>(ws + Q.off_grid);
@@ -3719,13 +3864,14 @@ cudaError_t launch_index_knn(const void* index_mem, const IndexLayout& X, const 
                              cudaStream_t s, bool sort_queries) {
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
-  cudaError_t e = launch_query_sort(xgrid, queries, m, 0.0, X.max_cells, workspace, Q, sm_count, s,
+  const int32_t* starts = reinterpret_cast<const int32_t*>(mem + X.off_starts);
+  const int32_t* sums = reinterpret_cast<const int32_t*>(mem + X.off_sums);
+  cudaError_t e = launch_query_sort(xgrid, IndexCells{starts, sums, X.n}, queries, m, 0.0,
+                                    knn_sampled(k, m) ? k : 0, X.max_cells, workspace, Q, sm_count, s,
                                     sort_queries && m > kUnsortedKnn);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const float4* qrec = reinterpret_cast<const float4*>(ws + Q.off_qrec);
-  const int32_t* starts = reinterpret_cast<const int32_t*>(mem + X.off_starts);
-  const int32_t* sums = reinterpret_cast<const int32_t*>(mem + X.off_sums);
   const float4* sorted = reinterpret_cast<const float4*>(mem + X.off_sorted);
   const float* data = reinterpret_cast<const float*>(mem + X.off_data);
   const int32_t* bpre = reinterpret_cast<const int32_t*>(mem + X.off_bpre);

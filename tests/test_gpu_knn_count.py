@@ -73,3 +73,59 @@ def test_scales(scale):
     prob = synthetic.uniform_problem(3000, 40000, seed=4)
     prob["data"][:, :2] *= np.float32(scale)
     _compare(prob["data"], prob["queries"] * np.float32(scale), 20)
+
+
+def test_up_to_32_neighbours_counted_from_114689_queries():
+    """k = 17 .. 32 are counted above 7 * 2^14 queries."""
+    m = 7 * (1 << 14) + 1
+    for k in (17, 24, 32):
+        prob = synthetic.uniform_problem(6000, m, seed=k, exact_hits=100)
+        Z = _compare(prob["data"], prob["queries"], k)
+        part = slice(0, None, 997)
+        want = oracle.idw_knn(prob["data"], prob["queries"][part], 2.0, k)["Z"]
+        assert np.max(np.abs(Z[part] - want)) <= 2e-6 * np.max(np.abs(prob["data"][:, 2]))
+
+
+@pytest.mark.parametrize("share", [0.3, 0.45, 0.7])
+def test_queries_beyond_the_edge(share):
+    """120,000 queries, k = 20, a share of them beyond the data: the counting
+    search leaves them to warps (36,000), to threads (54,000), or, where they
+    are most of the call, does not run."""
+    prob = synthetic.uniform_problem(5000, 120000, seed=8)
+    q = prob["queries"]
+    out = np.random.default_rng(8).random(len(q)) < share
+    q[out] = np.where(q[out] < 0.5, q[out] - 0.7, q[out] + 0.7)
+    Z = _compare(prob["data"], q, 20)
+    part = slice(0, None, 499)
+    want = oracle.idw_knn(prob["data"], np.ascontiguousarray(q[part]), 2.0, 20)["Z"]
+    assert np.max(np.abs(Z[part] - want)) <= 2e-6 * np.max(np.abs(prob["data"][:, 2]))
+
+
+def test_uneven_rims():
+    """Data in a disc: even by the count of filled cells, with a fifth of the
+    box empty; its queries are left over from the counting search."""
+    prob = synthetic.uniform_problem(40000, 300000, seed=9)
+    xy = prob["data"][:, :2]
+    data = np.ascontiguousarray(prob["data"][((xy - 0.5) ** 2).sum(1) < 0.25])
+    _compare(data, prob["queries"], 24)
+
+
+@pytest.mark.parametrize("m", [1 << 18, (1 << 18) + 1, 1 << 19])
+@pytest.mark.parametrize("clustered", [False, True])
+def test_where_the_heap_search_is_started_another_way(m, clustered):
+    prob = synthetic.config_local(n=20000, m=m, clustered=clustered)
+    _compare(prob["data"], prob["queries"], 18)
+
+
+def test_queries_beyond_the_edge_take_no_longer():
+    """131,072 queries, most of them beyond the data, k = 32: without lists (the
+    call that may count) against with lists (which never does).  About equal;
+    11 times as long when every such query ended up with a warp of its own."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    from test_gpu_knn_warp import _fastest
+    prob = synthetic.uniform_problem(1 << 20, 1 << 17, seed=3)
+    d = torch.from_numpy(prob["data"]).cuda()
+    q = torch.from_numpy(prob["queries"]).cuda() * 3.0 - 1.0
+    counted = _fastest(lambda: idw.interpolate_knn(d, q, 2.0, 32))
+    assert counted <= 3 * _fastest(lambda: idw.interpolate_knn(d, q, 2.0, 32, neighbours=True))

@@ -120,3 +120,37 @@ def test_more_ties_than_the_buffer_holds(k):
     data = synthetic.pack_xyz(xy, np.linspace(-1, 1, len(xy), dtype=np.float32))
     _check(data, np.zeros((33, 2), np.float32), k)
     _check(data, np.zeros((33, 2), np.float32), k, p=3.5, index=True)
+
+
+@pytest.mark.parametrize("k", [1, 2, 8])
+@pytest.mark.parametrize("m", [20480, 24577, 36864, 60000])
+def test_clustered_queries(m, k):
+    """Queries in the data's blobs: listed for warps up to a size (the first
+    three are limits for k = 1, 2 and 8), then a thread each.  The same queries
+    in calls of 8192 are all warps'."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    r = np.random.default_rng(m)
+    xy = synthetic.mixture_xy(r, 50000 + m).astype(np.float32)
+    data = synthetic.pack_xyz(xy[:50000], r.standard_normal(50000).astype(np.float32))
+    d, q = torch.from_numpy(data).cuda(), torch.from_numpy(np.ascontiguousarray(xy[50000:])).cuda()
+    Z, nbr, kd2 = idw.interpolate_knn(d, q, 2.0, k, neighbours=True, kth_d2=True)
+    for i in range(0, m, 8192):
+        part = q[i:i + 8192].contiguous()
+        Zp, nbrp, kd2p = idw.interpolate_knn(d, part, 2.0, k, neighbours=True, kth_d2=True)
+        assert torch.equal(nbr[i:i + 8192], nbrp) and torch.equal(kd2[i:i + 8192], kd2p)
+        assert float((Z[i:i + 8192] - Zp).abs().max()) <= 2e-6 * float(d[:, 2].abs().max())
+
+
+def test_half_the_queries_take_no_longer():
+    """Half a million queries in the blobs of a million points against twice as
+    many (0.7 of their time; twice their time when each had a warp)."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    n = 1 << 20
+    xy = synthetic.mixture_xy(np.random.default_rng(3), 2 * n).astype(np.float32)
+    data = synthetic.pack_xyz(xy[:n], xy[:n, 0])
+    d, q = torch.from_numpy(data).cuda(), torch.from_numpy(np.ascontiguousarray(xy[n:])).cuda()
+    half = q[:500000].contiguous()
+    few = _fastest(lambda: idw.interpolate_knn(d, half, 2.0, 8))
+    assert few <= 1.2 * _fastest(lambda: idw.interpolate_knn(d, q, 2.0, 8))
