@@ -110,7 +110,7 @@ struct GridDev {
   unsigned next;         // next group of queries of the uneven-data heap search
   unsigned next_left;    // next group of the queries left
   unsigned beyond;       // of kSampleQueries queries: those beyond the grid's edge,
-  unsigned dense;        // and those in dense surroundings (see knn_sample)
+  unsigned dense;        // and those in dense surroundings, or heavy (see sample_queries)
 };
 
 // Order-preserving unsigned key of a float (for atomic min).
@@ -511,93 +511,6 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   return r;
 }
 
-// Radius of the square of cells that holds 2k points at the mean density:
-// ceil((sqrt(2 k ca) - 1) / 2) with ca cells per point.
-__device__ __forceinline__ int knn_square(float cells_per_point, int k) {
-  return int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
-}
-// More than this in that square is dense.
-__device__ __forceinline__ int knn_dense(int k) { return 8 * k + 64; }
-
-// What kSampleQueries of the queries, by a block of as many threads, have
-// around them: counts those beyond the grid's edge and those in dense
-// surroundings, from the cells' starts.
-constexpr int kSampleQueries = 256;
-constexpr int kSampleK = 2;  // with one neighbour a thread is through a cluster soon
-__device__ __forceinline__ void knn_sample(GridDev* out, const GridDev& g, const int32_t* starts,
-                                           const int32_t* base, int64_t n, const float* queries,
-                                           int64_t m, int k) {
-  const int64_t j = m * threadIdx.x / kSampleQueries;
-  const float x = queries[2 * j], y = queries[2 * j + 1];
-  bool beyond = false, dense = false;
-  if (finite2(x, y)) {
-    const float u = cell_pos(x, g.hx0, g.inv2), v = cell_pos(y, g.hy0, g.inv2);
-    const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
-    const int re = knn_square(float(g.cells) * rcp_approx(float(n)), k);
-    int held = 0;
-    for (int yy = max(0, cy - re); yy <= min(g.gy - 1, cy + re); ++yy)
-      held += cell_start(starts, base, yy * g.gx + min(g.gx - 1, cx + re) + 1, g.cells) -
-              cell_start(starts, base, yy * g.gx + max(0, cx - re), g.cells);
-    beyond = beyond_grid(g, u, v);
-    dense = held > knn_dense(k);
-  }
-  const int nb = __syncthreads_count(beyond), nd = __syncthreads_count(dense);
-  if (threadIdx.x == 0) {
-    out->beyond = nb;
-    out->dense = nd;
-  }
-}
-
-// Threads [0, n) place data points as (x, y, z, index), [n, n + m) place
-// queries as (x, y, index, 0).  With sample_k > 0 the last block samples the
-// call's `all` queries instead.
-__global__ void __launch_bounds__(256)
-    scatter_kernel(GridDev* grid, const float* data, int64_t n,
-                   const float* queries, int64_t m, int64_t all, int sample_k,
-                   const int32_t* starts_d, const int32_t* starts_q,
-                   const int32_t* sums, int max_tiles,
-                   int32_t* cursor_d, int32_t* cursor_q,
-                   float4* sorted, float4* qrec) {
-  pdl_trigger();
-  pdl_wait();
-  const GridDev g = *grid;
-  if (sample_k > 0 && blockIdx.x == gridDim.x - 1) {
-    knn_sample(grid, g, starts_d, sums, n, queries, all, sample_k);
-    return;
-  }
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) {
-    const float x = data[3 * i], y = data[3 * i + 1];
-    const int c = data_cell(g, x, y);
-    if (c < 0) return;
-    const int pos = cell_start(starts_d, sums, c, g.cells) + atomicAdd(&cursor_d[c], 1);
-    if (!dcheck(pos >= 0 && pos < n, kSiteScatter)) return;
-    sorted[pos] = make_float4(x, y, data[3 * i + 2], __int_as_float(static_cast<int>(i)));
-  } else if (i < n + m) {
-    const int64_t j = i - n;
-    const float x = queries[2 * j], y = queries[2 * j + 1];
-    const int b = query_bucket(g, x, y);
-    const int pos = cell_start(starts_q, sums + max_tiles, b, g.cells) + atomicAdd(&cursor_q[b], 1);
-    if (!dcheck(pos >= 0 && pos < m, kSiteScatter)) return;
-    qrec[pos] = make_float4(x, y, __int_as_float(static_cast<int>(j)), 0.f);
-  }
-}
-
-template <int MODE>
-__device__ __forceinline__ float local_weight(float d2, float hp, float nhp) {
-  if (MODE == kPow2) return rcp_approx(d2);
-  const float L = lg2_approx(d2);
-  const float th = L * nhp;
-  const float tl = fmaf(L, nhp, L * hp);  // exact rounding error of th
-  const float e = ex2_approx(th);
-  return fmaf(e, tl * 0.6931471805599453f, e);
-}
-
-__device__ __forceinline__ float fp32_d2(float qx, float qy, float x, float y) {
-  const float dx = __fsub_rn(qx, x), dy = __fsub_rn(qy, y);
-  return __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
-}
-
 // The runs of sorted data a query's disc of radius R can reach: at most
 // five rows, each one contiguous run [a[r], b[r]) (empty runs have a == b).
 // All runs are looked up before any is walked, so their loads overlap.
@@ -640,6 +553,124 @@ struct Runs {
   }
 };
 
+// Heavy queries: those with more candidates than `heavy_candidates`.  A
+// thread walks its candidates one load after another while the other lanes
+// wait, so heavy queries are listed and each is given a whole warp by a
+// kernel of their own.  At the mean density a query has about 21 cells of
+// candidates.  Calls that do not fill the GPU (few = true) list queries a
+// little above that; others, whose warps hide each other's loads, only those
+// several times above it.  200,003 points in 64 blobs, 150,001 uniform
+// queries, R for 16 members at the mean density (up to 1400 candidates a
+// query, modified Shepard): values 178 -> 18 us for the heavy queries and
+// 60 us for the rest, query gradients 680 -> 47 and 150 us.
+__device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, bool few) {
+  const float per_cell = float(n) * rcp_approx(float(g.cells));
+  return int(few ? fminf(fmaf(24.f, per_cell, 32.f), 1e9f) : fminf(fmaf(64.f, per_cell, 256.f), 1e9f));
+}
+// Whether a query goes on the list: a heavy one, unless the sample shows that
+// the call has more than `most` of them, enough to fill the GPU a thread each.
+// Such calls (queries clustered like the data) keep every lane busy, and
+// neighbouring threads share the candidates that a warp per query loads for
+// each: 2^20 points and queries in the same 64 blobs, R for 32 members at the
+// mean density, threads / warps: values 1100 / 1880 us, gradients 4530 / 6160.
+// (150,001 queries: 390 / 344 and 1250 / 1060.)
+constexpr int kSampleQueries = 256;
+__device__ __forceinline__ bool list_if_heavy(const GridDev& g, const Runs& runs, int64_t n,
+                                              int64_t m, int64_t most) {
+  return runs.candidates() > heavy_candidates(g, n, m <= most) &&
+         g.dense * m <= kSampleQueries * most;
+}
+
+// Radius of the square of cells that holds 2k points at the mean density:
+// ceil((sqrt(2 k ca) - 1) / 2) with ca cells per point.
+__device__ __forceinline__ int knn_square(float cells_per_point, int k) {
+  return int(ceilf(0.5f * (sqrt_approx(2.f * float(k) * cells_per_point) - 1.f)));
+}
+// More than this in that square is dense.
+__device__ __forceinline__ int knn_dense(int k) { return 8 * k + 64; }
+
+// What kSampleQueries of the queries, by a block of as many threads, have
+// around them, from the cells' starts: counts those beyond the grid's edge and
+// those in dense surroundings (a k-NN call, k > 0), or the heavy ones (a radius
+// call, kSampleRadius).
+constexpr int kSampleK = 2;  // with one neighbour a thread is through a cluster soon
+constexpr int kSampleRadius = -1;
+__device__ __forceinline__ void sample_queries(GridDev* out, const GridDev& g,
+                                               const int32_t* starts, const int32_t* base,
+                                               int64_t n, const float* queries, int64_t m, int k) {
+  const int64_t j = m * threadIdx.x / kSampleQueries;
+  const float x = queries[2 * j], y = queries[2 * j + 1];
+  bool beyond = false, dense = false;
+  if (k == kSampleRadius) {
+    dense = Runs(g, x, y, starts, base).candidates() > heavy_candidates(g, n, false);
+  } else if (finite2(x, y)) {
+    const float u = cell_pos(x, g.hx0, g.inv2), v = cell_pos(y, g.hy0, g.inv2);
+    const int cx = clamp_floor(u, 0, g.gx - 1), cy = clamp_floor(v, 0, g.gy - 1);
+    const int re = knn_square(float(g.cells) * rcp_approx(float(n)), k);
+    int held = 0;
+    for (int yy = max(0, cy - re); yy <= min(g.gy - 1, cy + re); ++yy)
+      held += cell_start(starts, base, yy * g.gx + min(g.gx - 1, cx + re) + 1, g.cells) -
+              cell_start(starts, base, yy * g.gx + max(0, cx - re), g.cells);
+    beyond = beyond_grid(g, u, v);
+    dense = held > knn_dense(k);
+  }
+  const int nb = __syncthreads_count(beyond), nd = __syncthreads_count(dense);
+  if (threadIdx.x == 0) {
+    out->beyond = nb;
+    out->dense = nd;
+  }
+}
+
+// Threads [0, n) place data points as (x, y, z, index), [n, n + m) place
+// queries as (x, y, index, 0).  With `sample` not 0 (see sample_queries) the
+// last block samples the call's `all` queries instead.
+__global__ void __launch_bounds__(256)
+    scatter_kernel(GridDev* grid, const float* data, int64_t n,
+                   const float* queries, int64_t m, int64_t all, int sample,
+                   const int32_t* starts_d, const int32_t* starts_q,
+                   const int32_t* sums, int max_tiles,
+                   int32_t* cursor_d, int32_t* cursor_q,
+                   float4* sorted, float4* qrec) {
+  pdl_trigger();
+  pdl_wait();
+  const GridDev g = *grid;
+  if (sample != 0 && blockIdx.x == gridDim.x - 1) {
+    sample_queries(grid, g, starts_d, sums, n, queries, all, sample);
+    return;
+  }
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i < n) {
+    const float x = data[3 * i], y = data[3 * i + 1];
+    const int c = data_cell(g, x, y);
+    if (c < 0) return;
+    const int pos = cell_start(starts_d, sums, c, g.cells) + atomicAdd(&cursor_d[c], 1);
+    if (!dcheck(pos >= 0 && pos < n, kSiteScatter)) return;
+    sorted[pos] = make_float4(x, y, data[3 * i + 2], __int_as_float(static_cast<int>(i)));
+  } else if (i < n + m) {
+    const int64_t j = i - n;
+    const float x = queries[2 * j], y = queries[2 * j + 1];
+    const int b = query_bucket(g, x, y);
+    const int pos = cell_start(starts_q, sums + max_tiles, b, g.cells) + atomicAdd(&cursor_q[b], 1);
+    if (!dcheck(pos >= 0 && pos < m, kSiteScatter)) return;
+    qrec[pos] = make_float4(x, y, __int_as_float(static_cast<int>(j)), 0.f);
+  }
+}
+
+template <int MODE>
+__device__ __forceinline__ float local_weight(float d2, float hp, float nhp) {
+  if (MODE == kPow2) return rcp_approx(d2);
+  const float L = lg2_approx(d2);
+  const float th = L * nhp;
+  const float tl = fmaf(L, nhp, L * hp);  // exact rounding error of th
+  const float e = ex2_approx(th);
+  return fmaf(e, tl * 0.6931471805599453f, e);
+}
+
+__device__ __forceinline__ float fp32_d2(float qx, float qy, float x, float y) {
+  const float dx = __fsub_rn(qx, x), dy = __fsub_rn(qy, y);
+  return __fmaf_rn(dy, dy, __fmul_rn(dx, dx));
+}
+
 // A query's runs laid end to end: candidate s of `total` sits at at(s), so
 // that one lane, or the 32 lanes of a warp side by side, can walk them.
 struct FlatRuns {
@@ -663,20 +694,6 @@ struct FlatRuns {
   }
 };
 
-// Heavy queries: those with more candidates than `heavy_candidates`.  A
-// thread walks its candidates one load after another while the other lanes
-// wait, so heavy queries are listed and each is given a whole warp by a
-// kernel of their own.  At the mean density a query has about 21 cells of
-// candidates.  Calls that do not fill the GPU (few = true) list queries a
-// little above that; others, whose warps hide each other's loads, only those
-// several times above it.  200,003 points in 64 blobs, 150,001 uniform
-// queries, R for 16 members at the mean density (up to 1400 candidates a
-// query, modified Shepard): values 178 -> 18 us for the heavy queries and
-// 60 us for the rest, query gradients 680 -> 47 and 150 us.
-__device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, bool few) {
-  const float per_cell = float(n) * rcp_approx(float(g.cells));
-  return int(few ? fminf(fmaf(24.f, per_cell, 32.f), 1e9f) : fminf(fmaf(64.f, per_cell, 256.f), 1e9f));
-}
 // Lists query t (any subset of a warp's lanes may call it together) from
 // `list` on upwards, or downwards (step = -1).
 template <int step = 1>
@@ -831,7 +848,7 @@ __global__ void __launch_bounds__(kLocalThreads)
                        int64_t n, const int32_t* starts,
                        const int32_t* base, const float4* qrec,
                        int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
-                       int32_t* count_out, double radius, bool few,
+                       int32_t* count_out, double radius, int64_t most,
                        unsigned* heavy_count, int32_t* heavy) {
   pdl_trigger();
   pdl_wait();
@@ -842,7 +859,7 @@ __global__ void __launch_bounds__(kLocalThreads)
   const int j = __float_as_int(r.z);
   if (!dcheck(j >= 0 && j < m, kSiteOutput)) return;
   const Runs runs(*grid, qx, qy, starts, base);
-  if (runs.candidates() > heavy_candidates(*grid, n, few)) {
+  if (list_if_heavy(*grid, runs, n, m, most)) {
     list_heavy(t, m, heavy_count, heavy);
     return;
   }
@@ -1223,7 +1240,7 @@ __global__ void __launch_bounds__(kLocalThreads)
                             int64_t m, double p, float r2f, float r2t,
                             const float* grad_out, float* __restrict__ grad_q,
                             double* __restrict__ grad_p, LocalGradRec* rec,
-                            LocalGradRec64* rec64, double radius, bool few,
+                            LocalGradRec64* rec64, double radius, int64_t most,
                             unsigned* heavy_count, int32_t* heavy) {
   pdl_trigger();
   pdl_wait();
@@ -1236,7 +1253,7 @@ __global__ void __launch_bounds__(kLocalThreads)
     const int j = __float_as_int(r.z);
     if (dcheck(j >= 0 && j < m, kSiteOutput)) {
       const Runs runs(*grid, qx, qy, starts, base);
-      if (runs.candidates() > heavy_candidates(*grid, n, few)) {
+      if (list_if_heavy(*grid, runs, n, m, most)) {
         list_heavy(t, m, heavy_count, heavy);
       } else {
         const float gj = grad_out[j];
@@ -3174,8 +3191,9 @@ __global__ void __launch_bounds__(256)
 
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Calls whose queries, a thread each, leave most of the GPU's warps empty.
-bool few_queries(int64_t m, int sm_count) { return m <= int64_t(sm_count) * 1024; }
+// Queries that, a thread each, fill the GPU: up to as many heavy ones are listed
+// (see list_if_heavy).
+int64_t heavy_limit(int sm_count) { return int64_t(sm_count) * 1024; }
 
 // Up to this many queries that lie in dense surroundings, or that the search by
 // counts left, a warp searches for each (64 blobs, queries in the blobs too,
@@ -3254,15 +3272,16 @@ cudaError_t launch_grid_sort(const float* data, int64_t n, const float* queries,
   // Without the query sort, the queries join none of the three passes and
   // their records are written in the caller's order.
   const int64_t mq = sort_queries ? m : 0;
-  const int sample_k = knn_sampled(knn_k, m) ? knn_k : 0;
+  const int sample = knn_k > 0 ? (knn_sampled(knn_k, m) ? knn_k : 0)
+                               : m <= heavy_limit(sm_count) ? 0 : kSampleRadius;
   const unsigned pgrid = static_cast<unsigned>((n + mq + 255) / 256);
   e = launch_pdl(count_kernel, pgrid, 256, 0, s, grid, data, n, queries, mq, counts_d, counts_q);
   if (e == cudaSuccess)
     e = launch_pdl(scan_kernel, dim3(max_tiles, sort_queries ? 2 : 1), kScanBlock, 0, s, grid,
                    counts_d, counts_q, starts_d, starts_q, sums, max_tiles, 0);
   if (e == cudaSuccess)
-    e = launch_pdl(scatter_kernel, pgrid + (sample_k > 0 ? 1 : 0), kSampleQueries, 0, s, grid, data,
-                   n, queries, mq, m, sample_k, starts_d, starts_q, sums, max_tiles, counts_d,
+    e = launch_pdl(scatter_kernel, pgrid + (sample != 0 ? 1 : 0), kSampleQueries, 0, s, grid, data,
+                   n, queries, mq, m, sample, starts_d, starts_q, sums, max_tiles, counts_d,
                    counts_q, sorted, qrec);
   if (e == cudaSuccess && !sort_queries && m > 0)
     e = launch_pdl(query_identity_kernel, static_cast<unsigned>((m + 255) / 256), 256, 0, s, queries,
@@ -3295,7 +3314,7 @@ cudaError_t launch_radius_queries(const GridDev* grid, const float4* sorted, int
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
     const cudaError_t e = launch_pdl(
         local_query_kernel<M, W>, qgrid, kLocalThreads, 0, s, grid, sorted, n, starts, base, qrec, m,
-        p, r2f, r2t, out, count_out, radius, few_queries(m, sm_count), heavy_count, heavy);
+        p, r2f, r2t, out, count_out, radius, heavy_limit(sm_count), heavy_count, heavy);
     if (e != cudaSuccess) return e;
     return launch_pdl(local_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, 0, s, grid,
                       sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
@@ -3371,7 +3390,7 @@ cudaError_t launch_local_backward(const float* data, int64_t n, const float* que
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
     e = launch_pdl(local_grad_query_kernel<M, W>, qgrid, kLocalThreads, 0, s, grid, sorted, n,
                    starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p, rec, rec64, radius,
-                   few_queries(m, sm_count), heavy_count, heavy);
+                   heavy_limit(sm_count), heavy_count, heavy);
     if (e == cudaSuccess)
       e = launch_pdl(local_grad_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, 0, s,
                      grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, grad_out, grad_q, grad_p,
@@ -3694,35 +3713,36 @@ __device__ __forceinline__ void copy_plan(const GridDev* src,
 
 // First kernel of a query call on an index: the plan copy and, for the query
 // sort, the histogram's clearing, or else the records in the caller's order.
-// In both the first block also samples the queries of a k-NN call (sample_k > 0).
+// In both the first block also samples the call's queries (see sample_queries).
 struct IndexCells {
   const int32_t *starts, *base;
   int64_t n;
 };
 __device__ __forceinline__ void index_plan(const GridDev* src, GridDev* dst, double radius,
                                            const IndexCells& data, const float* queries, int64_t m,
-                                           int sample_k) {
+                                           int sample) {
   if (blockIdx.x != 0) return;
   if (threadIdx.x == 0) copy_plan(src, dst, radius);
-  if (sample_k > 0) {
+  if (sample != 0) {
     __syncthreads();
-    knn_sample(dst, *src, data.starts, data.base, data.n, queries, m, sample_k);
+    const GridDev g = *dst;
+    sample_queries(dst, g, data.starts, data.base, data.n, queries, m, sample);
   }
 }
 __global__ void __launch_bounds__(256)
     index_prep_kernel(const GridDev* src, GridDev* dst, double radius, const IndexCells data,
-                      const float* queries, int64_t m, int sample_k, int32_t* counts) {
+                      const float* queries, int64_t m, int sample, int32_t* counts) {
   pdl_trigger();
   pdl_wait();
-  index_plan(src, dst, radius, data, queries, m, sample_k);
+  index_plan(src, dst, radius, data, queries, m, sample);
   zero_counts(counts, count_int4s(src->cells));
 }
 __global__ void __launch_bounds__(256)
     index_identity_kernel(const GridDev* src, GridDev* dst, double radius, const IndexCells data,
-                          const float* queries, int64_t m, int sample_k, float4* qrec) {
+                          const float* queries, int64_t m, int sample, float4* qrec) {
   pdl_trigger();
   pdl_wait();
-  index_plan(src, dst, radius, data, queries, m, sample_k);
+  index_plan(src, dst, radius, data, queries, m, sample);
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= m) return;
   qrec[j] = make_float4(queries[2 * j], queries[2 * j + 1], __int_as_float(static_cast<int>(j)),
@@ -3733,7 +3753,7 @@ __global__ void __launch_bounds__(256)
 // sort of the queries alone (the scan runs its query half only), or their
 // records as they come.
 cudaError_t launch_query_sort(const GridDev* xgrid, const IndexCells& data, const float* queries,
-                              int64_t m, double radius, int sample_k, int64_t max_cells,
+                              int64_t m, double radius, int sample, int64_t max_cells,
                               void* workspace, const QueryLayout& Q, int sm_count, cudaStream_t s,
                               bool sort_queries) {
   unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -3746,11 +3766,11 @@ cudaError_t launch_query_sort(const GridDev* xgrid, const IndexCells& data, cons
   const unsigned qgrid = static_cast<unsigned>((m + 255) / 256);
   if (!sort_queries)
     return launch_pdl(index_identity_kernel, qgrid, kSampleQueries, 0, s, xgrid, grid, radius, data,
-                      queries, m, sample_k, qrec);
+                      queries, m, sample, qrec);
   const unsigned zgrid = static_cast<unsigned>(
       std::min<int64_t>(int64_t(sm_count) * 4, (count_int4s(max_cells) + 255) / 256));
   cudaError_t e = launch_pdl(index_prep_kernel, zgrid, kSampleQueries, 0, s, xgrid, grid, radius,
-                             data, queries, m, sample_k, counts);
+                             data, queries, m, sample, counts);
   if (e == cudaSuccess)
     e = launch_pdl(count_kernel, qgrid, 256, 0, s, grid, nullptr, 0, queries, m, counts, counts);
   if (e == cudaSuccess)
@@ -3841,14 +3861,15 @@ cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, cons
                                cudaStream_t s, bool sort_queries, bool modified) {
   const unsigned char* mem = static_cast<const unsigned char*>(index_mem);
   const GridDev* xgrid = reinterpret_cast<const GridDev*>(mem + X.off_grid);
-  cudaError_t e = launch_query_sort(xgrid, IndexCells{}, queries, m, radius, 0, X.max_cells, workspace,
-                                    Q, sm_count, s, sort_queries && m > kUnsortedRadius);
+  const int32_t* starts = reinterpret_cast<const int32_t*>(mem + X.off_starts);
+  const int32_t* sums = reinterpret_cast<const int32_t*>(mem + X.off_sums);
+  cudaError_t e = launch_query_sort(xgrid, IndexCells{starts, sums, X.n}, queries, m, radius,
+                                    m <= heavy_limit(sm_count) ? 0 : kSampleRadius, X.max_cells,
+                                    workspace, Q, sm_count, s, sort_queries && m > kUnsortedRadius);
   if (e != cudaSuccess) return e;
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   const GridDev* grid = reinterpret_cast<const GridDev*>(ws + Q.off_grid);
   const float4* qrec = reinterpret_cast<const float4*>(ws + Q.off_qrec);
-  const int32_t* starts = reinterpret_cast<const int32_t*>(mem + X.off_starts);
-  const int32_t* sums = reinterpret_cast<const int32_t*>(mem + X.off_sums);
   const float4* sorted = reinterpret_cast<const float4*>(mem + X.off_sorted);
   const float r2f = static_cast<float>(radius * radius);
   const float r2t = r2f > 0.f ? r2f : 0x1p-149f;

@@ -51,3 +51,36 @@ def test_values_counts_gradients(modified, n, m, radius, p):
         scale = np.max(np.abs(b))
         # the bar of the adjoints: 1e-4 of the largest magnitude
         assert np.max(np.abs(a - b)) <= 1e-4 * scale, name
+
+
+@pytest.mark.parametrize("modified", [False, True])
+def test_as_many_heavy_queries_as_fill_the_gpu(modified):
+    """170,000 queries in the blobs of 20,000 points: most are heavy, so none is
+    listed.  The same queries in calls of 85,000, which list theirs, give the
+    same members, values and gradients."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    m = 170000
+    r = np.random.default_rng(5)
+    xy = synthetic.mixture_xy(r, 20000 + m)
+    data = synthetic.pack_xyz(xy[:20000], r.standard_normal(20000).astype(np.float32))
+    d = torch.from_numpy(data).cuda()
+    q = torch.from_numpy(np.ascontiguousarray(xy[20000:])).cuda()
+    g = torch.from_numpy(r.standard_normal(m).astype(np.float32)).cuda()
+    radius = synthetic.local_radius(20000, 16.0)
+    call = idw.interpolate_modified if modified else idw.interpolate_local
+    parts = [slice(0, m // 2), slice(m // 2, m)]
+    Z, count = call(d, q, 2.5, radius, counts=True)
+    gz, gxy, gq, gp = idw.local_backward(d, q, 2.5, radius, g, modified=modified)
+    halves = [call(d, q[s].contiguous(), 2.5, radius, counts=True) for s in parts]
+    grads = [idw.local_backward(d, q[s].contiguous(), 2.5, radius, g[s].contiguous(),
+                                modified=modified) for s in parts]
+    assert torch.equal(count, torch.cat([h[1] for h in halves]))
+    Zh = torch.cat([h[0] for h in halves])
+    assert torch.equal(Z.isnan(), Zh.isnan())
+    assert float((Z - Zh).nan_to_num(0.0).abs().max()) <= 2e-6 * float(d[:, 2].abs().max())
+    want = (grads[0][0] + grads[1][0], grads[0][1] + grads[1][1],
+            torch.cat([grads[0][2], grads[1][2]]), grads[0][3] + grads[1][3])
+    for a, b in zip((gz, gxy, gq, gp), want):
+        # each within the adjoints' bar, 1e-4 of the largest magnitude
+        assert float((a - b).abs().max()) <= 2e-4 * float(b.abs().max())
