@@ -575,10 +575,18 @@ __device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, boo
 // mean density, threads / warps: values 1100 / 1880 us, gradients 4530 / 6160.
 // (150,001 queries: 390 / 344 and 1250 / 1060.)
 constexpr int kSampleQueries = 256;
+//
+// Queries in no spatial order (`scattered`) are heavy from 128 + m / 256
+// candidates on: threads of a warp then read from as many places, the 32 lanes
+// of one query from one.  More queries hide more of the threads' latency.
+// Index of 2^20 uniform points, R for 128 / 512 / 2048 members, us sorted first / a
+// thread each / by this rule: 10,007 queries 74 / 176 / 576, 74 / 219 / 914 and
+// 31 / 32 / 75; 131,072 queries 92 / 240 / 799, 107 / 381 / 1456 and 107 / 300 / 830.
 __device__ __forceinline__ bool list_if_heavy(const GridDev& g, const Runs& runs, int64_t n,
-                                              int64_t m, int64_t most) {
-  return runs.candidates() > heavy_candidates(g, n, m <= most) &&
-         g.dense * m <= kSampleQueries * most;
+                                              int64_t m, int64_t most, bool scattered = false) {
+  int bound = heavy_candidates(g, n, m <= most);
+  if (scattered) bound = min(bound, 128 + int(m / 256));
+  return runs.candidates() > bound && g.dense * m <= kSampleQueries * most;
 }
 
 // Radius of the square of cells that holds 2k points at the mean density:
@@ -848,7 +856,7 @@ __global__ void __launch_bounds__(kLocalThreads)
                        int64_t n, const int32_t* starts,
                        const int32_t* base, const float4* qrec,
                        int64_t m, double p, float r2f, float r2t, float* __restrict__ out,
-                       int32_t* count_out, double radius, int64_t most,
+                       int32_t* count_out, double radius, int64_t most, bool scattered,
                        unsigned* heavy_count, int32_t* heavy) {
   pdl_trigger();
   pdl_wait();
@@ -859,7 +867,7 @@ __global__ void __launch_bounds__(kLocalThreads)
   const int j = __float_as_int(r.z);
   if (!dcheck(j >= 0 && j < m, kSiteOutput)) return;
   const Runs runs(*grid, qx, qy, starts, base);
-  if (list_if_heavy(*grid, runs, n, m, most)) {
+  if (list_if_heavy(*grid, runs, n, m, most, scattered)) {
     list_heavy(t, m, heavy_count, heavy);
     return;
   }
@@ -3308,13 +3316,13 @@ cudaError_t launch_radius_queries(const GridDev* grid, const float4* sorted, int
                                   const int32_t* starts, const int32_t* base, const float4* qrec,
                                   int64_t m, double p, float r2f, float r2t, float* out,
                                   int32_t* count_out, double radius, bool modified, int32_t* heavy,
-                                  unsigned qgrid, int sm_count, cudaStream_t s) {
+                                  bool scattered, unsigned qgrid, int sm_count, cudaStream_t s) {
   unsigned* heavy_count = &const_cast<GridDev*>(grid)->hard;
   auto run = [&](auto mode, auto wmode) {
     constexpr int M = decltype(mode)::value, W = decltype(wmode)::value;
     const cudaError_t e = launch_pdl(
         local_query_kernel<M, W>, qgrid, kLocalThreads, 0, s, grid, sorted, n, starts, base, qrec, m,
-        p, r2f, r2t, out, count_out, radius, heavy_limit(sm_count), heavy_count, heavy);
+        p, r2f, r2t, out, count_out, radius, heavy_limit(sm_count), scattered, heavy_count, heavy);
     if (e != cudaSuccess) return e;
     return launch_pdl(local_heavy_kernel<M, W>, unsigned(sm_count) * 8, kHeavyThreads, 0, s, grid,
                       sorted, n, starts, base, qrec, m, p, r2f, r2t, out, count_out, radius,
@@ -3346,8 +3354,8 @@ cudaError_t launch_local(const float* data, int64_t n, const float* queries, int
   const float r2t = r2f > 0.f ? r2f : 0x1p-149f;
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
   return launch_radius_queries(grid, sorted, n, starts_d, sums, qrec, m, p, r2f, r2t, out, count_out,
-                               radius, modified, reinterpret_cast<int32_t*>(ws + L.off_hard), qgrid,
-                               sm_count, s);
+                               radius, modified, reinterpret_cast<int32_t*>(ws + L.off_hard), false,
+                               qgrid, sm_count, s);
 }
 
 size_t local_grad_record_bytes(int64_t m) {
@@ -3875,7 +3883,8 @@ cudaError_t launch_index_local(const void* index_mem, const IndexLayout& X, cons
   const float r2t = r2f > 0.f ? r2f : 0x1p-149f;
   const unsigned qgrid = static_cast<unsigned>((m + kLocalThreads - 1) / kLocalThreads);
   return launch_radius_queries(grid, sorted, X.n, starts, sums, qrec, m, p, r2f, r2t, out, count_out,
-                               radius, modified, reinterpret_cast<int32_t*>(ws + Q.off_hard), qgrid,
+                               radius, modified, reinterpret_cast<int32_t*>(ws + Q.off_hard),
+                               sort_queries && m <= kUnsortedRadius, qgrid,
                                sm_count, s);
 }
 
