@@ -233,6 +233,22 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
   return false;
 }
 
+// Waits until the counter at `p` reaches `target`, giving up in the same way
+// after `limit_ns`.
+__device__ __forceinline__ bool wait_count_bounded(unsigned* p, unsigned target,
+                                                   unsigned long long limit_ns, unsigned* err) {
+  const unsigned long long t0 = global_ns();
+  for (uint32_t it = 1; it < (1u << 30); ++it) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (v >= target) return true;
+    __nanosleep(64);
+    if ((it & 63u) == 0 && global_ns() - t0 > limit_ns) break;
+  }
+  atomicOr(err, kErrWaitTimeout);
+  return false;
+}
+
 // ------------------------------------------------------ tile ring
 // A ring of ST shared-memory stages fed by one 1-D bulk copy per work unit.
 // Thread 0 produces; every thread consumes.  `src(u)` gives the global

@@ -107,15 +107,15 @@ __device__ __forceinline__ float mul_ftz(float a, float b) {
 }
 
 // Largest finite |x|, |y| over each problem's data and queries.  Also clears
-// `flagged`, the call's count of queries listed for the slow path (nullable).
+// the call's counts of the slow path's list in `ctrl` (nullable).
 template <int CAP>
 __global__ void __launch_bounds__(256) range_kernel(const __grid_constant__ Table<CAP> t,
-                                                    unsigned* maxbits,
-                                                    unsigned* flagged) {
+                                                    unsigned* maxbits, Control* ctrl) {
   __shared__ float red[8];
   pdl_trigger();
   pdl_wait();
-  if (flagged && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *flagged = 0u;
+  if (ctrl && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+    ctrl->flagged = ctrl->slow_drawn = ctrl->slow_done = 0u;
   const Instance& I = t.inst[blockIdx.y];
   float mx = 0.f;
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;

@@ -4,8 +4,8 @@
 // Pipeline (one call): coordinate range scan -> staging -> persistent
 // all-pairs sweep -> combine (FP64 division) -> for problems of more than
 // 2048 points, the search for the exact hits among the flagged queries and
-// the results of those queries (smaller problems' flagged queries are
-// finished by the combine).
+// the results of those queries, in one kernel (smaller problems' flagged queries
+// are finished by the combine).
 //
 // The sweep is the paper's tiled kernel (Sec. 4.2: the data are read once
 // per block of prediction points, tile by tile) rebuilt for sm_103a:
@@ -410,8 +410,8 @@ __global__ void __launch_bounds__(Var<V>::NT, 512 / Var<V>::NT)
 // sums are added in a fixed order, so the result is deterministic.  The
 // CTA's flagged queries are then redone one after another by all 256
 // threads when their problem is small; a query's slow path reads all n
-// points, so those of a larger problem are listed for the two kernels after
-// this one, which spread each search over the GPU.  Block 0 finally clears
+// points, so those of a larger problem are listed for the kernel after
+// this one, which spreads each search over the GPU.  Block 0 finally clears
 // the per-problem range words the range scan and staging of this call used,
 // so the next call (or graph replay) starts from zero without a memset.
 //
@@ -427,8 +427,8 @@ static_assert(kCombineThreads == kSlowThreads, "the combine CTA runs the slow pa
 
 // Flagged queries of problems up to this many points stay with their CTA:
 // one FP64 recomputation of 2048 points keeps one SM's FP64 pipe busy for
-// about 14 us (100,003 points: 690 us), and the two kernels that share larger
-// ones out cost about 3 us a call.
+// about 14 us (100,003 points: 690 us), and the kernel that shares larger ones
+// out costs about 1.3 us a call.
 constexpr int kSlowInlinePoints = 2048;
 
 // A listed query: problem, query, the lowest coincident data index found so
@@ -527,77 +527,114 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
     for (int c = threadIdx.x; c < t.count; c += blockDim.x) ctrl->maxbits[c] = 0u;
 }
 
-// Exact hits of the listed queries.  A work item is a group of up to 32
-// listed queries and one of S equal slices of their problem's points, S
-// chosen so that the items fill the grid: every point is read once per group
-// and compared with the group's queries from shared memory, and the lowest
-// coincident index is kept with an atomic minimum.
+// The listed queries, in one launch of two steps.
+//
+// First the exact hits.  A work item is a group of up to 32 listed queries and
+// one of S equal slices of their problem's points, S chosen so that the items
+// fill the grid: every point is read once per group and compared with the
+// group's queries from shared memory, and the lowest coincident index is kept
+// with an atomic minimum.
+//
+// Then the results: a hit's z, or Eq. 1 in FP64.  A query without a hit is one
+// whose FP32 sums left FP32's range; among them are the queries that shared a
+// reciprocal with a hit (their weight there is NaN).  Its points are cut into
+// S slices, S chosen so that all such queries' slices fill the grid (counted
+// when the list is short; a list of more than kSlowThreads queries fills it by
+// itself); each slice's sums are scaled by its own d2_min, and a warp of the
+// CTA that finishes a query's last slice rescales and adds them in a fixed
+// order.  A 100,003-point, 65,537-query call with 16 hits spent 860 us on them in
+// the combine, one CTA a query: the FP64 pipe of one SM bounds a query; spread
+// over the GPU they take under 30 us.
+//
+// The second step waits for all of the first.  CTAs draw its items from a
+// counter, and one waits only when none is left: what it waits for has been
+// drawn by CTAs that run, so the wait ends wherever the others are scheduled.
+// One launch and not one for each step, because most calls list nothing and pay
+// for the launches alone (p = 2 without hits, no list / two launches / this one:
+// 12,000 x 12,000 48.9 / 51.0 / 50.2 us, 20,000 x 20,000 109.9 / 112.2 / 111.3).
 constexpr int kSlowGroup = 32;
+// One item over all points of the largest problem (2^31) takes several seconds.
+constexpr unsigned long long kSlowWaitNs = 60000000000ull;
 
+struct SlowShared {
+  float2 q[kSlowGroup];
+  int prob[kSlowGroup];
+  int work[kSlowThreads];
+  int warp_count[kSlowThreads / 32];
+  unsigned drawn;
+  bool last;
+};
+
+// Item w of `slices` to a group: marks its queries' hits among the slice's points.
 template <int CAP>
-__global__ void __launch_bounds__(kSlowThreads)
-    slow_search_kernel(const __grid_constant__ Table<CAP> t, const Control* ctrl,
-                       const SlowList slow) {
-  __shared__ float2 q[kSlowGroup];
-  __shared__ int prob[kSlowGroup];
-  pdl_trigger();
-  pdl_wait();
-  const int64_t count = min(ctrl->flagged, slow.cap);
-  const int64_t groups = (count + kSlowGroup - 1) / kSlowGroup;
-  if (groups == 0) return;
-  const int64_t slices = max(int64_t(1), gridDim.x / groups);
-  for (int64_t w = blockIdx.x; w < groups * slices; w += gridDim.x) {
-    const int64_t e0 = w / slices * kSlowGroup, sl = w % slices;
-    const int ne = static_cast<int>(min(int64_t(kSlowGroup), count - e0));
-    __syncthreads();  // the previous item's group is no longer read
-    if (threadIdx.x < ne) {
-      const SlowItem it = slow.item[e0 + threadIdx.x];
-      const float* p = t.inst[it.problem].queries + 2 * int64_t(it.query);
-      q[threadIdx.x] = make_float2(p[0], p[1]);
-      prob[threadIdx.x] = it.problem;
-    }
-    __syncthreads();
-    for (int a = 0; a < ne;) {  // runs of the same problem (uniform across the CTA)
-      int b = a + 1;
-      while (b < ne && prob[b] == prob[a]) ++b;
-      const Instance& I = t.inst[prob[a]];
-      slow_scan(I.data, sl * I.n / slices, (sl + 1) * I.n / slices,
-                [&](int64_t i, float x, float y) {
-                  for (int e = a; e < b; ++e)
-                    if (q[e].x == x && q[e].y == y)
-                      atomicMin(&slow.item[e0 + e].hit, static_cast<int32_t>(i));
-                  return false;
-                });
-      a = b;
-    }
+__device__ void slow_search(const Table<CAP>& t, const SlowList& slow, int64_t count, int64_t slices,
+                            int64_t w, SlowShared& sh) {
+  const int64_t e0 = w / slices * kSlowGroup, sl = w % slices;
+  const int ne = static_cast<int>(min(int64_t(kSlowGroup), count - e0));
+  if (threadIdx.x < ne) {
+    const SlowItem it = slow.item[e0 + threadIdx.x];
+    const float* p = t.inst[it.problem].queries + 2 * int64_t(it.query);
+    sh.q[threadIdx.x] = make_float2(p[0], p[1]);
+    sh.prob[threadIdx.x] = it.problem;
+  }
+  __syncthreads();
+  for (int a = 0; a < ne;) {  // runs of the same problem (uniform across the CTA)
+    int b = a + 1;
+    while (b < ne && sh.prob[b] == sh.prob[a]) ++b;
+    const Instance& I = t.inst[sh.prob[a]];
+    slow_scan(I.data, sl * I.n / slices, (sl + 1) * I.n / slices,
+              [&](int64_t i, float x, float y) {
+                for (int e = a; e < b; ++e)
+                  if (sh.q[e].x == x && sh.q[e].y == y)
+                    atomicMin(&slow.item[e0 + e].hit, static_cast<int32_t>(i));
+                return false;
+              });
+    a = b;
   }
 }
 
-// Results of the listed queries: a hit's z, or Eq. 1 in FP64.  A query
-// without a hit is one whose FP32 sums left FP32's range; among them are the
-// queries that shared a reciprocal with a hit (their weight there is NaN).
-// Its points are cut into S slices, S chosen so that all such queries'
-// slices fill the grid (counted when the list is short; a list of more than
-// kSlowThreads queries fills it by itself); each slice's sums are scaled by
-// its own d2_min, and a warp of the CTA that finishes a query's last slice
-// rescales and adds them in a fixed order.  A 100,003-point, 65,537-query call with 16
-// hits spent 860 us on them in the combine, one CTA a query: the FP64 pipe
-// of one SM bounds a query; spread over the GPU they take under 30 us.
+// Listed query f as other CTAs have left it (past this SM's cache).
+__device__ __forceinline__ SlowItem slow_item(const SlowList& slow, int64_t f) {
+  const int4 v = __ldcg(reinterpret_cast<const int4*>(slow.item + f));
+  return SlowItem{v.x, v.y, v.z, static_cast<unsigned>(v.w)};
+}
+
 template <int CAP>
 __global__ void __launch_bounds__(kSlowThreads)
-    slow_finish_kernel(const __grid_constant__ Table<CAP> t, const Control* ctrl,
-                       const SlowList slow, double p) {
-  __shared__ int work[kSlowThreads];
-  __shared__ int warp_count[kSlowThreads / 32];
-  __shared__ bool last;
-  pdl_trigger();
+    slow_kernel(const __grid_constant__ Table<CAP> t, Control* ctrl, const SlowList slow, double p) {
+  __shared__ SlowShared sh;
+  // The kernels behind this one start only when it has gone this far: held back
+  // early, they, and the next call's sweep with them, were placed around its
+  // CTAs (13,000 x 500, p = 2.5: 45 us a call, 37 so).
   pdl_wait();
+  pdl_trigger();
   const int count = static_cast<int>(min(ctrl->flagged, slow.cap));
   if (count == 0) return;
   const int tid = threadIdx.x;
+
+  const int64_t groups = (count + kSlowGroup - 1) / kSlowGroup;
+  const int64_t cuts = max(int64_t(1), gridDim.x / groups), searches = groups * cuts;
+  for (;;) {
+    __syncthreads();  // the previous item's group and number are no longer read
+    if (tid == 0) sh.drawn = atomicAdd(&ctrl->slow_drawn, 1u);
+    __syncthreads();
+    if (sh.drawn >= searches) break;
+    slow_search<CAP>(t, slow, count, cuts, sh.drawn, sh);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) atomicAdd(&ctrl->slow_done, 1u);
+  }
+  if (tid == 0) {
+    sh.last = wait_count_bounded(&ctrl->slow_done, static_cast<unsigned>(searches), kSlowWaitNs,
+                                 &ctrl->error);
+    __threadfence();
+  }
+  __syncthreads();
+  if (!sh.last) return;  // gave up; recorded
+
   // Hits: one thread each.
   for (int f = blockIdx.x * kSlowThreads + tid; f < count; f += gridDim.x * kSlowThreads) {
-    const SlowItem it = slow.item[f];
+    const SlowItem it = slow_item(slow, f);
     if (it.hit == INT_MAX) continue;
     const Instance& I = t.inst[it.problem];
     const int64_t j = it.query;
@@ -607,25 +644,25 @@ __global__ void __launch_bounds__(kSlowThreads)
   const bool short_list = count <= kSlowThreads;
   int sums = count;
   if (short_list) {  // the queries without a hit, in list order
-    const bool mine = tid < count && slow.item[tid].hit == INT_MAX;
+    const bool mine = tid < count && slow_item(slow, tid).hit == INT_MAX;
     const unsigned vote = __ballot_sync(0xffffffffu, mine);
-    if ((tid & 31) == 0) warp_count[tid >> 5] = __popc(vote);
+    if ((tid & 31) == 0) sh.warp_count[tid >> 5] = __popc(vote);
     __syncthreads();
     int before = 0;
     sums = 0;
     for (int w = 0; w < kSlowThreads / 32; ++w) {
-      if (w < (tid >> 5)) before += warp_count[w];
-      sums += warp_count[w];
+      if (w < (tid >> 5)) before += sh.warp_count[w];
+      sums += sh.warp_count[w];
     }
-    if (mine) work[before + __popc(vote & ((1u << (tid & 31)) - 1))] = tid;
+    if (mine) sh.work[before + __popc(vote & ((1u << (tid & 31)) - 1))] = tid;
     __syncthreads();
     if (sums == 0) return;
   }
   const int slices = max(1, int(gridDim.x) / sums);
   for (int64_t w = blockIdx.x; w < int64_t(sums) * slices; w += gridDim.x) {
     const int e = static_cast<int>(w / slices), sl = static_cast<int>(w % slices);
-    const int f = short_list ? work[e] : e;
-    const SlowItem it = slow.item[f];
+    const int f = short_list ? sh.work[e] : e;
+    const SlowItem it = slow_item(slow, f);
     if (it.hit != INT_MAX) continue;  // uniform across the CTA
     const Instance& I = t.inst[it.problem];
     const int64_t j = it.query;
@@ -635,10 +672,10 @@ __global__ void __launch_bounds__(kSlowThreads)
     if (tid == 0) {
       slow.part[w] = s;
       __threadfence();
-      last = atomicAdd(&slow.item[f].done, 1u) + 1u == unsigned(slices);
+      sh.last = atomicAdd(&slow.item[f].done, 1u) + 1u == unsigned(slices);
     }
     __syncthreads();
-    if (last && tid < 32) {  // one warp, lanes over the slices, a fixed shuffle tree
+    if (sh.last && tid < 32) {  // one warp, lanes over the slices, a fixed shuffle tree
       __threadfence();
       const double* P = reinterpret_cast<const double*>(slow.part + (w - sl));
       double dmin = INFINITY;
@@ -661,18 +698,22 @@ __global__ void __launch_bounds__(kSlowThreads)
         slow_write_sums<float>(sum, p, &I.out[j], I.s0_out ? &I.s0_out[j] : nullptr,
                                I.hit_out ? &I.hit_out[j] : nullptr);
     }
-    __syncthreads();  // `last` is rewritten by the next item
+    __syncthreads();  // sh.last is rewritten by the next item
   }
 }
 
-// One thread waits, with the sweep kernels' bounded wait, on a barrier whose
-// phase nothing completes; it gives up and records kErrWaitTimeout.
-__global__ void bounded_wait_selftest_kernel(unsigned* err) {
+// One thread waits, as the slow list's kernel does, for a count that nothing
+// reaches, and then, with the sweep kernels' bounded wait, on a barrier whose
+// phase nothing completes; both give up, and the second records
+// kErrWaitTimeout for good.
+__global__ void bounded_wait_selftest_kernel(Control* ctrl) {
   __shared__ __align__(8) unsigned long long bar;
   if (threadIdx.x == 0) {
+    if (wait_count_bounded(&ctrl->slow_done, ~0u, 1000000, &ctrl->error)) return;
+    if (!(atomicAnd(&ctrl->error, ~kErrWaitTimeout) & kErrWaitTimeout)) return;
     mbar_init(smem_u32(&bar), 1);
     fence_barrier_init();
-    mbar_wait_bounded(smem_u32(&bar), 0, err);
+    mbar_wait_bounded(smem_u32(&bar), 0, &ctrl->error);
   }
 }
 
@@ -1017,7 +1058,7 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
 
   const unsigned gx = static_cast<unsigned>(std::min<int64_t>(1024, (longest + 255) / 256));
   if ((e = launch_pdl(range_kernel<CAP>, dim3(gx, plan.count), dim3(256), 0, stream, t,
-                      maxbits, &ctrl->flagged)) != cudaSuccess)
+                      maxbits, ctrl)) != cudaSuccess)
     return e;
   const int64_t records = plan.total_stage_tiles * TB;
   const unsigned sgrid = static_cast<unsigned>((records + 255) / 256);
@@ -1073,11 +1114,7 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
   int64_t most_points = 0;
   for (int k = 0; k < plan.count; ++k) most_points = std::max(most_points, probs[k].n);
   if (most_points <= kSlowInlinePoints || slow.cap == 0) return cudaSuccess;  // nothing is listed
-  if ((e = launch_pdl(slow_search_kernel<CAP>, dim3(slow_grid), dim3(kSlowThreads), 0, stream, t,
-                      static_cast<const Control*>(ctrl), slow)) != cudaSuccess)
-    return e;
-  return launch_pdl(slow_finish_kernel<CAP>, dim3(slow_grid), dim3(kSlowThreads), 0, stream, t,
-                    static_cast<const Control*>(ctrl), slow, p);
+  return launch_pdl(slow_kernel<CAP>, dim3(slow_grid), dim3(kSlowThreads), 0, stream, t, ctrl, slow, p);
 }
 
 }  // namespace
@@ -1316,7 +1353,7 @@ int occupancy_forward_f32(bool general_p, int variant) {
 }
 
 cudaError_t launch_bounded_wait_selftest(Control* ctrl, cudaStream_t stream) {
-  bounded_wait_selftest_kernel<<<1, 32, 0, stream>>>(&ctrl->error);
+  bounded_wait_selftest_kernel<<<1, 32, 0, stream>>>(ctrl);
   return cudaGetLastError();
 }
 

@@ -65,6 +65,8 @@ constexpr int32_t kRecomputedF64 = -2;
 struct Control {
   unsigned flagged;  // number of queries routed to the slow path this call
   unsigned error;    // sticky error bits (kErrWaitTimeout, ...)
+  // Searches of this call's FP32 slow list that CTAs have drawn, and finished.
+  unsigned slow_drawn, slow_done;
   // Per-problem largest |coordinate| (float bits) of the FP32 forward's
   // range scan; every call leaves them zero (its combine clears them).
   unsigned maxbits[kBatchCap];

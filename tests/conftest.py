@@ -1,6 +1,9 @@
 """Shared pytest configuration: the ``gpu`` marker and the repo on sys.path."""
+import contextlib
 import os
 import sys
+
+import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 if ROOT not in sys.path:
@@ -11,3 +14,21 @@ def pytest_configure(config):
     config.addinivalue_line(
         "markers", "gpu: needs a CUDA GPU (sm_103a) and the compiled library; "
         "run with -m gpu on a GB300")
+
+
+@pytest.fixture
+def swept():
+    """``with swept():`` runs FP32 calls through the all-pairs sweep of the default
+    rule where small ones would take the one launch without a sweep (profiling
+    brackets the sweep, so it asks for one), and checks that they did."""
+    @contextlib.contextmanager
+    def run():
+        import paper_1402_4986_gb300 as idw
+        idw.profile_enable(True)
+        idw.profile_read()
+        try:
+            yield
+            assert idw.profile_read()[1] > 0
+        finally:
+            idw.profile_enable(False)
+    return run

@@ -1,8 +1,10 @@
 """Flagged queries of large problems (exact hits, FP64 recomputations): listed
-by the combine and finished by the two kernels after it, against the oracle.
+by the combine and finished by the kernel after it, against the oracle.
 Problems of up to 2048 points keep them in the combine; a list that is full
 (more flagged queries than the staged tiles' memory holds records) leaves the
-rest there too."""
+rest there too.  Calls within the limits of the one launch without a sweep (up
+to 12,288 points and 100 * 2^20 pairs) finish their own: the tests that name a
+sweep ask for one."""
 import numpy as np
 import pytest
 
@@ -16,7 +18,9 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("m,p", [(33, 2.0), (700, 3.5), (20000, 2.0)])
 def test_hits(n, m, p):
     """Every query on a data point, half of the points duplicated (the lowest
-    index wins); 20000 hits overflow the list of 2049 and of 8193 points (1046 and 4886 records)."""
+    index wins).  By default only 20,011 points and 20,000 queries on 8193 reach
+    the list, which the latter overflow (4886 records); the rest take the one
+    launch."""
     import torch
     import paper_1402_4986_gb300 as idw
     prob = synthetic.uniform_problem(n, m, seed=n + m)
@@ -49,3 +53,39 @@ def test_mixed_batch():
             assert np.array_equal(z[on], Z64[on].astype(np.float32))
             # the bar of the FP32 form; FP64 results carry only their rounding
             assert np.max(np.abs(z - Z64)) <= 2e-6 * np.max(np.abs(q["data"][:, 2]))
+
+
+@pytest.mark.parametrize("n", [2048, 2049, 8193, 20011])
+@pytest.mark.parametrize("m,p", [(1, 2.0), (33, 2.0), (257, 1.0), (700, 3.5), (20000, 2.0)])
+def test_hits_of_a_sweep(n, m, p, swept):
+    """As test_hits, by the sweep at every size: the combine alone up to 2048
+    points, then the list, whose kernel cuts few queries' points into many
+    slices and draws many groups of queries one by one; 20,000 hits overflow
+    the lists of 2049 and 8193 points."""
+    with swept():
+        test_hits(n, m, p)
+
+
+def test_mixed_batch_of_a_sweep(swept):
+    with swept():
+        test_mixed_batch()
+
+
+@pytest.mark.parametrize("hits", [0, 1, 300, 4000])
+def test_hits_among_others_of_a_sweep(hits, swept):
+    """Lists of no entry, of one, of more than a block's threads and of several
+    rounds; the neighbours of a hit, whose sums it spoils, are on them too."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(30011, 8000, seed=hits, exact_hits=hits)
+    Z64, hit64 = oracle.idw(prob["data"], prob["queries"], 2.0)
+    d, q = torch.from_numpy(prob["data"]).cuda(), torch.from_numpy(prob["queries"]).cuda()
+    with swept():
+        for _ in range(2):  # the counts start over with each call
+            Z, _, hit = idw.interpolate_saved(d, q, 2.0)
+            on = hit64 >= 0
+            assert np.array_equal(hit.cpu().numpy()[on], hit64[on])
+            assert not (hit.cpu().numpy()[~on] >= 0).any()
+            Zc = Z.cpu().numpy()
+            assert np.array_equal(Zc[on], Z64[on].astype(np.float32))
+            assert np.max(np.abs(Zc - Z64)) <= 2e-6 * np.max(np.abs(prob["data"][:, 2]))
