@@ -22,13 +22,13 @@ def swept():
     rule where small ones would take the one launch without a sweep (profiling
     brackets the sweep, so it asks for one), and checks that they did."""
     @contextlib.contextmanager
-    def run():
+    def run(handle=None):
         import paper_1402_4986_gb300 as idw
-        idw.profile_enable(True)
-        idw.profile_read()
+        idw.profile_enable(True, handle=handle)
+        idw.profile_read(handle=handle)
         try:
             yield
-            assert idw.profile_read()[1] > 0
+            assert idw.profile_read(handle=handle)[1] > 0
         finally:
-            idw.profile_enable(False)
+            idw.profile_enable(False, handle=handle)
     return run

@@ -113,3 +113,71 @@ def test_debug_build_index_checks_stay_clean(idw):
     assert res["status"] == 0, res
     assert res["sites"] == 0, f"index checks failed at sites {res['sites']:#x}"
     assert res["worst"] <= 1e-5
+
+
+LARGE = r"""
+import ctypes, json
+import numpy as np
+import torch
+import synthetic
+import paper_1402_4986_gb300 as idw
+from paper_1402_4986_gb300 import _lib
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+rng = np.random.default_rng(84)
+worst, calls = 0.0, 0
+xy = synthetic.mixture_xy(rng, 300000)
+blobs = synthetic.pack_xyz(xy[:20000], rng.standard_normal(20000).astype(np.float32))
+flat = synthetic.uniform_problem(6000, 300000, seed=85)
+outside = flat["queries"].copy()
+outside[::5] += 0.9; outside[1::5] -= 0.9
+far = flat["queries"] * 3.0 - 1.0
+grid = synthetic.grid_xy(70)
+lattice = synthetic.pack_xyz(grid, rng.standard_normal(len(grid)).astype(np.float32))
+on = grid[rng.integers(0, len(grid), 300000)]
+on[7] = np.nan
+for data, q in ((flat["data"], flat["queries"]), (flat["data"], outside), (flat["data"], far),
+                (blobs, flat["queries"]), (blobs, xy), (lattice, on)):
+    d, top = dev(data), float(np.abs(data[:, 2]).max())
+    for k, m in ((3, 30000), (9, 60000), (20, 120000), (20, 300000), (40, 90000)):
+        qq = dev(q[:m])
+        kix = idw.LocalIndex(d, k=k)
+        Z, kd2 = idw.interpolate_knn(d, qq, 2.0, k, kth_d2=True)
+        Zl, nbr, kd2l = idw.interpolate_knn(d, qq, 2.0, k, neighbours=True, kth_d2=True)
+        Zi, kd2i = kix.knn(qq, 2.0, k, kth_d2=True)
+        for a, b in ((Zl, kd2l), (Zi, kd2i)):
+            assert torch.equal(kd2.nan_to_num(-1.0), b.nan_to_num(-1.0)), (k, m)
+            worst = max(worst, float((Z - a).nan_to_num(0.0).abs().max()) / top)
+        calls += 3
+    for members, m in ((20.0, 300000), (200.0, 100000), (20.0, 100000)):
+        qq, R = dev(q[:m]), synthetic.local_radius(len(data), members)
+        Z, cnt = idw.interpolate_local(d, qq, 2.0, R, counts=True)
+        Zi, cnti = idw.LocalIndex(d, radius=R).interpolate(qq, 2.0, counts=True)
+        assert torch.equal(cnt, cnti)
+        worst = max(worst, float((Z - Zi).nan_to_num(0.0).abs().max()) / top)
+        idw.local_backward(d, qq, 2.0, R, torch.ones(m, device="cuda"), modified=members > 100)
+        calls += 3
+torch.cuda.synchronize()
+sites = ctypes.c_uint32(0)
+st = _lib.load().idw_debug_check_failures(torch.cuda.current_device(), ctypes.byref(sites))
+print(json.dumps({"status": st, "sites": sites.value, "worst": worst, "calls": calls,
+                  "lib": _lib.library_path()}))
+"""
+
+
+def test_large_calls_stay_clean(idw):
+    """The searches that only larger calls reach: by counts, by threads that
+    list hard queries, by threads for what is left, large and unsorted discs;
+    the routes of one input agree and no check fails."""
+    env = dict(os.environ, IDW_DEBUG_CHECKS="1")
+    env["PYTHONPATH"] = ROOT + os.pathsep + env.get("PYTHONPATH", "")
+    out = subprocess.run([sys.executable, "-c", LARGE], cwd=ROOT, env=env, capture_output=True,
+                         text=True, timeout=600)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    res = json.loads(out.stdout.strip().splitlines()[-1])
+    assert res["lib"].endswith("_debug.so")
+    assert res["status"] == 0 and res["calls"] == 144, res
+    assert res["sites"] == 0, f"index checks failed at sites {res['sites']:#x}"
+    assert res["worst"] <= 4e-6, res  # two values, each within the FP32 form's bar

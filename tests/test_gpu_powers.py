@@ -1,6 +1,8 @@
 """p = 1, 3 and 4 as powers of one reciprocal (square root): parity with the
 FP64 oracle at the edges of chunks, tiles and query tiles, hits, batches,
-points at infinity, NaN, and against the log2/exp2 form."""
+points at infinity, NaN, and against the log2/exp2 form.  Calls with default
+options lie within the one launch without a sweep; the tests that name a sweep
+run the default sweep (512-query tiles) or a forced one at the same inputs."""
 import numpy as np
 import pytest
 
@@ -67,3 +69,42 @@ def test_extreme_scales(p, scale):
     z = idw.interpolate(_dev(d), _dev(q), p).cpu().numpy()
     Z64, _ = oracle.idw(prob["data"], prob["queries"], p)
     assert np.max(np.abs(z - Z64)) <= TOL * np.max(np.abs(d[:, 2]))
+
+
+@pytest.mark.parametrize("p", [1.0, 3.0, 4.0])
+@pytest.mark.parametrize("n,m", [(1, 3), (32, 2049), (33, 4097), (257, 100), (5003, 777)])
+def test_parity_of_a_sweep(p, n, m, swept):
+    import paper_1402_4986_gb300 as idw
+    h = idw.Handle(0)
+    prob = synthetic.uniform_problem(n, m, seed=n + m, exact_hits=min(n, m, 4))
+    with swept(h):
+        Z, s0, hit = idw.interpolate_saved(_dev(prob["data"]), _dev(prob["queries"]), p, handle=h)
+    Z64, hit64 = oracle.idw(prob["data"], prob["queries"], p)
+    assert np.max(np.abs(Z.cpu().numpy() - Z64)) <= TOL * np.max(np.abs(prob["data"][:, 2]))
+    hit = hit.cpu().numpy()
+    assert np.array_equal(hit[hit >= 0], hit64[hit64 >= 0])
+
+
+@pytest.mark.parametrize("p", [1.0, 3.0, 4.0])
+def test_batch_and_infinite_points_of_a_sweep(p, swept):
+    with swept():
+        test_batch_and_infinite_points(p)
+
+
+@pytest.mark.parametrize("p", [1.0, 3.0, 4.0])
+@pytest.mark.parametrize("variant", [-1, 0, 4])
+@pytest.mark.parametrize("scale", [2.0 ** -60, 1.0, 2.0 ** 60])
+def test_extreme_scales_of_a_sweep(p, scale, variant, swept):
+    """Far padding (p = 4 shares reciprocals, p = 1 and 3 do not) against
+    coordinates at both ends, a point at infinity among them."""
+    import paper_1402_4986_gb300 as idw
+    h = idw.Handle(0)
+    idw.set_option("sweep_variant", variant, handle=h)
+    prob = synthetic.uniform_problem(900, 500, seed=3)
+    d, q = prob["data"].copy(), prob["queries"] * np.float32(scale)
+    d[:, :2] *= np.float32(scale)
+    d = np.concatenate([d, np.array([[np.inf, 0.0, 5.0]], np.float32)])  # weight 0
+    with swept(h):
+        z = idw.interpolate(_dev(d), _dev(q), p, handle=h).cpu().numpy()
+    Z64, _ = oracle.idw(prob["data"], prob["queries"], p)
+    assert np.max(np.abs(z - Z64)) <= TOL * np.max(np.abs(prob["data"][:, 2]))
