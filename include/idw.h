@@ -215,7 +215,7 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *       problem or batch of n <= 12,288 each, n m <= 100 2^20 and 256 tiles of
  *       128 queries in all, and p <= 4, takes one launch without a sweep,
  *       unless a variant, a staging layout, the autotuner or IDW_OPT_FMA_LOG2
- *       is set) or:
+ *       is set, or profiling is on: see idw_profile_enable) or:
  *       0: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal;
  *       1: 2048 queries per CTA, no shared reciprocal;
  *       2: 2048 queries per CTA, 1 of 4 query pairs shares a reciprocal
@@ -290,9 +290,10 @@ idw_status idw_plan_forward(int32_t sm_count, int32_t ctas_per_sm, int64_t n, in
  *   IDW_OPT_KNN_SEARCH          0 (default) or 1.  The k-NN search of
  *                               idw_interpolate_knn and idw_knn_backward: 0
  *                               one thread per query, each growing its own
- *                               square of cells at its own pace, or a warp per
+ *                               square of cells at its own pace, a warp per
  *                               query where there are few queries or the
- *                               points around one are far or dense; 1 the
+ *                               points around some are far or dense, or
+ *                               counts (see idw_interpolate_knn); 1 the
  *                               per-thread search with the 32 lanes of a warp
  *                               kept in step (the same step and row order,
  *                               each lane's row runs walked as one stream,
@@ -326,7 +327,9 @@ idw_status idw_get_option(idw_handle_t handle, idw_option option, int64_t *value
 
 /*
  * Kernel timing (tracing).  While enabled, every forward call records a pair
- * of CUDA events around its all-pairs sweep kernel on the call's stream.
+ * of CUDA events around its all-pairs sweep kernel on the call's stream; small
+ * calls that would take one launch without a sweep run the sweep instead
+ * (results within the same bound, the last bits may differ).
  * idw_profile_read synchronises those events, returns the summed sweep time
  * in milliseconds and the number of sweep launches, and clears the record.
  */
@@ -503,12 +506,13 @@ idw_status idw_noalloc_selftest_bounded_wait(void *stream);
  * of cells about R/2 wide (at most 2048 per axis and one cell per two data
  * points), planned by one device thread; a counting sort of the data and of
  * the queries into the cells; then one thread per query, in cell order,
- * walks the rows of cells its disc of radius R reaches.  Weights are summed
+ * walks the rows of cells its disc of radius R reaches, or a warp where a
+ * query has many more candidates than others.  Weights are summed
  * as compensated FP32 pairs; a query whose sums leave FP32's range is
  * redone in FP64.  Scatter positions come from atomics, so candidates may be
  * summed in a different order from call to call: results can differ in the
  * last bit.
- * Workspace (the handle's): 16 bytes per data point, 16 per query and 16 per
+ * Workspace (the handle's): 16 bytes per data point, 20 per query and 16 per
  * cell, for at most min(2^22, max(1024, n/2)) cells.  Errors as in
  * idw_interpolate, plus IDW_ERR_INVALID_ARG for radius <= 0 or NaN; the
  * kernels run asynchronously after it returns.
@@ -565,11 +569,15 @@ idw_status idw_interpolate_modified(idw_handle_t handle, const float *data_xyz, 
  * cells; once k keys are held, cells whose points provably lie beyond the
  * k-th key are skipped; the search stops once the k-th key is below a
  * conservative FP32 lower bound on the key of any point not yet seen.  For
- * few queries, and for those whose surroundings are empty or dense, a warp
- * takes the query instead: it walks the cells of a disc that the table shows
- * to hold k points.
- * Workspace as idw_interpolate_local and 4 bytes per query.  Errors as in
- * idw_interpolate, plus IDW_ERR_INVALID_ARG for k outside [1, 64].
+ * few queries, and in calls of up to 2^19 for those in empty surroundings and
+ * for some 20,000 to 65,000 (by k) in dense ones, a warp takes the query
+ * instead: it walks the cells of a disc that the table shows to hold k points.
+ * Without nbr_out, evenly spread data
+ * and k > 32 (k > 16 above 114,688 queries) are searched by counting the
+ * candidates of a disc by d2, without a heap, unless most queries lie beyond
+ * the data.
+ * Workspace as idw_interpolate_local.  Errors as in idw_interpolate, plus
+ * IDW_ERR_INVALID_ARG for k outside [1, 64].
  */
 idw_status idw_interpolate_knn(idw_handle_t handle, const float *data_xyz, int64_t n,
                                const float *queries_xy, int64_t m, double p, int32_t k,

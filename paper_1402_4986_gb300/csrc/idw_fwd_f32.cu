@@ -1167,7 +1167,9 @@ double sweep_clocks(const F32Problem* probs, int count, int variant, int threads
 // Measured, rule of thumb / 512-query tiles, whole call: p = 2: n = 20,000,
 // m = 1000 35.4 / 30.7 us; n = 70,000, m = 3000 88.7 / 78.6; n = m = 20,000
 // 113.5 / 126.4 (not taken).  p = 3.5: n = m = 4000 70.7 / 38.0; 64 problems of
-// 256 to 8192 points 320 / 275; n = m = 40,000 648 / 687 (not taken).
+// 256 to 8192 points 320 / 275; n = m = 40,000 648 / 687 (not taken).  p = 1, 3
+// and 4 go by the general form's rates: their sweeps are about 1.4 times as fast
+// with every tile, and only the rates' ratios matter here.
 int default_sweep_variant(const F32Problem* probs, int count, bool general_form, int sm_count) {
   const int64_t q4 = qt_of<4>(), q0 = qt_of<0>();
   double pad4 = 0, pad0 = 0, units0 = 0;
@@ -1263,8 +1265,8 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   // 641 / 700 / 651 us, against 1007 us through log2 and exp2, with errors
   // against 64 bits at or below that form's (it keeps that form's 32-point
   // chunks: the 64-point ones of p = 2 were 3% faster and 5% less exact).
-  // Aligned records beat duplicated pairs by 1-2% here as at p = 2.  Forced
-  // variants and layouts, made to study the general form, keep it.
+  // Aligned records beat duplicated pairs by 1-2% here as at p = 2.  Variants
+  // 1, 2, 3 and 5 and a forced layout, made to study the general form, keep it.
   if (!plan.force_general && plan.layout < 0 && !plan.fma_log2 &&
       (plan.variant == 0 || plan.variant == 4 || plan.variant == 7)) {
 #define IDW_LAUNCH_POWER(M)                                                                     \

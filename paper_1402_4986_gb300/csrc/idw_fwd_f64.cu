@@ -50,14 +50,17 @@ __device__ __forceinline__ void tile_record(const unsigned char* tile, int r, do
   }
 }
 
-// 1/a for a >= 0 by one third-order step from the hardware's approximation y
-// (at least 20 bits): with e = 1 - a y, 1/a = y (1 + e + e^2 + ...), and the
-// terms kept leave a relative error of e^3 <= 2^-60, so the result is within
-// half an ulp and 2^-60 of the quotient.  Three FP64 operations where the
-// division took five: the FP64 pipe (2 per SM and clock) bounds the sweep at
-// 9 operations a pair instead of 11.  n = 20,000, m = 10,007, p = 2:
-// 4722 -> 3824 us.  a = +inf gives 0; a = 0, a subnormal or NaN gives NaN
-// (the query then goes to the slow path).
+// 1/a for a >= 0 by one third-order step (Chebyshev's iteration for the
+// reciprocal) from the hardware's approximation y: with e = 1 - a y,
+// 1/a = y (1 + e + e^2 + ...), of which the terms up to e^2 are kept.  PTX
+// describes y as computed from the upper 32 bits of a and returned to 20
+// mantissa bits, so |e| stays below 2^-19 and the cut below 2^-57 of the
+// result: within 0.5 + 2^-4 ulp of the quotient, where the division it
+// replaces rounds to 0.5.  Z's largest error against 64 bits is the same with
+// either (4.8e-16 of the largest |z|, n = 20,000).  Three FP64 operations; the
+// FP64 pipe (2 per SM and clock) bounds the sweep at 9 a pair.  n = 20,000,
+// m = 10,007, p = 2: 4722 us with the division, 3824 so.  a = +inf gives 0;
+// a = 0, a subnormal or NaN gives NaN (the query then goes to the slow path).
 __device__ __forceinline__ double reciprocal(double a) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));

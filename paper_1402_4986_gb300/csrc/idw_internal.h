@@ -41,8 +41,7 @@ constexpr int kBatchCap = 256;
 // variant 0 is the default tiling above.
 constexpr int kNumSweepVariants = 6;
 // Two more that only the default rule picks, for small problems: 512 queries
-// per CTA (64 threads), work units of 64 (6; p = 2 and p = 1, 3, 4 only) or
-// 256 points (7).
+// per CTA (64 threads), work units of 64 (6; p = 2 only) or 256 points (7).
 constexpr int kSmallTileFine = 6, kSmallTile = 7, kNumAllVariants = 8;
 
 // Plain FP64 forward: kQueriesF64 queries per thread; tiles of (x,y) + z.
