@@ -157,6 +157,11 @@ idw_status idw_interpolate_batched(idw_handle_t handle, int32_t count,
  *   grad_z (n), grad_data_xy (n x 2), grad_query_xy (m x 2) : device float,
  *   grad_p (1) : device double; each nullable (NULL skips that gradient).
  *   The gradient buffers are overwritten, not accumulated into.
+ * Workspace (the handle's): about 24 bytes per data point and 32 per query,
+ * and 96 KiB per tile of 4096 queries (points) and per persistent CTA.  Where
+ * gradients of both sides are wanted and p >= 1, one sweep computes them and
+ * adds up to 256 MiB of per-tile sums and 24 bytes per data point; if that
+ * cannot be allocated, two sweeps run without it.
  */
 idw_status idw_backward(idw_handle_t handle, const float *data_xyz, int64_t n,
                         const float *queries_xy, int64_t m, double p, const float *Z,

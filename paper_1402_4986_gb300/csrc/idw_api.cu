@@ -657,6 +657,12 @@ idw_status idw_backward(idw_handle_t h, const float* data, int64_t n, const floa
   const bool both = (grad_query_xy || grad_p) && (grad_z || grad_data_xy);
   idw::plan_backward_f32(n, m, p, both, h->sm_count, h->occ_bwd, &bp);
   st = ensure_buffer(h, &h->ws, &h->ws_bytes, bp.workspace_bytes);
+  if (st == IDW_ERR_WORKSPACE && bp.fused) {  // no room for its partial sums
+    cudaGetLastError();  // that error is dealt with
+    bp = idw::BwdPlan();
+    idw::plan_backward_f32(n, m, p, false, h->sm_count, h->occ_bwd, &bp);
+    st = ensure_buffer(h, &h->ws, &h->ws_bytes, bp.workspace_bytes);
+  }
   if (st != IDW_OK) return st;
   idw::BwdProblem pb{static_cast<const float*>(data), n, static_cast<const float*>(queries), m, p,
                      Z, s0, hit, grad_out, grad_z, grad_data_xy, grad_query_xy, grad_p};

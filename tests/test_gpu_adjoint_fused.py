@@ -110,3 +110,31 @@ def test_extreme_pairs():
         G = oracle.idw_grad(prob["data"], prob["queries"], p, gn)
         assert _rel(gz.cpu().numpy(), G["grad_z"]) <= TOL
         assert _rel(gq.cpu().numpy(), G["grad_q"]) <= TOL
+
+
+def test_without_room_for_the_partial_sums():
+    """2^20 points want 252 MiB of them and 24 MiB of sums over panels, 403 MiB in
+    all with the quarter that a handle adds; with 256 MiB of the device's memory
+    left the two sweeps run, which need 86."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    torch.manual_seed(4)
+    n, m = 1 << 20, 90000
+    d, q = torch.rand(n, 3, device="cuda"), torch.rand(m, 2, device="cuda")
+    g = torch.randn(m, device="cuda")
+    roomy, tight = idw.Handle(0), idw.Handle(0)
+    Z, s0, hit = idw.interpolate_saved(d, q, 2.0, handle=roomy)
+    want = idw.backward(d, q, 2.0, Z, s0, hit, g, handle=roomy)
+    got = idw.backward(d[:1000].contiguous(), q, 2.0, Z, s0, hit, g, handle=tight)  # outputs' memory
+    del got
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    held = torch.empty(free - (256 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = idw.backward(d, q, 2.0, Z, s0, hit, g, handle=tight)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    for a, b in zip(got, want):
+        assert float((a.double() - b).norm()) <= 1e-5 * float(b.double().norm())
