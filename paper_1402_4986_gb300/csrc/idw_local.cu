@@ -107,8 +107,7 @@ struct GridDev {
   int gx, gy, cells;
   unsigned hard;         // queries the per-thread kernels left to warps
   unsigned left;         // queries the search by counts left to warps or threads
-  unsigned next;         // next group of queries of the uneven-data heap search
-  unsigned next_left;    // next group of the queries left
+  unsigned next;         // next group of queries of the fetching heap search
   unsigned beyond;       // of kSampleQueries queries: those beyond the grid's edge,
   unsigned dense;        // and those in dense surroundings, or heavy (see sample_queries)
 };
@@ -195,7 +194,7 @@ __device__ void plan_grid(GridDev* grid, double radius, double inv_max_cells, in
   grid->gx = gx;
   grid->gy = gy;
   grid->cells = gx * gy;
-  grid->hard = grid->left = grid->next = grid->next_left = 0u;
+  grid->hard = grid->left = grid->next = 0u;
   grid->beyond = grid->dense = 0u;
 }
 
@@ -288,9 +287,9 @@ __device__ __forceinline__ int query_bucket(const GridDev& g, float x, float y) 
   return cy * g.gx + cx;
 }
 
-// Whether a position in cells lies beyond the grid's edge.
-__device__ __forceinline__ bool beyond_grid(const GridDev& g, float u, float v) {
-  return fmaxf(fmaxf(-u, u - float(g.gx)), fmaxf(-v, v - float(g.gy))) > 0.f;
+// Whether a position in cells lies more than `cells` beyond the grid's edge.
+__device__ __forceinline__ bool beyond_grid(const GridDev& g, float u, float v, float cells = 0.f) {
+  return fmaxf(fmaxf(-u, u - float(g.gx)), fmaxf(-v, v - float(g.gy))) > cells;
 }
 
 // Threads [0, n) count data points, [n, n + m) count queries.
@@ -631,7 +630,7 @@ __device__ __forceinline__ void sample_queries(GridDev* out, const GridDev& g,
 
 // Threads [0, n) place data points as (x, y, z, index), [n, n + m) place
 // queries as (x, y, index, 0).  With `sample` not 0 (see sample_queries) the
-// last block samples the call's `all` queries instead.
+// first block samples the call's `all` queries instead.
 __global__ void __launch_bounds__(256)
     scatter_kernel(GridDev* grid, const float* data, int64_t n,
                    const float* queries, int64_t m, int64_t all, int sample,
@@ -642,11 +641,11 @@ __global__ void __launch_bounds__(256)
   pdl_trigger();
   pdl_wait();
   const GridDev g = *grid;
-  if (sample != 0 && blockIdx.x == gridDim.x - 1) {
+  if (sample != 0 && blockIdx.x == 0) {
     sample_queries(grid, g, starts_d, sums, n, queries, all, sample);
     return;
   }
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t i = int64_t(blockIdx.x - (sample != 0)) * blockDim.x + threadIdx.x;
   if (i < n) {
     const float x = data[3 * i], y = data[3 * i + 1];
     const int c = data_cell(g, x, y);
@@ -1662,10 +1661,9 @@ __device__ __forceinline__ bool knn_by_counts(const GridDev& g, int64_t n) {
   return knn_even(g, n) && 2 * g.beyond <= kSampleQueries;
 }
 
-// The queries that the heap search lists for warps, besides those in sparse
-// surroundings.
+// The queries that the heap search lists for warps.
 struct KnnListed {
-  bool dense, beyond;  // in dense surroundings; beyond the grid's edge
+  bool sparse, dense, beyond;  // in such surroundings; two cells beyond the grid's edge
 };
 
 // Query t, by one thread (no block-wide barrier; `return`s are its own).
@@ -1722,8 +1720,8 @@ __device__ __forceinline__ void knn_thread_query(
       const KnnSurroundings at =
           knn_surroundings(g, sat, float(g.cells) * rcp_approx(float(n)), cx, cy, k);
       // One branch, so that the warp comes together again behind it.
-      const bool away = (at == kSparse) | (listed.dense & (at == kDense)) |
-                        (listed.beyond & beyond_grid(g, u, v));
+      const bool away = (listed.sparse & (at == kSparse)) | (listed.dense & (at == kDense)) |
+                        (listed.beyond & beyond_grid(g, u, v, 2.f));
       if (away) {
         list_heavy(t, m, lists.hard, lists.query);
         return;
@@ -1879,11 +1877,11 @@ __device__ __forceinline__ void knn_thread_query(
 // again for each (64 blobs, n = 2^20, queries in the blobs too, threads / warps:
 // m = 500,000 k = 8 520 / 1605 us, k = 32 880 / 1826; m = 100,000 293 / 440 and
 // 391 / 554; m = 30,000 252 / 235 and 393 / 155).  FROM says which queries it
-// takes: all of them, a block's 32 each; all of them unless they are searched
-// by counts; or those that search left, if they are not few.  In the latter two
-// its blocks, as many as fit the GPU, fetch groups of 32 queries from a counter:
-// 32,768 blocks that return at once take 34 us.
-enum KnnFrom : int { kFromAll, kFromUneven, kFromUnevenFetched, kFromLeft };
+// takes: all of them, a block's 32 each; or, after the search by counts, those
+// that it left, if they are not few, and all of them where it does not run.  In
+// the last form the blocks, as many as fit the GPU, fetch groups of 32 queries
+// from a counter: 32,768 blocks that return at once take 34 us.
+enum KnnFrom : int { kFromAll, kFromLeft, kFromLeftFetched };
 template <int MODE, bool LIST, int FROM>
 __global__ void __maxnreg__(64)
     knn_query_kernel(const GridDev* grid, const float4* sorted,
@@ -1896,16 +1894,20 @@ __global__ void __maxnreg__(64)
                      bool sort_rows, const KnnLists lists, unsigned* next) {
   pdl_trigger();
   pdl_wait();
-  constexpr bool fetch = FROM >= kFromUnevenFetched;
-  if ((FROM == kFromUneven || FROM == kFromUnevenFetched) && knn_by_counts(*grid, n)) return;
-  const int64_t count = FROM == kFromLeft ? int64_t(*lists.left) : m;
-  if (FROM == kFromLeft && count <= lists.few) return;
-  KnnListed listed{false, false};
-  if (LIST) {
+  const bool counted = FROM != kFromAll && knn_by_counts(*grid, n);
+  int64_t count = m;
+  if (counted) {
+    count = *lists.left;
+    if (count <= lists.few) return;
+  }
+  KnnListed listed{false, false, false};
+  if (LIST && !counted) {
+    listed.sparse = true;
     listed.beyond = m <= kUnsortedKnn;
     listed.dense = m <= lists.few ||
                    (k >= kSampleK && grid->dense * m <= int64_t(kSampleQueries) * lists.few);
   }
+  constexpr bool fetch = FROM == kFromLeftFetched;
   const int lane = threadIdx.x;
   int64_t group = blockIdx.x;
   for (;;) {
@@ -1917,7 +1919,7 @@ __global__ void __maxnreg__(64)
     int64_t t = group * kKnnThreads + lane;
     if (fetch && group * kKnnThreads >= count) break;
     if (t < count) {
-      if (FROM == kFromLeft) t = lists.query[m - 1 - t];
+      if (counted) t = lists.query[m - 1 - t];
       if (dcheck(t >= 0 && t < m, kSiteScatter))
         knn_thread_query<MODE, LIST>(grid, sorted, starts, base, bpre, sat, qrec, data, n, m, p, k,
                                      out, nbr_out, kd2_out, hit_out, sort_rows, lists, listed, t);
@@ -3573,7 +3575,17 @@ int64_t knn_warp_queries(int k) { return std::min<int64_t>(8192 + 1024 * int64_t
 // the GPU is full either way (64 blobs, n = 2^20, k = 8, threads alone / with
 // warps: m = 10,007 1010 / 74 us, 100,000 1090 / 263 us, 2^20 1440 / 1770 us).
 constexpr int64_t kKnnHardQueries = int64_t(1) << 19;
+
+// Above this many queries k <= 32 is counted too: below it the counts' two walks
+// are bound by latency as the heaps are (100,000 queries, k = 32, uniform 143 us
+// by counts and 141 by heaps, on a lattice 124 and 102; 131,072: 140 and 196,
+// 127 and 134).
 constexpr int64_t kCountQueries = 7 * (int64_t(1) << 14);
+
+// Up to this many queries the heap search after the counts has a block for each
+// 32 of them, which is 5-10% faster where it has them all to do (64 blobs, queries
+// in the blobs too, k = 64, m = 100,000: 862 us, 934 fetched) and costs a
+// nanosecond each where it has none.
 constexpr int64_t kUnfetchedQueries = int64_t(1) << 18;
 static_assert(kUnfetchedQueries <= kKnnHardQueries, "these list their hard queries");
 
@@ -3604,7 +3616,8 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
   // Without lists and from k = 17 on, evenly spread data are searched by counts
   // (uniform n = m = 2^20, heaps / counts: k = 16 389 / 383 us, 24 550 / 454,
   // 32 723 / 475, 64 1552 / 718); the device decides which of the two runs.
-  const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16 && (a.k > 32 || a.m > kCountQueries);
+  const bool counted = !all_warps && !a.nbr_out && !a.hit_out && a.k > 16 &&
+                       (a.k > 32 || a.m > kCountQueries);
   const bool list = warps && !all_warps && a.m <= kKnnHardQueries;
   const KnnLists lists{&a.grid->hard, &a.grid->left, all_warps ? nullptr : a.hard,
                        static_cast<unsigned>(knn_few(a.k))};
@@ -3623,34 +3636,31 @@ cudaError_t launch_knn_search(const KnnArgs& a, int sm_count, cudaStream_t s) {
       constexpr bool L = decltype(list_these)::value;
       constexpr int F = decltype(from)::value;
       auto kernel = pow2 ? knn_query_kernel<kPow2, L, F> : knn_query_kernel<kPowGeneral, L, F>;
-      const unsigned blocks = F < kFromUnevenFetched ? groups : std::min(groups, resident);
-      unsigned* next = F == kFromLeft ? &a.grid->next_left : &a.grid->next;
+      const unsigned blocks = F == kFromLeftFetched ? std::min(groups, resident) : groups;
       // A kernel that starts early has its first blocks placed on the SMs that
       // the one before it leaves free; where all blocks fit at once, they stay
       // so (uniform m = 30,000, k = 32, gradient call: 270 us, 204 started
       // plainly; index call of 100,000, k = 16: 99 and 89).  The short searches
       // for a few neighbours gain more from the early start (m = 10,007, k = 1:
       // 18 us, 22 plainly).
-      if (groups >= resident || F == kFromLeft || a.k < 4)
+      if (groups >= resident || a.k < 4)
         return launch_pdl(kernel, blocks, kKnnThreads, smem, s, a.grid, a.sorted, a.starts, a.base,
                           a.bpre, a.sat, a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                          a.kd2_out, a.hit_out, a.sort_rows, lists, next);
+                          a.kd2_out, a.hit_out, a.sort_rows, lists, &a.grid->next);
       kernel<<<blocks, kKnnThreads, smem, s>>>(a.grid, a.sorted, a.starts, a.base, a.bpre, a.sat,
                                                a.qrec, a.data, a.n, a.m, a.p, a.k, a.out, a.nbr_out,
-                                               a.kd2_out, a.hit_out, a.sort_rows, lists, next);
+                                               a.kd2_out, a.hit_out, a.sort_rows, lists, &a.grid->next);
       return cudaGetLastError();
     };
     using All = std::integral_constant<int, kFromAll>;
-    using Uneven = std::integral_constant<int, kFromUneven>;
-    using Fetched = std::integral_constant<int, kFromUnevenFetched>;
     using Left = std::integral_constant<int, kFromLeft>;
+    using Fetched = std::integral_constant<int, kFromLeftFetched>;
     if (counted && a.m <= kUnfetchedQueries)
-      e = heap(std::true_type{}, Uneven{});
+      e = heap(std::true_type{}, Left{});
     else if (counted)
       e = list ? heap(std::true_type{}, Fetched{}) : heap(std::false_type{}, Fetched{});
     else
       e = list ? heap(std::true_type{}, All{}) : heap(std::false_type{}, All{});
-    if (e == cudaSuccess && counted && a.m > knn_few(a.k)) e = heap(std::false_type{}, Left{});
   }
   if (e != cudaSuccess || (!all_warps && !list && !counted)) return e;
   constexpr int per_block = kKnnWarpThreads / 32;
@@ -3715,7 +3725,7 @@ __device__ __forceinline__ void copy_plan(const GridDev* src,
   GridDev g = *src;
   g.box_ticket = 0xffffffffu;
   g.scan_ticket = 0xffffffffu;
-  g.hard = g.left = g.next = g.next_left = 0u;
+  g.hard = g.left = g.next = 0u;
   g.beyond = g.dense = 0u;
   if (radius > 0.0 && g.inv2 > 0.f)
     g.rho = __fmaf_ru(__fmul_ru(__double2float_ru(radius), g.inv2), 0.5f + 0x1p-9f, 0x1p-8f);
