@@ -448,8 +448,11 @@ def run_ours(args, ws, rank, local):
                    "n": n, "m": m, "p": 2.0, "parallelism": f"query shards x{ws}, data replicated",
                    "l2": "flushed between steps (256 MiB write; inputs are 36 MiB)"},
         "e2e": e2e,
-        # range, stage, sweep, combine; above 2048 points the slow list's search and finish.
-        "gpu_launches": (6 if n > 2048 else 4) * args.steps,
+        # range, stage, sweep, combine, and above 2048 points the slow list's.  The timed
+        # steps record the sweep's events, so a size within the one launch without a
+        # sweep (n <= 12,288, n m <= 100 * 2^20, 256 tiles of 128 queries) runs them too:
+        # its sweep figures are not those of a call without profiling.
+        "gpu_launches": (5 if n > 2048 else 4) * args.steps,
         "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
         "error_vs_fp64_oracle": err,
         **({"full_check": full} if full else {}),

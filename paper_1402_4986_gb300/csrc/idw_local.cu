@@ -2152,9 +2152,10 @@ __global__ void __launch_bounds__(kCountThreads)
 //    full its k smallest keys are kept and the bound drops to the k-th key;
 // 3. the k smallest of the buffer are the selection (keys are distinct, so
 //    the order of candidates does not matter), and the lanes share the sums.
-// Bound by instruction issue (66% of issue slots, 30 of 32 lanes active,
-// about 1250 instructions a query at k = 8); a query costs about as many
-// whether its points lie near or far, which is what the hard queries need.
+// About 1500 instructions a query at k = 8, with 29 of 32 lanes active; a query
+// costs about as many whether its points lie near or far, which is what the
+// hard queries need.  A call of 10,000 is bound by latency (a third of the warps
+// resident, loads the first stall).
 constexpr unsigned kWarp = 0xffffffffu;
 
 // kRegs keys per lane: the buffer of 32 kRegs keys is cut back to k when
