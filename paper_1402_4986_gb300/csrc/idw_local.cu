@@ -575,16 +575,18 @@ __device__ __forceinline__ int heavy_candidates(const GridDev& g, int64_t n, boo
 // (150,001 queries: 390 / 344 and 1250 / 1060.)
 constexpr int kSampleQueries = 256;
 //
-// Queries in no spatial order (`scattered`) are heavy from 128 + m / 256
+// Queries in no spatial order (`scattered`) are heavy from 128 + 3 m / 1024
 // candidates on: threads of a warp then read from as many places, the 32 lanes
 // of one query from one.  More queries hide more of the threads' latency.
 // Index of 2^20 uniform points, R for 128 / 512 / 2048 members, us sorted first / a
 // thread each / by this rule: 10,007 queries 74 / 176 / 576, 74 / 219 / 914 and
-// 31 / 32 / 75; 131,072 queries 92 / 240 / 799, 107 / 381 / 1456 and 107 / 300 / 830.
+// 31 / 32 / 75; 131,072 queries 92 / 240 / 799, 107 / 381 / 1456 and 107 / 335 / 830.
+// (A bound of 128 + m / 256 just missed the second: 382; and 10,007 queries with
+// 256 members in 2^24 points 147 us, 29 so.)
 __device__ __forceinline__ bool list_if_heavy(const GridDev& g, const Runs& runs, int64_t n,
                                               int64_t m, int64_t most, bool scattered = false) {
   int bound = heavy_candidates(g, n, m <= most);
-  if (scattered) bound = min(bound, 128 + int(m / 256));
+  if (scattered) bound = min(bound, 128 + int(3 * m / 1024));
   return runs.candidates() > bound && g.dense * m <= kSampleQueries * most;
 }
 
