@@ -2174,10 +2174,13 @@ struct KnnBuffer {
   // below) and hi (at least k) in the order of the float's bits; the probe
   // between them assumes keys spread evenly in d^2, as points of even density
   // are, and every third probe halves the bracket instead.  No probe separates
-  // keys of equal d^2 (data on a lattice): after kProbes of them the bracket's
-  // ends move to keys, so that it closes on a tie at once, not bit by bit
-  // (lattice of 2^20 points, queries on it, m = 50,000, k = 64: 212 us, 170 so).
-  static constexpr int kProbes = 6;
+  // keys of equal d^2 (data on a lattice): after kProbes of them the rest of the
+  // bracket is gone through key by key, which closes on a tie at once, not bit by
+  // bit (lattice of 2^20 points, queries on it, m = 50,000, k = 64: 176 us, 130 so).
+  // With four keys a lane six probes often stop short of a bracket that a few more
+  // would close (uniform data, m = 10,007, k = 64: six 37.8, eight 36.5, ten 34.2 us;
+  // m = 10,007 on the lattice 34.1, 35.5, 37.6); with fewer, ten gain nothing.
+  static constexpr int kProbes = kRegs > 3 ? 9 : 6;
   __device__ u64 prune(int& cnt, int k) {
     __syncwarp();
     if (cnt <= 32) return prune_regs<1>(cnt, k);
@@ -2220,23 +2223,21 @@ struct KnnBuffer {
           clo = c;
         }
       }
-      while (hi - lo > 1 && chi != k) {  // ties: the end that moves goes on to a key
-        const int mid = lo + ((hi - lo) >> 1);
-        int c = 0, at = -1, above = INT_MAX;
+      while (hi - lo > 1 && chi != k) {  // ties: on to the next key, until k are covered
+        int next = INT_MAX, c = 0;
 #pragma unroll
-        for (int i = 0; i < R; ++i) {
-          c += d[i] <= mid;
-          at = max(at, d[i] <= mid ? d[i] : -1);
-          above = min(above, d[i] > mid ? d[i] : INT_MAX);
-        }
+        for (int i = 0; i < R; ++i) next = min(next, d[i] > lo ? d[i] : INT_MAX);
+        next = __reduce_min_sync(kWarp, next);
+#pragma unroll
+        for (int i = 0; i < R; ++i) c += d[i] <= next;
         c = __reduce_add_sync(kWarp, c);
         if (c >= k) {
-          hi = __reduce_max_sync(kWarp, at);
+          hi = next;
           chi = c;
-        } else {
-          lo = __reduce_min_sync(kWarp, above) - 1;
-          clo = c;
+          break;
         }
+        lo = next;
+        clo = c;
       }
       int tie = INT_MAX;  // of keys with d^2 == hi, indices up to this one
       if (chi != k) {     // more than k: the lowest k - clo indices among the ties

@@ -1,7 +1,8 @@
-"""The k-NN search by counts (calls without neighbour lists above the
-all-warps size, k > 16, evenly spread data) and its neighbours, against the list-returning searches of the same call and the
-FP64 oracle: k-th keys equal, values within the last bits, hits, ties, edges of
-the data, clusters, fewer points than k, queries outside the box."""
+"""The k-NN search by counts (calls without neighbour lists on evenly spread
+data: k > 32 above the all-warps size, k > 16 above 114,688 queries) and its
+neighbours, against the list-returning searches of the same call and the FP64
+oracle: k-th keys equal, values within the last bits, hits, ties, edges of the
+data, clusters, fewer points than k, queries outside the box."""
 import numpy as np
 import pytest
 
@@ -29,7 +30,7 @@ def _compare(data, queries, k, p=2.0):
 @pytest.mark.parametrize("k", [1, 16, 17, 31, 32, 33, 64])
 @pytest.mark.parametrize("n", [200, 5000, 60000])
 def test_uniform(n, k):
-    m = 8192 + 1024 * k + 1  # the smallest such call, ending inside a warp
+    m = 8192 + 1024 * k + 1  # threads' (counted if k > 32), ending inside a warp
     prob = synthetic.uniform_problem(n, m, seed=n + k, exact_hits=100)
     Z = _compare(prob["data"], prob["queries"], k)
     part = slice(0, None, 97)
@@ -129,3 +130,30 @@ def test_queries_beyond_the_edge_take_no_longer():
     q = torch.from_numpy(prob["queries"]).cuda() * 3.0 - 1.0
     counted = _fastest(lambda: idw.interpolate_knn(d, q, 2.0, 32))
     assert counted <= 3 * _fastest(lambda: idw.interpolate_knn(d, q, 2.0, 32, neighbours=True))
+
+
+def test_counted_ties():
+    """As test_ties, with k and m that are counted: bins overflow on the ties."""
+    xy = synthetic.grid_xy(64)
+    xy = np.concatenate([xy, xy])
+    data = synthetic.pack_xyz(xy, np.arange(len(xy), dtype=np.float32) / len(xy))
+    queries = np.tile(np.concatenate([xy[:4096], synthetic.grid_xy(32)]), (24, 1))
+    for k in (17, 30, 40):
+        _compare(data, queries.astype(np.float32), k)
+
+
+def test_counted_few_points_and_bad_queries():
+    prob = synthetic.uniform_problem(5, 120000, seed=2)
+    prob["queries"][7] = np.nan
+    prob["queries"][8, 0] = np.inf
+    for k in (17, 40):
+        Z = _compare(prob["data"], prob["queries"], k)
+        assert np.isnan(Z[7]) and np.isnan(Z[8]) and np.isfinite(Z[9:]).all()
+
+
+@pytest.mark.parametrize("scale", [1e-15, 1e-30, 1e15])
+def test_counted_scales(scale):
+    prob = synthetic.uniform_problem(3000, 120000, seed=4)
+    prob["data"][:, :2] *= np.float32(scale)
+    for k in (20, 40):
+        _compare(prob["data"], prob["queries"] * np.float32(scale), k)
