@@ -530,10 +530,10 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
 // The listed queries, in one launch of two steps.
 //
 // First the exact hits.  A work item is a group of up to 32 listed queries and
-// one of S equal slices of their problem's points, S chosen so that the items
-// fill the grid: every point is read once per group and compared with the
-// group's queries from shared memory, and the lowest coincident index is kept
-// with an atomic minimum.
+// one of S equal slices of their problem's points, S chosen so that few groups'
+// items fill the grid and many groups' do so twice: every point is read once per
+// group and compared with the group's queries from shared memory, and the lowest
+// coincident index is kept with an atomic minimum.
 //
 // Then the results: a hit's z, or Eq. 1 in FP64.  A query without a hit is one
 // whose FP32 sums left FP32's range; among them are the queries that shared a
@@ -553,6 +553,10 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
 // for the launches alone (p = 2 without hits, no list / two launches / this one:
 // 12,000 x 12,000 48.9 / 51.0 / 50.2 us, 20,000 x 20,000 109.9 / 112.2 / 111.3).
 constexpr int kSlowGroup = 32;
+// CTAs to an SM: the FP64 sums wait on divisions and loads, and more warps hide
+// them, although four CTAs leave 64 registers and spill 40 bytes (p = 2, 30,000 x
+// 20,000, 1% of the queries hits: two 701 us, three 659, four 518).
+constexpr int kSlowCtas = 4;
 // One item over all points of the largest problem (2^31) takes several seconds.
 constexpr unsigned long long kSlowWaitNs = 60000000000ull;
 
@@ -600,7 +604,7 @@ __device__ __forceinline__ SlowItem slow_item(const SlowList& slow, int64_t f) {
 }
 
 template <int CAP>
-__global__ void __launch_bounds__(kSlowThreads)
+__global__ void __launch_bounds__(kSlowThreads, kSlowCtas)
     slow_kernel(const __grid_constant__ Table<CAP> t, Control* ctrl, const SlowList slow, double p) {
   __shared__ SlowShared sh;
   // The kernels behind this one start only when it has gone this far: held back
@@ -613,7 +617,9 @@ __global__ void __launch_bounds__(kSlowThreads)
   const int tid = threadIdx.x;
 
   const int64_t groups = (count + kSlowGroup - 1) / kSlowGroup;
-  const int64_t cuts = max(int64_t(1), gridDim.x / groups), searches = groups * cuts;
+  const int64_t cuts = 4 * groups < gridDim.x ? gridDim.x / groups
+                                              : (2 * int64_t(gridDim.x) + groups - 1) / groups;
+  const int64_t searches = groups * cuts;
   for (;;) {
     __syncthreads();  // the previous item's group and number are no longer read
     if (tid == 0) sh.drawn = atomicAdd(&ctrl->slow_drawn, 1u);
@@ -1092,7 +1098,7 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
   const int64_t slots = plan.total_query_tiles * QT;
   // Each listed query takes an item and a slice record; the grid's worth of
   // records more covers short lists cut into more slices.
-  const int slow_grid = 2 * sm_count;
+  const int slow_grid = kSlowCtas * sm_count;
   SlowList slow;
   const size_t spare = size_t(slow_grid) * sizeof(SlowSums);
   slow.cap = static_cast<unsigned>(std::min<size_t>(
