@@ -1086,8 +1086,14 @@ cudaError_t launch_impl(const F32Problem* probs, const BatchPlan& plan, double p
   if (ev && (e = cudaEventRecord(ev->start, stream)) != cudaSuccess) return e;
   constexpr int NT = Var<V>::NT, QT = qt_of<V>();
   // With profiling events the sweep is launched plainly, so that the events
-  // around it bracket it alone.
-  if (ev)
+  // around it bracket it alone.  So is one whose CTAs take between one place an SM
+  // and three quarters of all: launched early, they are placed around the kernels
+  // in flight, whose waiting CTAs hold places, and stay there, several on one SM
+  // with others idle (early / plainly: p = 3, 100,003 x 100 55.4 / 38.0 us; p = 2.5,
+  // 13,000 x 5000 73.8 / 48.8, 500 x 60,000 45.9 / 39.3).  A grid that fills every
+  // place cannot be uneven, and loses the early start (12,000 x 12,000, p = 2.5:
+  // 72 / 75).
+  if (ev || (plan.grid > sm_count && 4 * plan.grid < 3 * sm_count * (512 / NT)))
     sweep_kernel<MODE, CAP, V, LAYOUT, FMA_LOG2><<<plan.grid, NT, smem, stream>>>(a, t);
   else if ((e = launch_pdl(sweep_kernel<MODE, CAP, V, LAYOUT, FMA_LOG2>, dim3(plan.grid),
                            dim3(NT), smem, stream, a, t)) != cudaSuccess)
