@@ -744,12 +744,20 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Up to 100 M pairs the launch still wins (10,000 x 10,000: 37 against 42, all
 // hits 85 against 279; 3000 x 30,000: 36.5 against 42); beyond, and past 256
 // clusters, the sweep's larger tiles do more per load (12,000 x 12,000: level;
-// 1000 x 60,000: 42 against 33.5; batches of 4e8 pairs and more 5-10% slower).  Batches: 8 problems of 256 to 2048 points and queries
-// 22.3 us, from 34.1 (on the device 12.4 from 22.8), 128 of 16 to 64 on the
-// device 14.3 from 37.  Above p = 4 sums leave the fast form's range at ordinary
-// distances, and the slow list spreads their FP64 sums better.
+// 1000 x 60,000: 42 against 33.5; batches of 4e8 pairs and more 5-10% slower).
+// A single problem at p = 2, whose sweep is the fastest, does not pay for a second
+// wave of clusters (the GPU holds about 150) with few points (one launch / sweep: 16
+// x 20,000 15.0 / 14.4 us, 16 x 32,000 20.9 / 16.1, 1000 x 28,000 21.3 / 20.0, 2000
+// x 24,000 24.6 / 29.0; at p = 3, 16 x 32,000 21.4 / 29.2).  The line lies above
+// where the times cross, for the host's time in the sweep's launches: 16 x
+// 20,481, calls from Python back to back, 15.6 / 21.0.  Batches: 8 problems
+// of 256 to 2048 points and queries 22.3 us, from 34.1 (on the device 12.4 from
+// 22.8), 128 of 16 to 64 on the device 14.3 from 37.  Above p = 4 sums leave the
+// fast form's range at ordinary distances, and the slow list spreads their FP64
+// sums better.
 constexpr int kSmallQueries = 128, kSmallCluster = 8, kSmallThreads = 256;
 constexpr int64_t kSmallPoints = 12288, kSmallClusters = 256, kSmallPairs = int64_t(100) << 20;
+constexpr int64_t kSmallClustersPow2 = 192, kSmallPointsPow2 = 1500;
 constexpr double kSmallPower = 4.0;
 constexpr int kSmallChunk = 16, kSmallSubs = kSmallThreads / (kSmallQueries / 2);
 constexpr int kSmallStep = kSmallSubs * kSmallChunk;  // a CTA's points are padded to these
@@ -971,13 +979,15 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(kSmallTh
 
 int64_t small_clusters(int64_t m) { return (m + kSmallQueries - 1) / kSmallQueries; }
 
-bool small_problems(const F32Problem* probs, int count, double p) {
+bool small_problems(const F32Problem* probs, int count, double p, bool pow2) {
   int64_t clusters = 0, pairs = 0;
   for (int k = 0; k < count; ++k) {
     if (probs[k].n > kSmallPoints || probs[k].m > kSmallPairs) return false;
     clusters += small_clusters(probs[k].m);
     pairs += probs[k].n * probs[k].m;
   }
+  if (pow2 && count == 1 && clusters > kSmallClustersPow2 && probs[0].n < kSmallPointsPow2)
+    return false;
   return p <= kSmallPower && clusters <= kSmallClusters && pairs <= kSmallPairs;
 }
 
@@ -1260,10 +1270,10 @@ cudaError_t launch_batch_f32(const F32Problem* probs, const BatchPlan& plan, dou
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   if (plan.count < 1 || plan.count > kBatchCap) return cudaErrorInvalidValue;
   const bool one = plan.count == 1;
-  if (plan.small_ok && !ev && small_problems(probs, plan.count, p))
+  const bool pow2 = (p == 2.0) && !plan.force_general;
+  if (plan.small_ok && !ev && small_problems(probs, plan.count, p, pow2))
     return one ? launch_small<1>(probs, 1, p, plan.force_general, stream)
                : launch_small<kBatchCap>(probs, plan.count, p, plan.force_general, stream);
-  const bool pow2 = (p == 2.0) && !plan.force_general;
   // Default staging layout per weight form (measured fastest on GB300): the
   // aligned AoS record at p = 2, whose one shared load per point leaves the
   // special-function queue to the reciprocals; duplicated pair records for

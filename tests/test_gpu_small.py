@@ -1,5 +1,6 @@
 """Problems and batches that take the one-launch path (n <= 12288, at most 256
-tiles of 128 queries, n m <= 100 2^20, p <= 4): parity with
+tiles of 128 queries, n m <= 100 2^20, p <= 4; at p = 2 not those of fewer than
+1500 points and more than 192 tiles): parity with
 the FP64 oracle at its edges (cluster slices, chunks, query tiles, the largest
 sizes), hits, FP64 recomputations, saved outputs, NaN and infinities, scales,
 and the sizes just outside it."""
@@ -37,6 +38,13 @@ def test_parity(p, n, m):
     S0 = ((d ** 2).sum(-1) ** (-0.5 * p)).sum(1)
     assert np.allclose(s0.cpu().numpy()[on], S0, rtol=2e-6, atol=0.0)
     assert np.isinf(s0.cpu().numpy()[~on]).all()
+
+
+@pytest.mark.parametrize("n,m", [(16, 24576), (16, 24577), (1499, 24577), (1500, 24577),
+                                 (1499, 32768)])
+def test_parity_of_a_second_wave(n, m):
+    """Both sides of the limits for a single problem at p = 2."""
+    test_parity(2.0, n, m)
 
 
 @pytest.mark.parametrize("p,scale", [(2.0, 2.0 ** -60), (2.0, 2.0 ** 60), (64.0, 1.0), (0.1, 1.0)])
