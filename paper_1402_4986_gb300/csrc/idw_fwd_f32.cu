@@ -408,10 +408,13 @@ __global__ void __launch_bounds__(Var<V>::NT, 512 / Var<V>::NT)
 // (lanes x) and splits each query's pieces over 8 warps (lanes y, strided);
 // every warp's loads are coalesced across its 32 queries, and the 8 partial
 // sums are added in a fixed order, so the result is deterministic.  The
-// CTA's flagged queries are then redone one after another by all 256
-// threads when their problem is small; a query's slow path reads all n
-// points, so those of a larger problem are listed for the kernel after
-// this one, which spreads each search over the GPU.  Block 0 finally clears
+// CTA's flagged queries are then redone by all 256 threads when their problem
+// is small or the list full: one scan of the points for all their hits, then the
+// FP64 sums of the others one after another.  A query's slow path reads all n
+// points, so those of a larger problem are listed for the kernel after this one,
+// which spreads each search over the GPU.  (A scan for each query took 6 us of
+// 12,000 points, and the CTAs that find the list full have 32 of them: 12,000 x
+// 12,000, p = 3.5, all hits 429 us, 206 so.)  Block 0 finally clears
 // the per-problem range words the range scan and staging of this call used,
 // so the next call (or graph replay) starts from zero without a memset.
 //
@@ -456,7 +459,10 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
   constexpr int kCombineQueries = kCombineThreads / kCombineLanes;
   __shared__ float4 red[kCombineLanes][kCombineQueries];
   __shared__ int2 flagged[kCombineQueries];
+  __shared__ float2 flagged_q[kCombineQueries];
+  __shared__ int hit[kCombineQueries];
   __shared__ int nflagged;
+  static_assert(QT % kCombineQueries == 0, "a CTA's queries are of one problem");
   pdl_trigger();
   pdl_wait();
   const int lx = threadIdx.x % kCombineQueries, ly = threadIdx.x / kCombineQueries;
@@ -502,10 +508,14 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
     if (!(s0 > kTinySumPerPoint * double(I.n)) || !isfinite(s0) || !isfinite(s1) ||
         (p >= 2.0 && s0 > kHugeSumPow2Up)) {
       const unsigned slot = I.n > kSlowInlinePoints ? atomicAdd(&ctrl->flagged, 1u) : slow.cap;
-      if (slot < slow.cap)
+      if (slot < slow.cap) {
         slow.item[slot] = SlowItem{k, static_cast<int32_t>(j), INT_MAX, 0u};
-      else
-        flagged[atomicAdd(&nflagged, 1)] = make_int2(k, static_cast<int>(j));
+      } else {
+        const int f = atomicAdd(&nflagged, 1);
+        flagged[f] = make_int2(k, static_cast<int>(j));
+        flagged_q[f] = make_float2(I.queries[2 * j], I.queries[2 * j + 1]);
+        hit[f] = INT_MAX;
+      }
     } else {
       I.out[j] = static_cast<float>(s1 / s0);
       // Weights were computed on coordinates scaled by s: w = s^-p w_true.
@@ -515,13 +525,26 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
   }
   __syncthreads();
   const int nf = nflagged;
-  for (int f = 0; f < nf; ++f) {  // uniform across the CTA
-    const int2 e = flagged[f];
-    const Instance& F = t.inst[e.x];
-    const int64_t jf = e.y;
-    slow_one_query<float, float>(F.data, F.n, F.queries[2 * jf], F.queries[2 * jf + 1], p,
-                                 &F.out[jf], F.s0_out ? &F.s0_out[jf] : nullptr,
-                                 F.hit_out ? &F.hit_out[jf] : nullptr);
+  if (nf > 0) {  // uniform across the CTA
+    const Instance& F = t.inst[flagged[0].x];
+    slow_scan(F.data, 0, F.n, [&](int64_t i, float x, float y) {
+      for (int f = 0; f < nf; ++f)
+        if (flagged_q[f].x == x && flagged_q[f].y == y) atomicMin(&hit[f], static_cast<int>(i));
+      return false;
+    });
+    __syncthreads();
+    for (int f = 0; f < nf; ++f) {
+      const int64_t jf = flagged[f].y;
+      float* out = &F.out[jf];
+      double* s0_out = F.s0_out ? &F.s0_out[jf] : nullptr;
+      int32_t* hit_out = F.hit_out ? &F.hit_out[jf] : nullptr;
+      if (hit[f] != INT_MAX) {
+        if (threadIdx.x == f) slow_write_hit(F.data, hit[f], out, s0_out, hit_out);
+        continue;
+      }
+      const SlowSums sums = slow_sums<float>(F.data, 0, F.n, flagged_q[f].x, flagged_q[f].y, p);
+      if (threadIdx.x == 0) slow_write_sums(sums, p, out, s0_out, hit_out);
+    }
   }
   if (blockIdx.x == 0)
     for (int c = threadIdx.x; c < t.count; c += blockDim.x) ctrl->maxbits[c] = 0u;
