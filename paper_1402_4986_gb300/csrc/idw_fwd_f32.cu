@@ -577,9 +577,12 @@ __global__ void __launch_bounds__(kCombineThreads, 6)
 // 12,000 x 12,000 48.9 / 51.0 / 50.2 us, 20,000 x 20,000 109.9 / 112.2 / 111.3).
 constexpr int kSlowGroup = 32;
 // CTAs to an SM: the FP64 sums wait on divisions and loads, and more warps hide
-// them, although four CTAs leave 64 registers and spill 40 bytes (p = 2, 30,000 x
-// 20,000, 1% of the queries hits: two 701 us, three 659, four 518).
-constexpr int kSlowCtas = 4;
+// them where the list is long; where it is short, more slices cost more than they
+// spread, and four CTAs leave 64 registers and spill.  Two / three / four, p = 2:
+// 30,000 x 20,000, all hits, 608 / 561 / 515 us; 100,003 x 4096 with one hit 140 /
+// 144 / 150, with 16 149 / 152 / 155, with 200 372 / 370 / 383; p = 3.5: 100,003 x
+// 65,537, 20% hits, 3376 / 3026 / 3036; 30,000 x 20,000 with 2000 287 / 274 / 274.
+constexpr int kSlowCtas = 3;
 // One item over all points of the largest problem (2^31) takes several seconds.
 constexpr unsigned long long kSlowWaitNs = 60000000000ull;
 

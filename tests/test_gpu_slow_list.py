@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
 def test_hits(n, m, p):
     """Every query on a data point, half of the points duplicated (the lowest
     index wins).  By default only 20,011 points and 20,000 queries on 8193 reach
-    the list, which the latter overflow (4886 records); the rest take the one
+    the list, which the latter overflow (4795 records); the rest take the one
     launch."""
     import torch
     import paper_1402_4986_gb300 as idw
@@ -89,3 +89,21 @@ def test_hits_among_others_of_a_sweep(hits, swept):
             Zc = Z.cpu().numpy()
             assert np.array_equal(Zc[on], Z64[on].astype(np.float32))
             assert np.max(np.abs(Zc - Z64)) <= 2e-6 * np.max(np.abs(prob["data"][:, 2]))
+
+
+@pytest.mark.parametrize("n,hits", [(300, 40), (2048, 40), (2048, 900), (2049, 2049), (8193, 8000)])
+def test_hits_among_others_kept_by_the_combine(n, hits, swept):
+    """As test_hits_among_others_of_a_sweep, where the combine's CTAs find the
+    hits and sum the others in FP64: small problems, and lists that overflow."""
+    import torch
+    import paper_1402_4986_gb300 as idw
+    prob = synthetic.uniform_problem(n, 20000, seed=n, exact_hits=hits)
+    Z64, hit64 = oracle.idw(prob["data"], prob["queries"], 2.0)
+    d, q = torch.from_numpy(prob["data"]).cuda(), torch.from_numpy(prob["queries"]).cuda()
+    with swept():
+        Z, _, hit = idw.interpolate_saved(d, q, 2.0)
+    Z, hit, on = Z.cpu().numpy(), hit.cpu().numpy(), hit64 >= 0
+    assert np.array_equal(hit[on], hit64[on])
+    assert not (hit[~on] >= 0).any()
+    assert np.array_equal(Z[on], Z64[on].astype(np.float32))
+    assert np.max(np.abs(Z - Z64)) <= 2e-6 * np.max(np.abs(prob["data"][:, 2]))
